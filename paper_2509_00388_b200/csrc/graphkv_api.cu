@@ -1157,9 +1157,11 @@ static bool decode_shape(const graphkv_params *p, DecodeArgs *a)
     if (p->q_stride[0] < 0 || p->q_stride[1] < kHeadDim) return false;
     a->batch = p->batch; a->hq = p->n_q_heads; a->hkv = p->n_kv_heads; a->G = p->n_q_heads / p->n_kv_heads;
     a->rows = p->seq_len;
+    a->blocks_per_unit = ceil_div(p->seq_len, p->dtype == GRAPHKV_BF16 ? dec_rows<__nv_bfloat16>() : dec_rows<float>());
+    // one CTA per SM, each an equal run of blocks
+    // as many CTAs per unit as one wave holds (one per SM), with kDecMinBlocks blocks each or more
     const int units = p->batch * p->n_kv_heads;
-    const int tiles = ceil_div(p->seq_len, kDecTile);
-    a->splits = std::max(1, std::min(std::min(tiles, 256), ceil_div(4 * sm_count(), units)));
+    a->splits = std::max(1, std::min(sm_count() / units, ceil_div(a->blocks_per_unit, kDecMinBlocks)));
     a->qs[0] = p->q_stride[0]; a->qs[1] = p->q_stride[1];
     for (int i = 0; i < 3; ++i) { a->ks[i] = p->k_stride[i]; a->vs[i] = p->v_stride[i]; }
     return true;
@@ -1169,7 +1171,24 @@ size_t graphkv_decode_workspace_bytes(const graphkv_params *params)
 {
     DecodeArgs a;
     if (!decode_shape(params, &a)) return 0;
-    return align_up((size_t)a.batch * a.hkv * a.splits * a.G * (2 + kHeadDim) * sizeof(float));
+    return align_up((size_t)a.batch * a.hkv * sizeof(unsigned long long)) +
+           align_up((size_t)a.batch * a.hkv * a.splits * a.G * kDecPart * sizeof(float));
+}
+
+extern "C++" {
+template <typename T, int kG>
+static graphkv_status launch_decode(const DecodeArgs &a, const void *q, const void *K, const void *V, cudaStream_t st)
+{
+    static std::mutex mu;
+    static signed char state[64] = {};
+    if (!once_per_device(mu, state, [] { return set_smem(decode_kernel<T, kG>, kDecSmem); }))
+        return GRAPHKV_ERR_CUDA;
+    // (the kernel waits for the launches before it as its first step, so it may always be launched early)
+    t_launches_in_call = 1;
+    return launch_ex("decode_attention", decode_kernel<T, kG>, dim3(a.splits, a.batch * a.hkv), dim3(kDecThreads), kDecSmem,
+                     st, next_launch_is_dependent(), 1, a, static_cast<const T *>(q), static_cast<const T *>(K),
+                     static_cast<const T *>(V));
+}
 }
 
 graphkv_status graphkv_decode_attention(const graphkv_params *params, const void *q, const void *K,
@@ -1181,20 +1200,14 @@ graphkv_status graphkv_decode_attention(const graphkv_params *params, const void
                                                                                   : GRAPHKV_ERR_INVALID_ARG;
     if (!q || !K || !V || !out || !aligned16(K) || !aligned16(V)) return GRAPHKV_ERR_INVALID_ARG;
     if (!workspace || workspace_bytes < graphkv_decode_workspace_bytes(params)) return GRAPHKV_ERR_WORKSPACE;
-    a.part = static_cast<float *>(workspace);
+    a.arrived = static_cast<unsigned long long *>(workspace);
+    a.part = at<float>(workspace, align_up((size_t)a.batch * a.hkv * sizeof(unsigned long long)));
     a.out = out;
+    a.call_tag = next_call_tag();
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const dim3 grid(a.splits, a.batch * a.hkv);
     if (params->dtype == GRAPHKV_BF16)
-        GKV_LAUNCH("decode_partial", st, (decode_partial_kernel<__nv_bfloat16><<<grid, kDecThreads, 0, st>>>(
-                                             a, static_cast<const __nv_bfloat16 *>(q), static_cast<const __nv_bfloat16 *>(K),
-                                             static_cast<const __nv_bfloat16 *>(V))));
-    else
-        GKV_LAUNCH("decode_partial", st, (decode_partial_kernel<float><<<grid, kDecThreads, 0, st>>>(
-                                             a, static_cast<const float *>(q), static_cast<const float *>(K),
-                                             static_cast<const float *>(V))));
-    GKV_LAUNCH("decode_merge", st, (decode_merge_kernel<<<a.batch * a.hkv * a.G, kHeadDim, 0, st>>>(a)));
-    return launch_status();
+        return a.G <= 4 ? launch_decode<__nv_bfloat16, 4>(a, q, K, V, st) : launch_decode<__nv_bfloat16, 8>(a, q, K, V, st);
+    return a.G <= 4 ? launch_decode<float, 4>(a, q, K, V, st) : launch_decode<float, 8>(a, q, K, V, st);
 }
 
 graphkv_status graphkv_read_status(const void *workspace, void *stream)

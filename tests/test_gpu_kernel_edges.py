@@ -1,0 +1,39 @@
+"""GPU kernels at the sizes where their tiling can go wrong, against the CPU oracle."""
+import pytest
+import torch
+
+from oracle import graphkv_oracle as okv
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def gk():
+    from paper_2509_00388_b200 import binding
+    binding.lib()
+    return binding
+
+
+# rows around a warp's block (16 bf16 or 8 fp32 rows), around one ring of all warps and around the
+# least share of a CTA; one CTA per unit (units above half the SMs) and many; 1 to 8 query heads
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rows,g,hkv,batch", [(1, 1, 1, 1), (7, 3, 2, 1), (17, 4, 1, 1), (97, 5, 2, 2), (191, 8, 1, 1),
+                                              (193, 4, 8, 10), (400, 2, 8, 19), (3073, 7, 3, 1)])
+def test_decode_attention_edges(gk, dtype, rows, g, hkv, batch):
+    gen = torch.Generator().manual_seed(rows)
+    q = (2 * torch.randn((batch, hkv * g, 128), generator=gen)).to(dtype)
+    # token-major buffers, reached through the strides
+    K, V = (torch.randn((batch, rows, hkv, 128), generator=gen).to(dtype).transpose(1, 2) for _ in range(2))
+    want = okv.decode_attention(q, K.contiguous(), V.contiguous())
+    qd, Kd, Vd = q.to(DEV), K.to(DEV), V.to(DEV)
+    assert Kd.stride() == K.stride()
+    p = gk.decode_params(qd, Kd, Vd)
+    ws = gk.decode_workspace(p, DEV)
+    ws.random_(256)                                  # whatever the workspace holds
+    out = torch.empty((batch, hkv * g, 128), dtype=torch.float32, device=DEV)
+    for _ in range(2):
+        out.fill_(float("nan"))
+        gk.graphkv_decode_attention(p, qd, Kd, Vd, out, ws)
+        err = (out.cpu().double() - torch.as_tensor(want).double()).norm() / torch.as_tensor(want).double().norm()
+        assert err <= 2e-6
