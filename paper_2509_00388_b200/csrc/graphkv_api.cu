@@ -44,7 +44,6 @@ struct Layout {
     size_t src_cand;    // elements the emit sweep lists for the source selection [units][max_parts][kSrcCap]
     size_t src_cnt;     // [units][max_parts]
     size_t total;
-    int n_stat_chunks;  // key chunks of the SIMT statistics sweep
     int max_parts;      // partial statistics per row the region can hold
 };
 
@@ -222,8 +221,7 @@ Layout layout_of(const Dims &d)
     Layout l;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
-    l.n_stat_chunks = ceil_div(d.L, kStatsChunk);
-    l.max_parts = l.n_stat_chunks > 148 ? l.n_stat_chunks : 148;
+    l.max_parts = std::max(148, ceil_div(d.L, 1024));
     l.status = take(kAlign);
     l.arrivals = take((size_t)d.units * 2 * sizeof(int));
     l.a_hist = take((size_t)d.units * tc::kMassBins * sizeof(uint32_t));
@@ -406,36 +404,40 @@ inline graphkv_status reset_words(const Dims &d, const Layout &l, void *ws, cuda
 
 // ---- step (I) ------------------------------------------------------------------------------
 // Attention mass before pooling, a [units][N], SIMT path (any dtype).
+template <typename T, int kD, int kRT>
+graphkv_status launch_mass_simt(const Dims &d, const Layout &l, const T *Q, const T *K, float *a, void *ws,
+                                cudaStream_t st)
+{
+    const size_t smem = simt_smem_bytes<kD>(kRT);
+    static std::mutex mu;
+    static signed char state[64] = {};
+    if (!once_per_device(mu, state, [smem] {
+            return set_smem(score_stats_simt<T, kD, kRT>, smem) && set_smem(score_emit_simt<T, kD, kRT>, smem);
+        }))
+        return GRAPHKV_ERR_CUDA;
+    float *part = at<float>(ws, l.part);
+    // one wave of two CTAs per SM (what the registers hold) over all units, whole tiles each
+    const int row_tiles = ceil_div(d.GW, kRT), room = 2 * sm_count();
+    auto ctas = [&](int keys, int per_tile) {
+        const int tiles = ceil_div(keys, kSimtKeys);
+        return std::max(1, std::min(tiles, room / (d.units * per_tile)));
+    };
+    const int chunks = std::min(ctas(d.L, row_tiles), l.max_parts);
+    const graphkv_status rc = launch_ex("score_stats_simt", score_stats_simt<T, kD, kRT>, dim3(chunks, d.units, row_tiles),
+                                        dim3(kSimtThreads), smem, st, next_launch_is_dependent(), 1, d, Q, K, part,
+                                        chunks, at<int>(ws, l.status));
+    if (rc != GRAPHKV_OK) return rc;
+    return launch_ex("score_emit_simt", score_emit_simt<T, kD, kRT>, dim3(ctas(d.N, 1), d.units), dim3(kSimtThreads),
+                     smem, st, next_launch_is_dependent(), 1, d, Q, K, static_cast<const float *>(part), chunks, a);
+}
+
 template <typename T>
 graphkv_status run_mass_simt(const Dims &d, const Layout &l, const T *Q, const T *K, float *a,
                              void *ws, cudaStream_t st)
 {
-    if (reset_words(d, l, ws, st) != GRAPHKV_OK) return GRAPHKV_ERR_CUDA;
-    float *part = at<float>(ws, l.part);
-    const int threads = ceil_div(d.GW, 32) * 32;
-    const size_t smem = ((size_t)d.GW * d.D + 2 * d.GW) * sizeof(float);
-    static std::mutex mu;
-    static signed char state[64] = {};
-    if (!once_per_device(mu, state, [] {
-            const size_t mx = ((size_t)kMaxRows * kHeadDim + 2 * kMaxRows) * sizeof(float);
-            return set_smem(score_emit_simt<T, 128>, mx) && set_smem(score_emit_simt<T, 64>, mx);
-        }))
-        return GRAPHKV_ERR_CUDA;
-    const dim3 grid_s(l.n_stat_chunks, d.units), grid_e(ceil_div(d.N, kEmitChunk), d.units);
-    if (d.D == 64) {
-        GKV_LAUNCH("score_stats_simt", st,
-                   (score_stats_simt<T, 64><<<grid_s, threads, 0, st>>>(d, Q, K, part, l.n_stat_chunks,
-                                                                        at<int>(ws, l.status))));
-        GKV_LAUNCH("score_emit_simt", st,
-                   (score_emit_simt<T, 64><<<grid_e, kEmitThreads, smem, st>>>(d, Q, K, part, l.n_stat_chunks, a)));
-    } else {
-        GKV_LAUNCH("score_stats_simt", st,
-                   (score_stats_simt<T, 128><<<grid_s, threads, 0, st>>>(d, Q, K, part, l.n_stat_chunks,
-                                                                         at<int>(ws, l.status))));
-        GKV_LAUNCH("score_emit_simt", st,
-                   (score_emit_simt<T, 128><<<grid_e, kEmitThreads, smem, st>>>(d, Q, K, part, l.n_stat_chunks, a)));
-    }
-    return launch_status();
+    if (d.GW <= 32)
+        return d.D == 64 ? launch_mass_simt<T, 64, 32>(d, l, Q, K, a, ws, st) : launch_mass_simt<T, 128, 32>(d, l, Q, K, a, ws, st);
+    return d.D == 64 ? launch_mass_simt<T, 64, 64>(d, l, Q, K, a, ws, st) : launch_mass_simt<T, 128, 64>(d, l, Q, K, a, ws, st);
 }
 
 // ---- step (I), tensor-core path (bf16) -----------------------------------------------------------
@@ -694,18 +696,16 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
         return GRAPHKV_OK;
     }
     float *sims = at<float>(ws, l.sims);
-    const dim3 grid_sim(ceil_div(d.N, kSimChunk), d.units);
+    const dim3 grid_sim(ceil_div(d.N, kSimtKeys), d.units);
     const Strides3 st_s{{eo.ss[0], eo.ss[1], eo.ss[2]}}, st_a{{eo.as[0], eo.as[1], eo.as[2]}};
-    if (d.D == 64)
-        GKV_LAUNCH("similarity_simt", st,
-                   (similarity_simt<T, 64><<<grid_sim, kSimThreads, 0, st>>>(d, eo.S, st_s, eo.A, st_a, src, sims)));
-    else
-        GKV_LAUNCH("similarity_simt", st,
-                   (similarity_simt<T, 128><<<grid_sim, kSimThreads, 0, st>>>(d, eo.S, st_s, eo.A, st_a, src, sims)));
+    const auto sim = d.D == 64 ? similarity_simt<T, 64> : similarity_simt<T, 128>;
+    const size_t smem = d.D == 64 ? sim_simt_smem_bytes<64>() : sim_simt_smem_bytes<128>();
+    const graphkv_status rc = launch_ex("similarity_simt", sim, grid_sim, dim3(kSimtThreads), smem, st,
+                                        next_launch_is_dependent(), 1, d, eo.S, st_s, eo.A, st_a, src, sims);
+    if (rc != GRAPHKV_OK) return rc;
     SelectArgs na{sims, d.N, d.N, d.m, src, at<int>(ws, l.nbr_idx), at<float>(ws, l.nbr_e)};
-    GKV_LAUNCH("select_neighbors", st,
-               (topk_select_kernel<<<d.units * d.K_src, kSelectThreads, 0, st>>>(na)));
-    return launch_status();
+    return launch_ex("select_neighbors", topk_select_kernel, dim3(d.units * d.K_src), dim3(kSelectThreads), 0, st,
+                     next_launch_is_dependent(), 1, na);
 }
 
 // Decay rounds (when has_graph) on s in place, then (when do_select) the budget selection and

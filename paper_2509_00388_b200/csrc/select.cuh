@@ -55,6 +55,8 @@ __global__ void __launch_bounds__(kSelectThreads) topk_select_kernel(SelectArgs 
     __shared__ uint32_t hist[256];
     __shared__ uint32_t warp_tot[33];
     __shared__ uint32_t s_bin, s_remaining;
+    pdl_wait();
+    pdl_launch_dependents();
     const int row = blockIdx.x;
     const float *x = a.x + (long long)row * a.row_stride;
     const int skip = a.skip ? a.skip[row] : -1;

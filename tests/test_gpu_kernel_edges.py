@@ -3,6 +3,8 @@ import pytest
 import torch
 
 from oracle import graphkv_oracle as okv
+from paper_2509_00388_b200 import workloads as wl
+from tests.test_gpu_parity import check
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -37,3 +39,13 @@ def test_decode_attention_edges(gk, dtype, rows, g, hkv, batch):
         gk.graphkv_decode_attention(p, qd, Kd, Vd, out, ws)
         err = (out.cpu().double() - torch.as_tensor(want).double()).norm() / torch.as_tensor(want).double().norm()
         assert err <= 2e-6
+
+
+# the register-tiled fp32 sweeps: query rows around the row tiles (32, 64), keys around the 64-key
+# tiles, sources around the 16 of a pass
+@pytest.mark.parametrize("n,w,g,k,head_dim", [(31, 1, 1, 3, 128), (63, 32, 1, 16, 64), (64, 33, 1, 17, 128),
+                                              (129, 16, 4, 33, 128), (191, 13, 5, 1, 64), (1000, 64, 4, 40, 128)])
+def test_fp32_sweeps_edges(gk, n, w, g, k, head_dim):
+    cfg = wl.scaled(wl.TINY, n_prefix=n, window=w, n_q_heads=3 * g, n_kv_heads=3, head_dim=head_dim, topk_nodes=k,
+                    neighbors=min(n - 1, 5), budget=min(n, 20), batch=2)
+    check(gk, cfg, strict_overlap=False)
