@@ -67,7 +67,7 @@ typedef struct {
     int32_t batch;        /* independent sequences (or any independent units sharing the shape)  */
     int32_t n_q_heads;
     int32_t n_kv_heads;   /* must divide n_q_heads                                               */
-    int32_t head_dim;     /* D: 128, or 64 (served by the general kernels, not the tensor cores) */
+    int32_t head_dim;     /* D: 128 or 64                                                        */
     int32_t seq_len;      /* L = N + W rows present in K and V                                   */
     int32_t window;       /* W >= 1 observation-window rows: queried from, always kept           */
     int32_t budget;       /* B = k_l: prefix tokens kept, 1 <= B <= N; outputs hold B + W rows   */

@@ -31,7 +31,7 @@ struct Layout {
     size_t status;      // int status word (256 bytes reserved)
     size_t arrivals;    // counters of score CTAs per unit [2 * units] (directly after the status word)
     size_t a_hist;      // histogram of the attention mass [units][2048] (directly after the counters)
-    size_t row_c;       // softmax row constants [units][GW]
+    size_t row_c;       // softmax row constants [units][2][GW]
     size_t part;        // softmax row statistics per key chunk
     size_t a;           // attention mass before pooling [units][N]
     size_t s;           // scores when the caller gives no array [units][N]
@@ -196,7 +196,7 @@ struct SimPlan {
 SimPlan sim_plan(const Dims &d, bool bf16)
 {
     SimPlan p{false, 16, 1, ceil_div(d.N, tc::kTileKeys), 5};
-    if (!bf16 || d.D != kHeadDim || d.K_src < 1 || d.K_src > kSimMaxSources || d.m < 1 ||
+    if (!bf16 || d.K_src < 1 || d.K_src > kSimMaxSources || d.m < 1 ||
         d.m > tc::kSimMaxNeighbors)
         return p;
     if (env_int("GRAPHKV_FORCE_SIMT", 0)) return p;
@@ -208,7 +208,7 @@ SimPlan sim_plan(const Dims &d, bool bf16)
     // 32 sources per sweep (16 tiles, eight keys per thread) stay clear of it and measured faster
     // there at every source count, 64 faster for m = 16.
     p.NP = d.K_src <= 16 ? 16 : (d.K_src <= 32 || d.m > 16 ? 32 : 64);
-    p.stages = p.NP == 64 ? 4 : 5;
+    p.stages = d.D == 64 ? 8 : p.NP == 64 ? 4 : 5;      // (at least 80 KB: the queues take the ring's place after the sweep)
     const int cap = 512 / p.NP;
     const int group = units_per_group(d);
     p.chunks = sweep_chunks(group, p.n_tiles, ceil_div(p.n_tiles, cap), 1 << 20);
@@ -225,7 +225,7 @@ Layout layout_of(const Dims &d)
     l.status = take(kAlign);
     l.arrivals = take((size_t)d.units * 2 * sizeof(int));
     l.a_hist = take((size_t)d.units * tc::kMassBins * sizeof(uint32_t));
-    l.row_c = take((size_t)d.units * d.GW * sizeof(float));
+    l.row_c = take((size_t)d.units * d.GW * 2 * sizeof(float));
     l.part = take((size_t)d.units * l.max_parts * d.GW * 2 * sizeof(float));
     l.a = take((size_t)d.units * d.N * sizeof(float));
     l.s = take((size_t)d.units * d.N * sizeof(float));
@@ -460,7 +460,7 @@ EncodeTiledFn encode_tiled_fn()
     return fn;
 }
 
-// Tensor map over K [batch][hkv][rows][128] bf16 with the caller's strides; boxes of 128 rows x 64
+// Tensor map over K [batch][hkv][rows][D] bf16 with the caller's strides; boxes of 128 rows x 64
 // columns, 128-byte swizzle, zero fill past the last row.
 bool make_k_tensormap(CUtensorMap *tm, const void *K, const Dims &d, int rows, const long long *ks = nullptr)
 {
@@ -468,7 +468,7 @@ bool make_k_tensormap(CUtensorMap *tm, const void *K, const Dims &d, int rows, c
     if (!enc) return false;
     if (!ks) ks = d.ks;
     const cuuint64_t row_b = (cuuint64_t)ks[2] * 2;
-    cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)rows, (cuuint64_t)d.hkv, (cuuint64_t)d.batch};
+    cuuint64_t dims[4] = {(cuuint64_t)d.D, (cuuint64_t)rows, (cuuint64_t)d.hkv, (cuuint64_t)d.batch};
     cuuint64_t head_b = (cuuint64_t)ks[1] * 2, batch_b = (cuuint64_t)ks[0] * 2;
     if (d.hkv == 1 || head_b == 0) head_b = row_b * (cuuint64_t)rows;
     if (d.batch == 1 || batch_b == 0) batch_b = head_b * (cuuint64_t)d.hkv;
@@ -494,6 +494,7 @@ struct EmitExtras {
 };
 
 // Attention mass before pooling, a [units][N], tensor-core path (bf16).
+template <int kD>
 graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *Q,
                            const __nv_bfloat16 *K, float *a, void *ws, cudaStream_t st,
                            const EmitExtras &ex)
@@ -503,14 +504,14 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     const int row_tiles = d.GW <= 128 ? 1 : 2;
     const int rows_pad = 128 * row_tiles;
     const int stages = row_tiles == 1 ? 5 : 4;
-    const size_t smem = tc::score_smem_bytes(rows_pad, stages);
+    const size_t smem = tc::score_smem_bytes<kD>(rows_pad, stages);
     static std::mutex mu;
     static signed char state[64] = {};
     if (!once_per_device(mu, state, [] {
-        const size_t mx = std::max(tc::score_smem_bytes(256, 4), tc::score_smem_bytes(128, 5));
-        return set_smem(tc::score_stats_tc<1>, mx) && set_smem(tc::score_stats_tc<2>, mx) &&
-                  set_smem(tc::score_emit_tc<1>, mx) && set_smem(tc::score_emit_tc<2>, mx) &&
-                  set_smem(tc::score_fused_tc<1>, mx) && set_smem(tc::score_fused_tc<2>, mx);
+        const size_t mx = std::max(tc::score_smem_bytes<kD>(256, 4), tc::score_smem_bytes<kD>(128, 5));
+        return set_smem(tc::score_stats_tc<1, kD>, mx) && set_smem(tc::score_stats_tc<2, kD>, mx) &&
+                  set_smem(tc::score_emit_tc<1, kD>, mx) && set_smem(tc::score_emit_tc<2, kD>, mx) &&
+                  set_smem(tc::score_fused_tc<1, kD>, mx) && set_smem(tc::score_fused_tc<2, kD>, mx);
         }))
         return GRAPHKV_ERR_CUDA;
     const int tiles_stats = ceil_div(d.L, tc::kTileKeys), tiles_emit = ceil_div(d.N, tc::kTileKeys);
@@ -552,7 +553,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
             fa.call_tag = next_call_tag();
             fa.wait_prior = next_launch_is_dependent();
             t_cooperative = true;
-            rc = launch_ex("score_fused_tc", row_tiles == 1 ? tc::score_fused_tc<1> : tc::score_fused_tc<2>,
+            rc = launch_ex("score_fused_tc", row_tiles == 1 ? tc::score_fused_tc<1, kD> : tc::score_fused_tc<2, kD>,
                            dim3(chunks_s, nu), dim3(tc::kScoreThreads), smem, st, fa.wait_prior != 0, 1, tmK, fa);
             if (rc == GRAPHKV_OK) continue;
             cudaGetLastError();
@@ -560,11 +561,11 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
             rc = GRAPHKV_OK;
         }
         sa.wait_prior = next_launch_is_dependent();
-        rc = launch_ex("score_stats_tc", row_tiles == 1 ? tc::score_stats_tc<1> : tc::score_stats_tc<2>,
+        rc = launch_ex("score_stats_tc", row_tiles == 1 ? tc::score_stats_tc<1, kD> : tc::score_stats_tc<2, kD>,
                        dim3(chunks_s, nu), dim3(tc::kScoreThreads), smem, st, sa.wait_prior != 0, 1, tmK, sa);
         if (rc != GRAPHKV_OK) break;
         ea.wait_prior = next_launch_is_dependent();
-        rc = launch_ex("score_emit_tc", row_tiles == 1 ? tc::score_emit_tc<1> : tc::score_emit_tc<2>,
+        rc = launch_ex("score_emit_tc", row_tiles == 1 ? tc::score_emit_tc<1, kD> : tc::score_emit_tc<2, kD>,
                        dim3(chunks_e, nu), dim3(tc::kScoreThreads), smem, st, ea.wait_prior != 0, 1, tmK, ea);
     }
     return rc;
@@ -572,7 +573,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
 
 constexpr EmitExtras kPlainEmit{0, nullptr, nullptr, nullptr, 0, true};
 
-inline bool tc_mass(const __nv_bfloat16 *, const Dims &d) { return d.D == kHeadDim && !env_int("GRAPHKV_FORCE_SIMT", 0); }
+inline bool tc_mass(const __nv_bfloat16 *, const Dims &d) { (void)d; return !env_int("GRAPHKV_FORCE_SIMT", 0); }
 inline bool tc_mass(const float *, const Dims &) { return false; }
 
 inline graphkv_status run_mass(const Dims &d, const Layout &l, const __nv_bfloat16 *Q,
@@ -580,7 +581,7 @@ inline graphkv_status run_mass(const Dims &d, const Layout &l, const __nv_bfloat
                                const EmitExtras &ex = kPlainEmit)
 {
     if (!tc_mass(Q, d)) return run_mass_simt(d, l, Q, K, a, ws, st);
-    return run_mass_tc(d, l, Q, K, a, ws, st, ex);
+    return d.D == 64 ? run_mass_tc<64>(d, l, Q, K, a, ws, st, ex) : run_mass_tc<kHeadDim>(d, l, Q, K, a, ws, st, ex);
 }
 inline graphkv_status run_mass(const Dims &d, const Layout &l, const float *Q, const float *K,
                                float *a, void *ws, cudaStream_t st, const EmitExtras & = kPlainEmit)
@@ -653,6 +654,17 @@ template <typename T> struct EdgeOperands {
     const long long *as;
 };
 
+template <int NP, int kD>
+graphkv_status launch_similarity(const CUtensorMap &tmK, const tc::SimTcArgs &sa, dim3 grid, dim3 block, cudaStream_t st)
+{
+    static std::mutex mu;
+    static signed char state[64] = {};
+    if (!once_per_device(mu, state, [] { return set_smem(tc::similarity_tc<NP, kD>, tc::sim_smem_bytes<NP, kD>(kD == 64 ? 8 : NP == 64 ? 4 : 5)); }))
+        return GRAPHKV_ERR_CUDA;
+    return launch_ex("similarity_tc", tc::similarity_tc<NP, kD>, grid, block, tc::sim_smem_bytes<NP, kD>(sa.stages), st,
+                     sa.wait_prior != 0, 1, tmK, sa);
+}
+
 // `merge` (optional): the sources are still candidate lists the emit sweep left; the similarity
 // sweep merges them (tensor-core path, one sweep of at most 64 sources).
 template <typename T>
@@ -663,14 +675,6 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
     if (sp.ok) {
         CUtensorMap tmK;
         if (!make_k_tensormap(&tmK, eo.A, d, d.L, eo.as)) return GRAPHKV_ERR_CUDA;
-        static std::mutex mu;
-        static signed char state[64] = {};
-        if (!once_per_device(mu, state, [] {
-            return set_smem(tc::similarity_tc<16>, tc::sim_smem_bytes<16>(5)) &&
-                      set_smem(tc::similarity_tc<32>, tc::sim_smem_bytes<32>(5)) &&
-                      set_smem(tc::similarity_tc<64>, tc::sim_smem_bytes<64>(4));
-            }))
-            return GRAPHKV_ERR_CUDA;
         const int group = units_per_group(d);
         for (int u0 = 0; u0 < d.units; u0 += group) {
             const int nu = std::min(group, d.units - u0);
@@ -681,16 +685,11 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
                              merge ? *merge : tc::SourceArgs{0, 0, nullptr, nullptr, nullptr, 0, 0}, a_mass};
             sa.wait_prior = next_launch_is_dependent();
             const dim3 grid(sp.chunks, nu, ceil_div(d.K_src, sp.NP)), block(tc::kSimThreads);
-            graphkv_status rc;
-            if (sp.NP == 16)
-                rc = launch_ex("similarity_tc", tc::similarity_tc<16>, grid, block,
-                               tc::sim_smem_bytes<16>(sp.stages), st, sa.wait_prior != 0, 1, tmK, sa);
-            else if (sp.NP == 32)
-                rc = launch_ex("similarity_tc", tc::similarity_tc<32>, grid, block,
-                               tc::sim_smem_bytes<32>(sp.stages), st, sa.wait_prior != 0, 1, tmK, sa);
-            else
-                rc = launch_ex("similarity_tc", tc::similarity_tc<64>, grid, block,
-                               tc::sim_smem_bytes<64>(sp.stages), st, sa.wait_prior != 0, 1, tmK, sa);
+            const auto launch = d.D == 64 ? (sp.NP == 16 ? launch_similarity<16, 64> : sp.NP == 32 ? launch_similarity<32, 64>
+                                                                                                  : launch_similarity<64, 64>)
+                                          : (sp.NP == 16 ? launch_similarity<16, 128> : sp.NP == 32 ? launch_similarity<32, 128>
+                                                                                                   : launch_similarity<64, 128>);
+            const graphkv_status rc = launch(tmK, sa, grid, block, st);
             if (rc != GRAPHKV_OK) return rc;
         }
         return GRAPHKV_OK;
@@ -848,7 +847,7 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
     // (one sweep of at most 64 sources, one launch group, max pooling).  Measured on B200 the
     // merge in front of every similarity CTA costs what the pooling kernel takes (32K keys: 114
     // against 112 us per step; 131072 x 4: 1.25 against 1.13 ms), so it is off by default.
-    const bool tail_src = tc_mass(Q, d) && tc_graph && d.K_src <= tc::kSrcMaxK && !d.pool_avg &&
+    const bool tail_src = tc_mass(Q, d) && tc_graph && d.D == kHeadDim && d.K_src <= tc::kSrcMaxK && !d.pool_avg &&
                           units_per_group(d) >= d.units && env_int("GRAPHKV_TAIL_SOURCES", 0);
     const bool finish_pools = d.kp > 1 && !d.pool_avg && (tail_src || !graph) && finish_plan(d, halo).ok &&
                               cluster_plan(d).ok;

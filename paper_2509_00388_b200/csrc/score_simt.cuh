@@ -1,7 +1,6 @@
 // Step (I), SIMT fp32 path: SnapKV-style window-attention scores for any input dtype.
-// Used for fp32 inputs and for a head dimension of 64 (the tensor-core path takes bf16 and 128
-// only); kD = 64 or 128.  Two sweeps over the keys of a
-// head: (1) per-row softmax statistics, (2) the column sums of the normalised probabilities.
+// Used for fp32 inputs (the tensor-core path takes bf16 only); kD = 64 or 128.  Two sweeps over the
+// keys of a head: (1) per-row softmax statistics, (2) the column sums of the normalised probabilities.
 //
 // Bound: the FMA pipe (G*W*D multiply-adds per key and sweep, about 123 per clock and SM).  Both
 // sweeps are a register-tiled product: tiles of 64 keys in shared memory, 64 (or 32) query rows at a

@@ -1,4 +1,4 @@
-// Step (I) on the tensor cores (bf16 inputs): SnapKV-style window-attention scores.
+// Step (I) on the tensor cores (bf16 inputs, head dimension 128 or 64): SnapKV-style window-attention scores.
 //
 // Two sweeps over the keys of a head, both as TMA -> shared memory -> tcgen05.mma -> TMEM
 // pipelines with the softmax arithmetic done on the accumulators as they come out of TMEM:
@@ -30,13 +30,14 @@ namespace tc {
 constexpr int kScoreThreads = 576;       // producer warp, MMA warp, 16 epilogue warps
 constexpr int kMassBins = 2048;         // histogram of the attention mass: top 11 bits of float_to_key
 constexpr int kEpiWarps = 16;
-constexpr int kScratchBytes = 10240;     // row constants (1 KB) + four exchange buffers of 4 x 128 floats
+constexpr int kScratchBytes = 11264;     // row constants and weights (2 KB) + exchange buffers of 16 x 128 floats
 
 struct ScoreTcArgs {
     Dims d;
     const __nv_bfloat16 *Q;
     float *part;        // [units][stats_chunks][GW][2] row statistics (max, sum) per key chunk
-    float *row_c;       // [units][GW] c_r = max_r + log2(Z_r), written by the last stats CTA of a unit
+    float *row_c;       // [units][2][GW] c_r = max_r + log2(Z_r) (D = 64: max_r, then 1 / Z_r), written by the last
+                        // stats CTA of a unit
     int *arrivals;      // [2 * units] words: the two-kernel path counts finished statistics CTAs in [unit]
                         // (zero before the launch; reset on the way), the kernel of both sweeps keeps a
                         // 64-bit (tag, count) word per unit there
@@ -64,11 +65,20 @@ struct ScoreTcArgs {
                              // both sweeps): no CTA announces itself at the hand-over, so that wait runs out
 };
 
+// Of every four pairs of exponentials, how many the FMA pipe takes: one at D = 128.  At D = 64 the
+// sweep needs none (half the bytes per key, as many exponentials: MUFU and HBM are about even at 128
+// rows), and its probabilities are 2^(l2 - max_r) * (1 / Z_r) instead of 2^(l2 - c_r), which keeps
+// the rounding of c_r out of them.  (Eight heads of 8191 keys at D = 64, whole path: 166 us on the fp32
+// sweeps, 59 us here.)
+template <int kD> __host__ __device__ constexpr int poly_pairs() { return kD == 128 ? 1 : 0; }
+template <int kD> __host__ __device__ constexpr bool weighted() { return kD == 64; }
+
 struct ScoreSmem {
     uint32_t q, stage0, full0, empty0, tfull0, tempty0, tmem_slot, xbar0, misc;
 };
 
 // Carve dynamic shared memory (1024-byte aligned base): Q operand, K stages, barriers.
+template <int kD>
 __device__ __forceinline__ ScoreSmem score_smem_layout(uint8_t *raw, int rows_pad, int stages,
                                                        uint8_t **gen_base)
 {
@@ -76,8 +86,8 @@ __device__ __forceinline__ ScoreSmem score_smem_layout(uint8_t *raw, int rows_pa
     *gen_base = raw + (base - smem_u32(raw));
     ScoreSmem s;
     s.q = base;
-    s.stage0 = s.q + rows_pad * 256;
-    s.full0 = s.stage0 + stages * kTileBytes;
+    s.stage0 = s.q + rows_pad * 2 * kD;
+    s.full0 = s.stage0 + stages * tile_bytes<kD>();
     s.empty0 = s.full0 + 8 * 8;
     s.tfull0 = s.empty0 + 8 * 8;
     s.tempty0 = s.tfull0 + 4 * 8;
@@ -87,27 +97,29 @@ __device__ __forceinline__ ScoreSmem score_smem_layout(uint8_t *raw, int rows_pa
     return s;
 }
 
-__host__ __device__ inline size_t score_smem_bytes(int rows_pad, int stages)
+template <int kD> __host__ __device__ inline size_t score_smem_bytes(int rows_pad, int stages)
 {
-    return 1024 + (size_t)rows_pad * 256 + (size_t)stages * kTileBytes + 8 * 8 * 2 + 4 * 8 * 2 + 16 + 8 * 8 +
+    return 1024 + (size_t)rows_pad * 2 * kD + (size_t)stages * tile_bytes<kD>() + 8 * 8 * 2 + 4 * 8 * 2 + 16 + 8 * 8 +
            kScratchBytes + 8192 + 64;   // scratch: the CTA's row statistics / row constants and the
                                         // exchange buffers; 8 KB: the emit sweep's histogram of the mass
 }
 
 // Q rows of the unit -> K-major swizzled operand (rows >= GW zero-filled).  Threads tid of
 // nthreads; loads are issued four at a time ahead of the shared-memory stores.
+template <int kD>
 __device__ __forceinline__ void stage_q(uint8_t *q_gen, int rows_pad, const Dims &d,
                                         const __nv_bfloat16 *Q, int b, int h, int tid, int nthreads)
 {
+    constexpr int kPieces = kD / 8;                  // 16-byte pieces of a row
     const __nv_bfloat16 *Qh = Q + b * d.qs[0] + (long long)(h * d.G) * d.qs[1];
-    for (int i0 = tid; i0 < rows_pad * 16; i0 += 4 * nthreads) {
+    for (int i0 = tid; i0 < rows_pad * kPieces; i0 += 4 * nthreads) {
         uint4 v[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * nthreads;
-            const int r = i >> 4, c16 = i & 15;
+            const int r = i / kPieces, c16 = i % kPieces;
             v[k] = make_uint4(0, 0, 0, 0);
-            if (i < rows_pad * 16 && r < d.GW) {
+            if (i < rows_pad * kPieces && r < d.GW) {
                 const int g = r / d.W, rw = r - g * d.W;
                 v[k] = *reinterpret_cast<const uint4 *>(Qh + g * d.qs[1] + rw * d.qs[2] + c16 * 8);
             }
@@ -115,8 +127,8 @@ __device__ __forceinline__ void stage_q(uint8_t *q_gen, int rows_pad, const Dims
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * nthreads;
-            if (i < rows_pad * 16)
-                *reinterpret_cast<uint4 *>(q_gen + sw128_offset(rows_pad, i >> 4, i & 15)) = v[k];
+            if (i < rows_pad * kPieces)
+                *reinterpret_cast<uint4 *>(q_gen + sw128_offset(rows_pad, i / kPieces, i % kPieces)) = v[k];
         }
     }
 }
@@ -151,6 +163,7 @@ __device__ __forceinline__ uint32_t score_setup(const ScoreSmem &s, uint8_t *gen
 
 // TMA producer (one thread): key tiles t0+i of (h, b), i in [i_begin, i_end), into the stage ring.
 // The keys are an input of the call, so the producer never waits for the kernels before.
+template <int kD>
 __device__ __forceinline__ bool score_produce(const ScoreSmem &s, const CUtensorMap *tmK, int stages,
                                               int t0, int i_begin, int i_end, int h, int b, long long lim)
 {
@@ -159,10 +172,7 @@ __device__ __forceinline__ bool score_produce(const ScoreSmem &s, const CUtensor
     for (int i = i_begin; i < i_end; ++i) {
         const int st = i % stages, ph = (i / stages) & 1;
         if (!mbar_wait(s.empty0 + 8 * st, ph ^ 1, lim)) { ok = false; break; }
-        const uint32_t dst = s.stage0 + st * kTileBytes;
-        mbar_expect_tx(s.full0 + 8 * st, kTileBytes);
-        tma_load_4d(dst, tmK, s.full0 + 8 * st, 0, (t0 + i) * kTileKeys, h, b);
-        tma_load_4d(dst + kHalfBytes, tmK, s.full0 + 8 * st, 64, (t0 + i) * kTileKeys, h, b);
+        tma_load_tile<kD>(s.stage0 + st * tile_bytes<kD>(), tmK, s.full0 + 8 * st, (t0 + i) * kTileKeys, h, b);
         ++issued;
     }
     if (!ok)        // gave up: let the copies already in flight land before the CTA exits
@@ -179,6 +189,7 @@ __device__ __forceinline__ void tile_range(int n_tiles, int chunks, int chunk, i
 }
 
 // One x32 slice of a row's accumulator: fold into the running (max, sum).
+template <int kD>
 __device__ __forceinline__ void stats_fold(float (&v)[32], float scale, float &mx, float &z)
 {
     float cm = fmaxf(v[0], v[1]);
@@ -188,7 +199,8 @@ __device__ __forceinline__ void stats_fold(float (&v)[32], float scale, float &m
     z *= ex2(mx - mn);
     mx = mn;
     const uint64_t nm = pack2(-mn, -mn);
-    z += ex2_sum32(v, pack2(scale, scale), [&](int) { return make_ulonglong2(nm, nm); });
+    const auto neg = [&](int) { return make_ulonglong2(nm, nm); };
+    z += ex2_sum32<poly_pairs<kD>(), false>(v, pack2(scale, scale), neg, neg);
 }
 
 // (max, sum) of a row over the partials of all key chunks of a unit: kTpr consecutive threads of a
@@ -225,7 +237,7 @@ __device__ __forceinline__ float2 merge_row_partials(const float2 *pu, int chunk
 }
 
 // kRowTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid (chunks, units of the launch).
-template <int kRowTiles>
+template <int kRowTiles, int kD>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 {
@@ -242,7 +254,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const Dims &d = a.d;
     const long long lim = a.wait_cycles;
     uint8_t *gen;
-    const ScoreSmem s = score_smem_layout(smem_raw, kRowsPad, a.stages, &gen);
+    const ScoreSmem s = score_smem_layout<kD>(smem_raw, kRowsPad, a.stages, &gen);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x;
@@ -258,9 +270,9 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kGroups);
     bool ok = true;
     if (warp == 0) {
-        if (lane == 0) ok = score_produce(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
+        if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
     } else {
-        stage_q(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
+        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
         fence_proxy_async();
     }
     pc.mark();
@@ -271,7 +283,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     pc.mark();
 
     if (warp == 0) {
-        if (lane == 0 && ok) ok = score_produce(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim);
+        if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim);
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
@@ -281,11 +293,11 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                 if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
                 if (!mbar_wait(s.full0 + 8 * st, ph, lim)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t kt = s.stage0 + st * kTileBytes;
+                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
 #pragma unroll
                 for (int rt = 0; rt < kRowTiles; ++rt) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
+                    for (int k = 0; k < kD / 16; ++k) {
                         const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
                         const uint32_t qoff = (k >> 2) * (kRowsPad * 128) + rt * (128 * 128) + (k & 3) * 32;
                         umma_bf16(tmem_base + buf * kBufCols + rt * 128, umma_desc_sw128(s.q + qoff),
@@ -304,7 +316,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         const int grp = set / (4 / kGroups);               // tiles grp, grp + kGroups, ...
         const int row = quad * 32 + lane;
         const int col0 = (set % (4 / kGroups)) * kSetCols, rt = col0 >> 7, key_off = col0 & 127;
-        const float scale = rsqrtf((float)kHeadDim) * kLog2e;
+        const float scale = rsqrtf((float)kD) * kLog2e;
         float mx = kNegBig, z = 0.f;
         const int r = rt * 128 + row;
         const int lim = d.N + (r < d.GW ? r % d.W : 0);      // last visible key of the row
@@ -337,7 +349,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                     for (int e = 0; e < 32; ++e)
                         if (key0 + c * 32 + e > lim) v[e] = -INFINITY;
                 }
-                stats_fold(v, scale, mx, z);
+                stats_fold<kD>(v, scale, mx, z);
             }
         }
         ok = alive;
@@ -381,7 +393,11 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         if (threadIdx.x < kRowsPad * kTpr) {
             const int r = threadIdx.x / kTpr, sub = threadIdx.x % kTpr;
             const float2 mz = merge_row_partials<kTpr>(pu, a.chunks, d.GW, r, sub);
-            if (sub == 0 && r < d.GW) a.row_c[(long long)unit * d.GW + r] = mz.x + log2f(mz.y);
+            if (sub == 0 && r < d.GW) {
+                float *c = a.row_c + (long long)unit * 2 * d.GW + r;
+                c[0] = weighted<kD>() ? mz.x : mz.x + log2f(mz.y);
+                if (weighted<kD>()) c[d.GW] = 1.0f / mz.y;
+            }
         }
         if (threadIdx.x == 0) a.arrivals[unit] = 0;      // ready for the next launch
     }
@@ -390,7 +406,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 }
 
 // kColTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid (chunks, units of the launch).
-template <int kColTiles>
+template <int kColTiles, int kD>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 {
@@ -409,9 +425,10 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const Dims &d = a.d;
     const long long lim = a.wait_cycles;
     uint8_t *gen;
-    const ScoreSmem s = score_smem_layout(smem_raw, kRowsPad, a.stages, &gen);
+    const ScoreSmem s = score_smem_layout<kD>(smem_raw, kRowsPad, a.stages, &gen);
     float *row_c = reinterpret_cast<float *>(gen + (s.misc - s.q));      // [kRowsPad]
-    float *xchg = row_c + 256;                                          // [kXchg tiles][kSets][128]
+    float *row_w = row_c + 256;                                         // [kRowsPad] (D = 64)
+    float *xchg = row_w + 256;                                          // [kXchg tiles][kSets][128]
     uint32_t *mass_hist = reinterpret_cast<uint32_t *>(gen + (s.misc - s.q) + kScratchBytes);   // [kMassBins]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
@@ -425,9 +442,9 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kGroups);
     bool ok = true;
     if (warp == 0) {
-        if (lane == 0) ok = score_produce(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
+        if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
     } else {
-        stage_q(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
+        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
         fence_proxy_async();
     }
     pc.mark();
@@ -444,13 +461,16 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
             a.zero[(long long)unit * a.zero_words + i] = 0u;
     }
     // -c_r of the unit's rows; padding rows contribute 2^-inf = 0
-    for (int r = threadIdx.x; r < kRowsPad; r += kScoreThreads)
-        row_c[r] = r < d.GW ? -__ldcg(a.row_c + (long long)unit * d.GW + r) : -INFINITY;
+    for (int r = threadIdx.x; r < kRowsPad; r += kScoreThreads) {
+        const float *c = a.row_c + (long long)unit * 2 * d.GW + r;
+        row_c[r] = r < d.GW ? -__ldcg(c) : -INFINITY;
+        if (weighted<kD>()) row_w[r] = r < d.GW ? __ldcg(c + d.GW) : 0.f;
+    }
     __syncthreads();
     pc.mark();
 
     if (warp == 0) {
-        if (lane == 0 && ok) ok = score_produce(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim);
+        if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim);
     } else if (warp == 1) {
         if (lane == 0) {
             const uint32_t idesc = umma_idesc_bf16(128, n_cols);
@@ -460,9 +480,9 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                 if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
                 if (!mbar_wait(s.full0 + 8 * st, ph, lim)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t kt = s.stage0 + st * kTileBytes;
+                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
+                for (int k = 0; k < kD / 16; ++k) {
                     const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
                     const uint32_t qoff = (k >> 2) * (kRowsPad * 128) + (k & 3) * 32;
                     umma_bf16(tmem_base + buf * kBufCols, umma_desc_sw128(kt + koff),
@@ -478,7 +498,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         const int quad = warp & 3, set = (warp - 2) >> 2;
         const int grp = set / kSets, part = set % kSets;       // tiles grp, grp + kGroups, ...
         const int key_lane = quad * 32 + lane;
-        const float scale = rsqrtf((float)kHeadDim) * kLog2e;
+        const float scale = rsqrtf((float)kD) * kLog2e;
         const uint64_t scale2 = pack2(scale, scale);
         const int n_slices = (d.GW + 31) >> 5;                 // x32 column slices in use (<= 8)
         const int s_begin = (part * n_slices) / kSets, s_end = ((part + 1) * n_slices) / kSets;
@@ -492,7 +512,9 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 #pragma unroll
             for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(reg[e]);
             const ulonglong2 *c4 = reinterpret_cast<const ulonglong2 *>(row_c + sl * 32);
-            return ex2_sum32(v, scale2, [&](int q) { return c4[q]; });
+            const ulonglong2 *w4 = reinterpret_cast<const ulonglong2 *>(row_w + sl * 32);
+            return ex2_sum32<poly_pairs<kD>(), weighted<kD>()>(v, scale2, [&](int q) { return c4[q]; },
+                                                               [&](int q) { return w4[q]; });
         };
         for (int i = grp; i < n_local && alive; i += kGroups) {
             const int buf = i % kBufs;
@@ -577,7 +599,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 // the re-read of the ring's tiles.  kTiles = 1 (G*W <= 128) or 2 (G*W <= 256); grid (chunks,
 // units of the launch); a.arrivals holds one 64-bit word per unit (the call's tag and the count of
 // arrived CTAs), whatever its content before the launch.
-template <int kTiles>
+template <int kTiles, int kD>
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 {
@@ -593,7 +615,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const Dims &d = a.d;
     const long long lim = a.wait_cycles;
     uint8_t *gen;
-    const ScoreSmem s = score_smem_layout(smem_raw, kRowsPad, a.stages, &gen);
+    const ScoreSmem s = score_smem_layout<kD>(smem_raw, kRowsPad, a.stages, &gen);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x;
@@ -608,7 +630,8 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     // exchange buffers of the emit pass
     float2 *cta_part = reinterpret_cast<float2 *>(gen + (s.misc - s.q));      // [kParts][kRowsPad]
     float *row_c = reinterpret_cast<float *>(gen + (s.misc - s.q));           // [kRowsPad]
-    float *xchg = row_c + 256;                                                // [kXchg tiles][kSets][128]
+    float *row_w = row_c + 256;                                               // [kRowsPad] (D = 64)
+    float *xchg = row_w + 256;                                                // [kXchg tiles][kSets][128]
     uint32_t *mass_hist = reinterpret_cast<uint32_t *>(gen + (s.misc - s.q) + kScratchBytes);   // [kMassBins]
     int *s_flag = reinterpret_cast<int *>(gen + (s.tmem_slot - s.q)) + 2;
     const int n_ahead = min(n_local, S);
@@ -616,9 +639,9 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const uint32_t tmem_base = score_setup(s, gen, &tmK, S, kTmemCols, kEpiWarps / kGroups);
     bool ok = true;
     if (warp == 0) {
-        if (lane == 0) ok = score_produce(s, &tmK, S, t0, 0, n_ahead, h, b, lim);
+        if (lane == 0) ok = score_produce<kD>(s, &tmK, S, t0, 0, n_ahead, h, b, lim);
     } else {
-        stage_q(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
+        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
         fence_proxy_async();
     }
     pc.mark();
@@ -648,7 +671,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 
     // ---- statistics pass: D = Q K^T, tiles 0 .. n_local-1 in order ----
     if (warp == 0) {
-        if (lane == 0 && ok) ok = score_produce(s, &tmK, S, t0, n_ahead, n_local, h, b, lim);
+        if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, S, t0, n_ahead, n_local, h, b, lim);
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
@@ -658,11 +681,11 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                 if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
                 if (!mbar_wait(s.full0 + 8 * st, ph, lim)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t kt = s.stage0 + st * kTileBytes;
+                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
 #pragma unroll
                 for (int rt = 0; rt < kTiles; ++rt) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
+                    for (int k = 0; k < kD / 16; ++k) {
                         const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
                         const uint32_t qoff = (k >> 2) * (kRowsPad * 128) + rt * (128 * 128) + (k & 3) * 32;
                         umma_bf16(tmem_base + buf * kBufCols + rt * 128, umma_desc_sw128(s.q + qoff),
@@ -679,7 +702,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         const int grp = set / (4 / kGroups);
         const int row = quad * 32 + lane;
         const int col0 = (set % (4 / kGroups)) * kSetCols, rt = col0 >> 7, key_off = col0 & 127;
-        const float scale = rsqrtf((float)kHeadDim) * kLog2e;
+        const float scale = rsqrtf((float)kD) * kLog2e;
         float mx = kNegBig, z = 0.f;
         const int r = rt * 128 + row;
         const int last = d.N + (r < d.GW ? r % d.W : 0);      // last visible key of the row
@@ -710,7 +733,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                     for (int e = 0; e < 32; ++e)
                         if (key0 + c * 32 + e > last) v[e] = -INFINITY;
                 }
-                stats_fold(v, scale, mx, z);
+                stats_fold<kD>(v, scale, mx, z);
             }
         }
         ok = alive;
@@ -785,7 +808,10 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
             const int r = threadIdx.x / kTpr, sub = threadIdx.x % kTpr;
             const float2 mz = merge_row_partials<kTpr>(pu, a.chunks, d.GW, r, sub);
             // -c_r of the unit's rows; padding rows contribute 2^-inf = 0
-            if (sub == 0) row_c[r] = r < d.GW ? -(mz.x + log2f(mz.y)) : -INFINITY;
+            if (sub == 0) {
+                row_c[r] = r < d.GW ? -(weighted<kD>() ? mz.x : mz.x + log2f(mz.y)) : -INFINITY;
+                if (weighted<kD>()) row_w[r] = r < d.GW ? 1.0f / mz.y : 0.f;
+            }
         }
     }
     __syncthreads();
@@ -806,10 +832,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                 if (tl + S >= n_local) {
                     mbar_arrive(s.full0 + 8 * st);            // still there from the first pass
                 } else {
-                    const uint32_t dst = s.stage0 + st * kTileBytes;
-                    mbar_expect_tx(s.full0 + 8 * st, kTileBytes);
-                    tma_load_4d(dst, &tmK, s.full0 + 8 * st, 0, (t0 + tl) * kTileKeys, h, b);
-                    tma_load_4d(dst + kHalfBytes, &tmK, s.full0 + 8 * st, 64, (t0 + tl) * kTileKeys, h, b);
+                    tma_load_tile<kD>(s.stage0 + st * tile_bytes<kD>(), &tmK, s.full0 + 8 * st, (t0 + tl) * kTileKeys, h, b);
                 }
                 ++issued;
             }
@@ -829,9 +852,9 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                 if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
                 if (!mbar_wait(s.full0 + 8 * st, u & 1, lim)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t kt = s.stage0 + st * kTileBytes;
+                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
+                for (int kk = 0; kk < kD / 16; ++kk) {
                     const uint32_t koff = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
                     const uint32_t qoff = (kk >> 2) * (kRowsPad * 128) + (kk & 3) * 32;
                     umma_bf16(tmem_base + buf * kBufCols, umma_desc_sw128(kt + koff),
@@ -845,7 +868,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         const int quad = warp & 3, set = (warp - 2) >> 2;
         const int grp = set / kSets, part = set % kSets;
         const int key_lane = quad * 32 + lane;
-        const float scale = rsqrtf((float)kHeadDim) * kLog2e;
+        const float scale = rsqrtf((float)kD) * kLog2e;
         const uint64_t scale2 = pack2(scale, scale);
         const int n_slices = (d.GW + 31) >> 5;
         const int s_begin = (part * n_slices) / kSets, s_end = ((part + 1) * n_slices) / kSets;
@@ -857,7 +880,9 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 #pragma unroll
             for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(reg[e]);
             const ulonglong2 *c4 = reinterpret_cast<const ulonglong2 *>(row_c + sl * 32);
-            return ex2_sum32(v, scale2, [&](int q) { return c4[q]; });
+            const ulonglong2 *w4 = reinterpret_cast<const ulonglong2 *>(row_w + sl * 32);
+            return ex2_sum32<poly_pairs<kD>(), weighted<kD>()>(v, scale2, [&](int q) { return c4[q]; },
+                                                               [&](int q) { return w4[q]; });
         };
         for (int k = grp; k < n_emit && alive; k += kGroups) {
             const int i = n_local + k, buf = i % kBufs;

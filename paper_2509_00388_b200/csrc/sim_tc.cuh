@@ -58,9 +58,9 @@ template <int NP> __host__ __device__ constexpr int sim_tiles_cap() { return 512
 //   [0, NP*256)                      source keys, K-major 128-byte swizzle (two 64-column halves)
 //   [.., + stages*32 KB)             key tiles in flight; reused for the per-thread maxima
 //   barriers, inverse norms of the chunk's keys, source bookkeeping, candidate lists
-template <int NP> __host__ __device__ inline size_t sim_smem_bytes(int stages)
+template <int NP, int kD> __host__ __device__ inline size_t sim_smem_bytes(int stages)
 {
-    return 1024 + (size_t)NP * 256 + (size_t)stages * kTileBytes + (8 + 8 + kSimMaxTiles) * 8 + 16 +
+    return 1024 + (size_t)NP * 2 * kD + (size_t)stages * tile_bytes<kD>() + (8 + 8 + kSimMaxTiles) * 8 + 16 +
            (size_t)sim_tiles_cap<NP>() * 128 * 4 + (size_t)NP * 6 * 4 + (size_t)NP * kCandCap * 8 + 64;
 }
 
@@ -80,7 +80,7 @@ __device__ __forceinline__ void tmem_ld_np(uint32_t taddr, float (&v)[NP])
     }
 }
 
-template <int NP>
+template <int NP, int kD>
 __global__ void __launch_bounds__(kSimThreads, 1)
 similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
 {
@@ -91,8 +91,8 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t s_src = base;
-    const uint32_t s_stage0 = s_src + NP * 256;
-    const uint32_t s_full0 = s_stage0 + a.stages * kTileBytes;
+    const uint32_t s_stage0 = s_src + NP * 2 * kD;
+    const uint32_t s_full0 = s_stage0 + a.stages * tile_bytes<kD>();
     const uint32_t s_empty0 = s_full0 + 8 * 8;
     const uint32_t s_done0 = s_empty0 + 8 * 8;
     const uint32_t s_tmem = s_done0 + kSimMaxTiles * 8;
@@ -142,10 +142,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
         // (a merge of candidate lists borrows the last two stages as scratch first)
         n_ahead = min(a.merge.k > 0 ? a.stages - 2 : a.stages, n_local);
         for (int i = 0; i < n_ahead; ++i) {
-            const uint32_t dst = s_stage0 + i * kTileBytes;
-            mbar_expect_tx(s_full0 + 8 * i, kTileBytes);
-            tma_load_4d(dst, &tmK, s_full0 + 8 * i, 0, (t0 + i) * kTileKeys, h, b);
-            tma_load_4d(dst + kHalfBytes, &tmK, s_full0 + 8 * i, 64, (t0 + i) * kTileKeys, h, b);
+            tma_load_tile<kD>(s_stage0 + i * tile_bytes<kD>(), &tmK, s_full0 + 8 * i, (t0 + i) * kTileKeys, h, b);
         }
     }
     if (warp == 1) {
@@ -157,17 +154,18 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     pdl_launch_dependents();
     pc.mark();
     if (a.merge.k > 0) {
-        static_assert(2 * kTileBytes >= kSrcSmemBytes, "the merge's scratch fits two stages");
+        static_assert(kD == 64 || 2 * tile_bytes<kD>() >= kSrcSmemBytes, "the merge's scratch fits two stages");
         source_merge(a.merge, d, unit, a.a_mass + (long long)unit * d.N,
-                     gen + (s_stage0 - base) + (a.stages - 2) * kTileBytes, src_pos,
+                     gen + (s_stage0 - base) + (a.stages - 2) * tile_bytes<kD>(), src_pos,
                      chunk == 0 ? const_cast<int *>(src) : nullptr);
     }
     // source keys -> swizzled operand rows (rows >= K_src are zero), their positions and norms
-    // (16 consecutive threads share a row: the row's squared norm is reduced among them)
-    for (int i0 = 0; i0 < NP * 16; i0 += kSimThreads) {
+    // (kPieces consecutive threads share a row: the row's squared norm is reduced among them)
+    constexpr int kPieces = kD / 8;
+    for (int i0 = 0; i0 < NP * kPieces; i0 += kSimThreads) {
         const int i = i0 + threadIdx.x;
-        const int r = i >> 4, c16 = i & 15;
-        const bool in = i < NP * 16;
+        const int r = i / kPieces, c16 = i % kPieces;
+        const bool in = i < NP * kPieces;
         uint4 v = make_uint4(0, 0, 0, 0);
         int pos = -1;
         if (in && r < n_src) {
@@ -183,7 +181,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             n2 = fmaf(lo, lo, fmaf(hi, hi, n2));
         }
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        for (int o = kPieces / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         if (in && c16 == 0) {
             src_pos[r] = pos;
             src_norm[r] = fmaxf(sqrtf(n2), kNormEps);
@@ -206,10 +204,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             for (int i = n_ahead; i < n_local; ++i) {
                 const int st = i % a.stages, ph = (i / a.stages) & 1;
                 if (!mbar_wait(s_empty0 + 8 * st, ph ^ 1, lim)) { ok = false; break; }
-                const uint32_t dst = s_stage0 + st * kTileBytes;
-                mbar_expect_tx(s_full0 + 8 * st, kTileBytes);
-                tma_load_4d(dst, &tmK, s_full0 + 8 * st, 0, (t0 + i) * kTileKeys, h, b);
-                tma_load_4d(dst + kHalfBytes, &tmK, s_full0 + 8 * st, 64, (t0 + i) * kTileKeys, h, b);
+                tma_load_tile<kD>(s_stage0 + st * tile_bytes<kD>(), &tmK, s_full0 + 8 * st, (t0 + i) * kTileKeys, h, b);
                 ++issued;
             }
             if (!ok)        // gave up: let the copies already in flight land before the CTA exits
@@ -223,9 +218,9 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
                 const int st = i % a.stages, ph = (i / a.stages) & 1;
                 if (!mbar_wait(s_full0 + 8 * st, ph, lim)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t kt = s_stage0 + st * kTileBytes;
+                const uint32_t kt = s_stage0 + st * tile_bytes<kD>();
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
+                for (int k = 0; k < kD / 16; ++k) {
                     const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
                     const uint32_t soff = (k >> 2) * (NP * 128) + (k & 3) * 32;
                     umma_bf16(tmem_base + i * NP, umma_desc_sw128(kt + koff),
@@ -251,10 +246,10 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             if (alive) alive = __all_sync(0xffffffffu, mbar_wait(s_full0 + 8 * st, ph, lim));
             if (alive) {
                 // squared norm of this thread's key from the staged tile
-                const uint8_t *tile = gen + (s_stage0 - base) + st * kTileBytes;
+                const uint8_t *tile = gen + (s_stage0 - base) + st * tile_bytes<kD>();
                 float n0 = 0.f, n1 = 0.f;
 #pragma unroll
-                for (int c16 = 0; c16 < 16; ++c16) {
+                for (int c16 = 0; c16 < kPieces; ++c16) {
                     const uint4 raw = *reinterpret_cast<const uint4 *>(tile + sw128_offset(128, key_lane, c16));
                     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll

@@ -12,7 +12,7 @@ namespace tc {
 
 constexpr int kTileKeys = 128;                              // keys per MMA tile (UMMA M or N)
 constexpr int kHalfBytes = kTileKeys * 64 * 2;              // 128 rows x 64 bf16 (one swizzle atom wide)
-constexpr int kTileBytes = 2 * kHalfBytes;                  // 128 keys x 128 dims bf16
+template <int kD> __host__ __device__ constexpr int tile_bytes() { return (kD / 64) * kHalfBytes; }
 constexpr long long kWaitCycles = 4000000000LL;             // default limit of a wait: ~2 s at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
@@ -77,6 +77,15 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *tm,
         "[%0], [%1, {%3, %4, %5, %6}], [%2];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
         : "memory");
+}
+// One key tile: keys key0 .. key0 + 127 of (h, b), all kD dimensions, announced on `bar`.
+template <int kD>
+__device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap *tm, uint32_t bar, int key0, int h, int b)
+{
+    mbar_expect_tx(bar, tile_bytes<kD>());
+#pragma unroll
+    for (int half = 0; half < kD / 64; ++half)
+        tma_load_4d(dst + half * kHalfBytes, tm, bar, half * 64, key0, h, b);
 }
 // Generic-proxy writes to shared memory become visible to the async proxy (TMA, tensor core).
 __device__ __forceinline__ void fence_proxy_async()
@@ -298,13 +307,10 @@ __device__ __forceinline__ uint64_t ex2_poly3_pair(uint64_t x)
                  __int_as_float(__float_as_int(phi) + (__float_as_int(thi) << 23)));
 }
 
-#ifndef GRAPHKV_POLY_PAIRS
-#define GRAPHKV_POLY_PAIRS 1          // of every four pairs, how many take the polynomial
-#endif
-
-// sum over i < 32 of 2^(v[i] * scale + c[i]): nc(q) returns c[4q .. 4q+3] as two packed pairs
-template <class NegC>
-__device__ __forceinline__ float ex2_sum32(const float (&v)[32], uint64_t scale2, NegC nc)
+// sum over i < 32 of 2^(v[i] * scale + c[i]) (times w[i]): nc(q), and with kWeighted nw(q), return
+// elements 4q .. 4q+3 as two packed pairs.  kPoly of every four pairs take the polynomial.
+template <int kPoly, bool kWeighted, class NegC, class Weight>
+__device__ __forceinline__ float ex2_sum32(const float (&v)[32], uint64_t scale2, NegC nc, Weight nw)
 {
     uint64_t acc0 = 0ull, acc1 = 0ull;             // (0.f, 0.f)
 #pragma unroll
@@ -312,16 +318,24 @@ __device__ __forceinline__ float ex2_sum32(const float (&v)[32], uint64_t scale2
         const ulonglong2 c = nc(p >> 1);
         const uint64_t x0 = fma2(pack2(v[2 * p], v[2 * p + 1]), scale2, c.x);
         const uint64_t x1 = fma2(pack2(v[2 * p + 2], v[2 * p + 3]), scale2, c.y);
-        acc0 = add2(acc0, (p & 3) >= 4 - GRAPHKV_POLY_PAIRS ? ex2_poly3_pair(x0) : ex2_pair(x0));
-        acc1 = add2(acc1, ((p + 1) & 3) >= 4 - GRAPHKV_POLY_PAIRS ? ex2_poly3_pair(x1) : ex2_pair(x1));
+        const uint64_t e0 = (p & 3) >= 4 - kPoly ? ex2_poly3_pair(x0) : ex2_pair(x0);
+        const uint64_t e1 = ((p + 1) & 3) >= 4 - kPoly ? ex2_poly3_pair(x1) : ex2_pair(x1);
+        if constexpr (kWeighted) {
+            const ulonglong2 w = nw(p >> 1);
+            acc0 = fma2(e0, w.x, acc0);
+            acc1 = fma2(e1, w.y, acc1);
+        } else {
+            acc0 = add2(acc0, e0);
+            acc1 = add2(acc1, e1);
+        }
     }
     float lo, hi;
     unpack2(add2(acc0, acc1), lo, hi);
     return lo + hi;
 }
 
-// Byte offset of the 16-byte piece `c16` (0..15) of row `r` inside a K-major, 128-byte-swizzled
-// operand of `rows` rows x 128 bf16: two halves of 64 columns, rows 128 bytes apart.
+// Byte offset of the 16-byte piece `c16` of row `r` inside a K-major, 128-byte-swizzled operand of
+// `rows` rows x 128 (or 64) bf16: halves of 64 columns, rows 128 bytes apart.
 __device__ __forceinline__ uint32_t sw128_offset(int rows, int r, int c16)
 {
     return static_cast<uint32_t>((c16 >> 3) * rows * 128 + r * 128 + (((c16 & 7) ^ (r & 7)) << 4));

@@ -49,3 +49,13 @@ def test_fp32_sweeps_edges(gk, n, w, g, k, head_dim):
     cfg = wl.scaled(wl.TINY, n_prefix=n, window=w, n_q_heads=3 * g, n_kv_heads=3, head_dim=head_dim, topk_nodes=k,
                     neighbors=min(n - 1, 5), budget=min(n, 20), batch=2)
     check(gk, cfg, strict_overlap=False)
+
+
+# head dimension 64 on the tensor cores: one and two row tiles of queries, ragged key tiles, 16 / 32 / 64
+# sources per sweep and several sweeps
+@pytest.mark.parametrize("n,w,g,k,m", [(127, 1, 1, 3, 2), (128, 32, 4, 16, 8), (1281, 33, 4, 17, 32), (2900, 64, 4, 70, 8),
+                                       (2560, 50, 5, 40, 12)])
+def test_head_dimension_64_edges(gk, n, w, g, k, m):
+    cfg = wl.scaled(wl.LLAMA_32K, n_prefix=n, window=w, n_q_heads=2 * g, n_kv_heads=2, head_dim=64, topk_nodes=k,
+                    neighbors=m, budget=min(n, 90), batch=2, n_clusters=24)
+    check(gk, cfg, strict_overlap=False)
