@@ -825,6 +825,7 @@ struct PoolSelectArgs {
     uint32_t *zero;        // optional: [units][zero_words] words this launch clears for later kernels
     int zero_words;
     int wait_prior;        // launched with programmatic stream serialization
+    uint32_t *row_hist;    // optional [units][kBins], zero before: the scores' top digits are counted there
 };
 
 // grid = units * C CTAs in clusters of C; block kThreads.  kPer >= chunk / kThreads: elements of
@@ -1035,6 +1036,28 @@ __global__ void __launch_bounds__(kThreads, 1) pool_select_kernel(PoolSelectArgs
         }
     }
     pc.mark();
+    // The row's histogram for the finishing kernel: while the first CTA ranks the sources' candidates, the
+    // others count their chunks and share the first one's (in its shared memory).
+    if (a.row_hist && (rank > 0 || C == 1)) {
+        for (int i = tid; i < kBins; i += kThreads) s.fine[i] = 0u;
+        __syncthreads();
+        auto count = [&](const float *v, int lo, int hi) {
+            for (int i0 = lo + (tid & ~31); i0 < hi; i0 += kThreads) {
+                const int i = i0 + (tid & 31);
+                const uint32_t bin = i < hi ? float_to_key(v[i]) >> 21 : 0xffffffffu;
+                const unsigned peers = __match_any_sync(0xffffffffu, bin);
+                if (i < hi && (tid & 31) == __ffs(peers) - 1) atomicAdd(&s.fine[bin], (uint32_t)__popc(peers));
+            }
+        };
+        count(vals, 0, n_local);
+        if (C > 1) {
+            const int n0 = min(a.chunk, N), share = ceil_div(n0, C - 1);
+            count(cl.map_shared_rank(vals, 0), (rank - 1) * share, min(rank * share, n0));
+        }
+        __syncthreads();
+        for (int i = tid; i < kBins; i += kThreads)
+            if (s.fine[i]) atomicAdd(a.row_hist + (long long)unit * kBins + i, s.fine[i]);
+    }
     if (C > 1) cl.sync();      // no CTA leaves while its shared memory may still be read
     pc.mark();
     pc.flush(3);

@@ -12,6 +12,7 @@
 #include "common.cuh"
 #include "decode_attn.cuh"
 #include "gather.cuh"
+#include "row_finish.cuh"
 #include "propagate_simt.cuh"
 #include "score_simt.cuh"
 #include "score_tc.cuh"
@@ -32,6 +33,7 @@ struct Layout {
     size_t arrivals;    // counters of score CTAs per unit [2 * units] (directly after the status word)
     size_t a_hist;      // histogram of the attention mass [units][2048] (directly after the counters)
     size_t row_c;       // softmax row constants [units][2][GW]
+    size_t row_hist;    // histogram of the scores [units][2048], cleared by the sweeps
     size_t part;        // softmax row statistics per key chunk
     size_t a;           // attention mass before pooling [units][N]
     size_t s;           // scores when the caller gives no array [units][N]
@@ -225,6 +227,7 @@ Layout layout_of(const Dims &d)
     l.status = take(kAlign);
     l.arrivals = take((size_t)d.units * 2 * sizeof(int));
     l.a_hist = take((size_t)d.units * tc::kMassBins * sizeof(uint32_t));
+    l.row_hist = take((size_t)d.units * cs::kBins * sizeof(uint32_t));
     l.row_c = take((size_t)d.units * d.GW * 2 * sizeof(float));
     l.part = take((size_t)d.units * l.max_parts * d.GW * 2 * sizeof(float));
     l.a = take((size_t)d.units * d.N * sizeof(float));
@@ -614,12 +617,12 @@ graphkv_status launch_cluster(const char *name, void (*kern)(Args), Args args, i
 // `mass_hist` (optional): per unit, a histogram of values the scores dominate (see the kernel).
 graphkv_status run_pool_sources(const Dims &d, const float *a, float *s, int k, int *src,
                                 const uint32_t *mass_hist, uint32_t *zero, int zero_words,
-                                cudaStream_t st)
+                                cudaStream_t st, uint32_t *row_hist = nullptr)
 {
     if (!a && k == 0) return GRAPHKV_OK;
     const ClusterPlan cp = cluster_plan(d);
     if (cp.ok) {
-        cs::PoolSelectArgs pa{d, cp.C, cp.chunk, a ? cp.halo : 0, 0, a, s, k, src, mass_hist, zero, zero_words, 0};
+        cs::PoolSelectArgs pa{d, cp.C, cp.chunk, a ? cp.halo : 0, 0, a, s, k, src, mass_hist, zero, zero_words, 0, row_hist};
         const char *name = a ? (k ? "pool_select_sources" : "pool_max") : "select_sources";
         const size_t smem = cs::smem_bytes(cp.chunk, pa.halo);
         const int per = ceil_div(cp.chunk, cs::kThreads);
@@ -728,17 +731,94 @@ FinishPlan finish_plan(const Dims &d, int halo)
     return p;
 }
 
+// Rows up to this length are candidates as a whole: no histogram, no bits.
+constexpr int kDenseRow = 4096;
+
 // Per-batch-element budgets of the call in flight (graphkv_compress_layers), or none.
 thread_local const int32_t *t_budgets = nullptr;
 // The caller of the call in flight wants the final scores (graphkv_compress without scores_out
 // does not: its last kernel then leaves them in shared memory).
 thread_local bool t_keep_scores = true;
 
+// The finishing kernel that works on the candidates of a row (row_finish.cuh).
+struct CandidatePlan {
+    bool ok;
+    int C, chunk, dense, cap, sel_cap, list_bytes;
+    size_t smem;
+};
+
+CandidatePlan candidate_plan(const Dims &d, bool has_graph, bool do_select, bool keep_scores, int max_budget)
+{
+    CandidatePlan p{};
+    if (env_int("GRAPHKV_NO_CLUSTER", 0) || d.N > rf::kMaxRow) return p;
+    const long long pairs = has_graph ? (long long)d.K_src * d.m : 0;
+    if (pairs > 16384) return p;
+    const bool raises = has_graph && d.signal == GRAPHKV_SIGNAL_ENHANCE;
+    const int need = do_select ? (int)std::min<long long>(d.N, max_budget + (raises ? 0 : pairs)) : 0;
+    p.dense = d.N <= kDenseRow || (do_select && 2LL * need > d.N);
+    // room for half as many again: the digit of the last one needed brings its fellows along
+    p.sel_cap = p.dense ? d.N : std::min(d.N, need + need / 2 + 256);
+    p.cap = p.dense ? d.N : std::min<long long>(d.N, p.sel_cap + (has_graph && (keep_scores || !do_select || raises) ? pairs : 0));
+    p.cap = (p.cap + 31) & ~31;
+    p.list_bytes = (int)(std::max<long long>(8 * pairs, do_select ? 4LL * max_budget : 0) + 15) & ~15;
+    p.smem = rf::smem_bytes(d.N, p.cap, p.list_bytes, p.dense);
+    p.C = 1;
+    while (p.C < rf::kMaxCluster && d.units * p.C * 2 <= sm_count()) p.C *= 2;
+    p.chunk = (ceil_div(d.N, p.C) + 31) & ~31;
+    p.ok = p.smem <= kMaxSmem;
+    return p;
+}
+
 graphkv_status run_finish(const Dims &d, const Layout &l, int elem_bytes, const float *a, float *s,
                           bool has_graph, bool merge, bool do_select, const void *K, const void *V,
-                          void *K_out, void *V_out, int *idx_out, void *ws, cudaStream_t st)
+                          void *K_out, void *V_out, int *idx_out, void *ws, cudaStream_t st,
+                          const uint32_t *row_hist = nullptr)
 {
     if (!has_graph && !do_select && !a) return GRAPHKV_OK;
+    const bool keep = has_graph && (t_keep_scores || !do_select);
+    const CandidatePlan cd = a ? CandidatePlan{} : candidate_plan(d, has_graph, do_select, keep, d.B);
+    if (cd.ok) {
+        rf::FinishArgs fa{};
+        fa.d = d;
+        fa.C = cd.C;
+        fa.chunk = cd.chunk;
+        fa.dense = cd.dense;
+        fa.cap = cd.cap;
+        fa.sel_cap = cd.sel_cap;
+        fa.list_bytes = cd.list_bytes;
+        // enough groups for every source at once where that leaves a group more than one warp
+        fa.group_warps = d.K_src <= 4 * cd.C ? 4 : d.K_src <= 8 * cd.C ? 2 : 1;
+        fa.row_hist = row_hist;
+        fa.s = s;
+        fa.nbr_idx = at<int>(ws, l.nbr_idx);
+        fa.nbr_e = at<float>(ws, l.nbr_e);
+        fa.has_graph = has_graph;
+        fa.merge = has_graph && merge;
+        fa.cand = at<Cand>(ws, l.cand);
+        fa.cand_hist = at<uint32_t>(ws, l.cand_hist);
+        fa.cand_chunks = merge ? sim_plan(d, d.bf16 != 0).chunks : 0;
+        fa.do_select = do_select;
+        fa.idx_out = idx_out;
+        fa.elem_bytes = elem_bytes;
+        for (fa.vpr_log2 = 0; (16 << fa.vpr_log2) < d.D * elem_bytes;) ++fa.vpr_log2;
+        fa.K = static_cast<const unsigned char *>(K);
+        fa.V = static_cast<const unsigned char *>(V);
+        fa.K_out = static_cast<unsigned char *>(K_out);
+        fa.V_out = static_cast<unsigned char *>(V_out);
+        fa.early_row = has_graph;
+        fa.keep_scores = keep;
+        if (t_budgets && do_select) {
+            fa.per_batch_budget = 1;
+            for (int i = 0; i < d.batch; ++i) fa.budget_of[i] = t_budgets[i];
+        }
+        static std::mutex mu;
+        static signed char state[64] = {};
+        if (!once_per_device(mu, state, [] { return set_smem(rf::finish_kernel, kMaxSmem); })) return GRAPHKV_ERR_CUDA;
+        fa.wait_prior = next_launch_is_dependent();
+        const char *name = has_graph ? (do_select ? "decay_select_gather" : "decay_rounds") : "select_gather";
+        return launch_ex(name, rf::finish_kernel, dim3(d.units * cd.C), dim3(rf::kThreads), cd.smem, st,
+                         fa.wait_prior != 0, cd.C, fa);
+    }
     const int halo = a ? (d.kp - 1) / 2 : 0;
     const FinishPlan fp = finish_plan(d, halo);
     if (fp.ok && cluster_plan(d).ok) {
@@ -849,10 +929,11 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
     // against 112 us per step; 131072 x 4: 1.25 against 1.13 ms), so it is off by default.
     const bool tail_src = tc_mass(Q, d) && tc_graph && d.D == kHeadDim && d.K_src <= tc::kSrcMaxK && !d.pool_avg &&
                           units_per_group(d) >= d.units && env_int("GRAPHKV_TAIL_SOURCES", 0);
-    const bool finish_pools = d.kp > 1 && !d.pool_avg && (tail_src || !graph) && finish_plan(d, halo).ok &&
+    const bool finish_pools = d.kp > 1 && !d.pool_avg && (tail_src || (!graph && !candidate_plan(d, false, true, false, d.B).ok)) && finish_plan(d, halo).ok &&
                               cluster_plan(d).ok;
     graphkv_status rc;
     int list_chunks = 0;
+    uint32_t *row_hist = nullptr;
     if (tail_src || !graph) {
         const EmitExtras ex{tail_src ? d.K_src : 0, &list_chunks, src, tail_src ? at<uint32_t>(ws, l.cand_hist) : nullptr,
                             tail_src ? d.K_src * kCandBins : 0, false};
@@ -861,11 +942,19 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
             (rc = run_pool_sources(d, a, s, 0, nullptr, nullptr, nullptr, 0, st)) != GRAPHKV_OK)
             return rc;
     } else {
-        if ((rc = run_mass(d, l, Q, K, a, ws, st)) != GRAPHKV_OK) return rc;
+        // (the sweeps clear the words the pooling kernel counts the scores in)
+        if (cluster_plan(d).ok && tc_mass(Q, d) && (!d.reselect || d.T <= 1)) {
+            const CandidatePlan cd = candidate_plan(d, true, true, t_keep_scores, d.B);
+            if (cd.ok && !cd.dense) row_hist = at<uint32_t>(ws, l.row_hist);
+        }
+        EmitExtras ex = kPlainEmit;
+        ex.zero = row_hist;
+        ex.zero_words = cs::kBins;
+        if ((rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
         // the tensor-core emit sweep leaves a histogram of the attention mass behind
         rc = run_pool_sources(d, d.kp > 1 ? a : nullptr, s, d.K_src, src,
                               tc_mass(Q, d) ? at<uint32_t>(ws, l.a_hist) : nullptr,
-                              tc_graph ? at<uint32_t>(ws, l.cand_hist) : nullptr, d.K_src * kCandBins, st);
+                              tc_graph ? at<uint32_t>(ws, l.cand_hist) : nullptr, d.K_src * kCandBins, st, row_hist);
         if (rc != GRAPHKV_OK) return rc;
     }
     const EdgeOperands<T> eo{K, d.ks, K, d.ks};
@@ -889,7 +978,7 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
                                l.max_parts, list_chunks};
     if (graph && (rc = run_graph(d, l, eo, src, ws, st, tail_src ? &merge : nullptr, a)) != GRAPHKV_OK) return rc;
     return run_finish(d, l, (int)sizeof(T), finish_pools ? a : nullptr, s, graph, tc_graph, true, K, V,
-                      K_out, V_out, idx_out, ws, st);
+                      K_out, V_out, idx_out, ws, st, row_hist);
 }
 
 // ---- KNorm initial score ---------------------------------------------------------------------

@@ -59,3 +59,30 @@ def test_head_dimension_64_edges(gk, n, w, g, k, m):
     cfg = wl.scaled(wl.LLAMA_32K, n_prefix=n, window=w, n_q_heads=2 * g, n_kv_heads=2, head_dim=64, topk_nodes=k,
                     neighbors=m, budget=min(n, 90), batch=2, n_clusters=24)
     check(gk, cfg, strict_overlap=False)
+
+
+# the budget selection by candidates: rows around the length that is all candidates, budgets of one and
+# near the row's, ties that no digit separates (constant rows, few values), one and several CTAs per row
+@pytest.mark.parametrize("values", ["spread", "constant", "few", "negative"])
+@pytest.mark.parametrize("n,budget,heads", [(33, 33, 1), (4096, 1, 2), (4097, 700, 2), (8191, 4000, 3), (20000, 512, 2),
+                                            (9001, 257, 160), (262144, 4096, 1)])
+def test_select_by_candidates(gk, values, n, budget, heads):
+    gen = torch.Generator().manual_seed(n + budget)
+    s = torch.randn((1, heads, n), generator=gen).exp()
+    if values == "constant":
+        s.fill_(0.25)
+    elif values == "few":
+        s = torch.randint(0, 4, s.shape, generator=gen).float()
+    elif values == "negative":
+        s = -s
+        s[:, :, ::3] = float("-inf")
+    K = torch.randn((1, heads, n + 3, 64), generator=gen).to(torch.bfloat16)
+    Kd, sd = K.to(DEV), s.to(DEV)
+    p = gk.make_params(Kd, window=3, budget=budget)
+    K_out, _, idx, _ = gk.alloc_outputs(p, Kd)
+    gk.graphkv_select_gather(p, sd, Kd, None, K_out, None, idx, gk.alloc_workspace(p, DEV))
+    for h in range(heads) if heads < 8 else (0, heads // 2, heads - 1):
+        want = okv.topk(s[0, h], budget).long().sort().values
+        assert torch.equal(idx[0, h].cpu().long(), want)
+        rows = torch.cat([want, torch.arange(n, n + 3)])
+        assert torch.equal(K_out[0, h].cpu().view(torch.int16), K[0, h, rows].view(torch.int16))
