@@ -1,0 +1,787 @@
+// The whole path in one kernel, for few units with short rows (up to three key tiles
+// per CTA, 3072 tokens): one cluster of C CTAs
+// per (sequence, KV head) unit, each CTA owning a run of key tiles from the first score to the gather.
+//
+// Bound: latency.  At these sizes the four kernels of the general path take 8-20 us each for 1-3 us of
+// work: launch, set-up, the first loads, writes that the next kernel reads back, a tail.  Here the key
+// tiles come from memory once and stay in shared memory for all three sweeps, the row of scores is copied into every CTA, which then selects and decays it like the others without
+// asking them, and what the CTAs of a unit exchange goes through distributed shared memory behind cluster
+// barriers (0.3 us each, seven of them).
+//
+// Every arithmetic step is the general kernels': the same accumulators, the row statistics folded and
+// merged over the same key chunks in the same order (a CTA takes whole chunks), the same pooling, cosines
+// and decay order; so the results agree with them to the bit.
+// 512 threads; thread 0 issues copies and MMAs between the barriers of the sweeps.
+//
+// Measured on one B200 against the four kernels, 8 KV heads, W = 32, 16 sources: 500 tokens 40 -> 30 us,
+// 1003 tokens 43 -> 34, 2000 tokens 47 -> 40, 3000 tokens 53 -> 50; with four tiles per CTA and more the
+// sweeps' 64 CTAs lose to the general path's 128 to 148 (two heads of 4064 tokens 49 -> 55 us).
+#pragma once
+
+#include "row_finish.cuh"
+#include "score_tc.cuh"
+
+namespace graphkv {
+namespace cp {
+
+namespace cg = cooperative_groups;
+using rf::kThreads;
+using rf::kWarps;
+
+constexpr int kMaxCluster = 8;
+constexpr int kMaxTiles = 4;            // key tiles per CTA (whole chunks of the row statistics: they come out uneven)
+constexpr int kMeanTiles = 3;           // on average
+constexpr int kMaxSources = 64;
+constexpr int kMaxNeighbours = 32;
+constexpr int kMaxRow = kMaxCluster * kMeanTiles * tc::kTileKeys;    // tokens per row
+constexpr int kListCap = 64;            // listed edges per source and CTA
+
+struct PathArgs {
+    Dims d;
+    const __nv_bfloat16 *Q, *K;
+    int C;
+    int chunks, n_tiles;       // key chunks of the row statistics and key tiles, per unit
+    int tiles;                 // most key tiles a CTA owns
+    int np;                    // sources padded to 16, 32 or 64
+    int region;                // bytes of the lists' place
+    float *part;               // [units][chunks][GW][2] row statistics per chunk
+    int *status;
+    float *scores;             // optional [units][N]: final scores (scores_only: the pooled ones)
+    int scores_only;
+    int has_graph;
+    int *src_out, *nbr_idx;    // [units][K_src], [units][K_src][m]
+    float *nbr_e;
+    int *idx_out;
+    int vpr_log2;              // 16-byte pieces per row: 1 << vpr_log2
+    const unsigned char *Kb, *V;
+    unsigned char *K_out, *V_out;
+    long long wait_cycles;
+    int withhold_commit;       // test hook: 1: the first accumulator is never announced
+    int per_batch_budget;
+    int budget_of[rf::kMaxBudgets];
+};
+
+// Shared memory, from a 1024-byte aligned base.
+struct Layout {
+    int tiles, mass, inv, row, row_c, scratch, small, bars, total;
+};
+template <int kD, int kTiles> __host__ __device__ inline Layout layout(int tiles, int region, int N)
+{
+    Layout l;
+    int off = 128 * kTiles * 2 * kD;            // the queries; then source rows
+    l.tiles = off;                              // the tiles; then the region of the lists
+    off += tiles * tc::tile_bytes<kD>() > region ? tiles * tc::tile_bytes<kD>() : region;
+    const int keys = tiles * tc::kTileKeys;
+    l.mass = off;    off += keys * 4;           // this CTA's attention mass before pooling
+    l.inv = off;     off += keys * 4;           // 1 / |k|
+    l.row = off;     off += (N + 3) / 4 * 16;   // the unit's scores
+    l.row_c = off;   off += 2 * 128 * kTiles * 4;
+    l.scratch = off; off += 16384;              // partial statistics, exchange, histograms
+    l.small = off;   off += 2048;
+    l.bars = off;    off += (kMaxTiles + 2) * 8 + 16;
+    l.total = off + 1024;
+    return l;
+}
+
+__host__ __device__ inline int first_chunk(int chunks, int C, int rank) { return (int)((long long)chunks * rank / C); }
+__host__ __device__ inline int first_tile_of_chunk(int n_tiles, int chunks, int c)
+{
+    const int base = n_tiles / chunks, rem = n_tiles % chunks;
+    return c * base + (c < rem ? c : rem);
+}
+
+// After the sweeps the tiles' place holds the cosines [16][keys] (then the gangs' survivors), the CTA's lists
+// [k][kListCap], the merged lists of its sources [ceil(k / C)][kMaxNeighbours], all lists [k][m] and, at its
+// end, the kept positions [B].
+__host__ __device__ inline int region_bytes(int keys, int C, int k, int m, int B)
+{
+    const int cosines = 16 * keys * 4, tops = 4 * (kMaxCluster + 1) * kListCap * 8;
+    return ((cosines > tops ? cosines : tops) + k * kListCap * 8 + ((k + C - 1) / C) * kMaxNeighbours * 8 + k * m * 8 + B * 4 + 15) / 16 * 16;
+}
+
+// The edges of x(0 .. n) (lane-strided: element i * 32 + lane, kCandEmpty where there is none) that reach a
+// bound at which between m and kListCap of them do; with too many near-ties, exactly the m largest (lowest
+// positions first).  put(slot, e, i).  Returns their number, and in *bound a value that m of them reach (-1
+// with fewer than m).  `from`: -1, or a value that at least m of them are known to reach.  Rolled loops over
+// shared memory: the code runs once per source.
+template <typename At, typename Put>
+__device__ __forceinline__ int warp_list_top(int n, int m, float from, At x, Put put, float *bound)
+{
+    const int lane = threadIdx.x & 31;
+    // how many reach t0, t1 (packed)
+    auto reach2 = [&](float t0, float t1) {
+        uint32_t c = 0;
+#pragma unroll 4
+        for (int i = lane; i < n; i += 32) {
+            const float e = x(i);
+            c += (e >= t0 ? 1u : 0u) + (e >= t1 ? 0x10000u : 0u);
+        }
+        return __reduce_add_sync(0xffffffffu, c);
+    };
+    float lo = from, hi = 1.0f;
+    const float half = from + 0.5f * (1.0f - from);
+    uint32_t c = reach2(from, half);
+    int have = (int)(c & 0xffffu);
+    *bound = -1.0f;
+    if ((int)(c >> 16) >= m) lo = half, have = (int)(c >> 16);
+    else hi = half;
+    for (int it = 0; have > kListCap && it < 16; ++it) {
+        const float t0 = lo + (hi - lo) * (1.0f / 3.0f), t1 = lo + (hi - lo) * (2.0f / 3.0f);
+        c = reach2(t0, t1);
+        if ((int)(c >> 16) >= m) {
+            lo = t1;
+            have = (int)(c >> 16);
+        } else if ((int)(c & 0xffffu) >= m) {
+            lo = t0;
+            hi = t1;
+            have = (int)(c & 0xffffu);
+        } else {
+            hi = t0;
+        }
+    }
+    if (have >= m) *bound = lo;
+    uint32_t exact = 0;                         // with too many near-ties: the key of the m-th largest
+    int ties = 0;                               // and how many of its ties belong to the m
+    if (have > kListCap) {
+        uint32_t klo = float_to_key(lo), khi = float_to_key(1.0f) + 1u;
+        while (khi - klo > 1u) {
+            const uint32_t mid = klo + (khi - klo) / 2u;
+            uint32_t q = 0;
+            for (int i = lane; i < n; i += 32) q += float_to_key(x(i)) >= mid;
+            if ((int)__reduce_add_sync(0xffffffffu, q) >= m) klo = mid;
+            else khi = mid;
+        }
+        exact = klo;
+        uint32_t q = 0;
+        for (int i = lane; i < n; i += 32) q += float_to_key(x(i)) > exact;
+        ties = m - (int)__reduce_add_sync(0xffffffffu, q);
+    }
+    int at = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const float e = i0 + lane < n ? x(i0 + lane) : kCandEmpty;
+        bool keep = e >= lo;
+        if (exact) {
+            const uint32_t key = float_to_key(e);
+            const unsigned eq = __ballot_sync(0xffffffffu, key == exact);
+            keep = key > exact || (key == exact && __popc(eq & ((1u << lane) - 1u)) < ties);
+            ties -= min(ties, __popc(eq));
+        }
+        const unsigned bm = __ballot_sync(0xffffffffu, keep);
+        if (keep) put(at + __popc(bm & ((1u << lane) - 1u)), e, i0 + lane);
+        at += __popc(bm);
+    }
+    return at;
+}
+
+// kTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid = units * C CTAs in clusters of C.
+template <int kD, int kTiles>
+__global__ void __launch_bounds__(kThreads, 1)
+cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ PathArgs a)
+{
+    using namespace tc;
+    extern __shared__ uint8_t smem_raw[];
+    cg::cluster_group cl = cg::this_cluster();
+    constexpr int kRowsPad = 128 * kTiles, kBufCols = 128 * kTiles;
+    constexpr int kGroups = 2 / kTiles, kSets = 4 / kGroups, kParts = 4 / kTiles;     // as in the score kernels
+    constexpr int kTile = tile_bytes<kD>();
+    const Dims &d = a.d;
+    const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C;
+    const int b = unit / d.hkv, h = unit % d.hkv, N = d.N, keys = a.tiles * kTileKeys;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, quad = warp & 3, set = warp >> 2;
+    const long long lim = a.wait_cycles;
+    const uint32_t base_s = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t *gen = smem_raw + (base_s - smem_u32(smem_raw));
+    const Layout lay = layout<kD, kTiles>(a.tiles, a.region, N);
+    float *mass = reinterpret_cast<float *>(gen + lay.mass), *inv_norm = reinterpret_cast<float *>(gen + lay.inv);
+    float *row = reinterpret_cast<float *>(gen + lay.row);                // [N] the unit's scores, whole
+    float *row_c = reinterpret_cast<float *>(gen + lay.row_c), *row_w = row_c + kRowsPad;
+    uint8_t *scratch = gen + lay.scratch;
+    uint32_t *hist = reinterpret_cast<uint32_t *>(scratch);
+    uint32_t *wcnt = reinterpret_cast<uint32_t *>(gen + lay.small);       // [2 * kWarps]
+    uint32_t *misc = wcnt + 2 * kWarps;                                   // [32]
+    int *src_pos = reinterpret_cast<int *>(misc + 32);                    // [kMaxSources]
+    float *src_inv = reinterpret_cast<float *>(src_pos + kMaxSources);    // [kMaxSources]
+    int *list_n = reinterpret_cast<int *>(src_inv + kMaxSources);         // [kMaxSources]
+    float *list_bound = reinterpret_cast<float *>(list_n + kMaxSources);  // [kMaxSources]
+    int *start = reinterpret_cast<int *>(list_bound + kMaxSources);       // [kMaxCluster + 1] first key of each CTA
+    const uint32_t bar_full = base_s + lay.bars, bar_done = bar_full + 8 * kMaxTiles, tmem_slot = bar_done + 16;
+    PhaseClock pc(tid == 0);
+    pc.mark();
+    if (C > 1) cl.barrier_arrive();
+
+    const int c0 = first_chunk(a.chunks, C, rank), c1 = first_chunk(a.chunks, C, rank + 1);
+    const int t0 = first_tile_of_chunk(a.n_tiles, a.chunks, c0), n_tiles = first_tile_of_chunk(a.n_tiles, a.chunks, c1) - t0;
+    const int base = t0 * kTileKeys, n_local = max(0, min(N - base, n_tiles * kTileKeys));
+    const int n_emit = (n_local + kTileKeys - 1) / kTileKeys;             // tiles with prefix keys
+
+    // ---- set-up: barriers, tensor memory, the first tiles, the queries ----
+    auto tile_landed = [&](int t) { return mbar_wait(bar_full + 8 * t, 0, lim); };
+    if (tid == 0) {
+        for (int i = 0; i < kMaxTiles; ++i) mbar_init(bar_full + 8 * i, 1);
+        mbar_init(bar_done, 1);
+        mbar_init(bar_done + 8, 1);
+        mbar_fence_init();
+        tma_prefetch_desc(&tmK);
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
+    }
+    // (the launch may be early: nothing of the stream before it, inputs included, is touched ahead of this)
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tid == 0) {
+        for (int t = 0; t < n_tiles; ++t)
+            tma_load_tile<kD>(base_s + lay.tiles + t * kTile, &tmK, bar_full + 8 * t, (t0 + t) * kTileKeys, h, b);
+        if (rank == 0 && unit == 0) *a.status = 0;
+    }
+    if (tid <= C) start[tid] = first_tile_of_chunk(a.n_tiles, a.chunks, first_chunk(a.chunks, C, tid)) * kTileKeys;
+    stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, tid, kThreads);
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + (tmem_slot - base_s));
+    const uint32_t tmem_lane = tmem + ((uint32_t)(quad * 32) << 16);
+    bool alive = true;              // no wait of this CTA has run out (the same in all its threads)
+    int batch = 0;                  // batches of MMAs so far; the announcements alternate between two barriers
+    auto batch_done = [&](int bt) { return __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (bt & 1), (bt >> 1) & 1, lim)) != 0; };
+    pc.mark();
+
+    // ---- statistics: D = Q K^T, chunk by chunk, kGroups tiles per batch, two batches under way ----
+    const float scale = rsqrtf((float)kD) * kLog2e;
+    {
+        struct Cursor { int c, i; };                                      // chunk, first tile of the batch within it
+        auto chunk_tiles = [&](int c) { return first_tile_of_chunk(a.n_tiles, a.chunks, c + 1) - first_tile_of_chunk(a.n_tiles, a.chunks, c); };
+        auto next = [&](Cursor &u) {
+            u.i += kGroups;
+            if (u.i >= chunk_tiles(u.c)) u.i = 0, ++u.c;
+        };
+        bool ok = true, issued_ok = true;                                 // (issued_ok: thread 0's own waits)
+        auto issue = [&](Cursor u, int bt) {
+            const int first = first_tile_of_chunk(a.n_tiles, a.chunks, u.c) - t0 + u.i, n = min(kGroups, chunk_tiles(u.c) - u.i);
+            for (int g = 0; g < n && issued_ok; ++g) {
+                issued_ok = tile_landed(first + g);
+                if (!issued_ok) break;
+                tc_fence_after();
+                const uint32_t kt = base_s + lay.tiles + (first + g) * kTile;
+                const uint32_t out = tmem + ((bt & 1) * kGroups + g) * kBufCols;
+#pragma unroll
+                for (int rt = 0; rt < kTiles; ++rt)
+#pragma unroll
+                    for (int k = 0; k < kD / 16; ++k)
+                        umma_bf16(out + rt * 128, umma_desc_sw128(base_s + (k >> 2) * (kRowsPad * 128) + rt * (128 * 128) + (k & 3) * 32),
+                                  umma_desc_sw128(kt + (k >> 2) * kHalfBytes + (k & 3) * 32), umma_idesc_bf16(128, 128), k > 0);
+            }
+            if (issued_ok && !(a.withhold_commit == 1 && bt == 0)) umma_commit(bar_done + 8 * (bt & 1));
+        };
+        Cursor at{c0, 0}, ahead{c0, 0};
+        int n_issued = 0;
+        if (tid == 0)
+            for (; n_issued < 2 && ahead.c < c1; ++n_issued) {
+                issue(ahead, n_issued);
+                next(ahead);
+            }
+        const int grp = set / (4 / kGroups), col0 = (set % (4 / kGroups)) * 64, rt = col0 >> 7, key_off = col0 & 127;
+        const int r = rt * 128 + quad * 32 + lane, last = N + (r < d.GW ? r % d.W : 0);      // last visible key of the row
+        float mx = kNegBig, z = 0.f;
+        while (at.c < c1 && alive) {
+            const int nt = chunk_tiles(at.c);
+            const int tile = first_tile_of_chunk(a.n_tiles, a.chunks, at.c) - t0 + at.i + grp;
+            ok = batch_done(batch);
+            if (ok && at.i + grp < nt) {
+                tc_fence_after();
+                uint32_t raw[2][32];
+                const uint32_t from = tmem_lane + ((batch & 1) * kGroups + grp) * kBufCols + col0;
+                tmem_ld32_issue(from, raw[0]);
+                tmem_ld32_issue(from + 32, raw[1]);
+                tmem_ld_fence(raw[0]);
+                tmem_ld_fence(raw[1]);
+                const int key0 = (t0 + tile) * kTileKeys + key_off;
+                const bool masked = key0 + 63 > N;                          // window keys or the tail past L
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    float v[32];
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(raw[c][e]);
+                    if (masked) {
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (key0 + c * 32 + e > last) v[e] = -INFINITY;
+                    }
+                    stats_fold<kD>(v, scale, mx, z);
+                }
+            }
+            tc_fence_before();
+            const bool chunk_ends = at.i + kGroups >= nt;
+            // (two buffers in turn: the merge below may still read one while the next chunk ends)
+            float2 *cta_part = reinterpret_cast<float2 *>(scratch) + (at.c & 1) * (kParts * kRowsPad);
+            if (chunk_ends) {
+                cta_part[(kTiles == 1 ? set : set & 1) * kRowsPad + r] = make_float2(mx, z);
+                mx = kNegBig;
+                z = 0.f;
+            }
+            alive = __syncthreads_and(ok && issued_ok ? 1 : 0) != 0;
+            if (!alive) break;
+            if (chunk_ends && tid < d.GW) {
+                float2 p[kParts];
+                float m = kNegBig, sum = 0.f;
+#pragma unroll
+                for (int k = 0; k < kParts; ++k) {
+                    p[k] = cta_part[k * kRowsPad + tid];
+                    m = fmaxf(m, p[k].x);
+                }
+#pragma unroll
+                for (int k = 0; k < kParts; ++k) sum += p[k].y * ex2(p[k].x - m);
+                reinterpret_cast<float2 *>(a.part)[((long long)unit * a.chunks + at.c) * d.GW + tid] = make_float2(m, sum);
+            }
+            if (tid == 0) {
+                tc_fence_after();
+                if (ahead.c < c1) {
+                    issue(ahead, n_issued++);
+                    next(ahead);
+                }
+            }
+            ++batch;
+            next(at);
+        }
+    }
+    pc.mark();
+
+    // ---- row constants from all chunks of the unit ----
+    if (C > 1) {
+        cl.barrier_wait();              // (the start of the kernel)
+        cl.sync();                      // every chunk's statistics have been written
+    } else {
+        __syncthreads();
+    }
+    pc.mark();
+    {
+        constexpr int kTpr = 4 / kTiles;
+        static_assert(kRowsPad * kTpr == kThreads, "every thread has a share of a row");
+        const int r = tid / kTpr, sub = tid % kTpr;
+        const float2 mz = merge_row_partials<kTpr>(reinterpret_cast<const float2 *>(a.part) + (long long)unit * a.chunks * d.GW,
+                                                   a.chunks, d.GW, r, sub);
+        if (sub == 0) {
+            row_c[r] = r < d.GW ? -(weighted<kD>() ? mz.x : mz.x + log2f(mz.y)) : -INFINITY;
+            if (weighted<kD>()) row_w[r] = r < d.GW ? 1.0f / mz.y : 0.f;
+        }
+    }
+    __syncthreads();
+    pc.mark();
+
+    // ---- emission: D = K Q^T, the prefix tiles from the last to the first ----
+    if (alive && n_emit > 0) {
+        bool ok = true, issued_ok = true;
+        const int n_cols = (d.GW + 31) & ~31, n_batches = ceil_div(n_emit, kGroups), batch0 = batch;
+        const uint32_t idesc = umma_idesc_bf16(128, n_cols);
+        auto issue = [&](int q) {
+            const int bt = batch0 + q;
+            for (int g = 0; g < kGroups && q * kGroups + g < n_emit && issued_ok; ++g) {
+                const int t = n_emit - 1 - (q * kGroups + g);
+                issued_ok = tile_landed(t);
+                if (!issued_ok) break;
+                tc_fence_after();
+                const uint32_t kt = base_s + lay.tiles + t * kTile, out = tmem + ((bt & 1) * kGroups + g) * kBufCols;
+#pragma unroll
+                for (int k = 0; k < kD / 16; ++k)
+                    umma_bf16(out, umma_desc_sw128(kt + (k >> 2) * kHalfBytes + (k & 3) * 32),
+                              umma_desc_sw128(base_s + (k >> 2) * (kRowsPad * 128) + (k & 3) * 32), idesc, k > 0);
+            }
+            if (issued_ok) umma_commit(bar_done + 8 * (bt & 1));
+        };
+        if (tid == 0) {
+            tc_fence_after();
+            issue(0);
+            if (n_batches > 1) issue(1);
+        }
+        const int grp = set / kSets, part = set % kSets;
+        const int n_slices = (d.GW + 31) >> 5, s_begin = (part * n_slices) / kSets, s_end = ((part + 1) * n_slices) / kSets;
+        const uint64_t scale2 = pack2(scale, scale);
+        float *xchg = reinterpret_cast<float *>(scratch);                 // [2][kGroups][kSets][128]
+        for (int q = 0; q < n_batches; ++q) {
+            ok = batch_done(batch);
+            float acc[2] = {0.f, 0.f};
+            if (ok && q * kGroups + grp < n_emit) {
+                tc_fence_after();
+                const uint32_t from = tmem_lane + ((batch & 1) * kGroups + grp) * kBufCols + s_begin * 32;
+                uint32_t raw[2][32];
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    if (s_begin + c < s_end) tmem_ld32_issue(from + c * 32, raw[c]);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (s_begin + c >= s_end) continue;
+                    tmem_ld_fence(raw[c]);
+                    float v[32];
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(raw[c][e]);
+                    const ulonglong2 *c4 = reinterpret_cast<const ulonglong2 *>(row_c + (s_begin + c) * 32);
+                    const ulonglong2 *w4 = reinterpret_cast<const ulonglong2 *>(row_w + (s_begin + c) * 32);
+                    acc[c] = ex2_sum32<poly_pairs<kD>(), weighted<kD>()>(v, scale2, [&](int i) { return c4[i]; },
+                                                                         [&](int i) { return w4[i]; });
+                }
+            }
+            float *x = xchg + (batch & 1) * (4 * 128);
+            x[(grp * kSets + part) * 128 + quad * 32 + lane] = s_end - s_begin == 2 ? acc[0] + acc[1] : acc[0];
+            tc_fence_before();
+            alive = __syncthreads_and(ok && issued_ok ? 1 : 0) != 0;
+            if (!alive) break;
+            if (tid == 0) {
+                tc_fence_after();
+                if (q + 2 < n_batches) issue(q + 2);
+            }
+            if (tid < kGroups * 128 && q * kGroups + tid / 128 < n_emit) {
+                const int t = n_emit - 1 - (q * kGroups + tid / 128), key = tid & 127;
+                const float *xs = x + (tid / 128) * kSets * 128 + key;
+                mass[t * kTileKeys + key] = kSets == 4 ? (xs[0] + xs[128]) + (xs[256] + xs[384]) : xs[0] + xs[128];
+            }
+            ++batch;
+        }
+    }
+    if (!alive)
+        for (int i = tid; i < n_local; i += kThreads) mass[i] = 0.f;
+    pc.mark();
+
+    // ---- the row of masses, pooled: every CTA its own copy ----
+    auto peer = [&](auto *x, int p) { return p == rank ? x : cl.map_shared_rank(x, p); };
+    auto unit_sync = [&]() { if (C > 1) cl.sync(); else __syncthreads(); };
+    unit_sync();
+    const int half = (d.kp - 1) / 2;
+    {
+        float *raw = reinterpret_cast<float *>(scratch);                  // [N]
+        for (int p = 0; p < C; ++p) {
+            const int from = start[p], n = min(start[p + 1], N) - from;
+            const float *m = peer(mass, p);
+            for (int i = tid; i < n; i += kThreads) raw[from + i] = m[i];
+        }
+        __syncthreads();
+        for (int i = tid; i < N; i += kThreads) {
+            float best;
+            if (d.pool_avg) {
+                best = i >= half ? raw[i - half] : 0.f;
+                for (int t = 1 - half; t <= half; ++t) best += i + t >= 0 && i + t < N ? raw[i + t] : 0.f;
+                if (d.kp > 1) best /= (float)(2 * half + 1);
+            } else {
+                best = raw[i];
+                for (int j = max(i - half, 0); j <= min(i + half, N - 1); ++j) best = fmaxf(best, raw[j]);
+            }
+            row[i] = best;
+        }
+        __syncthreads();
+    }
+    const int s0 = (int)((long long)N * rank / C), s1 = (int)((long long)N * (rank + 1) / C);      // this CTA's share of what is written
+    if (a.scores_only)
+        for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
+    pc.mark();
+
+    uint8_t *region = gen + lay.tiles;                                    // once the sweeps are over
+    if (a.has_graph && !a.scores_only) {
+        // ---- Eq. 2 ----
+        const int k = d.K_src;
+        {
+            const rf::Threshold th = rf::block_threshold(row, N, (uint32_t)k, 0u, 0u, hist, wcnt, misc);
+            uint32_t gt, eq;
+            rf::kept_counts(row, N, th, gt, eq);
+            rf::kept_prefix(wcnt, gt, eq);
+            rf::emit_kept(row, N, th, gt, eq, [&](int t, int i) {
+                src_pos[t] = i;
+                if (rank == 0) a.src_out[(long long)unit * k + t] = i;
+            });
+        }
+        __syncthreads();
+        pc.mark();
+
+        // ---- Eq. 1: the sources' rows as an operand, all tiles against them ----
+        constexpr int kPieces = kD / 8;
+        const int np = a.np;
+        const __nv_bfloat16 *Kh = a.K + b * d.ks[0] + (long long)h * d.ks[1];
+        for (int i = tid; i < np * kPieces; i += kThreads) {
+            const int r = i / kPieces, c16 = i % kPieces;
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (r < k) v = *reinterpret_cast<const uint4 *>(Kh + (long long)src_pos[r] * d.ks[2] + c16 * 8);
+            *reinterpret_cast<uint4 *>(gen + sw128_offset(np, r, c16)) = v;
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            float n2 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float lo = __uint_as_float(w[q] << 16), hi = __uint_as_float(w[q] & 0xffff0000u);
+                n2 = fmaf(lo, lo, fmaf(hi, hi, n2));
+            }
+#pragma unroll
+            for (int o = kPieces / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+            if (c16 == 0) src_inv[r] = 1.0f / fmaxf(sqrtf(n2), kNormEps);
+        }
+        fence_proxy_async();
+        __syncthreads();
+        bool ok = true;
+        static_assert(kMaxTiles <= 4, "a warp set per tile");
+        if (n_emit > 0 && alive) {
+            if (tid == 0) {
+                tc_fence_after();
+                for (int t = 0; t < n_emit; ++t) {
+                    const uint32_t kt = base_s + lay.tiles + t * kTile;
+#pragma unroll
+                    for (int q = 0; q < kD / 16; ++q)
+                        umma_bf16(tmem + t * np, umma_desc_sw128(kt + (q >> 2) * kHalfBytes + (q & 3) * 32),
+                                  umma_desc_sw128(base_s + (q >> 2) * (np * 128) + (q & 3) * 32), umma_idesc_bf16(128, np), q > 0);
+                }
+                umma_commit(bar_done + 8 * (batch & 1));
+            }
+            __syncwarp();
+            // the keys' norms, a warp set per tile
+            const int t = set;
+            if (t < n_emit) {
+                ok = __all_sync(0xffffffffu, tile_landed(t));
+                if (ok) {
+                    const uint8_t *tile = gen + lay.tiles + t * kTile;
+                    float n0 = 0.f, n1 = 0.f;
+#pragma unroll
+                    for (int c16 = 0; c16 < kPieces; ++c16) {
+                        const uint4 raw = *reinterpret_cast<const uint4 *>(tile + sw128_offset(128, quad * 32 + lane, c16));
+                        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float lo = __uint_as_float(w[q] << 16), hi = __uint_as_float(w[q] & 0xffff0000u);
+                            n0 = fmaf(lo, lo, n0);
+                            n1 = fmaf(hi, hi, n1);
+                        }
+                    }
+                    inv_norm[t * kTileKeys + quad * 32 + lane] = 1.0f / fmaxf(sqrtf(n0 + n1), kNormEps);
+                }
+            }
+            ok = batch_done(batch) && ok;
+            tc_fence_before();
+            alive = __syncthreads_and(ok ? 1 : 0) != 0;
+            ++batch;
+        }
+        tc_fence_after();
+        pc.mark();
+
+        // ---- Eq. 3, first half: per source the CTA's own best edges, sixteen sources at a time, a warp each ----
+        float *cosines = reinterpret_cast<float *>(region);                                       // [16][keys]
+        unsigned long long *lists = reinterpret_cast<unsigned long long *>(cosines + max(16 * keys, 8 * (kMaxCluster + 1) * kListCap));     // [k][kListCap]
+        const int m = d.m;
+        for (int g0 = 0; g0 < k; g0 += 16) {
+            for (int t = set; t < n_emit && alive; t += 4) {
+                float v[16];
+                tmem_ld16(tmem_lane + t * np + g0, v);
+                const int i = t * kTileKeys + quad * 32 + lane, j = base + i;
+                const float inv = inv_norm[i];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    float e = kCandEmpty;
+                    if (g0 + c < k && j < N && j != src_pos[g0 + c])
+                        e = fminf(fmaxf(v[c] * inv * src_inv[g0 + c], -1.0f), 1.0f);
+                    cosines[c * keys + i] = e;
+                }
+            }
+            __syncthreads();
+            if (g0 + warp < k) {
+                const float *x = cosines + warp * keys;
+                unsigned long long *out = lists + (g0 + warp) * kListCap;
+                float bound;
+                const int n = warp_list_top(alive ? n_local : 0, m, -1.0f, [&](int i) { return x[i]; },
+                                            [&](int at, float e, int i) { out[at] = edge_key(e, base + i); }, &bound);
+                if (lane == 0) {
+                    list_n[g0 + warp] = n;
+                    list_bound[g0 + warp] = bound;
+                }
+            }
+            __syncthreads();
+        }
+        tc_fence_before();
+        unit_sync();
+        pc.mark();
+
+        // ---- Eq. 3, second half: source c is merged by CTA c % C, four warps each ----
+        // (m edges of one CTA reach its bound, so the highest of the CTAs' bounds bounds the unit's m-th edge)
+        const int fin_rows = ceil_div(k, C);
+        int *fin_j = reinterpret_cast<int *>(lists + k * kListCap);                   // [fin_rows][kMaxNeighbours]
+        float *fin_f = reinterpret_cast<float *>(fin_j + fin_rows * kMaxNeighbours);
+        constexpr int kGang = 128, kTops = kMaxCluster * kListCap;
+        const int gang = tid / kGang, gt = tid % kGang;
+        unsigned long long *all = reinterpret_cast<unsigned long long *>(cosines) + gang * (kTops + kListCap);      // [kTops] 0: no edge
+        unsigned long long *top = all + kTops;                                        // [kListCap]
+        uint32_t *top_n = misc + 8 + gang;
+        for (int c = rank + C * gang; c < k; c += C * (kThreads / kGang)) {
+            const int n_lane = lane < C ? peer(list_n, lane)[c] : 0;
+#pragma unroll
+            for (int q = 0; q < kTops / kGang; ++q) {                                 // peer 2 q + gt / 64, entry gt % 64
+                const int p = 2 * q + gt / kListCap, i = gt % kListCap, n = __shfl_sync(0xffffffffu, n_lane, p & 31);
+                all[q * kGang + gt] = p < C && i < n ? peer(lists, p)[c * kListCap + i] : 0ull;
+            }
+            rf::group_bar(1 + gang, kGang);
+            // thresholds tried by the whole gang, four edges per thread, until at most kListCap reach one
+            float bound = lane < C ? peer(list_bound, lane)[c] : -1.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) bound = fmaxf(bound, __shfl_xor_sync(0xffffffffu, bound, o));
+            float e[kTops / kGang];
+#pragma unroll
+            for (int q = 0; q < kTops / kGang; ++q) {
+                const unsigned long long key = all[q * kGang + gt];
+                e[q] = key ? rf::edge_of(key) : kCandEmpty;
+            }
+            float lo = bound, hi = 1.0f;
+            int have = kTops + 1;
+            for (int it = 0; it < 12 && have > kListCap; ++it) {
+                // (the first round counts the bound itself)
+                const float t0 = it == 0 ? lo : lo + (hi - lo) * (1.0f / 3.0f), t1 = lo + (hi - lo) * (it == 0 ? 0.5f : 2.0f / 3.0f);
+                uint32_t q2 = 0;
+#pragma unroll
+                for (int q = 0; q < kTops / kGang; ++q) q2 += (e[q] >= t0 ? 1u : 0u) + (e[q] >= t1 ? 0x10000u : 0u);
+                q2 = __reduce_add_sync(0xffffffffu, q2);
+                uint32_t *votes = reinterpret_cast<uint32_t *>(scratch) + gang * 8 + (it & 1) * 4;
+                if (lane == 0) votes[gt >> 5] = q2;
+                rf::group_bar(1 + gang, kGang);
+                const uint32_t n2 = votes[0] + votes[1] + votes[2] + votes[3];
+                const int n0 = (int)(n2 & 0xffffu), n1 = (int)(n2 >> 16);
+                if (n1 >= m) {
+                    lo = t1;
+                    have = n1;
+                } else if (n0 >= m || it == 0) {
+                    lo = t0;
+                    hi = t1;
+                    have = n0;
+                } else {
+                    hi = t0;
+                }
+            }
+            if (have > kListCap) {
+                // near-ties: one warp finds exactly the m
+                if (gt < 32) {
+                    float reached;
+                    const int n = warp_list_top(kTops, m, bound, [&](int i) { return all[i] ? rf::edge_of(all[i]) : kCandEmpty; },
+                                                [&](int at, float, int i) { top[at] = all[i]; }, &reached);
+                    if (lane == 0) *top_n = (uint32_t)n;
+                }
+            } else {
+                if (gt == 0) *top_n = 0u;
+                rf::group_bar(1 + gang, kGang);
+#pragma unroll
+                for (int q = 0; q < kTops / kGang; ++q)
+                    if (e[q] >= lo) top[atomicAdd(top_n, 1u)] = all[q * kGang + gt];
+            }
+            rf::group_bar(1 + gang, kGang);
+            const int n = (int)*top_n;                                                // at most kListCap: two threads per edge
+            const int i = gt >> 1;
+            const unsigned long long me = i < n ? top[i] : 0ull;
+            int r = 0;
+#pragma unroll 4
+            for (int u = gt & 1; u < n; u += 2) r += top[u] > me;
+            r += __shfl_xor_sync(0xffffffffu, r, 1);
+            if (i >= n) r = i;                                                        // (fewer than m edges: empty places)
+            if ((gt & 1) == 0 && r < m) {
+                int j = -1;
+                float f = 1.f;
+                if (i < n) {
+                    const float e = rf::edge_of(me);
+                    j = rf::position_of(me);
+                    f = signal_factor(e, d.lambda, d.T, d.signal);
+                    a.nbr_idx[((long long)unit * k + c) * m + r] = j;
+                    a.nbr_e[((long long)unit * k + c) * m + r] = e;
+                }
+                fin_j[(c / C) * kMaxNeighbours + r] = j;
+                fin_f[(c / C) * kMaxNeighbours + r] = f;
+            }
+            rf::group_bar(1 + gang, kGang);
+        }
+        unit_sync();
+        pc.mark();
+
+        // ---- Eq. 5: every CTA applies the unit's lists to its copy of the row, sources in order ----
+        int *nb_j = reinterpret_cast<int *>(fin_f + fin_rows * kMaxNeighbours);       // [k m]
+        float *nb_f = reinterpret_cast<float *>(nb_j + k * m);
+        for (int p = tid; p < k * m; p += kThreads) {
+            const int c = p / m, at = (c / C) * kMaxNeighbours + p % m;
+            nb_j[p] = peer(fin_j, c % C)[at];
+            nb_f[p] = peer(fin_f, c % C)[at];
+        }
+        __syncthreads();
+        const bool evict = d.signal == GRAPHKV_SIGNAL_EVICT;
+        for (int q0 = 0; q0 < k; q0 += 4) {
+            int slot[4];
+            float f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = lane < m && q0 + u < k;
+                slot[u] = in ? nb_j[(q0 + u) * m + lane] : -1;
+                f[u] = in ? nb_f[(q0 + u) * m + lane] : 1.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (slot[u] >= 0 && (slot[u] & (kWarps - 1)) == warp) row[slot[u]] = evict ? -INFINITY : row[slot[u]] * f[u];
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        pc.mark();
+    }
+    if (C > 1) cl.barrier_arrive();                 // nothing of another CTA is read after this
+
+    if (!a.scores_only) {
+        if (a.scores)
+            for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
+        // ---- the B largest, in ascending position; a CTA takes its share of them ----
+        const int B = a.per_batch_budget ? a.budget_of[b] : d.B;
+        const rf::Threshold th = rf::block_threshold(row, N, (uint32_t)B, 0u, 0u, hist, wcnt, misc);
+        pc.mark();
+        uint32_t gt, eq;
+        rf::kept_counts(row, N, th, gt, eq);
+        rf::kept_prefix(wcnt, gt, eq);
+        const int first = B * rank / C, count = B * (rank + 1) / C - first;
+        int *kept = reinterpret_cast<int *>(region + a.region) - B;         // [count]
+        int *idx = a.idx_out + (long long)unit * d.B;
+        rf::emit_kept(row, N, th, gt, eq, [&](int t, int i) {
+            if (t >= first && t < first + count) {
+                idx[t] = i;
+                kept[t - first] = i;
+            }
+        });
+        __syncthreads();
+        pc.mark();
+        // ---- gather: the CTA's share of the kept rows and of the window rows ----
+        const int vl = a.vpr_log2, es = 2;
+        const unsigned char *k0 = a.Kb + (b * d.ks[0] + h * d.ks[1]) * es, *v0 = a.V + (b * d.vs[0] + h * d.vs[1]) * es;
+        const long long out0 = (long long)unit * (d.B + d.W);
+        const int w0 = d.W * rank / C, w1 = d.W * (rank + 1) / C, n_rows = count + (w1 - w0);
+        for (int p0 = tid; p0 < n_rows << (vl + 1); p0 += 4 * kThreads) {
+            uint4 v[4];
+            unsigned char *dst[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = p0 + u * kThreads, t = p >> (vl + 1), c = p & ((1 << vl) - 1);
+                dst[u] = nullptr;
+                if (t < n_rows) {
+                    const bool is_v = (p >> vl) & 1;
+                    const int w = w0 + (t - count);
+                    const long long from = t < count ? kept[t] : N + w, to = out0 + (t < count ? first + t : B + w);
+                    v[u] = *reinterpret_cast<const uint4 *>((is_v ? v0 + from * d.vs[2] * es : k0 + from * d.ks[2] * es) + c * 16);
+                    dst[u] = (is_v ? a.V_out : a.K_out) + ((to << vl) + c) * 16;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (dst[u]) *reinterpret_cast<uint4 *>(dst[u]) = v[u];
+        }
+    }
+    if (C > 1) cl.barrier_wait();
+    pc.mark();
+    // copies still under way after a wait that ran out land before the CTA exits
+    if (!alive) {
+        if (tid == 0) {
+            for (int t = 0; t < n_tiles; ++t) tile_landed(t);
+            atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+    pc.flush(7);
+}
+
+}  // namespace cp
+}  // namespace graphkv

@@ -8,6 +8,7 @@
 #include <mutex>
 #include <vector>
 
+#include "cluster_path.cuh"
 #include "cluster_select.cuh"
 #include "common.cuh"
 #include "decode_attn.cuh"
@@ -865,12 +866,152 @@ graphkv_status run_finish(const Dims &d, const Layout &l, int elem_bytes, const 
     return launch_status();
 }
 
+
+// ---- the whole path in one kernel (cluster_path.cuh) ------------------------------------------------
+template <int kD, int kTiles> bool cluster_path_ready()
+{
+    static std::mutex mu;
+    static signed char state[64] = {};
+    return once_per_device(mu, state, [] { return set_smem(cp::cluster_path_kernel<kD, kTiles>, kMaxSmem); });
+}
+
+// Largest power-of-two cluster size (up to 8) at which `units` clusters are all resident, one CTA per
+// SM: the device is asked once (15, 33 and 74 clusters of 8, 4 and 2 on a B200).
+int resident_cluster_size(int units)
+{
+    static std::mutex mu;
+    static int fits[64][4] = {};                    // [device][log2 C] clusters, 0: not asked yet
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lk(mu);
+    if (fits[dev][0] == 0) {
+        if (!cluster_path_ready<128, 1>()) return 0;
+        for (int q = 0; q < 4; ++q) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(1 << q);
+            cfg.blockDim = dim3(cp::kThreads);
+            cfg.dynamicSmemBytes = kMaxSmem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1 << q;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, cp::cluster_path_kernel<128, 1>, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = -1;
+            }
+            fits[dev][q] = n == 0 ? -1 : n;
+        }
+    }
+    for (int q = 3; q >= 0; --q)
+        if (fits[dev][q] >= units) return 1 << q;
+    return 0;
+}
+
+struct ClusterPathPlan {
+    bool ok;
+    int C, chunks, n_tiles, tiles, np, region;
+    size_t smem;
+};
+
+template <int kD, int kTiles> size_t cluster_path_smem(int tiles, int region, int N)
+{
+    return cp::layout<kD, kTiles>(tiles, region, N).total;
+}
+
+ClusterPathPlan cluster_path_plan(const Dims &d, const Layout &l, bool graph)
+{
+    ClusterPathPlan p{};
+    if (!d.bf16 || d.N > cp::kMaxRow || units_per_group(d) < d.units) return p;
+    for (const char *off : {"GRAPHKV_NO_CLUSTER", "GRAPHKV_FORCE_SIMT", "GRAPHKV_TAIL_SOURCES", "GRAPHKV_TWO_SCORE_KERNELS"})
+        if (env_int(off, 0)) return p;
+    if (env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) == 2) return p;
+    p.n_tiles = ceil_div(d.L, tc::kTileKeys);
+    if (graph && (d.K_src > cp::kMaxSources || d.m > cp::kMaxNeighbours || (d.reselect && d.T > 1))) return p;
+    p.C = resident_cluster_size(d.units);
+    if (p.C == 0) return p;
+    while (p.C > 1 && p.C / 2 >= p.n_tiles) p.C /= 2;
+    p.chunks = sweep_chunks(d.units, p.n_tiles, 1, l.max_parts);       // the general path's chunks
+    int tiles = 0;
+    for (int r = 0; r < p.C; ++r)
+        tiles = std::max(tiles, cp::first_tile_of_chunk(p.n_tiles, p.chunks, cp::first_chunk(p.chunks, p.C, r + 1)) -
+                                    cp::first_tile_of_chunk(p.n_tiles, p.chunks, cp::first_chunk(p.chunks, p.C, r)));
+    if (tiles > cp::kMaxTiles || p.n_tiles > cp::kMeanTiles * p.C) return p;
+    p.np = d.K_src <= 16 ? 16 : d.K_src <= 32 ? 32 : 64;
+    p.tiles = tiles;
+    p.region = cp::region_bytes(tiles * tc::kTileKeys, p.C, graph ? d.K_src : 0, graph ? d.m : 0, d.B);
+    const auto smem_of = d.D == 64 ? (d.GW <= 128 ? cluster_path_smem<64, 1> : cluster_path_smem<64, 2>)
+                                   : (d.GW <= 128 ? cluster_path_smem<128, 1> : cluster_path_smem<128, 2>);
+    p.smem = smem_of(tiles, p.region, d.N);
+    p.ok = p.smem <= kMaxSmem;
+    return p;
+}
+
+graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPathPlan &pl, const __nv_bfloat16 *Q,
+                                const __nv_bfloat16 *K, const void *V, void *K_out, void *V_out, int *idx_out, float *scores,
+                                bool scores_only, bool graph, void *ws, cudaStream_t st)
+{
+    CUtensorMap tmK;
+    if (!make_k_tensormap(&tmK, K, d, d.L)) return GRAPHKV_ERR_CUDA;
+    cp::PathArgs a{};
+    a.d = d;
+    a.Q = Q;
+    a.K = K;
+    a.C = pl.C;
+    a.chunks = pl.chunks;
+    a.n_tiles = pl.n_tiles;
+    a.tiles = pl.tiles;
+    a.np = pl.np;
+    a.region = pl.region;
+    a.part = at<float>(ws, l.part);
+    a.status = at<int>(ws, l.status);
+    a.scores = scores;
+    a.scores_only = scores_only;
+    a.has_graph = graph;
+    if (!scores_only) {
+        a.src_out = at<int>(ws, l.src);
+        a.nbr_idx = at<int>(ws, l.nbr_idx);
+        a.nbr_e = at<float>(ws, l.nbr_e);
+        a.idx_out = idx_out;
+        a.vpr_log2 = d.D == 64 ? 3 : 4;
+        a.Kb = reinterpret_cast<const unsigned char *>(K);
+        a.V = static_cast<const unsigned char *>(V);
+        a.K_out = static_cast<unsigned char *>(K_out);
+        a.V_out = static_cast<unsigned char *>(V_out);
+        if (t_budgets) {
+            a.per_batch_budget = 1;
+            for (int i = 0; i < d.batch; ++i) a.budget_of[i] = t_budgets[i];
+        }
+    }
+    a.wait_cycles = wait_cycles();
+    a.withhold_commit = env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0);
+    auto launch = [&](auto kern, bool ready) -> graphkv_status {
+        if (!ready) return GRAPHKV_ERR_CUDA;
+        // (its first step past the set-up is to wait for what the stream held before, so it may be launched early)
+        t_launches_in_call = 1;
+        return launch_ex("cluster_path", kern, dim3(d.units * pl.C), dim3(cp::kThreads), pl.smem, st,
+                         next_launch_is_dependent(), pl.C, tmK, a);
+    };
+    if (d.D == 64)
+        return d.GW <= 128 ? launch(cp::cluster_path_kernel<64, 1>, cluster_path_ready<64, 1>())
+                           : launch(cp::cluster_path_kernel<64, 2>, cluster_path_ready<64, 2>());
+    return d.GW <= 128 ? launch(cp::cluster_path_kernel<128, 1>, cluster_path_ready<128, 1>())
+                       : launch(cp::cluster_path_kernel<128, 2>, cluster_path_ready<128, 2>());
+}
+
 // ---- the calls, typed ---------------------------------------------------------------------------
 
 template <typename T>
 graphkv_status do_score(const Dims &d, const Layout &l, const T *Q, const T *K, float *scores,
                         void *ws, cudaStream_t st)
 {
+    if constexpr (sizeof(T) == 2) {
+        const ClusterPathPlan pl = cluster_path_plan(d, l, false);
+        if (pl.ok) return run_cluster_path(d, l, pl, Q, K, nullptr, nullptr, nullptr, nullptr, scores, true, false, ws, st);
+    }
     float *a = d.kp > 1 ? at<float>(ws, l.a) : scores;
     graphkv_status rc = run_mass(d, l, Q, K, a, ws, st);
     if (rc != GRAPHKV_OK || d.kp == 1) return rc;
@@ -918,6 +1059,11 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
                            cudaStream_t st)
 {
     const bool graph = graph_active(d);
+    if constexpr (sizeof(T) == 2) {
+        const ClusterPathPlan pl = cluster_path_plan(d, l, graph);
+        if (pl.ok)
+            return run_cluster_path(d, l, pl, Q, K, V, K_out, V_out, idx_out, t_keep_scores ? s : nullptr, false, graph, ws, st);
+    }
     float *a = d.kp > 1 ? at<float>(ws, l.a) : s;
     int *src = at<int>(ws, l.src);
     const bool tc_graph = graph && sim_plan(d, sizeof(T) == 2).ok;

@@ -86,3 +86,38 @@ def test_select_by_candidates(gk, values, n, budget, heads):
         assert torch.equal(idx[0, h].cpu().long(), want)
         rows = torch.cat([want, torch.arange(n, n + 3)])
         assert torch.equal(K_out[0, h].cpu().view(torch.int16), K[0, h, rows].view(torch.int16))
+
+
+# the one-kernel path for short rows against the general kernels (forced by a switch), to the bit: rows of
+# one token, of whole tiles and just past them, the longest it takes; one to 74 units (clusters of 8 to 2);
+# no sources, one, the most; ties of every key; mean pooling, evicted signal, window-only last tiles
+@pytest.mark.parametrize("n,w,g,hkv,batch,k,m,over", [
+    (1, 1, 1, 1, 1, 0, 0, {}), (2, 5, 2, 1, 1, 1, 1, {}), (127, 1, 1, 2, 1, 5, 3, {}), (128, 32, 4, 8, 1, 16, 32, {}),
+    (500, 12, 4, 2, 2, 64, 4, {}), (1003, 32, 4, 8, 1, 16, 32, {}), (1003, 64, 4, 8, 1, 33, 8, {"pool_mode": 1}),
+    (2300, 32, 4, 8, 1, 40, 32, {"signal": 2}), (3000, 32, 4, 8, 1, 16, 16, {"rounds": 0}), (3000, 32, 4, 8, 1, 16, 16, {"same": True}),
+    (1400, 64, 4, 8, 4, 16, 7, {"signal": 1}), (700, 8, 4, 37, 2, 9, 9, {}), (900, 16, 4, 8, 1, 16, 32, {"head_dim": 64})])
+def test_short_rows_in_one_kernel(gk, monkeypatch, n, w, g, hkv, batch, k, m, over):
+    cfg = wl.scaled(wl.LLAMA_32K, n_prefix=n, window=w, n_q_heads=g * hkv, n_kv_heads=hkv, batch=batch, n_clusters=16,
+                    head_dim=over.get("head_dim", 128))
+    inp = wl.make_inputs(cfg)
+    if over.get("same"):
+        inp["K"][:] = inp["K"][:, :, :1]
+    Q, K, V = (inp[x].to(DEV) for x in ("Qw", "K", "V"))
+    p = gk.make_params(K, Qw=Q, V=V, window=w, budget=max(1, n // 5), pool_kernel=7, topk_nodes=k, neighbors=m,
+                       rounds=over.get("rounds", 2), signal=over.get("signal", 0), pool_mode=over.get("pool_mode", 0))
+    ws = gk.alloc_workspace(p, DEV)
+    got = gk.alloc_outputs(p, K)
+    launches = gk.graphkv_launch_count()
+    gk.graphkv_compress(p, Q, K, V, *got, ws)
+    assert gk.graphkv_launch_count() == launches + 1
+    assert gk.graphkv_read_status(ws) == gk.OK
+    score = torch.empty_like(got[3])
+    gk.graphkv_score(p, Q, K, score, ws)
+    monkeypatch.setenv("GRAPHKV_TWO_SCORE_KERNELS", "1")
+    want = gk.alloc_outputs(p, K)
+    gk.graphkv_compress(p, Q, K, V, *want, ws)
+    for a, b in zip(got, want):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+    want_score = torch.empty_like(score)
+    gk.graphkv_score(p, Q, K, want_score, ws)
+    assert torch.equal(score, want_score)
