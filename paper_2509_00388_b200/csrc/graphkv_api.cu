@@ -312,16 +312,18 @@ template <typename T> inline T *at(void *ws, size_t off)
 }
 
 // ---- launches with attributes -------------------------------------------------------------------
-// Kernels of one API call after the first are launched with programmatic stream serialization:
-// their prologue (barriers, TMEM, operand staging, the first key tiles) overlaps the tail of the
-// kernel before, and they execute griddepcontrol.wait before touching anything an earlier kernel
-// of the call wrote.
+// Every kernel is launched with programmatic stream serialization: its prologue (barriers, TMEM and,
+// after the first launch of a call, operand staging and the first key tiles) overlaps the tail of the
+// kernel before, and it executes griddepcontrol.wait before touching anything an earlier kernel of
+// the call wrote.  The first launch of a call waits before it touches its inputs as well: whatever
+// the stream held before the call may have written them.
 thread_local int t_launches_in_call = 0;
 
-inline bool next_launch_is_dependent()
+inline bool next_launch_is_dependent(int *first = nullptr)
 {
     static const bool enabled = [] { const char *v = getenv("GRAPHKV_PDL"); return v ? atoi(v) != 0 : true; }();
-    const bool dep = enabled && t_launches_in_call > 0 && !g_trace_on.load(std::memory_order_relaxed);
+    const bool dep = enabled && !g_trace_on.load(std::memory_order_relaxed);
+    if (first) *first = t_launches_in_call == 0 ? 1 : 0;
     ++t_launches_in_call;
     return dep;
 }
@@ -533,7 +535,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
         const int chunks_e = sweep_chunks(nu, tiles_emit, 1, l.max_parts);
         tc::ScoreTcArgs sa{d, Q, at<float>(ws, l.part), at<float>(ws, l.row_c), at<int>(ws, l.arrivals), a,
                            ex.global_hist ? at<uint32_t>(ws, l.a_hist) : nullptr, at<int>(ws, l.status), u0,
-                           chunks_s, tiles_stats, chunks_s, stages, 0,
+                           chunks_s, tiles_stats, chunks_s, stages, 0, 0,
                            tc::SourceArgs{0, 0, nullptr, nullptr, nullptr, 0, 0}, nullptr, 0, 0,
                            wait_cycles(), 0, 0u, env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0)};
         tc::ScoreTcArgs ea = sa;
@@ -555,7 +557,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
             fa.n_tiles = tiles_stats;
             fa.clear_head = 1;
             fa.call_tag = next_call_tag();
-            fa.wait_prior = next_launch_is_dependent();
+            fa.wait_prior = next_launch_is_dependent(&fa.first);
             t_cooperative = true;
             rc = launch_ex("score_fused_tc", row_tiles == 1 ? tc::score_fused_tc<1, kD> : tc::score_fused_tc<2, kD>,
                            dim3(chunks_s, nu), dim3(tc::kScoreThreads), smem, st, fa.wait_prior != 0, 1, tmK, fa);
@@ -564,7 +566,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
             if (reset_words(d, l, ws, st) != GRAPHKV_OK) return GRAPHKV_ERR_CUDA;
             rc = GRAPHKV_OK;
         }
-        sa.wait_prior = next_launch_is_dependent();
+        sa.wait_prior = next_launch_is_dependent(&sa.first);
         rc = launch_ex("score_stats_tc", row_tiles == 1 ? tc::score_stats_tc<1, kD> : tc::score_stats_tc<2, kD>,
                        dim3(chunks_s, nu), dim3(tc::kScoreThreads), smem, st, sa.wait_prior != 0, 1, tmK, sa);
         if (rc != GRAPHKV_OK) break;
@@ -990,8 +992,6 @@ graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPat
     a.withhold_commit = env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0);
     auto launch = [&](auto kern, bool ready) -> graphkv_status {
         if (!ready) return GRAPHKV_ERR_CUDA;
-        // (its first step past the set-up is to wait for what the stream held before, so it may be launched early)
-        t_launches_in_call = 1;
         return launch_ex("cluster_path", kern, dim3(d.units * pl.C), dim3(cp::kThreads), pl.smem, st,
                          next_launch_is_dependent(), pl.C, tmK, a);
     };
@@ -1138,6 +1138,8 @@ __global__ void __launch_bounds__(256) knorm_score_kernel(Dims d, const T *__res
     const T *Kh = K + (unit / d.hkv) * d.ks[0] + (long long)(unit % d.hkv) * d.ks[1] + sub * 8;
     float *out = scores + (long long)unit * d.N;
     const int stride = (gridDim.x * blockDim.x) / kTpr;
+    pdl_wait();
+    pdl_launch_dependents();
     for (int j0 = (blockIdx.x * blockDim.x + threadIdx.x) / kTpr; j0 < d.N; j0 += 8 * stride) {
         float n2[8];
 #pragma unroll
@@ -1301,17 +1303,15 @@ graphkv_status graphkv_score_knorm(const graphkv_params *params, const void *K, 
     // about one wave of resident CTAs (eight of 256 threads per SM) over all units
     const int per_unit = std::max(1, std::min(ceil_div(d.N, 16 * 8), ceil_div(sm_count() * 8, d.units)));
     const dim3 grid(per_unit, d.units);
+    t_launches_in_call = 0;
+    auto launch = [&](auto kern, auto *keys) {
+        return launch_ex("knorm_score", kern, grid, dim3(256), 0, st, next_launch_is_dependent(), 1, d, keys, scores);
+    };
     const __nv_bfloat16 *Kb = static_cast<const __nv_bfloat16 *>(K);
     const float *Kf = static_cast<const float *>(K);
-    if (params->dtype == GRAPHKV_BF16 && d.D == 64)
-        GKV_LAUNCH("knorm_score", st, (knorm_score_kernel<__nv_bfloat16, 64><<<grid, 256, 0, st>>>(d, Kb, scores)));
-    else if (params->dtype == GRAPHKV_BF16)
-        GKV_LAUNCH("knorm_score", st, (knorm_score_kernel<__nv_bfloat16, 128><<<grid, 256, 0, st>>>(d, Kb, scores)));
-    else if (d.D == 64)
-        GKV_LAUNCH("knorm_score", st, (knorm_score_kernel<float, 64><<<grid, 256, 0, st>>>(d, Kf, scores)));
-    else
-        GKV_LAUNCH("knorm_score", st, (knorm_score_kernel<float, 128><<<grid, 256, 0, st>>>(d, Kf, scores)));
-    return launch_status();
+    if (params->dtype == GRAPHKV_BF16)
+        return d.D == 64 ? launch(knorm_score_kernel<__nv_bfloat16, 64>, Kb) : launch(knorm_score_kernel<__nv_bfloat16, 128>, Kb);
+    return d.D == 64 ? launch(knorm_score_kernel<float, 64>, Kf) : launch(knorm_score_kernel<float, 128>, Kf);
 }
 
 graphkv_status graphkv_select_gather(const graphkv_params *params, const float *scores,
@@ -1417,8 +1417,6 @@ static graphkv_status launch_decode(const DecodeArgs &a, const void *q, const vo
     static signed char state[64] = {};
     if (!once_per_device(mu, state, [] { return set_smem(decode_kernel<T, kG>, kDecSmem); }))
         return GRAPHKV_ERR_CUDA;
-    // (the kernel waits for the launches before it as its first step, so it may always be launched early)
-    t_launches_in_call = 1;
     return launch_ex("decode_attention", decode_kernel<T, kG>, dim3(a.splits, a.batch * a.hkv), dim3(kDecThreads), kDecSmem,
                      st, next_launch_is_dependent(), 1, a, static_cast<const T *>(q), static_cast<const T *>(K),
                      static_cast<const T *>(V));

@@ -50,6 +50,7 @@ struct ScoreTcArgs {
     int stats_chunks;   // key chunks of the statistics sweep (partials per row)
     int stages;         // shared-memory K tiles in flight
     int wait_prior;     // launched with programmatic stream serialization: wait for the kernels before
+    int first;          // the first launch of a call: what is before it is not this call's, so inputs wait too
     // emit sweep only: candidate lists for the source nodes of Eq. 2 at its tail (src.k = 0: none), and words to clear
     // for the kernels that follow
     SourceArgs src;
@@ -162,7 +163,7 @@ __device__ __forceinline__ uint32_t score_setup(const ScoreSmem &s, uint8_t *gen
 }
 
 // TMA producer (one thread): key tiles t0+i of (h, b), i in [i_begin, i_end), into the stage ring.
-// The keys are an input of the call, so the producer never waits for the kernels before.
+// The keys are an input of the call, so the producer waits for none of the call's kernels before.
 template <int kD>
 __device__ __forceinline__ bool score_produce(const ScoreSmem &s, const CUtensorMap *tmK, int stages,
                                               int t0, int i_begin, int i_end, int h, int b, long long lim)
@@ -269,6 +270,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 
     const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kGroups);
     bool ok = true;
+    if (a.first && a.wait_prior) pdl_wait();
     if (warp == 0) {
         if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
     } else {
@@ -276,7 +278,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         fence_proxy_async();
     }
     pc.mark();
-    if (a.wait_prior) pdl_wait();
+    if (a.wait_prior && !a.first) pdl_wait();
     pc.mark();
     pdl_launch_dependents();
     __syncthreads();
@@ -441,6 +443,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const int n_ahead = min(n_local, a.stages);
     const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kGroups);
     bool ok = true;
+    if (a.first && a.wait_prior) pdl_wait();
     if (warp == 0) {
         if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
     } else {
@@ -448,7 +451,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         fence_proxy_async();
     }
     pc.mark();
-    if (a.wait_prior) pdl_wait();
+    if (a.wait_prior && !a.first) pdl_wait();
     pc.mark();
     pdl_launch_dependents();
     const bool want_hist = a.a_hist != nullptr || a.local_hist;
@@ -638,6 +641,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 
     const uint32_t tmem_base = score_setup(s, gen, &tmK, S, kTmemCols, kEpiWarps / kGroups);
     bool ok = true;
+    if (a.first && a.wait_prior) pdl_wait();
     if (warp == 0) {
         if (lane == 0) ok = score_produce<kD>(s, &tmK, S, t0, 0, n_ahead, h, b, lim);
     } else {
@@ -645,7 +649,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         fence_proxy_async();
     }
     pc.mark();
-    if (a.wait_prior) pdl_wait();
+    if (a.wait_prior && !a.first) pdl_wait();
     pc.mark();
     pdl_launch_dependents();
     const bool want_hist = a.a_hist != nullptr || a.local_hist;
