@@ -18,6 +18,7 @@
 // sweeps' 64 CTAs lose to the general path's 128 to 148 (two heads of 4064 tokens 49 -> 55 us).
 #pragma once
 
+#include "edge_search.cuh"
 #include "row_finish.cuh"
 #include "score_tc.cuh"
 
@@ -34,7 +35,7 @@ constexpr int kMeanTiles = 3;           // on average
 constexpr int kMaxSources = 64;
 constexpr int kMaxNeighbours = 32;
 constexpr int kMaxRow = kMaxCluster * kMeanTiles * tc::kTileKeys;    // tokens per row
-constexpr int kListCap = 64;            // listed edges per source and CTA
+constexpr int kListCap = kCandCap;      // listed edges per source and CTA
 
 struct PathArgs {
     Dims d;
@@ -97,80 +98,6 @@ __host__ __device__ inline int region_bytes(int keys, int C, int k, int m, int B
 {
     const int cosines = 16 * keys * 4, tops = 4 * (kMaxCluster + 1) * kListCap * 8;
     return ((cosines > tops ? cosines : tops) + k * kListCap * 8 + ((k + C - 1) / C) * kMaxNeighbours * 8 + k * m * 8 + B * 4 + 15) / 16 * 16;
-}
-
-// The edges of x(0 .. n) (lane-strided: element i * 32 + lane, kCandEmpty where there is none) that reach a
-// bound at which between m and kListCap of them do; with too many near-ties, exactly the m largest (lowest
-// positions first).  put(slot, e, i).  Returns their number, and in *bound a value that m of them reach (-1
-// with fewer than m).  `from`: -1, or a value that at least m of them are known to reach.  Rolled loops over
-// shared memory: the code runs once per source.
-template <typename At, typename Put>
-__device__ __forceinline__ int warp_list_top(int n, int m, float from, At x, Put put, float *bound)
-{
-    const int lane = threadIdx.x & 31;
-    // how many reach t0, t1 (packed)
-    auto reach2 = [&](float t0, float t1) {
-        uint32_t c = 0;
-#pragma unroll 4
-        for (int i = lane; i < n; i += 32) {
-            const float e = x(i);
-            c += (e >= t0 ? 1u : 0u) + (e >= t1 ? 0x10000u : 0u);
-        }
-        return __reduce_add_sync(0xffffffffu, c);
-    };
-    float lo = from, hi = 1.0f;
-    const float half = from + 0.5f * (1.0f - from);
-    uint32_t c = reach2(from, half);
-    int have = (int)(c & 0xffffu);
-    *bound = -1.0f;
-    if ((int)(c >> 16) >= m) lo = half, have = (int)(c >> 16);
-    else hi = half;
-    for (int it = 0; have > kListCap && it < 16; ++it) {
-        const float t0 = lo + (hi - lo) * (1.0f / 3.0f), t1 = lo + (hi - lo) * (2.0f / 3.0f);
-        c = reach2(t0, t1);
-        if ((int)(c >> 16) >= m) {
-            lo = t1;
-            have = (int)(c >> 16);
-        } else if ((int)(c & 0xffffu) >= m) {
-            lo = t0;
-            hi = t1;
-            have = (int)(c & 0xffffu);
-        } else {
-            hi = t0;
-        }
-    }
-    if (have >= m) *bound = lo;
-    uint32_t exact = 0;                         // with too many near-ties: the key of the m-th largest
-    int ties = 0;                               // and how many of its ties belong to the m
-    if (have > kListCap) {
-        uint32_t klo = float_to_key(lo), khi = float_to_key(1.0f) + 1u;
-        while (khi - klo > 1u) {
-            const uint32_t mid = klo + (khi - klo) / 2u;
-            uint32_t q = 0;
-            for (int i = lane; i < n; i += 32) q += float_to_key(x(i)) >= mid;
-            if ((int)__reduce_add_sync(0xffffffffu, q) >= m) klo = mid;
-            else khi = mid;
-        }
-        exact = klo;
-        uint32_t q = 0;
-        for (int i = lane; i < n; i += 32) q += float_to_key(x(i)) > exact;
-        ties = m - (int)__reduce_add_sync(0xffffffffu, q);
-    }
-    int at = 0;
-    for (int i0 = 0; i0 < n; i0 += 32) {
-        const float e = i0 + lane < n ? x(i0 + lane) : kCandEmpty;
-        bool keep = e >= lo;
-        if (exact) {
-            const uint32_t key = float_to_key(e);
-            const unsigned eq = __ballot_sync(0xffffffffu, key == exact);
-            keep = key > exact || (key == exact && __popc(eq & ((1u << lane) - 1u)) < ties);
-            ties -= min(ties, __popc(eq));
-        }
-        const unsigned bm = __ballot_sync(0xffffffffu, keep);
-        if (keep) put(at + __popc(bm & ((1u << lane) - 1u)), e, i0 + lane);
-        at += __popc(bm);
-    }
-    return at;
 }
 
 // kTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid = units * C CTAs in clusters of C.

@@ -44,8 +44,6 @@ struct Layout {
     size_t nbr_e;
     size_t cand;        // per-chunk neighbour candidates [units][K_src][sim_chunks][kCandCap]
     size_t cand_hist;   // [units][K_src][kCandBins]
-    size_t src_cand;    // elements the emit sweep lists for the source selection [units][max_parts][kSrcCap]
-    size_t src_cnt;     // [units][max_parts]
     size_t total;
     int max_parts;      // partial statistics per row the region can hold
 };
@@ -204,17 +202,17 @@ SimPlan sim_plan(const Dims &d, bool bf16)
         return p;
     if (env_int("GRAPHKV_FORCE_SIMT", 0)) return p;
     if (!cluster_plan(d).ok) return p;          // its candidate lists are merged by the cluster kernel
-    // 64 sources per sweep leave a CTA 8 key tiles (the tensor memory holds 512 columns): four keys per
-    // epilogue thread, of which the m + 1 best maxima set each source's threshold.  With more than 16
-    // neighbours the chunk's candidates then crowd its 64-entry lists and the threads' queues, and
-    // overflows take the slow exact path (450 sources, m = 32 at 32K keys: 2.1 ms against 0.35 ms);
-    // 32 sources per sweep (16 tiles, eight keys per thread) stay clear of it and measured faster
-    // there at every source count, 64 faster for m = 16.
-    p.NP = d.K_src <= 16 ? 16 : (d.K_src <= 32 || d.m > 16 ? 32 : 64);
-    p.stages = d.D == 64 ? 8 : p.NP == 64 ? 4 : 5;      // (at least 80 KB: the queues take the ring's place after the sweep)
-    const int cap = 512 / p.NP;
+    // Sources per sweep when there are more than 32.  The tensor memory (512 columns) holds 8 key tiles of 64
+    // sources or 16 of 32.  Where 8 tiles per CTA are enough to take the rows in one wave, 64 halve the
+    // sweeps and their fixed cost (64 sources: 25 us against 31 at 8K keys x 8 heads, 33 against 39 at
+    // 16K).  Beyond that the CTAs of 64 queue for the SMs and their maxima, of half as many keys, bound
+    // the neighbours less tightly (50 us against 56 at 32K x 8, 154 sources 111 against 158, 64 sources
+    // at 128K x 32: 617 against 721).
     const int group = units_per_group(d);
-    p.chunks = sweep_chunks(group, p.n_tiles, ceil_div(p.n_tiles, cap), 1 << 20);
+    p.NP = d.K_src <= 16 ? 16 : d.K_src <= 32 || (long long)group * ceil_div(p.n_tiles, 8) > sm_count() ? 32 : 64;
+    p.stages = d.D == 64 ? 8 : 5;
+    const int cap = 512 / p.NP;
+    p.chunks = sweep_chunks(group * ceil_div(d.K_src, p.NP), p.n_tiles, ceil_div(p.n_tiles, cap), 1 << 20);
     p.ok = true;
     return p;
 }
@@ -244,9 +242,6 @@ Layout layout_of(const Dims &d)
     const size_t slots = sp.ok ? (size_t)d.units * d.K_src * sp.chunks : 1;
     l.cand = take(slots * kCandCap * sizeof(Cand));
     l.cand_hist = take((size_t)d.units * (d.K_src > 0 ? d.K_src : 1) * kCandBins * sizeof(uint32_t));
-    const bool tail = d.bf16 && d.K_src > 0 && d.K_src <= tc::kSrcMaxK;
-    l.src_cand = take(tail ? (size_t)d.units * l.max_parts * tc::kSrcCap * sizeof(tc::SrcCand) : kAlign);
-    l.src_cnt = take(tail ? (size_t)d.units * l.max_parts * sizeof(int) : kAlign);
     l.total = off;
     return l;
 }
@@ -487,16 +482,10 @@ bool make_k_tensormap(CUtensorMap *tm, const void *K, const Dims &d, int rows, c
 }
 
 
-// What the emit sweep does besides the attention mass: the source nodes of Eq. 2 at its tail
-// (k > 0), words cleared for the kernels that follow, the unit's mass histogram for a pooling
-// kernel that follows.
+// What the sweeps do besides the attention mass: words cleared for the kernels that follow.
 struct EmitExtras {
-    int k;
-    int *list_chunks;   // out: candidate lists per unit the emit sweep leaves (its key chunks)
-    int *src_out;
     uint32_t *zero;
     int zero_words;
-    bool global_hist;
 };
 
 // Attention mass before pooling, a [units][N], tensor-core path (bf16).
@@ -525,7 +514,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     graphkv_status rc = GRAPHKV_OK;
     // the kernel of both sweeps (one launch of all units, all CTAs resident) clears the head of the
     // workspace itself; every other form gets a memset first
-    const bool one_kernel = ex.k == 0 && group >= d.units &&
+    const bool one_kernel = group >= d.units &&
                             d.units * sweep_chunks(d.units, tiles_stats, 1, l.max_parts) <= sm_count() &&
                             !env_int("GRAPHKV_TWO_SCORE_KERNELS", 0);
     if (!one_kernel && reset_words(d, l, ws, st) != GRAPHKV_OK) return GRAPHKV_ERR_CUDA;
@@ -534,19 +523,14 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
         const int chunks_s = sweep_chunks(nu, tiles_stats, 1, l.max_parts);
         const int chunks_e = sweep_chunks(nu, tiles_emit, 1, l.max_parts);
         tc::ScoreTcArgs sa{d, Q, at<float>(ws, l.part), at<float>(ws, l.row_c), at<int>(ws, l.arrivals), a,
-                           ex.global_hist ? at<uint32_t>(ws, l.a_hist) : nullptr, at<int>(ws, l.status), u0,
+                           at<uint32_t>(ws, l.a_hist), at<int>(ws, l.status), u0,
                            chunks_s, tiles_stats, chunks_s, stages, 0, 0,
-                           tc::SourceArgs{0, 0, nullptr, nullptr, nullptr, 0, 0}, nullptr, 0, 0,
-                           wait_cycles(), 0, 0u, env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0)};
+                           nullptr, 0, wait_cycles(), 0, 0u, env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0)};
         tc::ScoreTcArgs ea = sa;
         ea.chunks = chunks_e;
         ea.n_tiles = tiles_emit;
-        ea.src = tc::SourceArgs{ex.k, (d.kp - 1) / 2, ex.src_out, at<tc::SrcCand>(ws, l.src_cand),
-                                at<int>(ws, l.src_cnt), l.max_parts, chunks_e};
-        if (ex.list_chunks) *ex.list_chunks = chunks_e;
         ea.zero = ex.zero;
         ea.zero_words = ex.zero_words;
-        ea.local_hist = ex.k > 0 ? 1 : 0;
         // one kernel for both sweeps when all its CTAs are resident at once (one per SM): the CTAs
         // of a unit wait for one another between the passes, so the launch is a cooperative one
         // (the device starts the grid only when all of it fits beside whatever else is running);
@@ -577,7 +561,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     return rc;
 }
 
-constexpr EmitExtras kPlainEmit{0, nullptr, nullptr, nullptr, 0, true};
+constexpr EmitExtras kPlainEmit{nullptr, 0};
 
 inline bool tc_mass(const __nv_bfloat16 *, const Dims &d) { (void)d; return !env_int("GRAPHKV_FORCE_SIMT", 0); }
 inline bool tc_mass(const float *, const Dims &) { return false; }
@@ -665,17 +649,15 @@ graphkv_status launch_similarity(const CUtensorMap &tmK, const tc::SimTcArgs &sa
 {
     static std::mutex mu;
     static signed char state[64] = {};
-    if (!once_per_device(mu, state, [] { return set_smem(tc::similarity_tc<NP, kD>, tc::sim_smem_bytes<NP, kD>(kD == 64 ? 8 : NP == 64 ? 4 : 5)); }))
+    if (!once_per_device(mu, state, [] { return set_smem(tc::similarity_tc<NP, kD>, tc::sim_smem_bytes<NP, kD>()); }))
         return GRAPHKV_ERR_CUDA;
-    return launch_ex("similarity_tc", tc::similarity_tc<NP, kD>, grid, block, tc::sim_smem_bytes<NP, kD>(sa.stages), st,
+    return launch_ex("similarity_tc", tc::similarity_tc<NP, kD>, grid, block, tc::sim_smem_bytes<NP, kD>(), st,
                      sa.wait_prior != 0, 1, tmK, sa);
 }
 
-// `merge` (optional): the sources are still candidate lists the emit sweep left; the similarity
-// sweep merges them (tensor-core path, one sweep of at most 64 sources).
 template <typename T>
 graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &eo, const int *src, void *ws,
-                         cudaStream_t st, const tc::SourceArgs *merge = nullptr, const float *a_mass = nullptr)
+                         cudaStream_t st)
 {
     const SimPlan sp = sim_plan(d, sizeof(T) == 2);
     if (sp.ok) {
@@ -687,8 +669,7 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
             // one launch takes every source: grid.z counts the sweeps of sp.NP sources each
             tc::SimTcArgs sa{d, reinterpret_cast<const __nv_bfloat16 *>(eo.S), {eo.ss[0], eo.ss[1], eo.ss[2]}, src, at<Cand>(ws, l.cand),
                              at<uint32_t>(ws, l.cand_hist), at<int>(ws, l.status), u0, sp.chunks,
-                             sp.n_tiles, sp.stages, 0, wait_cycles(),
-                             merge ? *merge : tc::SourceArgs{0, 0, nullptr, nullptr, nullptr, 0, 0}, a_mass};
+                             sp.n_tiles, sp.stages, 0, wait_cycles()};
             sa.wait_prior = next_launch_is_dependent();
             const dim3 grid(sp.chunks, nu, ceil_div(d.K_src, sp.NP)), block(tc::kSimThreads);
             const auto launch = d.D == 64 ? (sp.NP == 16 ? launch_similarity<16, 64> : sp.NP == 32 ? launch_similarity<32, 64>
@@ -928,7 +909,7 @@ ClusterPathPlan cluster_path_plan(const Dims &d, const Layout &l, bool graph)
 {
     ClusterPathPlan p{};
     if (!d.bf16 || d.N > cp::kMaxRow || units_per_group(d) < d.units) return p;
-    for (const char *off : {"GRAPHKV_NO_CLUSTER", "GRAPHKV_FORCE_SIMT", "GRAPHKV_TAIL_SOURCES", "GRAPHKV_TWO_SCORE_KERNELS"})
+    for (const char *off : {"GRAPHKV_NO_CLUSTER", "GRAPHKV_FORCE_SIMT", "GRAPHKV_TWO_SCORE_KERNELS"})
         if (env_int(off, 0)) return p;
     if (env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) == 2) return p;
     p.n_tiles = ceil_div(d.L, tc::kTileKeys);
@@ -1067,23 +1048,13 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
     float *a = d.kp > 1 ? at<float>(ws, l.a) : s;
     int *src = at<int>(ws, l.src);
     const bool tc_graph = graph && sim_plan(d, sizeof(T) == 2).ok;
-    const int halo = (d.kp - 1) / 2;
-    // The tensor-core emit sweep can leave candidate lists for the sources at its tail, the
-    // similarity sweep merge them and the finishing kernel pool, which saves the pooling kernel
-    // (one sweep of at most 64 sources, one launch group, max pooling).  Measured on B200 the
-    // merge in front of every similarity CTA costs what the pooling kernel takes (32K keys: 114
-    // against 112 us per step; 131072 x 4: 1.25 against 1.13 ms), so it is off by default.
-    const bool tail_src = tc_mass(Q, d) && tc_graph && d.D == kHeadDim && d.K_src <= tc::kSrcMaxK && !d.pool_avg &&
-                          units_per_group(d) >= d.units && env_int("GRAPHKV_TAIL_SOURCES", 0);
-    const bool finish_pools = d.kp > 1 && !d.pool_avg && (tail_src || (!graph && !candidate_plan(d, false, true, false, d.B).ok)) && finish_plan(d, halo).ok &&
-                              cluster_plan(d).ok;
+    // without a graph (plain top-B) the old finishing kernel pools where the new one does not apply
+    const bool finish_pools = !graph && d.kp > 1 && !d.pool_avg && !candidate_plan(d, false, true, false, d.B).ok &&
+                              finish_plan(d, (d.kp - 1) / 2).ok && cluster_plan(d).ok;
     graphkv_status rc;
-    int list_chunks = 0;
     uint32_t *row_hist = nullptr;
-    if (tail_src || !graph) {
-        const EmitExtras ex{tail_src ? d.K_src : 0, &list_chunks, src, tail_src ? at<uint32_t>(ws, l.cand_hist) : nullptr,
-                            tail_src ? d.K_src * kCandBins : 0, false};
-        if ((rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
+    if (!graph) {
+        if ((rc = run_mass(d, l, Q, K, a, ws, st)) != GRAPHKV_OK) return rc;
         if (d.kp > 1 && !finish_pools &&
             (rc = run_pool_sources(d, a, s, 0, nullptr, nullptr, nullptr, 0, st)) != GRAPHKV_OK)
             return rc;
@@ -1109,9 +1080,7 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
         // after it start from the scores in `s`; the last pass also selects and gathers
         Dims one = d;
         one.T = 1;
-        const tc::SourceArgs merge1{d.K_src, halo, src, at<tc::SrcCand>(ws, l.src_cand), at<int>(ws, l.src_cnt),
-                                    l.max_parts, list_chunks};
-        if ((rc = run_graph(one, l, eo, src, ws, st, tail_src ? &merge1 : nullptr, a)) != GRAPHKV_OK) return rc;
+        if ((rc = run_graph(one, l, eo, src, ws, st)) != GRAPHKV_OK) return rc;
         if ((rc = run_finish(one, l, (int)sizeof(T), finish_pools ? a : nullptr, s, true, tc_graph, false,
                              nullptr, nullptr, nullptr, nullptr, nullptr, ws, st)) != GRAPHKV_OK)
             return rc;
@@ -1120,9 +1089,7 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
         return run_finish(one, l, (int)sizeof(T), nullptr, s, false, false, true, K, V, K_out, V_out, idx_out,
                           ws, st);
     }
-    const tc::SourceArgs merge{d.K_src, halo, src, at<tc::SrcCand>(ws, l.src_cand), at<int>(ws, l.src_cnt),
-                               l.max_parts, list_chunks};
-    if (graph && (rc = run_graph(d, l, eo, src, ws, st, tail_src ? &merge : nullptr, a)) != GRAPHKV_OK) return rc;
+    if (graph && (rc = run_graph(d, l, eo, src, ws, st)) != GRAPHKV_OK) return rc;
     return run_finish(d, l, (int)sizeof(T), finish_pools ? a : nullptr, s, graph, tc_graph, true, K, V,
                       K_out, V_out, idx_out, ws, st, row_hist);
 }

@@ -21,7 +21,6 @@
 // sets share a tile, the two pairs take alternate tiles and four buffers rotate).
 #pragma once
 
-#include "source_select.cuh"
 #include "tc_common.cuh"
 
 namespace graphkv {
@@ -51,12 +50,8 @@ struct ScoreTcArgs {
     int stages;         // shared-memory K tiles in flight
     int wait_prior;     // launched with programmatic stream serialization: wait for the kernels before
     int first;          // the first launch of a call: what is before it is not this call's, so inputs wait too
-    // emit sweep only: candidate lists for the source nodes of Eq. 2 at its tail (src.k = 0: none), and words to clear
-    // for the kernels that follow
-    SourceArgs src;
-    uint32_t *zero;     // optional [units][zero_words]
+    uint32_t *zero;     // optional [units][zero_words]: words to clear for the kernels that follow
     int zero_words;
-    int local_hist;     // build the per-CTA mass histogram even without a_hist
     long long wait_cycles;   // limit of every wait of the kernel, in clocks
     int clear_head;          // kernel of both sweeps: clear the status word and the unit's mass histogram on
                              // the way (the caller then needs no memset ahead of the launch)
@@ -454,7 +449,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     if (a.wait_prior && !a.first) pdl_wait();
     pc.mark();
     pdl_launch_dependents();
-    const bool want_hist = a.a_hist != nullptr || a.local_hist;
+    const bool want_hist = a.a_hist != nullptr;
     if (want_hist)
         for (int i = threadIdx.x; i < kMassBins; i += kScoreThreads) mass_hist[i] = 0u;
     if (a.zero) {
@@ -571,7 +566,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     }
     if (!ok && a.status) atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
     tc_fence_before();
-    const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    __syncthreads();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
@@ -582,11 +577,6 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         for (int i = threadIdx.x; i < kMassBins; i += kScoreThreads)
             if (mass_hist[i]) atomicAdd(a.a_hist + (long long)unit * kMassBins + i, mass_hist[i]);
     pc.mark();
-    // Eq. 2, first half: this chunk's candidates for the unit's source nodes (the stage ring is idle
-    // by now and serves as scratch); the similarity sweep merges the lists
-    if (a.src.k > 0 && all_ok)
-        source_list_chunk(a.src, d, unit, chunk, t0 * kTileKeys, min(t1 * kTileKeys, d.N),
-                          a.a_out + (long long)unit * d.N, mass_hist, gen + (s.stage0 - s.q));
     pc.mark();
     pc.flush(1);
 }
@@ -652,7 +642,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     if (a.wait_prior && !a.first) pdl_wait();
     pc.mark();
     pdl_launch_dependents();
-    const bool want_hist = a.a_hist != nullptr || a.local_hist;
+    const bool want_hist = a.a_hist != nullptr;
     if (want_hist)
         for (int i = threadIdx.x; i < kMassBins; i += kScoreThreads) mass_hist[i] = 0u;
     if (a.clear_head) {

@@ -121,3 +121,42 @@ def test_short_rows_in_one_kernel(gk, monkeypatch, n, w, g, hkv, batch, k, m, ov
     want_score = torch.empty_like(score)
     gk.graphkv_score(p, Q, K, want_score, ws)
     assert torch.equal(score, want_score)
+
+
+# the similarity sweep beyond short rows: one tile per CTA up to all its tensor memory (4096 keys at 16 sources,
+# reached with many units), the three source paddings and several sweeps, ties that no bound separates
+@pytest.mark.parametrize("n,hkv,batch,k,m,same", [(3500, 8, 1, 16, 32, False), (4160, 8, 20, 3, 16, False), (3300, 37, 4, 17, 32, False),
+                                                  (3201, 8, 1, 64, 16, False), (3201, 2, 1, 130, 5, False), (8200, 1, 1, 16, 1, False),
+                                                  (4000, 8, 16, 20, 32, True)])
+def test_similarity_sweep_edges(gk, n, hkv, batch, k, m, same):
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    K = torch.randn((batch, hkv, n + 4, 128), generator=gen, device=DEV)
+    K += 2.0 * torch.randn((batch, hkv, 40, 128), generator=gen, device=DEV)[:, :, torch.arange(n + 4) % 40]
+    if same:
+        K[:, :, ::2] = K[:, :, :1]
+    K = K.to(torch.bfloat16)
+    s = torch.rand((batch, hkv, n), generator=gen, device=DEV)
+    p = gk.make_params(K, window=4, topk_nodes=k, neighbors=m, rounds=1)
+    ws = gk.alloc_workspace(p, DEV)
+    src = torch.empty((batch, hkv, k), dtype=torch.int32, device=DEV)
+    gk.graphkv_propagate(p, K, s, src, ws)
+    nbr = torch.empty((batch, hkv, k, m), dtype=torch.int32, device=DEV)
+    e = torch.empty((batch, hkv, k, m), dtype=torch.float32, device=DEV)
+    gk.graphkv_read_neighbors(p, ws, nbr, e)
+    assert gk.graphkv_read_status(ws) == gk.OK
+    for u in {0, batch * hkv // 2, batch * hkv - 1}:
+        b, h = divmod(u, hkv)
+        x = torch.nn.functional.normalize(K[b, h, :n].double(), dim=1)
+        cos = x[src[b, h].long()] @ x.T
+        cos.scatter_(1, src[b, h].long()[:, None], -2.0)
+        want, at = cos.topk(m + 1, dim=1)
+        got = cos.gather(1, nbr[b, h].long())
+        assert torch.all(got >= want[:, m - 1:m] - 4e-6)             # members of the m largest, up to near-ties
+        assert torch.all((got - e[b, h].double()).abs() <= 4e-6)
+        assert all(len(set(r)) == m for r in nbr[b, h].tolist())
+        if same:                                                     # equal cosines: the lowest positions
+            even = src[b, h] % 2 == 0
+            first = torch.arange(0, 2 * (m + 1), 2, device=DEV)
+            for i in torch.nonzero(even).flatten().tolist():
+                low = first[first != src[b, h, i]][:m]
+                assert sorted(nbr[b, h, i].tolist()) == low.tolist()
