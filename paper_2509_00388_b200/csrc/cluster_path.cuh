@@ -287,8 +287,9 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         constexpr int kTpr = 4 / kTiles;
         static_assert(kRowsPad * kTpr == kThreads, "every thread has a share of a row");
         const int r = tid / kTpr, sub = tid % kTpr;
-        const float2 mz = merge_row_partials<kTpr>(reinterpret_cast<const float2 *>(a.part) + (long long)unit * a.chunks * d.GW,
-                                                   a.chunks, d.GW, r, sub);
+        const float2 *pu = reinterpret_cast<const float2 *>(a.part) + (long long)unit * a.chunks * d.GW;
+        const float2 mz = merge_row_partials<kTpr>([&](int q) { return __ldcg(pu + (long long)q * d.GW + r); }, a.chunks,
+                                                   d.GW, r, sub);
         if (sub == 0) {
             row_c[r] = r < d.GW ? -(weighted<kD>() ? mz.x : mz.x + log2f(mz.y)) : -INFINITY;
             if (weighted<kD>()) row_w[r] = r < d.GW ? 1.0f / mz.y : 0.f;

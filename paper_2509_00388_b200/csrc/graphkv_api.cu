@@ -500,12 +500,15 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     const int rows_pad = 128 * row_tiles;
     const int stages = row_tiles == 1 ? 5 : 4;
     const size_t smem = tc::score_smem_bytes<kD>(rows_pad, stages);
+    constexpr int kStages2 = kD == 64 ? 5 : 2;       // two CTAs per SM: what fits half its shared memory
     static std::mutex mu;
     static signed char state[64] = {};
     if (!once_per_device(mu, state, [] {
         const size_t mx = std::max(tc::score_smem_bytes<kD>(256, 4), tc::score_smem_bytes<kD>(128, 5));
-        return set_smem(tc::score_stats_tc<1, kD>, mx) && set_smem(tc::score_stats_tc<2, kD>, mx) &&
-                  set_smem(tc::score_emit_tc<1, kD>, mx) && set_smem(tc::score_emit_tc<2, kD>, mx) &&
+        const size_t two = tc::score_smem_bytes<kD>(128, kStages2, 2);
+        return set_smem(tc::score_stats_tc<1, kD, 1>, mx) && set_smem(tc::score_stats_tc<2, kD, 1>, mx) &&
+                  set_smem(tc::score_emit_tc<1, kD, 1>, mx) && set_smem(tc::score_emit_tc<2, kD, 1>, mx) &&
+                  set_smem(tc::score_stats_tc<1, kD, 2>, two) && set_smem(tc::score_emit_tc<1, kD, 2>, two) &&
                   set_smem(tc::score_fused_tc<1, kD>, mx) && set_smem(tc::score_fused_tc<2, kD>, mx);
         }))
         return GRAPHKV_ERR_CUDA;
@@ -521,7 +524,11 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     for (int u0 = 0; u0 < d.units && rc == GRAPHKV_OK; u0 += group) {
         const int nu = std::min(group, d.units - u0);
         const int chunks_s = sweep_chunks(nu, tiles_stats, 1, l.max_parts);
-        const int chunks_e = sweep_chunks(nu, tiles_emit, 1, l.max_parts);
+        // The two separate kernels run two CTAs per SM: a launch of several waves then pays for its set-ups and
+        // tails once (256 units of 16K keys: 259 -> 229 us and 255 -> 228 us for the two sweeps).  A chunk
+        // leaves four partials per row, which a launch of few units and many chunks has no room for.
+        const bool two = !one_kernel && row_tiles == 1 && 4 * chunks_s <= l.max_parts;
+        const int chunks_e = sweep_chunks(two ? ceil_div(nu, 2) : nu, tiles_emit, 1, l.max_parts);
         tc::ScoreTcArgs sa{d, Q, at<float>(ws, l.part), at<float>(ws, l.row_c), at<int>(ws, l.arrivals), a,
                            at<uint32_t>(ws, l.a_hist), at<int>(ws, l.status), u0,
                            chunks_s, tiles_stats, chunks_s, stages, 0, 0,
@@ -551,12 +558,17 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
             rc = GRAPHKV_OK;
         }
         sa.wait_prior = next_launch_is_dependent(&sa.first);
-        rc = launch_ex("score_stats_tc", row_tiles == 1 ? tc::score_stats_tc<1, kD> : tc::score_stats_tc<2, kD>,
-                       dim3(chunks_s, nu), dim3(tc::kScoreThreads), smem, st, sa.wait_prior != 0, 1, tmK, sa);
+        if (two) sa.stages = ea.stages = kStages2;
+        const dim3 block(two ? tc::score_threads<2>() : tc::kScoreThreads);
+        const size_t bytes = two ? tc::score_smem_bytes<kD>(128, kStages2, 2) : smem;
+        rc = launch_ex("score_stats_tc", two ? tc::score_stats_tc<1, kD, 2> : row_tiles == 1 ? tc::score_stats_tc<1, kD, 1>
+                       : tc::score_stats_tc<2, kD, 1>,
+                       dim3(two ? 2 * chunks_s : chunks_s, nu), block, bytes, st, sa.wait_prior != 0, 1, tmK, sa);
         if (rc != GRAPHKV_OK) break;
         ea.wait_prior = next_launch_is_dependent();
-        rc = launch_ex("score_emit_tc", row_tiles == 1 ? tc::score_emit_tc<1, kD> : tc::score_emit_tc<2, kD>,
-                       dim3(chunks_e, nu), dim3(tc::kScoreThreads), smem, st, ea.wait_prior != 0, 1, tmK, ea);
+        rc = launch_ex("score_emit_tc", two ? tc::score_emit_tc<1, kD, 2> : row_tiles == 1 ? tc::score_emit_tc<1, kD, 1>
+                       : tc::score_emit_tc<2, kD, 1>,
+                       dim3(chunks_e, nu), block, bytes, st, ea.wait_prior != 0, 1, tmK, ea);
     }
     return rc;
 }

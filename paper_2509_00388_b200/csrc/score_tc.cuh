@@ -19,6 +19,9 @@
 // columns of a tile, copies them to registers and frees the TMEM buffer before the arithmetic.
 // At 256 query rows all four sets share each tile and two buffers alternate; at 128 or fewer two
 // sets share a tile, the two pairs take alternate tiles and four buffers rotate).
+//
+// At 128 query rows or fewer the two separate kernels run two CTAs per SM, each with half the warps, tensor memory
+// and ring, so that the set-up and the tail of one are covered by the other's sweep.
 #pragma once
 
 #include "tc_common.cuh"
@@ -30,11 +33,15 @@ constexpr int kScoreThreads = 576;       // producer warp, MMA warp, 16 epilogue
 constexpr int kMassBins = 2048;         // histogram of the attention mass: top 11 bits of float_to_key
 constexpr int kEpiWarps = 16;
 constexpr int kScratchBytes = 11264;     // row constants and weights (2 KB) + exchange buffers of 16 x 128 floats
+constexpr int kScratchBytes2 = 6144;     // the same with two CTAs per SM: exchange buffers of 8 x 128 floats
+// kCtas = 2 (two CTAs per SM, at most 128 query rows): producer warp, MMA warp, 8 epilogue warps
+template <int kCtas> __host__ __device__ constexpr int score_threads() { return kCtas == 2 ? 320 : kScoreThreads; }
 
 struct ScoreTcArgs {
     Dims d;
     const __nv_bfloat16 *Q;
-    float *part;        // [units][stats_chunks][GW][2] row statistics (max, sum) per key chunk
+    float *part;        // [units][stats_chunks][GW][2] row statistics (max, sum) per key chunk (two CTAs per SM:
+                        // [units][stats_chunks][4][GW][2], the four warp sets' of a chunk)
     float *row_c;       // [units][2][GW] c_r = max_r + log2(Z_r) (D = 64: max_r, then 1 / Z_r), written by the last
                         // stats CTA of a unit
     int *arrivals;      // [2 * units] words: the two-kernel path counts finished statistics CTAs in [unit]
@@ -93,10 +100,10 @@ __device__ __forceinline__ ScoreSmem score_smem_layout(uint8_t *raw, int rows_pa
     return s;
 }
 
-template <int kD> __host__ __device__ inline size_t score_smem_bytes(int rows_pad, int stages)
+template <int kD> __host__ __device__ inline size_t score_smem_bytes(int rows_pad, int stages, int ctas = 1)
 {
     return 1024 + (size_t)rows_pad * 2 * kD + (size_t)stages * tile_bytes<kD>() + 8 * 8 * 2 + 4 * 8 * 2 + 16 + 8 * 8 +
-           kScratchBytes + 8192 + 64;   // scratch: the CTA's row statistics / row constants and the
+           (ctas == 2 ? kScratchBytes2 : kScratchBytes) + 8192 + 64;   // scratch: the CTA's row statistics / row constants and the
                                         // exchange buffers; 8 KB: the emit sweep's histogram of the mass
 }
 
@@ -157,18 +164,19 @@ __device__ __forceinline__ uint32_t score_setup(const ScoreSmem &s, uint8_t *gen
     return *reinterpret_cast<volatile uint32_t *>(gen + (s.tmem_slot - s.q));
 }
 
-// TMA producer (one thread): key tiles t0+i of (h, b), i in [i_begin, i_end), into the stage ring.
+// TMA producer (one thread): key tiles t0 + i * step of (h, b), i in [i_begin, i_end), into the stage ring.
 // The keys are an input of the call, so the producer waits for none of the call's kernels before.
 template <int kD>
 __device__ __forceinline__ bool score_produce(const ScoreSmem &s, const CUtensorMap *tmK, int stages,
-                                              int t0, int i_begin, int i_end, int h, int b, long long lim)
+                                              int t0, int i_begin, int i_end, int h, int b, long long lim,
+                                              int step = 1)
 {
     bool ok = true;
     int issued = i_begin;
     for (int i = i_begin; i < i_end; ++i) {
         const int st = i % stages, ph = (i / stages) & 1;
         if (!mbar_wait(s.empty0 + 8 * st, ph ^ 1, lim)) { ok = false; break; }
-        tma_load_tile<kD>(s.stage0 + st * tile_bytes<kD>(), tmK, s.full0 + 8 * st, (t0 + i) * kTileKeys, h, b);
+        tma_load_tile<kD>(s.stage0 + st * tile_bytes<kD>(), tmK, s.full0 + 8 * st, (t0 + i * step) * kTileKeys, h, b);
         ++issued;
     }
     if (!ok)        // gave up: let the copies already in flight land before the CTA exits
@@ -203,8 +211,9 @@ __device__ __forceinline__ void stats_fold(float (&v)[32], float scale, float &m
 // warp share the row, thread `sub` of them takes chunks sub, sub + kTpr, ..., eight loads in flight,
 // and the shares are combined with shuffles (every thread of the warp calls this).  Both score
 // paths merge this way, so they agree to the bit.
-template <int kTpr>
-__device__ __forceinline__ float2 merge_row_partials(const float2 *pu, int chunks, int GW, int r, int sub)
+// part(q): the row's partial of chunk q.
+template <int kTpr, typename Part>
+__device__ __forceinline__ float2 merge_row_partials(Part part, int chunks, int GW, int r, int sub)
 {
     float mx = kNegBig, z = 0.f;
     if (r < GW) {
@@ -212,8 +221,7 @@ __device__ __forceinline__ float2 merge_row_partials(const float2 *pu, int chunk
             float2 v[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                v[k] = q0 + k * kTpr < chunks ? __ldcg(pu + (long long)(q0 + k * kTpr) * GW + r)
-                                              : make_float2(kNegBig, 0.f);
+                v[k] = q0 + k * kTpr < chunks ? part(q0 + k * kTpr) : make_float2(kNegBig, 0.f);
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const float mn = fmaxf(mx, v[k].x);
@@ -232,9 +240,12 @@ __device__ __forceinline__ float2 merge_row_partials(const float2 *pu, int chunk
     return make_float2(mx, z);
 }
 
-// kRowTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid (chunks, units of the launch).
-template <int kRowTiles, int kD>
-__global__ void __launch_bounds__(kScoreThreads, 1)
+// kRowTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid (chunks, units of the launch); with kCtas = 2
+// (kRowTiles = 1 only, half the tensor memory and epilogue warps per CTA) grid (2 * chunks, units): a
+// chunk's even tiles belong to one CTA, its odd tiles to the next, which are the tiles of the two groups of
+// warps otherwise, so every partial sum is over the same keys in the same order.
+template <int kRowTiles, int kD, int kCtas>
+__global__ void __launch_bounds__(score_threads<kCtas>(), kCtas)
 score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -242,34 +253,37 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     pc.mark();
     constexpr int kRowsPad = 128 * kRowTiles;
     constexpr int kBufCols = 128 * kRowTiles;        // TMEM columns per accumulator buffer
-    constexpr uint32_t kTmemCols = 512;
+    constexpr uint32_t kTmemCols = 512 / kCtas;
     // Every epilogue thread takes 64 accumulator columns of a tile.  With two row tiles the 16
     // warps share each tile (two buffers); with one, two groups of 8 warps take alternate tiles
     // (four buffers), so that a round of waiting, loading and releasing covers as much arithmetic.
-    constexpr int kBufs = 512 / kBufCols, kGroups = 2 / kRowTiles;
+    constexpr int kBufs = 512 / kCtas / kBufCols, kGroups = 2 / kRowTiles / kCtas;
+    constexpr int kThreads = score_threads<kCtas>();
+    static_assert(kGroups >= 1, "two CTAs per SM: one row tile");
     const Dims &d = a.d;
     const long long lim = a.wait_cycles;
     uint8_t *gen;
     const ScoreSmem s = score_smem_layout<kD>(smem_raw, kRowsPad, a.stages, &gen);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
-    const int chunk = blockIdx.x;
+    const int chunk = blockIdx.x / kCtas, half = blockIdx.x % kCtas;
     int t0, t1;
     tile_range(a.n_tiles, a.chunks, chunk, &t0, &t1);
-    const int n_local = t1 - t0;
+    t0 += half;                                      // tiles t0, t0 + kCtas, ...
+    const int n_local = (t1 - t0 + kCtas - 1) / kCtas;
 
-    constexpr int kParts = 4 / kRowTiles;            // partial statistics per row
+    constexpr int kParts = 4 / kRowTiles;            // partial statistics per row and chunk
     float2 *cta_part = reinterpret_cast<float2 *>(gen + (s.misc - s.q));      // [kParts][kRowsPad]
     int *s_flag = reinterpret_cast<int *>(gen + (s.tmem_slot - s.q)) + 2;
     const int n_ahead = min(n_local, a.stages);
 
-    const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kGroups);
+    const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kCtas / kGroups);
     bool ok = true;
     if (a.first && a.wait_prior) pdl_wait();
     if (warp == 0) {
-        if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
+        if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim, kCtas);
     } else {
-        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
+        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kThreads - 32);
         fence_proxy_async();
     }
     pc.mark();
@@ -280,7 +294,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     pc.mark();
 
     if (warp == 0) {
-        if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim);
+        if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim, kCtas);
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
@@ -310,9 +324,10 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         // columns (row tile, then keys).
         constexpr int kSetCols = 64;
         const int quad = warp & 3, set = (warp - 2) >> 2;
-        const int grp = set / (4 / kGroups);               // tiles grp, grp + kGroups, ...
+        constexpr int kSets = 4 / kCtas / kGroups;
+        const int grp = set / kSets;                       // tiles grp, grp + kGroups, ...
         const int row = quad * 32 + lane;
-        const int col0 = (set % (4 / kGroups)) * kSetCols, rt = col0 >> 7, key_off = col0 & 127;
+        const int col0 = (set % kSets) * kSetCols, rt = col0 >> 7, key_off = col0 & 127;
         const float scale = rsqrtf((float)kD) * kLog2e;
         float mx = kNegBig, z = 0.f;
         const int r = rt * 128 + row;
@@ -334,7 +349,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(s.tempty0 + 8 * buf);
-            const int key0 = (t0 + i) * kTileKeys + key_off;
+            const int key0 = (t0 + i * kCtas) * kTileKeys + key_off;
             const bool masked = key0 + kSetCols - 1 > d.N;      // window keys or the tail past L
 #pragma unroll
             for (int c = 0; c < kSetCols / 32; ++c) {
@@ -352,7 +367,10 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         ok = alive;
         pc.mark();
         // partial p of row r: the sets (of every group) that hold columns of the row's tile
-        cta_part[(kRowTiles == 1 ? set : set & 1) * kRowsPad + r] = make_float2(mx, z);
+        if constexpr (kCtas == 1) cta_part[(kRowTiles == 1 ? set : set & 1) * kRowsPad + r] = make_float2(mx, z);
+        else if (r < d.GW)
+            reinterpret_cast<float2 *>(a.part)[(((long long)unit * a.stats_chunks + chunk) * kParts + 2 * half + set) * d.GW + r] =
+                make_float2(mx, z);
     }
     if (!ok && a.status) atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
     tc_fence_before();
@@ -362,34 +380,42 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         tc_fence_after();
         tmem_dealloc(tmem_base, kTmemCols);
     }
-    // this CTA's statistics of each row; the last CTA of the unit to get here merges all chunks
-    // into the unit's row constants c_r
-    for (int r = threadIdx.x; r < d.GW; r += kScoreThreads) {
+    // the statistics of a chunk's row from those of the warp sets
+    auto chunk_part = [&](auto part_of) {
         float2 p[kParts];
         float mx = kNegBig;
 #pragma unroll
         for (int k = 0; k < kParts; ++k) {
-            p[k] = cta_part[k * kRowsPad + r];
+            p[k] = part_of(k);
             mx = fmaxf(mx, p[k].x);
         }
         float z = 0.f;
 #pragma unroll
         for (int k = 0; k < kParts; ++k) z += p[k].y * ex2(p[k].x - mx);
-        reinterpret_cast<float2 *>(a.part)[((long long)unit * a.stats_chunks + chunk) * d.GW + r] =
-            make_float2(mx, z);
-    }
+        return make_float2(mx, z);
+    };
+    // this CTA's statistics of each row (one CTA per chunk); the last CTA of the unit to get here merges
+    // all chunks into the unit's row constants c_r
+    if constexpr (kCtas == 1)
+        for (int r = threadIdx.x; r < d.GW; r += kThreads)
+            reinterpret_cast<float2 *>(a.part)[((long long)unit * a.stats_chunks + chunk) * d.GW + r] =
+                chunk_part([&](int k) { return cta_part[k * kRowsPad + r]; });
     pc.mark();
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) *s_flag = atomicAdd(a.arrivals + unit, 1) == a.chunks - 1;
+    if (threadIdx.x == 0) *s_flag = atomicAdd(a.arrivals + unit, 1) == kCtas * a.chunks - 1;
     __syncthreads();
     if (*s_flag) {
         __threadfence();
-        const float2 *pu = reinterpret_cast<const float2 *>(a.part) + (long long)unit * a.stats_chunks * d.GW;
+        const float2 *pu = reinterpret_cast<const float2 *>(a.part) +
+                           (long long)unit * a.stats_chunks * (kCtas == 1 ? 1 : kParts) * d.GW;
         constexpr int kTpr = 4 / kRowTiles;
-        if (threadIdx.x < kRowsPad * kTpr) {
-            const int r = threadIdx.x / kTpr, sub = threadIdx.x % kTpr;
-            const float2 mz = merge_row_partials<kTpr>(pu, a.chunks, d.GW, r, sub);
+        for (int t = threadIdx.x; t < kRowsPad * kTpr; t += kThreads) {     // (whole warps)
+            const int r = t / kTpr, sub = t % kTpr;
+            const float2 mz = merge_row_partials<kTpr>([&](int q) {
+                if constexpr (kCtas == 1) return __ldcg(pu + (long long)q * d.GW + r);
+                else return chunk_part([&](int k) { return __ldcg(pu + (long long)(q * kParts + k) * d.GW + r); });
+            }, a.chunks, d.GW, r, sub);
             if (sub == 0 && r < d.GW) {
                 float *c = a.row_c + (long long)unit * 2 * d.GW + r;
                 c[0] = weighted<kD>() ? mz.x : mz.x + log2f(mz.y);
@@ -402,9 +428,10 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     pc.flush(0);
 }
 
-// kColTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid (chunks, units of the launch).
-template <int kColTiles, int kD>
-__global__ void __launch_bounds__(kScoreThreads, 1)
+// kColTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid (chunks, units of the launch).  kCtas = 2 (kColTiles =
+// 1 only): two CTAs per SM, half the tensor memory and epilogue warps each.
+template <int kColTiles, int kD, int kCtas>
+__global__ void __launch_bounds__(score_threads<kCtas>(), kCtas)
 score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -412,13 +439,16 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     pc.mark();
     constexpr int kRowsPad = 128 * kColTiles;        // rows of the Q operand (UMMA N)
     constexpr int kBufCols = 128 * kColTiles;
-    constexpr uint32_t kTmemCols = 512;
+    constexpr uint32_t kTmemCols = 512 / kCtas;
     // Every epilogue thread takes up to 64 accumulator columns of a tile.  With two column tiles
     // the 16 warps share each tile (two buffers); with one, two groups of 8 warps take alternate
     // tiles (four buffers), so that a round of waiting, loading and releasing covers as much
     // arithmetic.
-    constexpr int kBufs = 512 / kBufCols, kGroups = 2 / kColTiles, kSets = 4 / kGroups;
-    constexpr int kXchg = 16 / kSets;                // exchange buffers in rotation
+    constexpr int kBufs = 512 / kCtas / kBufCols, kGroups = 2 / kColTiles / kCtas, kSets = 4 / kCtas / kGroups;
+    constexpr int kXchg = 16 / kCtas / kSets;        // exchange buffers in rotation
+    constexpr int kThreads = score_threads<kCtas>();
+    static_assert(kGroups >= 1, "two CTAs per SM: one column tile");
+    static_assert(kXchg >= kBufs + kGroups, "a buffer comes round after every warp has left the tile that used it");
     const Dims &d = a.d;
     const long long lim = a.wait_cycles;
     uint8_t *gen;
@@ -426,7 +456,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     float *row_c = reinterpret_cast<float *>(gen + (s.misc - s.q));      // [kRowsPad]
     float *row_w = row_c + 256;                                         // [kRowsPad] (D = 64)
     float *xchg = row_w + 256;                                          // [kXchg tiles][kSets][128]
-    uint32_t *mass_hist = reinterpret_cast<uint32_t *>(gen + (s.misc - s.q) + kScratchBytes);   // [kMassBins]
+    uint32_t *mass_hist = reinterpret_cast<uint32_t *>(gen + (s.misc - s.q) + (kCtas == 2 ? kScratchBytes2 : kScratchBytes));   // [kMassBins]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x;
@@ -436,13 +466,13 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const int n_cols = (d.GW + 31) & ~31;            // UMMA N: every x32 slice read below is written
 
     const int n_ahead = min(n_local, a.stages);
-    const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kGroups);
+    const uint32_t tmem_base = score_setup(s, gen, &tmK, a.stages, kTmemCols, kEpiWarps / kCtas / kGroups);
     bool ok = true;
     if (a.first && a.wait_prior) pdl_wait();
     if (warp == 0) {
         if (lane == 0) ok = score_produce<kD>(s, &tmK, a.stages, t0, 0, n_ahead, h, b, lim);
     } else {
-        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kScoreThreads - 32);
+        stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, threadIdx.x - 32, kThreads - 32);
         fence_proxy_async();
     }
     pc.mark();
@@ -451,15 +481,15 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     pdl_launch_dependents();
     const bool want_hist = a.a_hist != nullptr;
     if (want_hist)
-        for (int i = threadIdx.x; i < kMassBins; i += kScoreThreads) mass_hist[i] = 0u;
+        for (int i = threadIdx.x; i < kMassBins; i += kThreads) mass_hist[i] = 0u;
     if (a.zero) {
         // this CTA's share of the unit's words to clear
         const int per_cta = ceil_div(a.zero_words, a.chunks);
-        for (int i = chunk * per_cta + threadIdx.x; i < min((chunk + 1) * per_cta, a.zero_words); i += kScoreThreads)
+        for (int i = chunk * per_cta + threadIdx.x; i < min((chunk + 1) * per_cta, a.zero_words); i += kThreads)
             a.zero[(long long)unit * a.zero_words + i] = 0u;
     }
     // -c_r of the unit's rows; padding rows contribute 2^-inf = 0
-    for (int r = threadIdx.x; r < kRowsPad; r += kScoreThreads) {
+    for (int r = threadIdx.x; r < kRowsPad; r += kThreads) {
         const float *c = a.row_c + (long long)unit * 2 * d.GW + r;
         row_c[r] = r < d.GW ? -__ldcg(c) : -INFINITY;
         if (weighted<kD>()) row_w[r] = r < d.GW ? __ldcg(c + d.GW) : 0.f;
@@ -574,9 +604,8 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     }
     // this CTA's share of the unit's mass histogram (pooling and source selection start from it)
     if (a.a_hist)
-        for (int i = threadIdx.x; i < kMassBins; i += kScoreThreads)
+        for (int i = threadIdx.x; i < kMassBins; i += kThreads)
             if (mass_hist[i]) atomicAdd(a.a_hist + (long long)unit * kMassBins + i, mass_hist[i]);
-    pc.mark();
     pc.mark();
     pc.flush(1);
 }
@@ -800,7 +829,8 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
         static_assert(kRowsPad * kTpr <= (kScoreThreads & ~31), "whole warps take the rows");
         if (threadIdx.x < kRowsPad * kTpr) {
             const int r = threadIdx.x / kTpr, sub = threadIdx.x % kTpr;
-            const float2 mz = merge_row_partials<kTpr>(pu, a.chunks, d.GW, r, sub);
+            const float2 mz = merge_row_partials<kTpr>([&](int q) { return __ldcg(pu + (long long)q * d.GW + r); }, a.chunks,
+                                                       d.GW, r, sub);
             // -c_r of the unit's rows; padding rows contribute 2^-inf = 0
             if (sub == 0) {
                 row_c[r] = r < d.GW ? -(weighted<kD>() ? mz.x : mz.x + log2f(mz.y)) : -INFINITY;

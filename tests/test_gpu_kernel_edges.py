@@ -160,3 +160,24 @@ def test_similarity_sweep_edges(gk, n, hkv, batch, k, m, same):
             for i in torch.nonzero(even).flatten().tolist():
                 low = first[first != src[b, h, i]][:m]
                 assert sorted(nbr[b, h, i].tolist()) == low.tolist()
+
+
+# the two score sweeps as kernels of their own, two CTAs per SM up to 128 query rows: one tile (the second CTA of
+# the chunk has none), odd and even tiles per chunk, few rows and all 128, more CTAs than the GPU holds at once
+@pytest.mark.parametrize("n,w,g,hkv,batch,d", [(70, 1, 1, 1, 1, 128), (129, 32, 4, 8, 1, 128), (390, 8, 3, 2, 2, 64), (5003, 32, 4, 8, 1, 128),
+                                               (1100, 16, 4, 37, 4, 128), (700, 32, 4, 8, 40, 64), (1500, 32, 4, 8, 40, 128)])
+def test_score_in_two_kernels(gk, monkeypatch, n, w, g, hkv, batch, d):
+    monkeypatch.setenv("GRAPHKV_TWO_SCORE_KERNELS", "1")
+    gen = torch.Generator().manual_seed(n)
+    Q = (3 * torch.randn((batch, g * hkv, w, d), generator=gen)).to(torch.bfloat16)
+    K = torch.randn((batch, hkv, n + w, d), generator=gen).to(torch.bfloat16)
+    Qd, Kd = Q.to(DEV), K.to(DEV)
+    p = gk.make_params(Kd, Qw=Qd, window=w)
+    ws = gk.alloc_workspace(p, DEV)
+    ws[256:].random_(256)                            # whatever the workspace holds
+    s = torch.empty((batch, hkv, n), dtype=torch.float32, device=DEV)
+    gk.graphkv_score(p, Qd, Kd, s, ws)
+    assert gk.graphkv_read_status(ws) == gk.OK
+    for b in {0, batch - 1}:
+        want = okv.score(Q[b:b + 1], K[b:b + 1], w, 1).double()
+        assert (s[b:b + 1].cpu().double() - want).norm() / want.norm() < 2e-4
