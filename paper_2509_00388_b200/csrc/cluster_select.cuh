@@ -830,14 +830,21 @@ struct PoolSelectArgs {
 
 // grid = units * C CTAs in clusters of C; block kThreads.  kPer >= chunk / kThreads: elements of
 // the chunk a thread pools (a power of two up to kMaxPerThread).
+constexpr int kRankDirect = 128;
+constexpr int kRankList = 2 * kThreads;  // candidates, of a CTA and in all
+constexpr int kPosBits = 18;             // a row's positions (its length is at most 2^18)
+static_assert(kFineBins >= kThreads && kBins >= kRankList && kTotWords >= kRankList && kStage >= kThreads, "bins, lists, kept");
+static_assert(4 * kRankDirect <= kThreads, "four threads per candidate");
+
 // Top-k of the cluster's row when a histogram of values that the row dominates elementwise is at
 // hand (the pooled scores against the histogram of the attention mass before pooling: pooling only
 // raises values, so the k-th largest pooled score is at least the k-th largest mass).  The highest
 // digit b with k histogram entries in digits >= b therefore bounds the k-th largest row value from
 // below; the row's elements with digit >= b are few (at most pool_kernel times the histogram's
 // count); each CTA lists its own, the first CTA pulls the lists through distributed shared memory
-// and ranks them by counting.  Returns false (in every CTA alike, nothing written) when they exceed kThreads; the
-// caller then runs the radix search.  `mass_hist`: kBins counts of the top 11 bits.
+// and ranks them by counting, more than kRankDirect of them after cutting them into bins (ranking n costs n^2:
+// 600 candidates of 38 sources took 9 us of the kernel's 13, now 4).  Returns false (in every CTA alike,
+// nothing written) when they exceed kRankList; the caller then runs the radix search.  `mass_hist`: kBins counts of the top 11 bits.
 // c0, c1: the histogram's counts of digits kBins-1-2t and kBins-2-2t for thread t (the caller loads
 // them early, ahead of the pooling).
 __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, const Smem &s,
@@ -851,6 +858,8 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
     if (tid == 0) {
         s.misc[0] = 0u;          // digit 0 when the histogram holds fewer than k entries
         s.misc[7] = 0u;          // this CTA's candidate counter
+        s.misc[3] = s.misc[4] = 0u;
+        s.misc[5] = kBins;       // one past the highest digit in use
     }
     __syncthreads();
     if (warp == 0) s.wcnt[lane] = warp_incl_scan(s.wcnt[lane], lane);
@@ -859,6 +868,7 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
     const uint32_t before0 = incl - c0 - c1, before1 = before0 + c0;
     if (before0 < (uint32_t)k && before0 + c0 >= (uint32_t)k) s.misc[0] = kBins - 1 - 2 * tid;
     else if (before1 < (uint32_t)k && before1 + c1 >= (uint32_t)k) s.misc[0] = kBins - 2 - 2 * tid;
+    if (before0 == 0u && c0 + c1 > 0u) s.misc[5] = kBins - 2 * tid;
     __syncthreads();
     const uint32_t bdigit = s.misc[0];
     // this CTA's candidates -> its own lists (keys in hist, positions in tot)
@@ -876,7 +886,7 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
             if (lane == 0) basep = atomicAdd(&s.misc[7], (uint32_t)__popc(bm));
             basep = __shfl_sync(0xffffffffu, basep, 0);
             const uint32_t pos = basep + __popc(bm & ((1u << lane) - 1u));
-            if (cand && pos < (uint32_t)kThreads) {
+            if (cand && pos < (uint32_t)kRankList) {
                 s.hist[pos] = key;
                 s.tot[pos] = (uint32_t)(base + i);
             }
@@ -889,64 +899,99 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
     uint32_t n_lane = 0;
     if (lane < C) n_lane = C > 1 ? cl.map_shared_rank(s.misc, lane)[7] : s.misc[7];
     uint32_t total = 0;
-    int mine_p = -1, mine_j = 0;
+    int mine_p[2] = {-1, -1}, mine_j[2] = {0, 0};            // thread's candidates: tid and tid + kThreads
     for (int p = 0; p < C; ++p) {
         const uint32_t n_p = __shfl_sync(0xffffffffu, n_lane, p);
-        if (n_p > (uint32_t)kThreads) total = 0x40000000u;       // a list overflowed
-        if (tid >= (int)total && tid < (int)(total + n_p)) {
-            mine_p = p;
-            mine_j = tid - (int)total;
+        if (n_p > (uint32_t)kRankList) total = 0x40000000u;      // a list overflowed
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int t = tid + q * kThreads;
+            if (t >= (int)total && t < (int)(total + n_p)) {
+                mine_p[q] = p;
+                mine_j[q] = t - (int)total;
+            }
         }
         total += n_p;
     }
-    if (total > (uint32_t)kThreads || total < (uint32_t)k) {
+    if (total > (uint32_t)kRankList || total < (uint32_t)k) {
         if (C > 1) cl.sync();                              // nobody still reads another CTA's counter
         return false;
     }
     if (rank == 0) {
-        uint32_t key = 0, pos = 0;
-        if (mine_p >= 0) {
-            key = (C > 1 ? cl.map_shared_rank(s.hist, mine_p) : s.hist)[mine_j];
-            pos = (C > 1 ? cl.map_shared_rank(s.tot, mine_p) : s.tot)[mine_j];
+        uint32_t key[2] = {0u, 0u}, pos[2] = {0u, 0u};
+        bool live[2];                                      // not yet known to be kept or dropped
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            live[q] = mine_p[q] >= 0;
+            if (live[q]) {
+                key[q] = (C > 1 ? cl.map_shared_rank(s.hist, mine_p[q]) : s.hist)[mine_j[q]];
+                pos[q] = (C > 1 ? cl.map_shared_rank(s.tot, mine_p[q]) : s.tot)[mine_j[q]];
+            }
         }
         __syncthreads();                                   // own list read before it is overwritten
-        uint32_t *ck = s.hist, *ci = s.tot;
-        if (mine_p >= 0) {
-            ck[tid] = key;
-            ci[tid] = pos;
-        }
-        __syncthreads();
-        // a warp per candidate: its rank among all (value descending, position ascending)
+        uint32_t *ck = s.hist, *ci = s.tot;                // what is ranked by counting: n of them, `need` to keep
         int *kept = s.st_idx;                              // [k] positions of the kept, unordered
-        if (tid == 0) s.misc[3] = 0u;      // (word 7 may still be read by the other CTAs)
+        int n = (int)total, need = k;
+        // Cut into 1024 bins by ten bits of (value above the bound, position) at a time while there are many:
+        // those above the bin that holds the last one to keep are kept, those in it go on.
+        const uint32_t lo = bdigit << 21, span = (s.misc[5] - bdigit) << 21;      // (0: 2^32)
+        for (int bits = 32 - __clz(span - 1u) + kPosBits; n > kRankDirect; bits = max(bits - 10, 0)) {
+            const int shift = max(bits - 10, 0);
+            s.fine[tid] = 0u;
+            __syncthreads();
+            uint32_t bin[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const unsigned long long v = (unsigned long long)(key[q] - lo) << kPosBits | ((1u << kPosBits) - 1u - pos[q]);
+                bin[q] = (uint32_t)(v >> shift) & (uint32_t)(kThreads - 1);
+                if (live[q]) atomicAdd(&s.fine[bin[q]], 1u);
+            }
+            __syncthreads();
+            const uint32_t c = s.fine[kThreads - 1 - tid];
+            uint32_t before = warp_incl_scan(c, lane);
+            if (lane == 31) s.wcnt[warp] = before;
+            __syncthreads();
+            if (warp == 0) s.wcnt[lane] = warp_incl_scan(s.wcnt[lane], lane);
+            __syncthreads();
+            before += (warp == 0 ? 0u : s.wcnt[warp - 1]) - c;
+            if (before < (uint32_t)need && before + c >= (uint32_t)need) {
+                s.misc[0] = (uint32_t)(kThreads - 1 - tid);
+                s.misc[1] = before;
+                s.misc[2] = c;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (live[q] && bin[q] > s.misc[0]) kept[atomicAdd(&s.misc[3], 1u)] = (int)pos[q];
+                live[q] = live[q] && bin[q] == s.misc[0];
+            }
+            need -= (int)s.misc[1];
+            n = (int)s.misc[2];
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            if (live[q]) {
+                const uint32_t at = atomicAdd(&s.misc[4], 1u);
+                ck[at] = key[q];
+                ci[at] = pos[q];
+            }
         __syncthreads();
-        if (total <= (uint32_t)(kThreads / 4)) {
-            // few candidates: four threads each, every one walking a quarter of the list
+        // rank among the n (value descending, position ascending): four threads each, every one walking a
+        // quarter of the list
+        {
             const int t = tid >> 2, sub = tid & 3;
-            const bool live = t < (int)total;
-            const uint32_t kt = live ? ck[t] : 0u, pt = live ? ci[t] : 0u;
+            const uint32_t kt = t < n ? ck[t] : 0u, pt = t < n ? ci[t] : 0u;
             int r = 0;
-            if (live) {
+            if (t < n) {
 #pragma unroll 4
-                for (int u = sub; u < (int)total; u += 4) {
+                for (int u = sub; u < n; u += 4) {
                     const uint32_t ku = ck[u], pu = ci[u];
                     r += (int)(ku > kt) | ((int)(ku == kt) & (int)(pu < pt));
                 }
             }
             r += __shfl_xor_sync(0xffffffffu, r, 1);
             r += __shfl_xor_sync(0xffffffffu, r, 2);
-            if (live && sub == 0 && r < k) kept[atomicAdd(&s.misc[3], 1u)] = (int)pt;
-        } else {
-            for (int t = warp; t < (int)total; t += kWarps) {
-                const uint32_t kt = ck[t], pt = ci[t];
-                int r = 0;
-                for (int u = lane; u < (int)total; u += 32) {
-                    const uint32_t ku = ck[u], pu = ci[u];
-                    r += (int)(ku > kt) | ((int)(ku == kt) & (int)(pu < pt));
-                }
-                r = __reduce_add_sync(0xffffffffu, r);
-                if (lane == 0 && r < k) kept[atomicAdd(&s.misc[3], 1u)] = (int)pt;
-            }
+            if (t < n && sub == 0 && r < need) kept[atomicAdd(&s.misc[3], 1u)] = (int)pt;
         }
         __syncthreads();
         // ascending positions: thread t places kept[t] by counting the smaller ones

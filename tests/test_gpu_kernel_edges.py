@@ -181,3 +181,27 @@ def test_score_in_two_kernels(gk, monkeypatch, n, w, g, hkv, batch, d):
     for b in {0, batch - 1}:
         want = okv.score(Q[b:b + 1], K[b:b + 1], w, 1).double()
         assert (s[b:b + 1].cpu().double() - want).norm() / want.norm() < 2e-4
+
+
+# the sources among few and many candidates (pooling widens the bound's list), with and without plateaus of equal
+# scores: one call against the stages, whose selection has no histogram of the mass and searches digit by digit
+@pytest.mark.parametrize("n,hkv,batch,k,pool,same", [(3500, 8, 1, 1, 1, 0), (3500, 8, 1, 38, 7, 0), (5000, 2, 1, 150, 7, 0), (8160, 8, 1, 38, 13, 0),
+                                                     (8160, 1, 1, 600, 3, 0), (4000, 8, 1, 38, 7, 300), (6000, 8, 2, 20, 7, 900),
+                                                     (20000, 1, 1, 1000, 1, 0), (9000, 8, 1, 38, 7, 1900)])
+def test_sources_by_bins(gk, n, hkv, batch, k, pool, same):
+    cfg = wl.scaled(wl.LLAMA_32K, n_prefix=n, n_q_heads=4 * hkv, n_kv_heads=hkv, batch=batch, n_clusters=64)
+    inp = wl.make_inputs(cfg)
+    if same:
+        inp["K"][:, :, 100:100 + same] = inp["K"][:, :, 50:51]
+    Q, K, V = (inp[x].to(DEV) for x in ("Qw", "K", "V"))
+    p = gk.make_params(K, Qw=Q, V=V, window=cfg.window, budget=n // 4, pool_kernel=pool, topk_nodes=k, neighbors=4, rounds=1)
+    ws = gk.alloc_workspace(p, DEV)
+    got = gk.alloc_outputs(p, K)
+    gk.graphkv_compress(p, Q, K, V, *got, ws)
+    assert gk.graphkv_read_status(ws) == gk.OK
+    want = gk.alloc_outputs(p, K)
+    gk.graphkv_score(p, Q, K, want[3], ws)
+    gk.graphkv_propagate(p, K, want[3], None, ws)
+    gk.graphkv_select_gather(p, want[3], K, V, *want[:3], ws)
+    for a, b in zip(got, want):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
