@@ -1380,12 +1380,16 @@ static bool decode_shape(const graphkv_params *p, DecodeArgs *a)
     return true;
 }
 
+static size_t decode_bytes(const DecodeArgs &a)
+{
+    return align_up((size_t)a.batch * a.hkv * sizeof(unsigned long long)) +
+           align_up((size_t)a.batch * a.hkv * a.splits * a.G * kDecPart * sizeof(float));
+}
+
 size_t graphkv_decode_workspace_bytes(const graphkv_params *params)
 {
     DecodeArgs a;
-    if (!decode_shape(params, &a)) return 0;
-    return align_up((size_t)a.batch * a.hkv * sizeof(unsigned long long)) +
-           align_up((size_t)a.batch * a.hkv * a.splits * a.G * kDecPart * sizeof(float));
+    return decode_shape(params, &a) ? decode_bytes(a) : 0;
 }
 
 extern "C++" {
@@ -1410,7 +1414,7 @@ graphkv_status graphkv_decode_attention(const graphkv_params *params, const void
     if (!decode_shape(params, &a)) return params && params->head_dim != kHeadDim ? GRAPHKV_ERR_UNSUPPORTED
                                                                                   : GRAPHKV_ERR_INVALID_ARG;
     if (!q || !K || !V || !out || !aligned16(K) || !aligned16(V)) return GRAPHKV_ERR_INVALID_ARG;
-    if (!workspace || workspace_bytes < graphkv_decode_workspace_bytes(params)) return GRAPHKV_ERR_WORKSPACE;
+    if (!workspace || workspace_bytes < decode_bytes(a)) return GRAPHKV_ERR_WORKSPACE;
     a.arrived = static_cast<unsigned long long *>(workspace);
     a.part = at<float>(workspace, align_up((size_t)a.batch * a.hkv * sizeof(unsigned long long)));
     a.out = out;
