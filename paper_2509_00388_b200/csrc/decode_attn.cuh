@@ -10,15 +10,17 @@
 // warp takes whole blocks through a ring of asynchronous copies of its own (two blocks: twelve warps
 // keep 96 to 192 KB in flight per SM) and keeps a running softmax of its own, so the loop has no
 // barrier.  The warps of a CTA merge in shared memory; a unit that several CTAs share is merged by
-// the last of them to finish, in the same launch.
+// the first of them where they fit a cluster, else by the last to finish, in the same launch.
 //
 // Measured on one B200, bf16, 8 KV heads, 4 query heads each (plain loads, a barrier per 32 rows and
 // a second kernel for the merge before -> now): 32800 rows 145 -> 28 us (4.8 TB/s), 16 x 2080 rows
 // 137 -> 25.5 us (5.4 TB/s), 4 x 32800 rows 89 us (6.0 TB/s, 92 % of the copy bandwidth), 544 rows
-// 15.4 -> 6.9 us (the host's time for a call).  About 8 us of a launch are its start, the first
+// 15.4 -> 5.8 us.  About 8 us of a launch are its start, the first
 // loads' latency and the merge.  Runs of blocks cut without regard to units (an equal share for
 // every SM, but two units in some CTAs, one after the other) measured 34 and 28 us.
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 
@@ -42,6 +44,7 @@ struct DecodeArgs {
     int batch, hq, hkv, G, rows;
     int blocks_per_unit;               // blocks of a unit
     int splits;                        // CTAs that share a unit
+    int cluster;                       // they are one cluster
     long long qs[2];                   // element strides of q: batch, head
     long long ks[3], vs[3];            // element strides of K and V: batch, head, row
     unsigned long long *arrived;       // [units] (call tag, count of CTAs that left their part), splits > 1
@@ -407,6 +410,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
     extern __shared__ __align__(128) uint8_t dec_smem[];         // [kDecWarps][kDecStages][kDecStage]
     __shared__ __align__(16) float s_x[kDecSplit * kG * kDecPart];
     __shared__ __align__(16) float s_q[sizeof(T) == 4 ? kG * kHeadDim : 4];
+    __shared__ __align__(16) float s_part[kG * kDecPart];
     __shared__ int s_last;
     constexpr int kRows = dec_rows<T>(), kPieces = kHeadDim * (int)sizeof(T) / 16;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, G = a.G, unit = blockIdx.y;
@@ -423,7 +427,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
     const uint32_t ring_s = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
     pdl_wait();
     pdl_launch_dependents();
-    if (a.splits > 1 && tid == kDecThreads - 1) {
+    if (a.splits > 1 && !a.cluster && tid == kDecThreads - 1) {
         // this call's tag into the unit's arrival word (nobody waits for it: a word that changes in
         // between has been tagged by another CTA of this call)
         const unsigned long long seen = *reinterpret_cast<volatile unsigned long long *>(a.arrived + unit);
@@ -477,6 +481,19 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
     };
     if (a.splits == 1) {
         decode_merge(n_warps, G, of_warp, s_x, true, out, kHeadDim);
+        return;
+    }
+    if (a.cluster) {
+        // the parts stay in shared memory, where the first CTA of the unit's cluster reads them
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl = cg::this_cluster();
+        decode_merge(n_warps, G, of_warp, s_x, false, s_part, kDecPart);
+        cl.sync();
+        if (blockIdx.x == 0) {
+            auto of_peer = [&](int i, int w) { return *reinterpret_cast<const float4 *>(cl.map_shared_rank(s_part, i) + w); };
+            decode_merge(a.splits, G, of_peer, s_x, true, out, kHeadDim);
+        }
+        cl.sync();                                               // nobody leaves while its part is read
         return;
     }
     // this CTA's part goes to memory; the last CTA of the unit to get here merges them

@@ -1375,6 +1375,12 @@ static bool decode_shape(const graphkv_params *p, DecodeArgs *a)
     // as many CTAs per unit as one wave holds (one per SM), with kDecMinBlocks blocks each or more
     const int units = p->batch * p->n_kv_heads;
     a->splits = std::max(1, std::min(sm_count() / units, ceil_div(a->blocks_per_unit, kDecMinBlocks)));
+    // CTAs of a unit that fit a cluster merge through shared memory instead of global memory and a counter
+    // (544 rows 6.5 -> 5.8 us).  Up to 24 blocks per CTA a cluster of eight also beats more CTAs that do not
+    // fit one (1032 rows 6.8 -> 6.4 us, 3032 rows 8.5 -> 8.2; 4132 rows 9.0 -> 9.2; clusters of four lose).
+    const int C = resident_cluster_size(units);
+    if (C == 8 && a->splits > C && a->blocks_per_unit <= 24 * C) a->splits = C;
+    a->cluster = a->splits > 1 && a->splits <= C ? 1 : 0;
     a->qs[0] = p->q_stride[0]; a->qs[1] = p->q_stride[1];
     for (int i = 0; i < 3; ++i) { a->ks[i] = p->k_stride[i]; a->vs[i] = p->v_stride[i]; }
     return true;
@@ -1401,7 +1407,7 @@ static graphkv_status launch_decode(const DecodeArgs &a, const void *q, const vo
     if (!once_per_device(mu, state, [] { return set_smem(decode_kernel<T, kG>, kDecSmem); }))
         return GRAPHKV_ERR_CUDA;
     return launch_ex("decode_attention", decode_kernel<T, kG>, dim3(a.splits, a.batch * a.hkv), dim3(kDecThreads), kDecSmem,
-                     st, next_launch_is_dependent(), 1, a, static_cast<const T *>(q), static_cast<const T *>(K),
+                     st, next_launch_is_dependent(), a.cluster ? a.splits : 1, a, static_cast<const T *>(q), static_cast<const T *>(K),
                      static_cast<const T *>(V));
 }
 }

@@ -21,7 +21,8 @@ def gk():
 # least share of a CTA; one CTA per unit (units above half the SMs) and many; 1 to 8 query heads
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("rows,g,hkv,batch", [(1, 1, 1, 1), (7, 3, 2, 1), (17, 4, 1, 1), (97, 5, 2, 2), (191, 8, 1, 1),
-                                              (193, 4, 8, 10), (400, 2, 8, 19), (3073, 7, 3, 1)])
+                                              (193, 4, 8, 10), (400, 2, 8, 19), (3073, 7, 3, 1), (1500, 4, 8, 1),
+                                              (2000, 8, 16, 1), (300, 3, 11, 3)])
 def test_decode_attention_edges(gk, dtype, rows, g, hkv, batch):
     gen = torch.Generator().manual_seed(rows)
     q = (2 * torch.randn((batch, hkv * g, 128), generator=gen)).to(dtype)
