@@ -1,23 +1,27 @@
-// The whole path in one kernel, for few units with short rows (up to three key tiles
-// per CTA, 3072 tokens): one cluster of C CTAs
-// per (sequence, KV head) unit, each CTA owning a run of key tiles from the first score to the gather.
+// The whole path in one kernel, for few units with short rows: one cluster of C CTAs (any C up to 16 of which as many
+// clusters as units are resident) per (sequence, KV head) unit, each CTA owning a run of key tiles from the first
+// score to the gather.
 //
 // Bound: latency.  At these sizes the four kernels of the general path take 8-20 us each for 1-3 us of
 // work: launch, set-up, the first loads, writes that the next kernel reads back, a tail.  Here the key
-// tiles come from memory once and stay in shared memory for all three sweeps, the row of scores is copied into every CTA, which then selects and decays it like the others without
-// asking them, and what the CTAs of a unit exchange goes through distributed shared memory behind cluster
-// barriers (0.3 us each, seven of them).
+// tiles come from memory once and stay in shared memory for all three sweeps (which limits the row: four tiles per CTA,
+// eight at D = 64), and every CTA holds the unit's row of scores, selects and decays it without asking the others.
+// What the CTAs exchange is pushed: the one that has it stores it into the shared memory of those that
+// need it (row statistics, masses and neighbour lists into all, the cosines of a source with all keys into the one CTA that picks
+// its neighbours), so that an exchange is stores and one cluster barrier (0.3 us); reading from the others after
+// the barrier took 1 to 2 us more each time.
 //
 // Every arithmetic step is the general kernels': the same accumulators, the row statistics folded and
-// merged over the same key chunks in the same order (a CTA takes whole chunks), the same pooling, cosines
+// merged over the same key chunks in the same order (one chunk per CTA), the same pooling, cosines
 // and decay order; so the results agree with them to the bit.
 // 512 threads; thread 0 issues copies and MMAs between the barriers of the sweeps.
 //
-// Measured on one B200 against the four kernels, 8 KV heads, W = 32, 16 sources: 1003 tokens 43 -> 31.5 us,
-// 2000 tokens 47 -> 37.4, 3000 tokens 53 -> 45.9; with four tiles per CTA and more the sweeps' 64 CTAs lose to
-// the general path's 128 to 148 (two heads of 4064 tokens 49 -> 55 us).
+// Measured on one B200, 8 KV heads, W = 32, 16 sources (four kernels; this kernel with clusters of 2, 4 or 8 that read from
+// one another and per-CTA lists of edges; now): 1003 tokens 43, 31.6, 24.1 us; 2000 tokens 47, 37.1, 28.1; 3000 tokens 53,
+// 46.0, 33.0; 4060 tokens 55.6, -, 38.0; 5000 tokens 53.6, -, 44.5; 8191 tokens at D = 64 51.5, -, 46.0.
 #pragma once
 
+#include "block_select.cuh"
 #include "edge_search.cuh"
 #include "row_finish.cuh"
 #include "score_tc.cuh"
@@ -29,23 +33,59 @@ namespace cg = cooperative_groups;
 using rf::kThreads;
 using rf::kWarps;
 
-constexpr int kMaxCluster = 8;
-constexpr int kMaxTiles = 4;            // key tiles per CTA (whole chunks of the row statistics: they come out uneven)
-constexpr int kMeanTiles = 3;           // on average
+constexpr int kMaxCluster = 16;
+constexpr int kMaxTiles = 8;            // key tiles per CTA: all of them stay in its shared memory
+__host__ __device__ constexpr int max_tiles(int D) { return D == 64 ? kMaxTiles : kMaxTiles / 2; }
 constexpr int kMaxSources = 64;
 constexpr int kMaxNeighbours = 32;
-constexpr int kMaxRow = kMaxCluster * kMeanTiles * tc::kTileKeys;    // tokens per row
-constexpr int kListCap = kCandCap;      // listed edges per source and CTA
+
+// Shared memory, from a 1024-byte aligned base.  What is dead is used again: the queries' place holds the source rows
+// and, behind them, the unit's scores where they fit; the tiles' place, once the sweeps are over, the unit's
+// neighbour lists [k][m] (position, factor) and, at its end, the kept positions [B]; the place of the row statistics
+// [C][GW] the cosines [rows][N].  Those come from other CTAs, which do not know whether this one's sweep is over:
+// in the tiles' place (behind the lists) they cost one more cluster barrier, so only where nothing else fits.
+struct Layout {
+    int tiles, mass, row, inv, row_c, parts, cosines, scratch, small, bars, total;
+};
+constexpr int kScratch = 6656;                  // partial statistics or exchange (4 KB each), histogram, groups' lists
+static_assert(kScratch >= 4 * bs::GroupScratch<128>::kBytes && kScratch >= bs::GroupScratch<kThreads>::kBytes &&
+                  kScratch >= (bs::kBins + bs::kRankCap) * 4, "scratch");
+struct Sizes {                                  // what the layout follows from
+    int N, C, GW, tiles, np, rows, lists, kept, cosines_in_tiles;
+};
+template <int kD, int kTiles> __host__ __device__ inline Layout layout(const Sizes &z)
+{
+    Layout l;
+    const int row = (z.N + 3) / 4 * 16, parts = (z.C * z.GW * 8 + 15) / 16 * 16, queries = 128 * kTiles * 2 * kD;
+    const int cosines = z.rows * row, region = z.lists + z.kept + (z.cosines_in_tiles ? cosines : 0);
+    int off = queries;
+    l.tiles = off;
+    off += z.tiles * tc::tile_bytes<kD>() > region ? z.tiles * tc::tile_bytes<kD>() : region;
+    l.mass = off;    off += row;                // the unit's attention mass before pooling
+    l.row = z.np * 2 * kD;                      // the unit's scores
+    if (l.row + row > queries) {
+        l.row = off;
+        off += row;
+    }
+    l.inv = off;     off += z.tiles * tc::kTileKeys * 4;    // 1 / |k| of this CTA's keys
+    l.row_c = off;   off += 2 * 128 * kTiles * 4;
+    l.parts = off;
+    l.cosines = z.cosines_in_tiles ? l.tiles + z.lists : off;
+    off += z.cosines_in_tiles || cosines < parts ? parts : cosines;
+    l.scratch = off; off += kScratch;
+    l.small = off;   off += 1024;
+    l.bars = off;    off += (kMaxTiles + 2) * 8 + 16;
+    l.total = off + 1024;
+    return l;
+}
 
 struct PathArgs {
     Dims d;
     const __nv_bfloat16 *Q, *K;
-    int C;
-    int chunks, n_tiles;       // key chunks of the row statistics and key tiles, per unit
-    int tiles;                 // most key tiles a CTA owns
-    int np;                    // sources padded to 16, 32 or 64
-    int region;                // bytes of the lists' place
-    float *part;               // [units][chunks][GW][2] row statistics per chunk
+    int C;                     // CTAs per unit, and key chunks of the row statistics
+    int n_tiles;               // key tiles per unit
+    Sizes z;                   // tiles: most key tiles a CTA owns; np: sources padded to 16, 32 or 64; rows: sources whose
+                               // cosines a CTA holds at a time; lists, kept: bytes; cosines_in_tiles: they take the tiles' place
     int *status;
     float *scores;             // optional [units][N]: final scores (scores_only: the pooled ones)
     int scores_only;
@@ -62,42 +102,20 @@ struct PathArgs {
     int budget_of[rf::kMaxBudgets];
 };
 
-// Shared memory, from a 1024-byte aligned base.
-struct Layout {
-    int tiles, mass, inv, row, row_c, scratch, small, bars, total;
-};
-template <int kD, int kTiles> __host__ __device__ inline Layout layout(int tiles, int region, int N)
+// ---- stores into another CTA of the cluster -----------------------------------------------------
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank)
 {
-    Layout l;
-    int off = 128 * kTiles * 2 * kD;            // the queries; then source rows
-    l.tiles = off;                              // the tiles; then the region of the lists
-    off += tiles * tc::tile_bytes<kD>() > region ? tiles * tc::tile_bytes<kD>() : region;
-    const int keys = tiles * tc::kTileKeys;
-    l.mass = off;    off += keys * 4;           // this CTA's attention mass before pooling
-    l.inv = off;     off += keys * 4;           // 1 / |k|
-    l.row = off;     off += (N + 3) / 4 * 16;   // the unit's scores
-    l.row_c = off;   off += 2 * 128 * kTiles * 4;
-    l.scratch = off; off += 16384;              // partial statistics, exchange, histograms
-    l.small = off;   off += 2048;
-    l.bars = off;    off += (kMaxTiles + 2) * 8 + 16;
-    l.total = off + 1024;
-    return l;
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
 }
-
-__host__ __device__ inline int first_chunk(int chunks, int C, int rank) { return (int)((long long)chunks * rank / C); }
-__host__ __device__ inline int first_tile_of_chunk(int n_tiles, int chunks, int c)
+__device__ __forceinline__ void peer_store(uint32_t addr, float x)
 {
-    const int base = n_tiles / chunks, rem = n_tiles % chunks;
-    return c * base + (c < rem ? c : rem);
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(x) : "memory");
 }
-
-// After the sweeps the tiles' place holds the cosines [16][keys] (then the gangs' survivors), the CTA's lists
-// [k][kListCap], the merged lists of its sources [ceil(k / C)][kMaxNeighbours], all lists [k][m] and, at its
-// end, the kept positions [B].
-__host__ __device__ inline int region_bytes(int keys, int C, int k, int m, int B)
+__device__ __forceinline__ void peer_store(uint32_t addr, float2 x)
 {
-    const int cosines = 16 * keys * 4, tops = 4 * (kMaxCluster + 1) * kListCap * 8;
-    return ((cosines > tops ? cosines : tops) + k * kListCap * 8 + ((k + C - 1) / C) * kMaxNeighbours * 8 + k * m * 8 + B * 4 + 15) / 16 * 16;
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x.x), "f"(x.y) : "memory");
 }
 
 // kTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid = units * C CTAs in clusters of C.
@@ -113,13 +131,14 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     constexpr int kTile = tile_bytes<kD>();
     const Dims &d = a.d;
     const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C;
-    const int b = unit / d.hkv, h = unit % d.hkv, N = d.N, keys = a.tiles * kTileKeys;
+    const int b = unit / d.hkv, h = unit % d.hkv, N = d.N;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, quad = warp & 3, set = warp >> 2;
     const long long lim = a.wait_cycles;
     const uint32_t base_s = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base_s - smem_u32(smem_raw));
-    const Layout lay = layout<kD, kTiles>(a.tiles, a.region, N);
-    float *mass = reinterpret_cast<float *>(gen + lay.mass), *inv_norm = reinterpret_cast<float *>(gen + lay.inv);
+    const Layout lay = layout<kD, kTiles>(a.z);
+    const float *mass = reinterpret_cast<const float *>(gen + lay.mass);  // [N] the unit's masses, written by all its CTAs
+    float *inv_norm = reinterpret_cast<float *>(gen + lay.inv);
     float *row = reinterpret_cast<float *>(gen + lay.row);                // [N] the unit's scores, whole
     float *row_c = reinterpret_cast<float *>(gen + lay.row_c), *row_w = row_c + kRowsPad;
     uint8_t *scratch = gen + lay.scratch;
@@ -128,16 +147,15 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     uint32_t *misc = wcnt + 2 * kWarps;                                   // [32]
     int *src_pos = reinterpret_cast<int *>(misc + 32);                    // [kMaxSources]
     float *src_inv = reinterpret_cast<float *>(src_pos + kMaxSources);    // [kMaxSources]
-    int *list_n = reinterpret_cast<int *>(src_inv + kMaxSources);         // [kMaxSources]
-    float *list_bound = reinterpret_cast<float *>(list_n + kMaxSources);  // [kMaxSources]
-    int *start = reinterpret_cast<int *>(list_bound + kMaxSources);       // [kMaxCluster + 1] first key of each CTA
+    uint32_t *range = reinterpret_cast<uint32_t *>(src_inv + kMaxSources);      // [2 * kWarps] least and greatest pooled score per warp
     const uint32_t bar_full = base_s + lay.bars, bar_done = bar_full + 8 * kMaxTiles, tmem_slot = bar_done + 16;
     PhaseClock pc(tid == 0);
     pc.mark();
     if (C > 1) cl.barrier_arrive();
 
-    const int c0 = first_chunk(a.chunks, C, rank), c1 = first_chunk(a.chunks, C, rank + 1);
-    const int t0 = first_tile_of_chunk(a.n_tiles, a.chunks, c0), n_tiles = first_tile_of_chunk(a.n_tiles, a.chunks, c1) - t0;
+    int t0, n_tiles;
+    tile_range(a.n_tiles, C, rank, &t0, &n_tiles);
+    n_tiles -= t0;
     const int base = t0 * kTileKeys, n_local = max(0, min(N - base, n_tiles * kTileKeys));
     const int n_emit = (n_local + kTileKeys - 1) / kTileKeys;             // tiles with prefix keys
 
@@ -162,12 +180,12 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             tma_load_tile<kD>(base_s + lay.tiles + t * kTile, &tmK, bar_full + 8 * t, (t0 + t) * kTileKeys, h, b);
         if (rank == 0 && unit == 0) *a.status = 0;
     }
-    if (tid <= C) start[tid] = first_tile_of_chunk(a.n_tiles, a.chunks, first_chunk(a.chunks, C, tid)) * kTileKeys;
     stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, tid, kThreads);
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (C > 1) cl.barrier_wait();   // (every CTA of the unit has started: its shared memory may be written to)
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + (tmem_slot - base_s));
     const uint32_t tmem_lane = tmem + ((uint32_t)(quad * 32) << 16);
     bool alive = true;              // no wait of this CTA has run out (the same in all its threads)
@@ -175,24 +193,18 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     auto batch_done = [&](int bt) { return __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (bt & 1), (bt >> 1) & 1, lim)) != 0; };
     pc.mark();
 
-    // ---- statistics: D = Q K^T, chunk by chunk, kGroups tiles per batch, two batches under way ----
+    // ---- statistics: D = Q K^T, kGroups tiles per batch, two batches under way ----
     const float scale = rsqrtf((float)kD) * kLog2e;
     {
-        struct Cursor { int c, i; };                                      // chunk, first tile of the batch within it
-        auto chunk_tiles = [&](int c) { return first_tile_of_chunk(a.n_tiles, a.chunks, c + 1) - first_tile_of_chunk(a.n_tiles, a.chunks, c); };
-        auto next = [&](Cursor &u) {
-            u.i += kGroups;
-            if (u.i >= chunk_tiles(u.c)) u.i = 0, ++u.c;
-        };
         bool ok = true, issued_ok = true;                                 // (issued_ok: thread 0's own waits)
-        auto issue = [&](Cursor u, int bt) {
-            const int first = first_tile_of_chunk(a.n_tiles, a.chunks, u.c) - t0 + u.i, n = min(kGroups, chunk_tiles(u.c) - u.i);
-            for (int g = 0; g < n && issued_ok; ++g) {
-                issued_ok = tile_landed(first + g);
+        const int n_batches = ceil_div(n_tiles, kGroups);
+        auto issue = [&](int bt) {
+            for (int t = bt * kGroups; t < min((bt + 1) * kGroups, n_tiles) && issued_ok; ++t) {
+                issued_ok = tile_landed(t);
                 if (!issued_ok) break;
                 tc_fence_after();
-                const uint32_t kt = base_s + lay.tiles + (first + g) * kTile;
-                const uint32_t out = tmem + ((bt & 1) * kGroups + g) * kBufCols;
+                const uint32_t kt = base_s + lay.tiles + t * kTile;
+                const uint32_t out = tmem + ((bt & 1) * kGroups + t % kGroups) * kBufCols;
 #pragma unroll
                 for (int rt = 0; rt < kTiles; ++rt)
 #pragma unroll
@@ -202,21 +214,15 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             if (issued_ok && !(a.withhold_commit == 1 && bt == 0)) umma_commit(bar_done + 8 * (bt & 1));
         };
-        Cursor at{c0, 0}, ahead{c0, 0};
-        int n_issued = 0;
         if (tid == 0)
-            for (; n_issued < 2 && ahead.c < c1; ++n_issued) {
-                issue(ahead, n_issued);
-                next(ahead);
-            }
+            for (int bt = 0; bt < min(2, n_batches); ++bt) issue(bt);
         const int grp = set / (4 / kGroups), col0 = (set % (4 / kGroups)) * 64, rt = col0 >> 7, key_off = col0 & 127;
         const int r = rt * 128 + quad * 32 + lane, last = N + (r < d.GW ? r % d.W : 0);      // last visible key of the row
         float mx = kNegBig, z = 0.f;
-        while (at.c < c1 && alive) {
-            const int nt = chunk_tiles(at.c);
-            const int tile = first_tile_of_chunk(a.n_tiles, a.chunks, at.c) - t0 + at.i + grp;
+        for (; batch < n_batches && alive; ++batch) {
+            const int tile = batch * kGroups + grp;
             ok = batch_done(batch);
-            if (ok && at.i + grp < nt) {
+            if (ok && tile < n_tiles) {
                 tc_fence_after();
                 uint32_t raw[2][32];
                 const uint32_t from = tmem_lane + ((batch & 1) * kGroups + grp) * kBufCols + col0;
@@ -240,56 +246,66 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
             }
             tc_fence_before();
-            const bool chunk_ends = at.i + kGroups >= nt;
-            // (two buffers in turn: the merge below may still read one while the next chunk ends)
-            float2 *cta_part = reinterpret_cast<float2 *>(scratch) + (at.c & 1) * (kParts * kRowsPad);
-            if (chunk_ends) {
-                cta_part[(kTiles == 1 ? set : set & 1) * kRowsPad + r] = make_float2(mx, z);
-                mx = kNegBig;
-                z = 0.f;
-            }
+            float2 *cta_part = reinterpret_cast<float2 *>(scratch);
+            if (batch == n_batches - 1) cta_part[(kTiles == 1 ? set : set & 1) * kRowsPad + r] = make_float2(mx, z);
             alive = __syncthreads_and(ok && issued_ok ? 1 : 0) != 0;
-            if (!alive) break;
-            if (chunk_ends && tid < d.GW) {
-                float2 p[kParts];
-                float m = kNegBig, sum = 0.f;
-#pragma unroll
-                for (int k = 0; k < kParts; ++k) {
-                    p[k] = cta_part[k * kRowsPad + tid];
-                    m = fmaxf(m, p[k].x);
-                }
-#pragma unroll
-                for (int k = 0; k < kParts; ++k) sum += p[k].y * ex2(p[k].x - m);
-                reinterpret_cast<float2 *>(a.part)[((long long)unit * a.chunks + at.c) * d.GW + tid] = make_float2(m, sum);
-            }
-            if (tid == 0) {
+            if (alive && tid == 0) {
                 tc_fence_after();
-                if (ahead.c < c1) {
-                    issue(ahead, n_issued++);
-                    next(ahead);
-                }
+                if (batch + 2 < n_batches) issue(batch + 2);
             }
-            ++batch;
-            next(at);
+        }
+        if (alive && tid < d.GW) {
+            // the chunk's statistics of this row, to every CTA of the unit
+            const float2 *cta_part = reinterpret_cast<const float2 *>(scratch);
+            float2 p[kParts];
+            float m = kNegBig, sum = 0.f;
+#pragma unroll
+            for (int k = 0; k < kParts; ++k) {
+                p[k] = cta_part[k * kRowsPad + tid];
+                m = fmaxf(m, p[k].x);
+            }
+#pragma unroll
+            for (int k = 0; k < kParts; ++k) sum += p[k].y * ex2(p[k].x - m);
+            const uint32_t to = base_s + lay.parts + (rank * d.GW + tid) * 8;
+            for (int p = 0; p < C; ++p) peer_store(peer_addr(to, p), make_float2(m, sum));
         }
     }
     pc.mark();
 
     // ---- row constants from all chunks of the unit ----
-    if (C > 1) {
-        cl.barrier_wait();              // (the start of the kernel)
-        cl.sync();                      // every chunk's statistics have been written
-    } else {
-        __syncthreads();
+    if (C > 1) cl.barrier_arrive(); // (this CTA's statistics are with everybody)
+    // the keys' norms meanwhile, a warp set per tile
+    constexpr int kPieces = kD / 8;
+    if (a.has_graph && !a.scores_only && alive) {
+        bool ok = true;
+        for (int t = set; t < n_emit && ok; t += 4) {
+            ok = __all_sync(0xffffffffu, tile_landed(t));
+            if (!ok) break;
+            const uint8_t *tile = gen + lay.tiles + t * kTile;
+            float n0 = 0.f, n1 = 0.f;
+#pragma unroll
+            for (int c16 = 0; c16 < kPieces; ++c16) {
+                const uint4 raw = *reinterpret_cast<const uint4 *>(tile + sw128_offset(128, quad * 32 + lane, c16));
+                const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float lo = __uint_as_float(w[q] << 16), hi = __uint_as_float(w[q] & 0xffff0000u);
+                    n0 = fmaf(lo, lo, n0);
+                    n1 = fmaf(hi, hi, n1);
+                }
+            }
+            inv_norm[t * kTileKeys + quad * 32 + lane] = 1.0f / fmaxf(sqrtf(n0 + n1), kNormEps);
+        }
     }
+    if (C > 1) cl.barrier_wait();
+    else __syncthreads();
     pc.mark();
     {
         constexpr int kTpr = 4 / kTiles;
         static_assert(kRowsPad * kTpr == kThreads, "every thread has a share of a row");
         const int r = tid / kTpr, sub = tid % kTpr;
-        const float2 *pu = reinterpret_cast<const float2 *>(a.part) + (long long)unit * a.chunks * d.GW;
-        const float2 mz = merge_row_partials<kTpr>([&](int q) { return __ldcg(pu + (long long)q * d.GW + r); }, a.chunks,
-                                                   d.GW, r, sub);
+        const float2 *parts = reinterpret_cast<const float2 *>(gen + lay.parts);
+        const float2 mz = merge_row_partials<kTpr>([&](int q) { return parts[q * d.GW + r]; }, C, d.GW, r, sub);
         if (sub == 0) {
             row_c[r] = r < d.GW ? -(weighted<kD>() ? mz.x : mz.x + log2f(mz.y)) : -INFINITY;
             if (weighted<kD>()) row_w[r] = r < d.GW ? 1.0f / mz.y : 0.f;
@@ -362,42 +378,53 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             if (tid < kGroups * 128 && q * kGroups + tid / 128 < n_emit) {
                 const int t = n_emit - 1 - (q * kGroups + tid / 128), key = tid & 127;
                 const float *xs = x + (tid / 128) * kSets * 128 + key;
-                mass[t * kTileKeys + key] = kSets == 4 ? (xs[0] + xs[128]) + (xs[256] + xs[384]) : xs[0] + xs[128];
+                const float aj = kSets == 4 ? (xs[0] + xs[128]) + (xs[256] + xs[384]) : xs[0] + xs[128];
+                const uint32_t to = base_s + lay.mass + (base + t * kTileKeys + key) * 4;
+                if (t * kTileKeys + key < n_local)
+                    for (int p = 0; p < C; ++p) peer_store(peer_addr(to, p), aj);
             }
             ++batch;
         }
     }
-    if (!alive)
-        for (int i = tid; i < n_local; i += kThreads) mass[i] = 0.f;
+    if (!alive) {
+        // a wait ran out: no scores, and the copies still under way land before their place is used again
+        for (int i = tid; i < n_local; i += kThreads)
+            for (int p = 0; p < C; ++p) peer_store(peer_addr(base_s + lay.mass + (base + i) * 4, p), 0.f);
+        if (tid == 0)
+            for (int t = 0; t < n_tiles; ++t) tile_landed(t);
+    }
     pc.mark();
 
-    // ---- the row of masses, pooled: every CTA its own copy ----
-    auto peer = [&](auto *x, int p) { return p == rank ? x : cl.map_shared_rank(x, p); };
+    // ---- the row of masses, which every CTA now has, pooled ----
     auto unit_sync = [&]() { if (C > 1) cl.sync(); else __syncthreads(); };
     unit_sync();
+    pc.mark();
     const int half = (d.kp - 1) / 2;
-    {
-        float *raw = reinterpret_cast<float *>(scratch);                  // [N]
-        for (int p = 0; p < C; ++p) {
-            const int from = start[p], n = min(start[p + 1], N) - from;
-            const float *m = peer(mass, p);
-            for (int i = tid; i < n; i += kThreads) raw[from + i] = m[i];
+    uint32_t key_lo = 0xffffffffu, key_hi = 0u;
+    for (int i = tid; i < N; i += kThreads) {
+        float best;
+        if (d.pool_avg) {
+            best = i >= half ? mass[i - half] : 0.f;
+            for (int t = 1 - half; t <= half; ++t) best += i + t >= 0 && i + t < N ? mass[i + t] : 0.f;
+            if (d.kp > 1) best /= (float)(2 * half + 1);
+        } else {
+            best = mass[i];
+#pragma unroll 4
+            for (int j = max(i - half, 0); j <= min(i + half, N - 1); ++j) best = fmaxf(best, mass[j]);
         }
-        __syncthreads();
-        for (int i = tid; i < N; i += kThreads) {
-            float best;
-            if (d.pool_avg) {
-                best = i >= half ? raw[i - half] : 0.f;
-                for (int t = 1 - half; t <= half; ++t) best += i + t >= 0 && i + t < N ? raw[i + t] : 0.f;
-                if (d.kp > 1) best /= (float)(2 * half + 1);
-            } else {
-                best = raw[i];
-                for (int j = max(i - half, 0); j <= min(i + half, N - 1); ++j) best = fmaxf(best, raw[j]);
-            }
-            row[i] = best;
-        }
-        __syncthreads();
+        row[i] = best;
+        key_lo = min(key_lo, float_to_key(best));
+        key_hi = max(key_hi, float_to_key(best));
     }
+    key_lo = __reduce_min_sync(0xffffffffu, key_lo);
+    key_hi = __reduce_max_sync(0xffffffffu, key_hi);
+    if (lane == 0) {
+        range[warp] = key_lo;
+        range[kWarps + warp] = key_hi;
+    }
+    __syncthreads();
+    key_lo = __reduce_min_sync(0xffffffffu, range[lane & (kWarps - 1)]);
+    key_hi = __reduce_max_sync(0xffffffffu, range[kWarps + (lane & (kWarps - 1))]);
     const int s0 = (int)((long long)N * rank / C), s1 = (int)((long long)N * (rank + 1) / C);      // this CTA's share of what is written
     if (a.scores_only)
         for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
@@ -407,22 +434,31 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (a.has_graph && !a.scores_only) {
         // ---- Eq. 2 ----
         const int k = d.K_src;
-        {
-            const rf::Threshold th = rf::block_threshold(row, N, (uint32_t)k, 0u, 0u, hist, wcnt, misc);
-            uint32_t gt, eq;
-            rf::kept_counts(row, N, th, gt, eq);
-            rf::kept_prefix(wcnt, gt, eq);
-            rf::emit_kept(row, N, th, gt, eq, [&](int t, int i) {
-                src_pos[t] = i;
-                if (rank == 0) a.src_out[(long long)unit * k + t] = i;
-            });
+        auto take = [&](int t, int i) {
+            src_pos[t] = i;
+            if (rank == 0) a.src_out[(long long)unit * k + t] = i;
+        };
+        bool found = false;
+        if (k <= bs::kTopMax) {
+            const bs::GroupScratch<kThreads> gs(scratch);
+            found = bs::group_top<kThreads>(row, N, k, 0, tid, gs) <= kThreads;
+            if (found && warp == 0) {
+                const int pos = lane < k ? rf::position_of(gs.top[lane]) : 0x7fffffff;
+                int t = 0;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) t += __shfl_sync(0xffffffffu, pos, u) < pos;
+                if (lane < k) take(t, pos);
+            }
+        }
+        if (!found) {
+            const bs::Kept th = bs::block_kth(row, N, (uint32_t)k, key_lo, key_hi, hist, wcnt, misc);
+            bs::emit_kept(row, N, th, wcnt, take);
         }
         __syncthreads();
         pc.mark();
 
         // ---- Eq. 1: the sources' rows as an operand, all tiles against them ----
-        constexpr int kPieces = kD / 8;
-        const int np = a.np;
+        const int np = a.z.np;
         const __nv_bfloat16 *Kh = a.K + b * d.ks[0] + (long long)h * d.ks[1];
         for (int i = tid; i < np * kPieces; i += kThreads) {
             const int r = i / kPieces, c16 = i % kPieces;
@@ -443,7 +479,6 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         fence_proxy_async();
         __syncthreads();
         bool ok = true;
-        static_assert(kMaxTiles <= 4, "a warp set per tile");
         if (n_emit > 0 && alive) {
             if (tid == 0) {
                 tc_fence_after();
@@ -457,28 +492,7 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 umma_commit(bar_done + 8 * (batch & 1));
             }
             __syncwarp();
-            // the keys' norms, a warp set per tile
-            const int t = set;
-            if (t < n_emit) {
-                ok = __all_sync(0xffffffffu, tile_landed(t));
-                if (ok) {
-                    const uint8_t *tile = gen + lay.tiles + t * kTile;
-                    float n0 = 0.f, n1 = 0.f;
-#pragma unroll
-                    for (int c16 = 0; c16 < kPieces; ++c16) {
-                        const uint4 raw = *reinterpret_cast<const uint4 *>(tile + sw128_offset(128, quad * 32 + lane, c16));
-                        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float lo = __uint_as_float(w[q] << 16), hi = __uint_as_float(w[q] & 0xffff0000u);
-                            n0 = fmaf(lo, lo, n0);
-                            n1 = fmaf(hi, hi, n1);
-                        }
-                    }
-                    inv_norm[t * kTileKeys + quad * 32 + lane] = 1.0f / fmaxf(sqrtf(n0 + n1), kNormEps);
-                }
-            }
-            ok = batch_done(batch) && ok;
+            ok = batch_done(batch);
             tc_fence_before();
             alive = __syncthreads_and(ok ? 1 : 0) != 0;
             ++batch;
@@ -486,146 +500,82 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         tc_fence_after();
         pc.mark();
 
-        // ---- Eq. 3, first half: per source the CTA's own best edges, sixteen sources at a time, a warp each ----
-        float *cosines = reinterpret_cast<float *>(region);                                       // [16][keys]
-        unsigned long long *lists = reinterpret_cast<unsigned long long *>(cosines + max(16 * keys, 8 * (kMaxCluster + 1) * kListCap));     // [k][kListCap]
-        const int m = d.m;
-        for (int g0 = 0; g0 < k; g0 += 16) {
-            for (int t = set; t < n_emit && alive; t += 4) {
-                float v[16];
-                tmem_ld16(tmem_lane + t * np + g0, v);
+        // ---- Eq. 3: source c belongs to CTA c % C, which gets its cosines with all keys; a.z.rows sources per CTA at a time ----
+        const int m = d.m, per_cta = ceil_div(k, C);
+        int *nb_j = reinterpret_cast<int *>(region);                                  // [k m] the unit's lists, in every CTA
+        float *nb_f = reinterpret_cast<float *>(nb_j + k * m);                        // [k m]
+        const float *cosines = reinterpret_cast<const float *>(gen + lay.cosines);    // [rows][row_step]
+        const int row_step = (N + 3) & ~3;
+        for (int r0 = 0; r0 < per_cta; r0 += a.z.rows) {
+            const int c_first = r0 * C, c_last = min(k, (r0 + a.z.rows) * C);
+            if (r0 > 0 || a.z.cosines_in_tiles) unit_sync();    // (the round before has been read; nobody reads tiles any more)
+            for (int t = set; t < n_emit; t += 4) {
                 const int i = t * kTileKeys + quad * 32 + lane, j = base + i;
                 const float inv = inv_norm[i];
+                const uint32_t to = base_s + lay.cosines + j * 4;
+                int slot = (c_first & ~7) / C, owner = (c_first & ~7) - slot * C;
+                for (int g0 = c_first & ~7; g0 < c_last; g0 += 8) {
+                    uint32_t raw[8];
+                    __syncwarp();
+                    tmem_ld8_issue(tmem_lane + t * np + g0, raw);
+                    tmem_ld_fence(raw);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    float e = kCandEmpty;
-                    if (g0 + c < k && j < N && j != src_pos[g0 + c])
-                        e = fminf(fmaxf(v[c] * inv * src_inv[g0 + c], -1.0f), 1.0f);
-                    cosines[c * keys + i] = e;
+                    for (int q = 0; q < 8; ++q) {
+                        const int c = g0 + q;
+                        if (c >= c_first && c < c_last && i < n_local) {
+                            float e = fminf(fmaxf(__uint_as_float(raw[q]) * inv * src_inv[c], -1.0f), 1.0f);
+                            if (j == src_pos[c] || !alive) e = kCandEmpty;
+                            peer_store(peer_addr(to + (slot - r0) * row_step * 4, owner), e);
+                        }
+                        if (++owner == C) owner = 0, ++slot;
+                    }
                 }
             }
-            __syncthreads();
-            if (g0 + warp < k) {
-                const float *x = cosines + warp * keys;
-                unsigned long long *out = lists + (g0 + warp) * kListCap;
-                float bound;
-                const int n = warp_list_top(alive ? n_local : 0, m, -1.0f, [&](int i) { return x[i]; },
-                                            [&](int at, float e, int i) { out[at] = edge_key(e, base + i); }, &bound);
-                if (lane == 0) {
-                    list_n[g0 + warp] = n;
-                    list_bound[g0 + warp] = bound;
+            tc_fence_before();
+            unit_sync();
+            pc.mark();
+            // the sources' lists, a group of threads each, and each list to all CTAs of the unit
+            constexpr int T = 128;
+            const int mine = min(a.z.rows, per_cta - r0), gang = tid / T, gt = tid % T;
+            const bs::GroupScratch<T> gs(scratch + gang * bs::GroupScratch<T>::kBytes);
+            for (int s = gang; s < mine; s += kThreads / T) {
+                const int c = (r0 + s) * C + rank;
+                if (c >= k) break;
+                const float *x = cosines + s * row_step;
+                if (bs::group_top<T>(x, N, m, 1 + gang, gt, gs) > T) {
+                    // ties: one warp finds exactly the m
+                    if (gt < 32) {
+                        float reached;
+                        const int n = warp_list_top(N, m, -1.0f, [&](int i) { return x[i]; },
+                                                    [&](int at, float e, int i) { gs.cand[at] = edge_key(e, i); }, &reached);
+                        if (lane == 0) gs.word[0] = (uint32_t)n;
+                    }
+                    bs::group_bar<T>(1 + gang);
+                    bs::group_rank(gs, (int)gs.word[0], m, 1 + gang, gt);
                 }
-            }
-            __syncthreads();
-        }
-        tc_fence_before();
-        unit_sync();
-        pc.mark();
-
-        // ---- Eq. 3, second half: source c is merged by CTA c % C, four warps each ----
-        // (m edges of one CTA reach its bound, so the highest of the CTAs' bounds bounds the unit's m-th edge)
-        const int fin_rows = ceil_div(k, C);
-        int *fin_j = reinterpret_cast<int *>(lists + k * kListCap);                   // [fin_rows][kMaxNeighbours]
-        float *fin_f = reinterpret_cast<float *>(fin_j + fin_rows * kMaxNeighbours);
-        constexpr int kGang = 128, kTops = kMaxCluster * kListCap;
-        const int gang = tid / kGang, gt = tid % kGang;
-        unsigned long long *all = reinterpret_cast<unsigned long long *>(cosines) + gang * (kTops + kListCap);      // [kTops] 0: no edge
-        unsigned long long *top = all + kTops;                                        // [kListCap]
-        uint32_t *top_n = misc + 8 + gang;
-        for (int c = rank + C * gang; c < k; c += C * (kThreads / kGang)) {
-            const int n_lane = lane < C ? peer(list_n, lane)[c] : 0;
-#pragma unroll
-            for (int q = 0; q < kTops / kGang; ++q) {                                 // peer 2 q + gt / 64, entry gt % 64
-                const int p = 2 * q + gt / kListCap, i = gt % kListCap, n = __shfl_sync(0xffffffffu, n_lane, p & 31);
-                all[q * kGang + gt] = p < C && i < n ? peer(lists, p)[c * kListCap + i] : 0ull;
-            }
-            rf::group_bar(1 + gang, kGang);
-            // thresholds tried by the whole gang, four edges per thread, until at most kListCap reach one
-            float bound = lane < C ? peer(list_bound, lane)[c] : -1.0f;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) bound = fmaxf(bound, __shfl_xor_sync(0xffffffffu, bound, o));
-            float e[kTops / kGang];
-#pragma unroll
-            for (int q = 0; q < kTops / kGang; ++q) {
-                const unsigned long long key = all[q * kGang + gt];
-                e[q] = key ? rf::edge_of(key) : kCandEmpty;
-            }
-            float lo = bound, hi = 1.0f;
-            int have = kTops + 1;
-            for (int it = 0; it < 12 && have > kListCap; ++it) {
-                // (the first round counts the bound itself)
-                const float t0 = it == 0 ? lo : lo + (hi - lo) * (1.0f / 3.0f), t1 = lo + (hi - lo) * (it == 0 ? 0.5f : 2.0f / 3.0f);
-                uint32_t q2 = 0;
-#pragma unroll
-                for (int q = 0; q < kTops / kGang; ++q) q2 += (e[q] >= t0 ? 1u : 0u) + (e[q] >= t1 ? 0x10000u : 0u);
-                q2 = __reduce_add_sync(0xffffffffu, q2);
-                uint32_t *votes = reinterpret_cast<uint32_t *>(scratch) + gang * 8 + (it & 1) * 4;
-                if (lane == 0) votes[gt >> 5] = q2;
-                rf::group_bar(1 + gang, kGang);
-                const uint32_t n2 = votes[0] + votes[1] + votes[2] + votes[3];
-                const int n0 = (int)(n2 & 0xffffu), n1 = (int)(n2 >> 16);
-                if (n1 >= m) {
-                    lo = t1;
-                    have = n1;
-                } else if (n0 >= m || it == 0) {
-                    lo = t0;
-                    hi = t1;
-                    have = n0;
-                } else {
-                    hi = t0;
+                if (lane < m) {
+                    const unsigned long long key = gs.top[lane];
+                    const float e = rf::edge_of(key);
+                    const bool is = key != 0ull && e >= -1.0f;
+                    const int j = is ? rf::position_of(key) : -1;
+                    const float f = is ? signal_factor(e, d.lambda, d.T, d.signal) : 1.f;
+                    if (gt < 32 && is) {
+                        a.nbr_idx[((long long)unit * k + c) * m + lane] = j;
+                        a.nbr_e[((long long)unit * k + c) * m + lane] = e;
+                    }
+                    const uint32_t to = base_s + lay.tiles + (c * m + lane) * 4;
+                    for (int p = gt >> 5; p < C; p += T / 32) {
+                        peer_store(peer_addr(to, p), __int_as_float(j));
+                        peer_store(peer_addr(to + k * m * 4, p), f);
+                    }
                 }
+                bs::group_bar<T>(1 + gang);
             }
-            if (have > kListCap) {
-                // near-ties: one warp finds exactly the m
-                if (gt < 32) {
-                    float reached;
-                    const int n = warp_list_top(kTops, m, bound, [&](int i) { return all[i] ? rf::edge_of(all[i]) : kCandEmpty; },
-                                                [&](int at, float, int i) { top[at] = all[i]; }, &reached);
-                    if (lane == 0) *top_n = (uint32_t)n;
-                }
-            } else {
-                if (gt == 0) *top_n = 0u;
-                rf::group_bar(1 + gang, kGang);
-#pragma unroll
-                for (int q = 0; q < kTops / kGang; ++q)
-                    if (e[q] >= lo) top[atomicAdd(top_n, 1u)] = all[q * kGang + gt];
-            }
-            rf::group_bar(1 + gang, kGang);
-            const int n = (int)*top_n;                                                // at most kListCap: two threads per edge
-            const int i = gt >> 1;
-            const unsigned long long me = i < n ? top[i] : 0ull;
-            int r = 0;
-#pragma unroll 4
-            for (int u = gt & 1; u < n; u += 2) r += top[u] > me;
-            r += __shfl_xor_sync(0xffffffffu, r, 1);
-            if (i >= n) r = i;                                                        // (fewer than m edges: empty places)
-            if ((gt & 1) == 0 && r < m) {
-                int j = -1;
-                float f = 1.f;
-                if (i < n) {
-                    const float e = rf::edge_of(me);
-                    j = rf::position_of(me);
-                    f = signal_factor(e, d.lambda, d.T, d.signal);
-                    a.nbr_idx[((long long)unit * k + c) * m + r] = j;
-                    a.nbr_e[((long long)unit * k + c) * m + r] = e;
-                }
-                fin_j[(c / C) * kMaxNeighbours + r] = j;
-                fin_f[(c / C) * kMaxNeighbours + r] = f;
-            }
-            rf::group_bar(1 + gang, kGang);
         }
         unit_sync();
         pc.mark();
 
         // ---- Eq. 5: every CTA applies the unit's lists to its copy of the row, sources in order ----
-        int *nb_j = reinterpret_cast<int *>(fin_f + fin_rows * kMaxNeighbours);       // [k m]
-        float *nb_f = reinterpret_cast<float *>(nb_j + k * m);
-        for (int p = tid; p < k * m; p += kThreads) {
-            const int c = p / m, at = (c / C) * kMaxNeighbours + p % m;
-            nb_j[p] = peer(fin_j, c % C)[at];
-            nb_f[p] = peer(fin_f, c % C)[at];
-        }
-        __syncthreads();
         const bool evict = d.signal == GRAPHKV_SIGNAL_EVICT;
         for (int q0 = 0; q0 < k; q0 += 4) {
             int slot[4];
@@ -638,29 +588,25 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (slot[u] >= 0 && (slot[u] & (kWarps - 1)) == warp) row[slot[u]] = evict ? -INFINITY : row[slot[u]] * f[u];
+                if ((uint32_t)slot[u] < (uint32_t)N && (slot[u] & (kWarps - 1)) == warp)
+                    row[slot[u]] = evict ? -INFINITY : row[slot[u]] * f[u];
                 __syncwarp();
             }
         }
         __syncthreads();
         pc.mark();
     }
-    if (C > 1) cl.barrier_arrive();                 // nothing of another CTA is read after this
-
     if (!a.scores_only) {
         if (a.scores)
             for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
         // ---- the B largest, in ascending position; a CTA takes its share of them ----
         const int B = a.per_batch_budget ? a.budget_of[b] : d.B;
-        const rf::Threshold th = rf::block_threshold(row, N, (uint32_t)B, 0u, 0u, hist, wcnt, misc);
+        const bs::Kept th = bs::block_kth(row, N, (uint32_t)B, key_lo, key_hi, hist, wcnt, misc);
         pc.mark();
-        uint32_t gt, eq;
-        rf::kept_counts(row, N, th, gt, eq);
-        rf::kept_prefix(wcnt, gt, eq);
         const int first = B * rank / C, count = B * (rank + 1) / C - first;
-        int *kept = reinterpret_cast<int *>(region + a.region) - B;         // [count]
+        int *kept = reinterpret_cast<int *>(region + a.z.lists + (a.z.cosines_in_tiles ? a.z.rows * ((N + 3) / 4 * 16) : 0));         // [count]
         int *idx = a.idx_out + (long long)unit * d.B;
-        rf::emit_kept(row, N, th, gt, eq, [&](int t, int i) {
+        bs::emit_kept(row, N, th, wcnt, [&](int t, int i) {
             if (t >= first && t < first + count) {
                 idx[t] = i;
                 kept[t - first] = i;
@@ -693,15 +639,8 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (dst[u]) *reinterpret_cast<uint4 *>(dst[u]) = v[u];
         }
     }
-    if (C > 1) cl.barrier_wait();
     pc.mark();
-    // copies still under way after a wait that ran out land before the CTA exits
-    if (!alive) {
-        if (tid == 0) {
-            for (int t = 0; t < n_tiles; ++t) tile_landed(t);
-            atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
-        }
-    }
+    if (!alive && tid == 0) atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {

@@ -440,6 +440,86 @@ graphkv_status run_mass_simt(const Dims &d, const Layout &l, const T *Q, const T
     return d.D == 64 ? launch_mass_simt<T, 64, 64>(d, l, Q, K, a, ws, st) : launch_mass_simt<T, 128, 64>(d, l, Q, K, a, ws, st);
 }
 
+// ---- clusters: what the device holds ---------------------------------------------------------------
+template <int kD, int kTiles> bool cluster_path_ready()
+{
+    static std::mutex mu;
+    static signed char state[64] = {};
+    return once_per_device(mu, state, [] {
+        return set_smem(cp::cluster_path_kernel<kD, kTiles>, kMaxSmem) &&
+               cudaFuncSetAttribute(cp::cluster_path_kernel<kD, kTiles>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    });
+}
+
+// Clusters of C CTAs that are all resident, one CTA per SM, for C = 1 .. cp::kMaxCluster (nullptr: no device): the device
+// is asked once (148, 74, 33, 15, 11, 7 clusters of 1, 2, 4, 8, 10, 16 on a B200).
+const int *resident_clusters()
+{
+    static std::once_flag once[64];
+    static int fits[64][cp::kMaxCluster + 1] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::call_once(once[dev], [dev] {
+        if (!cluster_path_ready<128, 1>()) return;
+        for (int q = 1; q <= cp::kMaxCluster; ++q) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(q);
+            cfg.blockDim = dim3(cp::kThreads);
+            cfg.dynamicSmemBytes = kMaxSmem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = q;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, cp::cluster_path_kernel<128, 1>, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            fits[dev][q] = n;
+        }
+    });
+    return fits[dev];
+}
+
+// Largest power-of-two cluster size (up to 8) at which `units` clusters are all resident.
+int resident_cluster_size(int units)
+{
+    const int *fits = resident_clusters();
+    for (int C = 8; fits && C >= 1; C /= 2)
+        if (fits[C] >= units) return C;
+    return 0;
+}
+
+// How the cluster path cuts a row of n_tiles key tiles: the smallest cluster whose CTAs have the fewest tiles, all
+// clusters resident (C = 0: none).
+struct ShortRow {
+    int C, tiles;
+};
+
+ShortRow short_row(const Dims &d)
+{
+    ShortRow s{0, 0};
+    const int n_tiles = ceil_div(d.L, tc::kTileKeys), most = cp::max_tiles(d.D);
+    if (!d.bf16 || n_tiles > cp::kMaxCluster * most || d.units > sm_count()) return s;
+    const int *fits = resident_clusters();
+    for (int C = 1; fits && C <= std::min(cp::kMaxCluster, n_tiles); ++C) {
+        if (fits[C] < d.units) continue;
+        const int tiles = ceil_div(n_tiles, C);
+        if (tiles <= most && (s.C == 0 || tiles < s.tiles)) s = ShortRow{C, tiles};
+    }
+    return s;
+}
+
+// The graph's parameters are ones the cluster path takes, and a call in stages would have its cosines from the tensor
+// cores too (wide pooling sends that to the register-tiled products, which round differently).
+inline bool short_row_graph(const Dims &d)
+{
+    return d.K_src <= cp::kMaxSources && d.m <= cp::kMaxNeighbours && !(d.reselect && d.T > 1) && cluster_plan(d).ok;
+}
+
 // ---- step (I), tensor-core path (bf16) -----------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                   const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -485,6 +565,7 @@ bool make_k_tensormap(CUtensorMap *tm, const void *K, const Dims &d, int rows, c
 struct EmitExtras {
     uint32_t *zero;
     int zero_words;
+    int stat_chunks;        // key chunks of the row statistics; 0: as suits the sweep
 };
 
 // Attention mass before pooling, a [units][N], tensor-core path (bf16).
@@ -517,12 +598,12 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     // the kernel of both sweeps (one launch of all units, all CTAs resident) clears the head of the
     // workspace itself; every other form gets a memset first
     const bool one_kernel = group >= d.units &&
-                            d.units * sweep_chunks(d.units, tiles_stats, 1, l.max_parts) <= sm_count() &&
+                            d.units * (ex.stat_chunks ? ex.stat_chunks : sweep_chunks(d.units, tiles_stats, 1, l.max_parts)) <= sm_count() &&
                             !env_int("GRAPHKV_TWO_SCORE_KERNELS", 0);
     if (!one_kernel && reset_words(d, l, ws, st) != GRAPHKV_OK) return GRAPHKV_ERR_CUDA;
     for (int u0 = 0; u0 < d.units && rc == GRAPHKV_OK; u0 += group) {
         const int nu = std::min(group, d.units - u0);
-        const int chunks_s = sweep_chunks(nu, tiles_stats, 1, l.max_parts);
+        const int chunks_s = ex.stat_chunks ? ex.stat_chunks : sweep_chunks(nu, tiles_stats, 1, l.max_parts);
         // The two separate kernels run two CTAs per SM: a launch of several waves then pays for its set-ups and
         // tails once (256 units of 16K keys: 259 -> 229 us and 255 -> 228 us for the two sweeps).  A chunk
         // leaves four partials per row, which a launch of few units and many chunks has no room for.
@@ -572,7 +653,7 @@ graphkv_status run_mass_tc(const Dims &d, const Layout &l, const __nv_bfloat16 *
     return rc;
 }
 
-constexpr EmitExtras kPlainEmit{nullptr, 0};
+constexpr EmitExtras kPlainEmit{nullptr, 0, 0};
 
 inline bool tc_mass(const __nv_bfloat16 *, const Dims &d) { (void)d; return !env_int("GRAPHKV_FORCE_SIMT", 0); }
 inline bool tc_mass(const float *, const Dims &) { return false; }
@@ -861,86 +942,48 @@ graphkv_status run_finish(const Dims &d, const Layout &l, int elem_bytes, const 
 
 
 // ---- the whole path in one kernel (cluster_path.cuh) ------------------------------------------------
-template <int kD, int kTiles> bool cluster_path_ready()
-{
-    static std::mutex mu;
-    static signed char state[64] = {};
-    return once_per_device(mu, state, [] { return set_smem(cp::cluster_path_kernel<kD, kTiles>, kMaxSmem); });
-}
-
-// Largest power-of-two cluster size (up to 8) at which `units` clusters are all resident, one CTA per
-// SM: the device is asked once (15, 33 and 74 clusters of 8, 4 and 2 on a B200).
-int resident_cluster_size(int units)
-{
-    static std::mutex mu;
-    static int fits[64][4] = {};                    // [device][log2 C] clusters, 0: not asked yet
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::lock_guard<std::mutex> lk(mu);
-    if (fits[dev][0] == 0) {
-        if (!cluster_path_ready<128, 1>()) return 0;
-        for (int q = 0; q < 4; ++q) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(1 << q);
-            cfg.blockDim = dim3(cp::kThreads);
-            cfg.dynamicSmemBytes = kMaxSmem;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1 << q;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, cp::cluster_path_kernel<128, 1>, &cfg) != cudaSuccess) {
-                cudaGetLastError();
-                n = -1;
-            }
-            fits[dev][q] = n == 0 ? -1 : n;
-        }
-    }
-    for (int q = 3; q >= 0; --q)
-        if (fits[dev][q] >= units) return 1 << q;
-    return 0;
-}
-
 struct ClusterPathPlan {
     bool ok;
-    int C, chunks, n_tiles, tiles, np, region;
+    int C, n_tiles;
+    cp::Sizes z;
     size_t smem;
 };
 
-template <int kD, int kTiles> size_t cluster_path_smem(int tiles, int region, int N)
-{
-    return cp::layout<kD, kTiles>(tiles, region, N).total;
-}
-
-ClusterPathPlan cluster_path_plan(const Dims &d, const Layout &l, bool graph)
+ClusterPathPlan cluster_path_plan(const Dims &d, bool graph)
 {
     ClusterPathPlan p{};
-    if (!d.bf16 || d.N > cp::kMaxRow || units_per_group(d) < d.units) return p;
-    for (const char *off : {"GRAPHKV_NO_CLUSTER", "GRAPHKV_FORCE_SIMT", "GRAPHKV_TWO_SCORE_KERNELS"})
-        if (env_int(off, 0)) return p;
-    if (env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) == 2) return p;
+    if (units_per_group(d) < d.units || (graph && !short_row_graph(d))) return p;
+    const ShortRow sr = short_row(d);
+    if (sr.C == 0) return p;
+    p.C = sr.C;
     p.n_tiles = ceil_div(d.L, tc::kTileKeys);
-    if (graph && (d.K_src > cp::kMaxSources || d.m > cp::kMaxNeighbours || (d.reselect && d.T > 1))) return p;
-    p.C = resident_cluster_size(d.units);
-    if (p.C == 0) return p;
-    while (p.C > 1 && p.C / 2 >= p.n_tiles) p.C /= 2;
-    p.chunks = sweep_chunks(d.units, p.n_tiles, 1, l.max_parts);       // the general path's chunks
-    int tiles = 0;
-    for (int r = 0; r < p.C; ++r)
-        tiles = std::max(tiles, cp::first_tile_of_chunk(p.n_tiles, p.chunks, cp::first_chunk(p.chunks, p.C, r + 1)) -
-                                    cp::first_tile_of_chunk(p.n_tiles, p.chunks, cp::first_chunk(p.chunks, p.C, r)));
-    if (tiles > cp::kMaxTiles || p.n_tiles > cp::kMeanTiles * p.C) return p;
-    p.np = d.K_src <= 16 ? 16 : d.K_src <= 32 ? 32 : 64;
-    p.tiles = tiles;
-    p.region = cp::region_bytes(tiles * tc::kTileKeys, p.C, graph ? d.K_src : 0, graph ? d.m : 0, d.B);
-    const auto smem_of = d.D == 64 ? (d.GW <= 128 ? cluster_path_smem<64, 1> : cluster_path_smem<64, 2>)
-                                   : (d.GW <= 128 ? cluster_path_smem<128, 1> : cluster_path_smem<128, 2>);
-    p.smem = smem_of(tiles, p.region, d.N);
-    p.ok = p.smem <= kMaxSmem;
+    p.z = cp::Sizes{d.N, sr.C, d.GW, sr.tiles, !graph || d.K_src <= 16 ? 16 : d.K_src <= 32 ? 32 : 64, 0,
+                    graph ? (d.K_src * d.m * 8 + 15) / 16 * 16 : 0, (d.B * 4 + 15) / 16 * 16, 0};
+    const auto layout_of_path = d.D == 64 ? (d.GW <= 128 ? cp::layout<64, 1> : cp::layout<64, 2>)
+                                          : (d.GW <= 128 ? cp::layout<128, 1> : cp::layout<128, 2>);
+    // the cosines of all a CTA's sources at once where that fits
+    const int per_cta = graph ? ceil_div(d.K_src, p.C) : 0;
+    for (int in_tiles = 0; in_tiles <= (graph ? 1 : 0) && !p.ok; ++in_tiles)
+        for (int rounds = 1; rounds <= std::max(1, std::min(2, per_cta)) && !p.ok; ++rounds) {
+            p.z.cosines_in_tiles = in_tiles;
+            p.z.rows = ceil_div(per_cta, rounds);
+            p.smem = layout_of_path(p.z).total;
+            p.ok = p.smem <= kMaxSmem;
+        }
     return p;
+}
+bool cluster_path_on()
+{
+    for (const char *off : {"GRAPHKV_NO_CLUSTER", "GRAPHKV_FORCE_SIMT", "GRAPHKV_TWO_SCORE_KERNELS"})
+        if (env_int(off, 0)) return false;
+    return env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) != 2;
+}
+// Key chunks of the row statistics of a row whose scores the cluster path can take (0: as suits the sweep): the general
+// kernels cut it the same way, so that a call has the same bits on either path, in stages or fused, whatever its graph.
+inline int short_row_chunks(const Dims &d)
+{
+    const ClusterPathPlan p = cluster_path_plan(d, false);
+    return p.ok ? p.C : 0;
 }
 
 graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPathPlan &pl, const __nv_bfloat16 *Q,
@@ -954,12 +997,8 @@ graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPat
     a.Q = Q;
     a.K = K;
     a.C = pl.C;
-    a.chunks = pl.chunks;
     a.n_tiles = pl.n_tiles;
-    a.tiles = pl.tiles;
-    a.np = pl.np;
-    a.region = pl.region;
-    a.part = at<float>(ws, l.part);
+    a.z = pl.z;
     a.status = at<int>(ws, l.status);
     a.scores = scores;
     a.scores_only = scores_only;
@@ -999,12 +1038,14 @@ template <typename T>
 graphkv_status do_score(const Dims &d, const Layout &l, const T *Q, const T *K, float *scores,
                         void *ws, cudaStream_t st)
 {
+    EmitExtras ex = kPlainEmit;
     if constexpr (sizeof(T) == 2) {
-        const ClusterPathPlan pl = cluster_path_plan(d, l, false);
-        if (pl.ok) return run_cluster_path(d, l, pl, Q, K, nullptr, nullptr, nullptr, nullptr, scores, true, false, ws, st);
+        const ClusterPathPlan pl = cluster_path_plan(d, false);
+        ex.stat_chunks = pl.ok ? pl.C : 0;
+        if (pl.ok && cluster_path_on()) return run_cluster_path(d, l, pl, Q, K, nullptr, nullptr, nullptr, nullptr, scores, true, false, ws, st);
     }
     float *a = d.kp > 1 ? at<float>(ws, l.a) : scores;
-    graphkv_status rc = run_mass(d, l, Q, K, a, ws, st);
+    graphkv_status rc = run_mass(d, l, Q, K, a, ws, st, ex);
     if (rc != GRAPHKV_OK || d.kp == 1) return rc;
     return run_pool_sources(d, a, scores, 0, nullptr, nullptr, nullptr, 0, st);
 }
@@ -1050,10 +1091,12 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
                            cudaStream_t st)
 {
     const bool graph = graph_active(d);
+    EmitExtras ex = kPlainEmit;
     if constexpr (sizeof(T) == 2) {
-        const ClusterPathPlan pl = cluster_path_plan(d, l, graph);
-        if (pl.ok)
+        const ClusterPathPlan pl = cluster_path_plan(d, graph);
+        if (pl.ok && cluster_path_on())
             return run_cluster_path(d, l, pl, Q, K, V, K_out, V_out, idx_out, t_keep_scores ? s : nullptr, false, graph, ws, st);
+        ex.stat_chunks = pl.ok ? pl.C : short_row_chunks(d);
     }
     float *a = d.kp > 1 ? at<float>(ws, l.a) : s;
     int *src = at<int>(ws, l.src);
@@ -1064,7 +1107,7 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
     graphkv_status rc;
     uint32_t *row_hist = nullptr;
     if (!graph) {
-        if ((rc = run_mass(d, l, Q, K, a, ws, st)) != GRAPHKV_OK) return rc;
+        if ((rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
         if (d.kp > 1 && !finish_pools &&
             (rc = run_pool_sources(d, a, s, 0, nullptr, nullptr, nullptr, 0, st)) != GRAPHKV_OK)
             return rc;
@@ -1074,7 +1117,6 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
             const CandidatePlan cd = candidate_plan(d, true, true, t_keep_scores, d.B);
             if (cd.ok && !cd.dense) row_hist = at<uint32_t>(ws, l.row_hist);
         }
-        EmitExtras ex = kPlainEmit;
         ex.zero = row_hist;
         ex.zero_words = cs::kBins;
         if ((rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
