@@ -161,7 +161,7 @@ __device__ __forceinline__ uint32_t score_setup(const ScoreSmem &s, uint8_t *gen
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    return *reinterpret_cast<volatile uint32_t *>(gen + (s.tmem_slot - s.q));
+    return __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(gen + (s.tmem_slot - s.q)), 0);
 }
 
 // TMA producer (one thread): key tiles t0 + i * step of (h, b), i in [i_begin, i_end), into the stage ring.
@@ -264,7 +264,7 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const long long lim = a.wait_cycles;
     uint8_t *gen;
     const ScoreSmem s = score_smem_layout<kD>(smem_raw, kRowsPad, a.stages, &gen);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x / kCtas, half = blockIdx.x % kCtas;
     int t0, t1;
@@ -296,28 +296,26 @@ score_stats_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     if (warp == 0) {
         if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim, kCtas);
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
-            for (int i = 0; i < n_local; ++i) {
-                const int st = i % a.stages, ph = (i / a.stages) & 1;
-                const int buf = i % kBufs, bph = (i / kBufs) & 1;
-                if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
-                if (!mbar_wait(s.full0 + 8 * st, ph, lim)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
+        // (all lanes: see umma_tile)
+        constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
+        const uint32_t q_lo = umma_desc_lo(s.q), ring_lo = umma_desc_lo(s.stage0);
+        int st = 0;
+        uint32_t ph = 0u;
+        for (int i = 0; i < n_local; ++i) {
+            const int buf = i % kBufs;
+            ok = mbar_wait(s.tempty0 + 8 * buf, ((i / kBufs) & 1) ^ 1, lim) && mbar_wait(s.full0 + 8 * st, ph, lim);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-                for (int rt = 0; rt < kRowTiles; ++rt) {
-#pragma unroll
-                    for (int k = 0; k < kD / 16; ++k) {
-                        const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
-                        const uint32_t qoff = (k >> 2) * (kRowsPad * 128) + rt * (128 * 128) + (k & 3) * 32;
-                        umma_bf16(tmem_base + buf * kBufCols + rt * 128, umma_desc_sw128(s.q + qoff),
-                                  umma_desc_sw128(kt + koff), idesc, k > 0);
-                    }
-                }
+                for (int rt = 0; rt < kRowTiles; ++rt)
+                    umma_tile<kD>(tmem_base + buf * kBufCols + rt * 128, q_lo + rt * (128 * 128 >> 4), kRowsPad * 128 >> 4,
+                                  ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, idesc);
                 umma_commit(s.empty0 + 8 * st);
                 if (!(a.withhold_commit == 1 && i == 0)) umma_commit(s.tfull0 + 8 * buf);
             }
+            __syncwarp();
+            if (++st == a.stages) st = 0, ph ^= 1u;
         }
     } else {
         // epilogue: thread = query row (TMEM lane); the four warp sets split the accumulator's
@@ -457,7 +455,7 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     float *row_w = row_c + 256;                                         // [kRowsPad] (D = 64)
     float *xchg = row_w + 256;                                          // [kXchg tiles][kSets][128]
     uint32_t *mass_hist = reinterpret_cast<uint32_t *>(gen + (s.misc - s.q) + (kCtas == 2 ? kScratchBytes2 : kScratchBytes));   // [kMassBins]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x;
     int t0, t1;
@@ -500,25 +498,22 @@ score_emit_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     if (warp == 0) {
         if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, a.stages, t0, n_ahead, n_local, h, b, lim);
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(128, n_cols);
-            for (int i = 0; i < n_local; ++i) {
-                const int st = i % a.stages, ph = (i / a.stages) & 1;
-                const int buf = i % kBufs, bph = (i / kBufs) & 1;
-                if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
-                if (!mbar_wait(s.full0 + 8 * st, ph, lim)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
-#pragma unroll
-                for (int k = 0; k < kD / 16; ++k) {
-                    const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
-                    const uint32_t qoff = (k >> 2) * (kRowsPad * 128) + (k & 3) * 32;
-                    umma_bf16(tmem_base + buf * kBufCols, umma_desc_sw128(kt + koff),
-                              umma_desc_sw128(s.q + qoff), idesc, k > 0);
-                }
+        const uint32_t idesc = umma_idesc_bf16(128, n_cols), q_lo = umma_desc_lo(s.q), ring_lo = umma_desc_lo(s.stage0);
+        int st = 0;
+        uint32_t ph = 0u;
+        for (int i = 0; i < n_local; ++i) {
+            const int buf = i % kBufs;
+            ok = mbar_wait(s.tempty0 + 8 * buf, ((i / kBufs) & 1) ^ 1, lim) && mbar_wait(s.full0 + 8 * st, ph, lim);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
+                umma_tile<kD>(tmem_base + buf * kBufCols, ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, q_lo,
+                              kRowsPad * 128 >> 4, idesc);
                 umma_commit(s.empty0 + 8 * st);
                 umma_commit(s.tfull0 + 8 * buf);
             }
+            __syncwarp();
+            if (++st == a.stages) st = 0, ph ^= 1u;
         }
     } else {
         // epilogue: thread = key (TMEM lane); the warp sets of a tile split the query rows (x32
@@ -638,7 +633,7 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     const long long lim = a.wait_cycles;
     uint8_t *gen;
     const ScoreSmem s = score_smem_layout<kD>(smem_raw, kRowsPad, a.stages, &gen);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x;
     const int S = a.stages;
@@ -696,28 +691,26 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
     if (warp == 0) {
         if (lane == 0 && ok) ok = score_produce<kD>(s, &tmK, S, t0, n_ahead, n_local, h, b, lim);
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
-            for (int i = 0; i < n_local; ++i) {
-                const int st = i % S, ph = (i / S) & 1;
-                const int buf = i % kBufs, bph = (i / kBufs) & 1;
-                if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
-                if (!mbar_wait(s.full0 + 8 * st, ph, lim)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
+        // (all lanes: see umma_tile)
+        constexpr uint32_t idesc = umma_idesc_bf16(128, 128);
+        const uint32_t q_lo = umma_desc_lo(s.q), ring_lo = umma_desc_lo(s.stage0);
+        int st = 0;
+        uint32_t ph = 0u;
+        for (int i = 0; i < n_local; ++i) {
+            const int buf = i % kBufs;
+            ok = mbar_wait(s.tempty0 + 8 * buf, ((i / kBufs) & 1) ^ 1, lim) && mbar_wait(s.full0 + 8 * st, ph, lim);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-                for (int rt = 0; rt < kTiles; ++rt) {
-#pragma unroll
-                    for (int k = 0; k < kD / 16; ++k) {
-                        const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
-                        const uint32_t qoff = (k >> 2) * (kRowsPad * 128) + rt * (128 * 128) + (k & 3) * 32;
-                        umma_bf16(tmem_base + buf * kBufCols + rt * 128, umma_desc_sw128(s.q + qoff),
-                                  umma_desc_sw128(kt + koff), idesc, k > 0);
-                    }
-                }
+                for (int rt = 0; rt < kTiles; ++rt)
+                    umma_tile<kD>(tmem_base + buf * kBufCols + rt * 128, q_lo + rt * (128 * 128 >> 4), kRowsPad * 128 >> 4,
+                                  ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, idesc);
                 umma_commit(s.empty0 + 8 * st);
                 if (!(a.withhold_commit == 1 && i == 0)) umma_commit(s.tfull0 + 8 * buf);
             }
+            __syncwarp();
+            if (++st == S) st = 0, ph ^= 1u;
         }
     } else {
         constexpr int kSetCols = 64;
@@ -875,26 +868,20 @@ score_fused_tc(const __grid_constant__ CUtensorMap tmK, ScoreTcArgs a)
                 }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(128, n_cols);
-            for (int k = 0; k < n_emit; ++k) {
-                const int tl = n_emit - 1 - k, st = tl % S, u = slot_use(tl, k);
-                const int i = n_local + k;                        // accumulator buffers keep rotating
-                const int buf = i % kBufs, bph = (i / kBufs) & 1;
-                if (!mbar_wait(s.tempty0 + 8 * buf, bph ^ 1, lim)) { ok = false; break; }
-                if (!mbar_wait(s.full0 + 8 * st, u & 1, lim)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t kt = s.stage0 + st * tile_bytes<kD>();
-#pragma unroll
-                for (int kk = 0; kk < kD / 16; ++kk) {
-                    const uint32_t koff = (kk >> 2) * kHalfBytes + (kk & 3) * 32;
-                    const uint32_t qoff = (kk >> 2) * (kRowsPad * 128) + (kk & 3) * 32;
-                    umma_bf16(tmem_base + buf * kBufCols, umma_desc_sw128(kt + koff),
-                              umma_desc_sw128(s.q + qoff), idesc, kk > 0);
-                }
+        const uint32_t idesc = umma_idesc_bf16(128, n_cols), q_lo = umma_desc_lo(s.q), ring_lo = umma_desc_lo(s.stage0);
+        for (int k = 0; k < n_emit; ++k) {
+            const int tl = n_emit - 1 - k, st = tl % S, u = slot_use(tl, k);
+            const int i = n_local + k, buf = i % kBufs;               // accumulator buffers keep rotating
+            ok = mbar_wait(s.tempty0 + 8 * buf, ((i / kBufs) & 1) ^ 1, lim) && mbar_wait(s.full0 + 8 * st, u & 1, lim);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
+                umma_tile<kD>(tmem_base + buf * kBufCols, ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, q_lo,
+                              kRowsPad * 128 >> 4, idesc);
                 umma_commit(s.empty0 + 8 * st);
                 umma_commit(s.tfull0 + 8 * buf);
             }
+            __syncwarp();
         }
     } else {
         const int quad = warp & 3, set = (warp - 2) >> 2;

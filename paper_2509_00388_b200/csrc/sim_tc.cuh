@@ -175,7 +175,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
 
     PhaseClock pc(threadIdx.x == 64);
     pc.mark();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int unit = a.unit0 + blockIdx.y, b = unit / d.hkv, h = unit % d.hkv;
     const int chunk = blockIdx.x;
     const int per = a.n_tiles / a.chunks, rem = a.n_tiles % a.chunks;
@@ -245,7 +245,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(gen + Sh::tmem);
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(gen + Sh::tmem), 0);
     bool ok = true;
     pc.mark();
 
@@ -263,23 +263,22 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
                     mbar_wait(s_full0 + 8 * (i % a.stages), (i / a.stages) & 1, lim);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, NP);
-            for (int i = 0; i < n_local; ++i) {
-                const int st = i % a.stages, ph = (i / a.stages) & 1;
-                if (!mbar_wait(s_full0 + 8 * st, ph, lim)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t kt = s_stage0 + st * tile_bytes<kD>();
-#pragma unroll
-                for (int k = 0; k < kD / 16; ++k) {
-                    const uint32_t koff = (k >> 2) * kHalfBytes + (k & 3) * 32;
-                    const uint32_t soff = (k >> 2) * (NP * 128) + (k & 3) * 32;
-                    umma_bf16(tmem_base + i * NP, umma_desc_sw128(kt + koff),
-                              umma_desc_sw128(base + soff), idesc, k > 0);
-                }
+        // (all lanes: see umma_tile)
+        constexpr uint32_t idesc = umma_idesc_bf16(128, NP);
+        const uint32_t src_lo = umma_desc_lo(base), ring_lo = umma_desc_lo(s_stage0);
+        int st = 0;
+        uint32_t ph = 0u;
+        for (int i = 0; i < n_local; ++i) {
+            ok = mbar_wait(s_full0 + 8 * st, ph, lim);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            tc_fence_after();
+            if (elect_one()) {
+                umma_tile<kD>(tmem_base + i * NP, ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, src_lo, NP * 128 >> 4, idesc);
                 umma_commit(s_empty0 + 8 * st);
                 umma_commit(s_done0 + 8 * i);
             }
+            __syncwarp();
+            if (++st == a.stages) st = 0, ph ^= 1u;
         }
     } else {
         // ---- epilogue: thread = key (TMEM lane), four sets of four warps.  With 64 sources a set takes 32 of

@@ -141,6 +141,38 @@ __device__ __forceinline__ void umma_bf16(uint32_t taddr, uint64_t adesc, uint64
         ::"r"(taddr), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// One thread of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(is));
+    return is != 0;
+}
+// This thread's warp, as a value the compiler knows to be the same in all its lanes.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
+
+// Low word of an operand descriptor (umma_desc_sw128); the high word is the same for all.  16 elements along K are 2
+// in it, 64 columns on half_bytes / 16.
+__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t addr) { return ((addr & 0x3ffffu) >> 4) | (1u << 16); }
+constexpr uint32_t kUmmaDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+// D[tmem] = A B^T over kD columns: A and B by the low words of their descriptors.  Called by all lanes of a warp, with the
+// same values: the operands then stay in uniform registers, where the instruction takes them from (issued from a branch
+// that one lane takes, with descriptors put together there, eight products took 1100 to 1400 clocks to issue).
+template <int kD>
+__device__ __forceinline__ void umma_tile(uint32_t taddr, uint32_t a_lo, uint32_t a_half, uint32_t b_lo, uint32_t b_half, uint32_t idesc)
+{
+#pragma unroll
+    for (int k = 0; k < kD / 16; ++k)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+            "mov.b64 a, {%1, %3};\n\t"
+            "mov.b64 b, {%2, %3};\n\t"
+            "setp.ne.u32 p, %5, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}"
+            ::"r"(taddr), "r"(a_lo + (k >> 2) * a_half + (k & 3) * 2), "r"(b_lo + (k >> 2) * b_half + (k & 3) * 2), "n"(kUmmaDescHi),
+              "r"(idesc), "r"((uint32_t)(k > 0))
+            : "memory");
+}
 // Arrive on `bar` once all MMAs issued so far by this thread have completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
