@@ -26,8 +26,8 @@
 
 namespace graphkv {
 
-constexpr int kDecWarps = 12;
-constexpr int kDecThreads = kDecWarps * 32;
+// Warps of a CTA: 12 where a CTA has an SM to itself, 6 where two share it.
+constexpr int kDecWarps = 12, kDecWarps2 = 6;
 constexpr int kDecStages = 2;          // blocks in a warp's ring
 constexpr int kDecHalf = 4096;         // bytes of K, and of V, in a block
 constexpr int kDecStage = 2 * kDecHalf;
@@ -37,7 +37,7 @@ template <typename T> __host__ __device__ constexpr int dec_rows() { return kDec
 constexpr int kDecMinBlocks = 6;
 constexpr int kDecMaxG = 8;            // query heads per KV head this kernel serves
 constexpr int kDecPart = 4 + kHeadDim; // floats of a partial result of one query head: max, sum, 2 unused, accumulator
-constexpr size_t kDecSmem = (size_t)kDecWarps * kDecStages * kDecStage;
+template <int kWarps> __host__ __device__ constexpr size_t dec_smem_bytes() { return (size_t)kWarps * kDecStages * kDecStage; }
 static_assert(kDecMaxG * kDecPart * 4 <= kDecStages * kDecStage, "a warp's result takes the place of its ring");
 
 struct DecodeArgs {
@@ -45,6 +45,7 @@ struct DecodeArgs {
     int blocks_per_unit;               // blocks of a unit
     int splits;                        // CTAs that share a unit
     int cluster;                       // they are one cluster
+    int two;                           // two CTAs per SM
     long long qs[2];                   // element strides of q: batch, head
     long long ks[3], vs[3];            // element strides of K and V: batch, head, row
     unsigned long long *arrived;       // [units] (call tag, count of CTAs that left their part), splits > 1; the call
@@ -344,12 +345,13 @@ template <int kG> struct DecodeSimt {
 // [G][kDecPart], into `dst` (the output rows, normalised, or a partial result).  All threads of the
 // CTA: kDecSplit groups of threads share the parts (four of them requested together), a thread of a group takes four
 // outputs; the groups' shares meet in `x` [kDecSplit][G][kDecPart] of shared memory.
-constexpr int kDecSplit = kDecThreads / 128;
-template <typename Part>
+constexpr int kDecSplit = 3;
+template <int kWarps, typename Part>
 __device__ __forceinline__ void decode_merge(int n, int G, Part part, float *x, bool normalise, float *dst,
                                              int dst_stride)
 {
-    const int grp = threadIdx.x >> 7, t = threadIdx.x & 127;
+    constexpr int kThreads = kWarps * 32, kWidth = kThreads / kDecSplit;
+    const int grp = threadIdx.x / kWidth, t = threadIdx.x % kWidth;
     auto fold = [&](int i0, int step, int count, auto get, int g, int d4, float &m, float &l, float4 &o) {
         for (int i = i0; i < count; i += 4 * step) {
             float4 pm[4], po[4];
@@ -376,7 +378,7 @@ __device__ __forceinline__ void decode_merge(int n, int G, Part part, float *x, 
             }
         }
     };
-    for (int u = t; u < G * 32; u += 128) {
+    for (int u = t; u < G * 32; u += kWidth) {
         const int g = u >> 5, d4 = u & 31;
         float m = kNegBig, l = 0.f;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -387,7 +389,7 @@ __device__ __forceinline__ void decode_merge(int n, int G, Part part, float *x, 
     }
     __syncthreads();
     auto shared = [&](int i, int w) { return *reinterpret_cast<const float4 *>(x + i * G * kDecPart + w); };
-    for (int u = threadIdx.x; u < G * 32; u += kDecThreads) {
+    for (int u = threadIdx.x; u < G * 32; u += kThreads) {
         const int g = u >> 5, d4 = u & 31;
         float m = kNegBig, l = 0.f;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -403,15 +405,16 @@ __device__ __forceinline__ void decode_merge(int n, int G, Part part, float *x, 
     }
 }
 
-// kG: query heads per KV head rounded up to 4 or 8.  grid (splits, units).
-template <typename T, int kG>
-__global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, const T *__restrict__ q,
+// kG: query heads per KV head rounded up to 4 or 8; kWarps 12, or 6 with two CTAs per SM.  grid (splits, units).
+template <typename T, int kG, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, kDecWarps / kWarps) decode_kernel(DecodeArgs a, const T *__restrict__ q,
                                                                 const T *__restrict__ K,
                                                                 const T *__restrict__ V)
 {
-    extern __shared__ __align__(128) uint8_t dec_smem[];         // [kDecWarps][kDecStages][kDecStage]
+    constexpr int kThreads = kWarps * 32;
+    extern __shared__ __align__(128) uint8_t dec_smem[];         // [kWarps][kDecStages][kDecStage]
     __shared__ __align__(16) float s_x[kDecSplit * kG * kDecPart];
-    __shared__ __align__(16) float s_q[sizeof(T) == 4 ? kG * kHeadDim : 4];
+    float *const s_q = s_x;                                      // fp32 rows: the queries [kG][kHeadDim], until the merges
     __shared__ __align__(16) float s_part[kG * kDecPart];
     __shared__ int s_last;
     constexpr int kRows = dec_rows<T>(), kPieces = kHeadDim * (int)sizeof(T) / 16;
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
     const int b = unit / a.hkv, h = unit % a.hkv;
     const int nb = a.blocks_per_unit;
     const int b0 = (int)((long long)nb * blockIdx.x / a.splits), b1 = (int)((long long)nb * (blockIdx.x + 1) / a.splits);
-    const int n_warps = min(kDecWarps, b1 - b0);                 // warps with rows
+    const int n_warps = min(kWarps, b1 - b0);                 // warps with rows
     const float scale = rsqrtf((float)kHeadDim) * kLog2e;
     const T *qu = q + b * a.qs[0] + (long long)(h * G) * a.qs[1];
     const T *Ku = K + b * a.ks[0] + (long long)h * a.ks[1];
@@ -429,7 +432,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
     const uint32_t ring_s = static_cast<uint32_t>(__cvta_generic_to_shared(ring));
     pdl_wait();
     pdl_launch_dependents();
-    if (a.splits > 1 && !a.cluster && tid == kDecThreads - 1) {
+    if (a.splits > 1 && !a.cluster && tid == kThreads - 1) {
         // this call's tag into the unit's arrival word (nobody waits for it: a word that changes in
         // between has been tagged by another CTA of this call)
         const unsigned long long seen = *reinterpret_cast<volatile unsigned long long *>(a.arrived + unit);
@@ -452,14 +455,14 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        for (int k = 0; k < kDecStages; ++k) request(b0 + warp + k * kDecWarps, k);
+        for (int k = 0; k < kDecStages; ++k) request(b0 + warp + k * kWarps, k);
         int stage = 0;
-        for (int i = b0 + warp; i < b1; i += kDecWarps) {
+        for (int i = b0 + warp; i < b1; i += kWarps) {
             asm volatile("cp.async.wait_group %0;" ::"n"(kDecStages - 1) : "memory");
             __syncwarp();
             run.block(ring_s + stage * kDecStage, i * kRows, a.rows, scale);
             __syncwarp();
-            request(i + kDecStages * kDecWarps, stage);
+            request(i + kDecStages * kWarps, stage);
             stage = stage + 1 == kDecStages ? 0 : stage + 1;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -470,7 +473,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
         run.load_q(qu, a.qs[1], G);
         walk(run);
     } else {
-        for (int i = tid; i < kG * kHeadDim; i += kDecThreads)
+        for (int i = tid; i < kG * kHeadDim; i += kThreads)
             s_q[i] = i / kHeadDim < G ? qu[(i / kHeadDim) * a.qs[1] + i % kHeadDim] : 0.f;
         __syncthreads();
         DecodeSimt<kG> run;
@@ -482,25 +485,25 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
         return *reinterpret_cast<const float4 *>(dec_smem + i * (kDecStages * kDecStage) + w * 4);
     };
     if (a.splits == 1) {
-        decode_merge(n_warps, G, of_warp, s_x, true, out, kHeadDim);
+        decode_merge<kWarps>(n_warps, G, of_warp, s_x, true, out, kHeadDim);
         return;
     }
     if (a.cluster) {
         // the parts stay in shared memory, where the first CTA of the unit's cluster reads them
         namespace cg = cooperative_groups;
         cg::cluster_group cl = cg::this_cluster();
-        decode_merge(n_warps, G, of_warp, s_x, false, s_part, kDecPart);
+        decode_merge<kWarps>(n_warps, G, of_warp, s_x, false, s_part, kDecPart);
         cl.sync();
         if (blockIdx.x == 0) {
             auto of_peer = [&](int i, int w) { return *reinterpret_cast<const float4 *>(cl.map_shared_rank(s_part, i) + w); };
-            decode_merge(a.splits, G, of_peer, s_x, true, out, kHeadDim);
+            decode_merge<kWarps>(a.splits, G, of_peer, s_x, true, out, kHeadDim);
         }
         cl.sync();                                               // nobody leaves while its part is read
         return;
     }
     // this CTA's part goes to memory; the last CTA of the unit to get here merges them
     float *parts = a.part + (long long)unit * a.splits * G * kDecPart;
-    decode_merge(n_warps, G, of_warp, s_x, false, parts + (long long)blockIdx.x * G * kDecPart, kDecPart);
+    decode_merge<kWarps>(n_warps, G, of_warp, s_x, false, parts + (long long)blockIdx.x * G * kDecPart, kDecPart);
     __syncthreads();
     if (tid == 0) {
         __threadfence();
@@ -512,7 +515,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(DecodeArgs a, co
         auto of_cta = [&](int i, int w) {
             return __ldcg(reinterpret_cast<const float4 *>(parts + (long long)i * G * kDecPart + w));
         };
-        decode_merge(a.splits, G, of_cta, s_x, true, out, kHeadDim);
+        decode_merge<kWarps>(a.splits, G, of_cta, s_x, true, out, kHeadDim);
         // (every CTA of the unit has added, so nobody else touches the word any more)
         if (tid == 0) a.arrived[unit] = 0ull;
     }

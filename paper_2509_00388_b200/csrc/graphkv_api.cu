@@ -1411,12 +1411,16 @@ static bool decode_shape(const graphkv_params *p, DecodeArgs *a)
     a->batch = p->batch; a->hq = p->n_q_heads; a->hkv = p->n_kv_heads; a->G = p->n_q_heads / p->n_kv_heads;
     a->rows = p->seq_len;
     a->blocks_per_unit = ceil_div(p->seq_len, p->dtype == GRAPHKV_BF16 ? dec_rows<__nv_bfloat16>() : dec_rows<float>());
-    // as many CTAs per unit as one wave holds (one per SM), with kDecMinBlocks blocks each or more.  (So a unit is
-    // one CTA from 75 units on, and a launch of somewhat more than 148 units pays for a second, short wave: 2080
-    // rows 19.4 us for 80 units, 25.6 for 128, 27.8 for 144, 40.4 for 152, 46.1 for 256, which is 4.4, 5.3, 5.5,
-    // 4.0 and 5.9 TB/s.  Weighing waves against parts to merge, as sweep_chunks does, is not done here.)
+    // As many CTAs per unit as one wave holds (one per SM), with kDecMinBlocks blocks each or more; a unit is one CTA from
+    // 75 units on.
     const int units = p->batch * p->n_kv_heads;
     a->splits = std::max(1, std::min(sm_count() / units, ceil_div(a->blocks_per_unit, kDecMinBlocks)));
+    // Somewhat more units than SMs: CTAs of half the warps, two per SM, so that no second, short wave follows (152 units
+    // of 2080 rows 40.5 -> 32.2 us, 200 units 42.2 -> 38.1; 256 units, where the second wave is fuller, 46.0 against 46.6, 224 of 4096
+    // rows 73.4 against 77.8).  Over short rows the waves' starts and merges weigh more, and overlap (256 units of 544 rows
+    // 18.0 -> 15.4, of 128 rows 9.9 -> 7.3).  Up to 148 units splitting each over two or three such CTAs loses (96 units of 2080
+    // rows 20.3 against 31.2, 128 units 25.5 against 27.1).
+    a->two = units > sm_count() && (20 * units <= 27 * sm_count() || a->blocks_per_unit <= 48);
     // CTAs of a unit that fit a cluster merge through shared memory instead of global memory and a counter
     // (544 rows 6.5 -> 5.8 us).  Up to 24 blocks per CTA a cluster of eight also beats more CTAs that do not
     // fit one (1032 rows 6.8 -> 6.4 us, 3032 rows 8.5 -> 8.2; 4132 rows 9.0 -> 9.2; clusters of four lose).
@@ -1442,16 +1446,21 @@ size_t graphkv_decode_workspace_bytes(const graphkv_params *params)
 }
 
 extern "C++" {
-template <typename T, int kG>
-static graphkv_status launch_decode(const DecodeArgs &a, const void *q, const void *K, const void *V, cudaStream_t st)
+template <typename T, int kG, int kWarps>
+static graphkv_status launch_decode_warps(const DecodeArgs &a, const void *q, const void *K, const void *V, cudaStream_t st)
 {
     static std::mutex mu;
     static signed char state[64] = {};
-    if (!once_per_device(mu, state, [] { return set_smem(decode_kernel<T, kG>, kDecSmem); }))
+    if (!once_per_device(mu, state, [] { return set_smem(decode_kernel<T, kG, kWarps>, dec_smem_bytes<kWarps>()); }))
         return GRAPHKV_ERR_CUDA;
-    return launch_ex("decode_attention", decode_kernel<T, kG>, dim3(a.splits, a.batch * a.hkv), dim3(kDecThreads), kDecSmem,
+    return launch_ex("decode_attention", decode_kernel<T, kG, kWarps>, dim3(a.splits, a.batch * a.hkv), dim3(kWarps * 32), dec_smem_bytes<kWarps>(),
                      st, next_launch_is_dependent(), a.cluster ? a.splits : 1, a, static_cast<const T *>(q), static_cast<const T *>(K),
                      static_cast<const T *>(V));
+}
+template <typename T, int kG>
+static graphkv_status launch_decode(const DecodeArgs &a, const void *q, const void *K, const void *V, cudaStream_t st)
+{
+    return a.two ? launch_decode_warps<T, kG, kDecWarps2>(a, q, K, V, st) : launch_decode_warps<T, kG, kDecWarps>(a, q, K, V, st);
 }
 }
 
