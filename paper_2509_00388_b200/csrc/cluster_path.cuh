@@ -14,7 +14,7 @@
 // Every arithmetic step is the general kernels': the same accumulators, the row statistics folded and
 // merged over the same key chunks in the same order (one chunk per CTA), the same pooling, cosines
 // and decay order; so the results agree with them to the bit.
-// 512 threads; thread 0 issues copies and MMAs between the barriers of the sweeps.
+// 512 threads; warp 0 issues copies and MMAs between the barriers of the sweeps.
 //
 // Measured on one B200, 8 KV heads, W = 32, 16 sources (four kernels; this kernel with clusters of 2, 4 or 8 that read from
 // one another and per-CTA lists of edges; now): 1003 tokens 43, 31.6, 24.1 us; 2000 tokens 47, 37.1, 28.1; 3000 tokens 53,
@@ -132,7 +132,7 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const Dims &d = a.d;
     const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C;
     const int b = unit / d.hkv, h = unit % d.hkv, N = d.N;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, quad = warp & 3, set = warp >> 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tc::warp_index(), quad = warp & 3, set = warp >> 2;
     const long long lim = a.wait_cycles;
     const uint32_t base_s = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base_s - smem_u32(smem_raw));
@@ -186,35 +186,36 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __syncthreads();
     tc_fence_after();
     if (C > 1) cl.barrier_wait();   // (every CTA of the unit has started: its shared memory may be written to)
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + (tmem_slot - base_s));
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(gen + (tmem_slot - base_s)), 0);
     const uint32_t tmem_lane = tmem + ((uint32_t)(quad * 32) << 16);
     bool alive = true;              // no wait of this CTA has run out (the same in all its threads)
     int batch = 0;                  // batches of MMAs so far; the announcements alternate between two barriers
     auto batch_done = [&](int bt) { return __all_sync(0xffffffffu, mbar_wait(bar_done + 8 * (bt & 1), (bt >> 1) & 1, lim)) != 0; };
     pc.mark();
 
+    const uint32_t q_lo = umma_desc_lo(base_s), tiles_lo = umma_desc_lo(base_s + lay.tiles);
     // ---- statistics: D = Q K^T, kGroups tiles per batch, two batches under way ----
     const float scale = rsqrtf((float)kD) * kLog2e;
     {
-        bool ok = true, issued_ok = true;                                 // (issued_ok: thread 0's own waits)
+        bool ok = true, issued_ok = true;                                 // (issued_ok: the issuing warp's own waits)
         const int n_batches = ceil_div(n_tiles, kGroups);
+        // (by all lanes of warp 0: see umma_tile)
         auto issue = [&](int bt) {
-            for (int t = bt * kGroups; t < min((bt + 1) * kGroups, n_tiles) && issued_ok; ++t) {
-                issued_ok = tile_landed(t);
-                if (!issued_ok) break;
-                tc_fence_after();
-                const uint32_t kt = base_s + lay.tiles + t * kTile;
-                const uint32_t out = tmem + ((bt & 1) * kGroups + t % kGroups) * kBufCols;
+            const int first = bt * kGroups, last = min(first + kGroups, n_tiles);
+            for (int t = first; t < last && issued_ok; ++t) issued_ok = __all_sync(0xffffffffu, tile_landed(t));
+            if (!issued_ok) return;
+            tc_fence_after();
+            if (elect_one()) {
+                for (int t = first; t < last; ++t)
 #pragma unroll
-                for (int rt = 0; rt < kTiles; ++rt)
-#pragma unroll
-                    for (int k = 0; k < kD / 16; ++k)
-                        umma_bf16(out + rt * 128, umma_desc_sw128(base_s + (k >> 2) * (kRowsPad * 128) + rt * (128 * 128) + (k & 3) * 32),
-                                  umma_desc_sw128(kt + (k >> 2) * kHalfBytes + (k & 3) * 32), umma_idesc_bf16(128, 128), k > 0);
+                    for (int rt = 0; rt < kTiles; ++rt)
+                        umma_tile<kD>(tmem + ((bt & 1) * kGroups + t - first) * kBufCols + rt * 128, q_lo + rt * (128 * 128 >> 4),
+                                      kRowsPad * 128 >> 4, tiles_lo + t * (kTile >> 4), kHalfBytes >> 4, umma_idesc_bf16(128, 128));
+                if (!(a.withhold_commit == 1 && bt == 0)) umma_commit(bar_done + 8 * (bt & 1));
             }
-            if (issued_ok && !(a.withhold_commit == 1 && bt == 0)) umma_commit(bar_done + 8 * (bt & 1));
+            __syncwarp();
         };
-        if (tid == 0)
+        if (warp == 0)
             for (int bt = 0; bt < min(2, n_batches); ++bt) issue(bt);
         const int grp = set / (4 / kGroups), col0 = (set % (4 / kGroups)) * 64, rt = col0 >> 7, key_off = col0 & 127;
         const int r = rt * 128 + quad * 32 + lane, last = N + (r < d.GW ? r % d.W : 0);      // last visible key of the row
@@ -249,10 +250,7 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             float2 *cta_part = reinterpret_cast<float2 *>(scratch);
             if (batch == n_batches - 1) cta_part[(kTiles == 1 ? set : set & 1) * kRowsPad + r] = make_float2(mx, z);
             alive = __syncthreads_and(ok && issued_ok ? 1 : 0) != 0;
-            if (alive && tid == 0) {
-                tc_fence_after();
-                if (batch + 2 < n_batches) issue(batch + 2);
-            }
+            if (alive && warp == 0 && batch + 2 < n_batches) issue(batch + 2);
         }
         if (alive && tid < d.GW) {
             // the chunk's statistics of this row, to every CTA of the unit
@@ -320,22 +318,19 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         const int n_cols = (d.GW + 31) & ~31, n_batches = ceil_div(n_emit, kGroups), batch0 = batch;
         const uint32_t idesc = umma_idesc_bf16(128, n_cols);
         auto issue = [&](int q) {
-            const int bt = batch0 + q;
-            for (int g = 0; g < kGroups && q * kGroups + g < n_emit && issued_ok; ++g) {
-                const int t = n_emit - 1 - (q * kGroups + g);
-                issued_ok = tile_landed(t);
-                if (!issued_ok) break;
-                tc_fence_after();
-                const uint32_t kt = base_s + lay.tiles + t * kTile, out = tmem + ((bt & 1) * kGroups + g) * kBufCols;
-#pragma unroll
-                for (int k = 0; k < kD / 16; ++k)
-                    umma_bf16(out, umma_desc_sw128(kt + (k >> 2) * kHalfBytes + (k & 3) * 32),
-                              umma_desc_sw128(base_s + (k >> 2) * (kRowsPad * 128) + (k & 3) * 32), idesc, k > 0);
-            }
-            if (issued_ok) umma_commit(bar_done + 8 * (bt & 1));
-        };
-        if (tid == 0) {
+            const int bt = batch0 + q, n = min(kGroups, n_emit - q * kGroups), last = n_emit - 1 - q * kGroups;
+            for (int g = 0; g < n && issued_ok; ++g) issued_ok = __all_sync(0xffffffffu, tile_landed(last - g));
+            if (!issued_ok) return;
             tc_fence_after();
+            if (elect_one()) {
+                for (int g = 0; g < n; ++g)
+                    umma_tile<kD>(tmem + ((bt & 1) * kGroups + g) * kBufCols, tiles_lo + (last - g) * (kTile >> 4), kHalfBytes >> 4, q_lo,
+                                  kRowsPad * 128 >> 4, idesc);
+                umma_commit(bar_done + 8 * (bt & 1));
+            }
+            __syncwarp();
+        };
+        if (warp == 0) {
             issue(0);
             if (n_batches > 1) issue(1);
         }
@@ -371,10 +366,7 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             tc_fence_before();
             alive = __syncthreads_and(ok && issued_ok ? 1 : 0) != 0;
             if (!alive) break;
-            if (tid == 0) {
-                tc_fence_after();
-                if (q + 2 < n_batches) issue(q + 2);
-            }
+            if (warp == 0 && q + 2 < n_batches) issue(q + 2);
             if (tid < kGroups * 128 && q * kGroups + tid / 128 < n_emit) {
                 const int t = n_emit - 1 - (q * kGroups + tid / 128), key = tid & 127;
                 const float *xs = x + (tid / 128) * kSets * 128 + key;
@@ -480,18 +472,15 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         __syncthreads();
         bool ok = true;
         if (n_emit > 0 && alive) {
-            if (tid == 0) {
+            if (warp == 0) {
                 tc_fence_after();
-                for (int t = 0; t < n_emit; ++t) {
-                    const uint32_t kt = base_s + lay.tiles + t * kTile;
-#pragma unroll
-                    for (int q = 0; q < kD / 16; ++q)
-                        umma_bf16(tmem + t * np, umma_desc_sw128(kt + (q >> 2) * kHalfBytes + (q & 3) * 32),
-                                  umma_desc_sw128(base_s + (q >> 2) * (np * 128) + (q & 3) * 32), umma_idesc_bf16(128, np), q > 0);
+                if (elect_one()) {
+                    for (int t = 0; t < n_emit; ++t)
+                        umma_tile<kD>(tmem + t * np, tiles_lo + t * (kTile >> 4), kHalfBytes >> 4, q_lo, np * 128 >> 4, umma_idesc_bf16(128, np));
+                    umma_commit(bar_done + 8 * (batch & 1));
                 }
-                umma_commit(bar_done + 8 * (batch & 1));
+                __syncwarp();
             }
-            __syncwarp();
             ok = batch_done(batch);
             tc_fence_before();
             alive = __syncthreads_and(ok ? 1 : 0) != 0;
