@@ -7,7 +7,9 @@
 // Measured for 1003 values on one SM: the 32 largest in order 4000 -> 1900 clocks.
 #pragma once
 
-#include "row_finish.cuh"
+#include <type_traits>
+
+#include "common.cuh"
 
 namespace graphkv {
 namespace bs {
@@ -19,10 +21,43 @@ constexpr int kRankCap = 128;           // elements of the threshold bin ranked 
 constexpr int kTopMax = 32;             // elements group_top takes at most
 constexpr uint32_t kAllTies = 0xffffffffu;
 
+__device__ __forceinline__ uint32_t incl_scan(uint32_t v, int lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
 // What a selection keeps: keys above thr, and of those equal to it the first `ties` by position (kAllTies: all).
 struct Kept {
     uint32_t thr, ties;
 };
+
+// The least and the greatest key of val[0 .. n).  wcnt: 2 * kWarps words.  Starts after and ends with a barrier.
+__device__ __forceinline__ void block_range(const float *val, int n, uint32_t *wcnt, uint32_t &lo, uint32_t &hi)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    lo = 0xffffffffu;
+    hi = 0u;
+    for (int i = threadIdx.x; i < n; i += kThreads) {
+        const uint32_t key = float_to_key(val[i]);
+        lo = min(lo, key);
+        hi = max(hi, key);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+        wcnt[warp] = lo;
+        wcnt[kWarps + warp] = hi;
+    }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, wcnt[lane & (kWarps - 1)]);
+    hi = __reduce_max_sync(0xffffffffu, wcnt[kWarps + (lane & (kWarps - 1))]);
+    __syncthreads();
+}
 
 // The k largest (1 <= k <= n) of val[0 .. n).  Where the threshold is expected to lie, lo .. hi in keys, is cut into
 // bins; the lowest bin takes all below, the highest all above, so any lo <= hi gives the right result.  hist: kBins words
@@ -55,7 +90,7 @@ __device__ __noinline__ Kept block_kth(const float *val, int n, uint32_t k, uint
         __syncthreads();
         const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wcnt[lane & (kWarps - 1)] : 0u);
         if (before < left && before + sum >= left) {
-            const uint32_t run = before + rf::incl_scan(c.x + c.y, lane) - (c.x + c.y);
+            const uint32_t run = before + incl_scan(c.x + c.y, lane) - (c.x + c.y);
             const uint32_t bin = 2u * (uint32_t)(kThreads - 1 - tid);
             if (run < left && run + c.y >= left) misc[0] = bin + 1u, misc[1] = run, misc[2] = c.y;
             else if (run + c.y < left && run + c.y + c.x >= left) misc[0] = bin, misc[1] = run + c.y, misc[2] = c.x;
@@ -107,18 +142,44 @@ __device__ __noinline__ Kept block_kth(const float *val, int n, uint32_t k, uint
 
 // put(t, i) for every element i that is kept, t its rank by position: every warp owns a contiguous run of elements.
 // wcnt: 2 * kWarps words.  Starts after a barrier; the words are free after the caller's next.
+__device__ __forceinline__ int run_length(int n) { return (ceil_div(n, kWarps) + 31) & ~31; }
+// ... where only the first of the ties are kept
+template <typename Put>
+__device__ __forceinline__ void emit_with_ties(const float *val, int n, Kept th, uint32_t *wcnt, Put put)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, seg = run_length(n), lo = min(warp * seg, n), hi = min(lo + seg, n);
+    const unsigned below = (1u << lane) - 1u;
+    uint32_t gt = 0, eq = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) {
+            if (lane == 0) {
+                wcnt[warp] = gt;
+                wcnt[kWarps + warp] = eq;
+            }
+            __syncthreads();
+            gt = __reduce_add_sync(0xffffffffu, lane < warp ? wcnt[lane] : 0u);
+            eq = __reduce_add_sync(0xffffffffu, lane < warp ? wcnt[kWarps + lane] : 0u);
+        }
+        for (int i0 = lo; i0 < hi; i0 += 32) {
+            const int i = i0 + lane;
+            const uint32_t key = i < hi ? float_to_key(val[i]) : 0u;
+            const bool is_gt = i < hi && key > th.thr, is_eq = i < hi && key == th.thr;
+            const unsigned bg = __ballot_sync(0xffffffffu, is_gt), be = __ballot_sync(0xffffffffu, is_eq);
+            const uint32_t g = gt + __popc(bg & below), e = eq + __popc(be & below);
+            if (pass == 1 && (is_gt || (is_eq && e < th.ties))) put((int)(g + min(e, th.ties)), i);
+            gt += __popc(bg);
+            eq += __popc(be);
+        }
+    }
+}
 template <typename Put>
 __device__ __forceinline__ void emit_kept(const float *val, int n, Kept th, uint32_t *wcnt, Put put)
 {
     if (th.ties != kAllTies) {
-        const rf::Threshold full{th.thr, 0xffffffffu, th.ties};
-        uint32_t gt, eq;
-        rf::kept_counts(val, n, full, gt, eq);
-        rf::kept_prefix(wcnt, gt, eq);
-        rf::emit_kept(val, n, full, gt, eq, put);
+        emit_with_ties(val, n, th, wcnt, put);
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, seg = rf::run_length(n);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, seg = run_length(n);
     const int lo = min(warp * seg, n), hi = min(lo + seg, n);
     constexpr int kQ = 4;
     unsigned bm[kQ];

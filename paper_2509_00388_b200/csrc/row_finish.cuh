@@ -25,21 +25,20 @@
 
 #include <type_traits>
 
-#include "common.cuh"
+#include "block_select.cuh"
 
 namespace graphkv {
 namespace rf {
 
 namespace cg = cooperative_groups;
 
-constexpr int kThreads = 512;
+constexpr int kThreads = bs::kThreads;      // 512
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCluster = 8;
 constexpr int kBins = 2048;
 constexpr int kSurvCap = 256;           // merged candidates a group ranks in shared memory
 constexpr int kMaxRow = 262144;         // scores per row
 constexpr int kMaxBudgets = 64;         // batch elements with a budget of their own per launch
-constexpr int kRankMax = 160;           // elements of the threshold digit ranked by counting (its square is what that costs)
 constexpr int kScratch = kWarps * kSurvCap * 8;     // bytes: histograms, the merges' survivors, the ranking's lists
 static_assert(kScratch >= 2 * kBins * 4, "two histograms");
 
@@ -94,22 +93,12 @@ struct Smem {
     uint32_t *misc;            // [16]
 };
 
-__device__ __forceinline__ uint32_t incl_scan(uint32_t v, int lane)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    return v;
-}
-
 // Exclusive prefix of v over the CTA's threads; *total: the sum.  One barrier; `wcnt` is free again
 // after the caller's next barrier.
 __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *wcnt, uint32_t *total)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t incl = incl_scan(v, lane);
+    const uint32_t incl = bs::incl_scan(v, lane);
     if (lane == 31) wcnt[warp] = incl;
     __syncthreads();
     const uint32_t w = lane < kWarps ? wcnt[lane] : 0u;
@@ -164,134 +153,6 @@ __device__ __forceinline__ void count_bin(uint32_t *hist, uint32_t bin, bool val
 __device__ __forceinline__ int digit_shift(int pass) { return pass <= 0 ? 21 : pass == 1 ? 10 : 0; }
 __device__ __forceinline__ int digit_count(int pass) { return pass == 2 ? 1024 : 2048; }
 
-// What a selection keeps: elements whose masked key exceeds `prefix`, and of those whose masked key equals it
-// the `remaining` first.
-struct Threshold {
-    uint32_t prefix, mask, remaining;
-};
-
-// The k largest of val[0 .. n) (shared memory): digits of the ordered image until few are left in the
-// threshold's, which are ranked by counting.  Where it is known in which digits the threshold lies
-// (`hi_digits` of them from the key lo_key on, 0: not known), those are cut into 2046 bins first (pass -1;
-// bins 0 and 2047 take what lies outside) and the plain digits follow only if that was not enough.
-// `hist`: 2 * kBins words.  Starts after and ends with a barrier.
-__device__ __noinline__ Threshold block_threshold(const float *val, int n, uint32_t k, uint32_t lo_key, uint32_t hi_digits,
-                                                  uint32_t *hist, uint32_t *wcnt, uint32_t *misc)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    Threshold th{0u, 0u, k};
-    const int fine = 32 - __clz(hi_digits * 1026u);        // (hi_digits << 21) >> fine <= 2046
-    for (int pass = hi_digits > 0 ? -1 : 0; pass < 3; ++pass) {
-        const int shift = digit_shift(pass), nb = digit_count(pass);
-        auto bin_of = [&](uint32_t key) {
-            if (pass >= 0) return (key >> shift) & (uint32_t)(nb - 1);
-            return key < lo_key ? 0u : min(1u + ((key - lo_key) >> fine), 2047u);
-        };
-        auto in_class = [&](uint32_t key) { return pass < 0 || (key & th.mask) == th.prefix; };
-        for (int i = tid; i < nb; i += kThreads) hist[i] = 0u;
-        __syncthreads();
-        for (int i0 = warp * 32; i0 < n; i0 += kThreads) {
-            const int i = i0 + lane;
-            const uint32_t key = i < n ? float_to_key(val[i]) : 0u;
-            count_bin(hist, bin_of(key), i < n && in_class(key));
-        }
-        __syncthreads();
-        if (tid == 0) misc[3] = 0u;
-        find_digit(hist, nb, th.remaining, wcnt, misc);
-        const uint32_t bin = misc[0], left = th.remaining - misc[1];
-        const int in = (int)misc[2];
-        if (pass < 0 && (bin == 0u || bin == 2047u || (in > kRankMax && in != (int)left))) {
-            __syncthreads();
-            continue;                                       // the plain digits, from the start
-        }
-        th.remaining = left;
-        if (in == (int)left) {                              // the whole class is kept
-            if (pass < 0) {
-                th = Threshold{lo_key + ((bin - 1u) << fine) - 1u, 0xffffffffu, 0u};        // everything above this
-            } else {
-                th.prefix |= bin << shift;
-                th.mask |= (uint32_t)(nb - 1) << shift;
-            }
-            break;
-        }
-        if (in <= kRankMax && pass < 2) {
-            uint32_t *list = hist + kBins;
-            for (int i = tid; i < n; i += kThreads) {
-                const uint32_t key = float_to_key(val[i]);
-                if (in_class(key) && bin_of(key) == bin) list[atomicAdd(&misc[3], 1u)] = key;
-            }
-            __syncthreads();
-            const int share = in * 4 <= kThreads ? 4 : in * 2 <= kThreads ? 2 : 1, i = tid / share, sub = tid & (share - 1);
-            const uint32_t me = i < in ? list[i] : 0xffffffffu;
-            uint32_t gt = 0, ge = 0;                        // larger ones; larger or equal
-#pragma unroll 4
-            for (int u = sub; u < in; u += share) {
-                const uint32_t x = list[u];
-                gt += x > me;
-                ge += x >= me;
-            }
-            if (share > 1) gt += __shfl_xor_sync(0xffffffffu, gt, 1), ge += __shfl_xor_sync(0xffffffffu, ge, 1);
-            if (share > 2) gt += __shfl_xor_sync(0xffffffffu, gt, 2), ge += __shfl_xor_sync(0xffffffffu, ge, 2);
-            if (i < in && gt < left && ge >= left) {
-                misc[4] = me;                               // the threshold (ties write the same)
-                misc[5] = left - gt;                        // of its ties, how many are kept
-            }
-            __syncthreads();
-            th = Threshold{misc[4], 0xffffffffu, misc[5]};
-            break;
-        }
-        th.prefix |= bin << shift;
-        th.mask |= (uint32_t)(nb - 1) << shift;
-        __syncthreads();
-    }
-    __syncthreads();
-    return th;
-}
-
-// Ordered output of what a selection keeps: every warp owns a contiguous run of elements.  Elements of
-// this warp's run above the threshold and equal to it ...
-__device__ __forceinline__ int run_length(int n) { return (ceil_div(n, kWarps) + 31) & ~31; }
-__device__ __forceinline__ void kept_counts(const float *val, int n, Threshold th, uint32_t &gt, uint32_t &eq)
-{
-    const int lane = threadIdx.x & 31, seg = run_length(n), lo = min((int)(threadIdx.x >> 5) * seg, n), hi = min(lo + seg, n);
-    gt = eq = 0;
-    for (int i0 = lo; i0 < hi; i0 += 32) {
-        const int i = i0 + lane;
-        const uint32_t key = i < hi ? float_to_key(val[i]) & th.mask : 0u;
-        gt += __popc(__ballot_sync(0xffffffffu, i < hi && key > th.prefix));
-        eq += __popc(__ballot_sync(0xffffffffu, i < hi && key == th.prefix));
-    }
-}
-// ... of the runs before it (the CTA's totals stay in wcnt[0 .. kWarps), wcnt[kWarps ..)) ...
-__device__ __forceinline__ void kept_prefix(uint32_t *wcnt, uint32_t &gt, uint32_t &eq)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        wcnt[warp] = gt;
-        wcnt[kWarps + warp] = eq;
-    }
-    __syncthreads();
-    gt = __reduce_add_sync(0xffffffffu, lane < warp ? wcnt[lane] : 0u);
-    eq = __reduce_add_sync(0xffffffffu, lane < warp ? wcnt[kWarps + lane] : 0u);
-}
-// ... and put(t, i) for every element i that is kept, t its rank by position.
-template <typename Put>
-__device__ __forceinline__ void emit_kept(const float *val, int n, Threshold th, uint32_t gt, uint32_t eq, Put put)
-{
-    const int lane = threadIdx.x & 31, seg = run_length(n), lo = min((int)(threadIdx.x >> 5) * seg, n), hi = min(lo + seg, n);
-    const unsigned below = (1u << lane) - 1u;
-    for (int i0 = lo; i0 < hi; i0 += 32) {
-        const int i = i0 + lane;
-        const uint32_t key = i < hi ? float_to_key(val[i]) & th.mask : 0u;
-        const bool is_gt = i < hi && key > th.prefix, is_eq = i < hi && key == th.prefix;
-        const unsigned bg = __ballot_sync(0xffffffffu, is_gt), be = __ballot_sync(0xffffffffu, is_eq);
-        const uint32_t g = gt + __popc(bg & below), e = eq + __popc(be & below);
-        if (is_gt || (is_eq && e < th.remaining)) put((int)(g + min(e, th.remaining)), i);
-        gt += __popc(bg);
-        eq += __popc(be);
-    }
-}
-
 __device__ __forceinline__ void group_bar(int id, int threads)
 {
     if (threads == 32) __syncwarp();
@@ -337,7 +198,7 @@ __device__ __noinline__ void merge_exact(const unsigned long long *cand, int slo
             // lane l holds digits 255 - 8 l - q (q < 8)
             uint32_t sum = 0;
             for (int q = 0; q < 8; ++q) sum += rh[255 - 8 * lane - q];
-            uint32_t run = incl_scan(sum, lane) - sum;
+            uint32_t run = bs::incl_scan(sum, lane) - sum;
             if (lane == 0) {
                 rh[256] = 0u;                                   // fewer edges than m: all are kept
                 rh[257] = remaining;
@@ -402,7 +263,7 @@ __device__ __forceinline__ void merge_source(const Dims &d, const Cand *cand_in,
     uint32_t mine = 0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) mine += h[q];
-    const uint32_t up_to = incl_scan(mine, lane), total = __shfl_sync(0xffffffffu, up_to, 31);
+    const uint32_t up_to = bs::incl_scan(mine, lane), total = __shfl_sync(0xffffffffu, up_to, 31);
     uint32_t run = total - up_to;               // listed edges in the bins above this lane's
     int bstar = -1;
 #pragma unroll
@@ -773,14 +634,16 @@ __global__ void __launch_bounds__(kThreads, 2) finish_kernel(FinishArgs a)
         pc.mark();
         if (a.do_select) {
             // ---- the B largest candidates, in ascending position ----
-            const Threshold th = block_threshold(s.val, n, (uint32_t)B, lo_key, lowers || !a.has_graph ? hi_digits : 0u, s.hist,
-                                                 s.wcnt, s.misc);
+            uint32_t lo = lo_key, hi = 0xffffffffu;
+            if (hi_digits > 0 && (lowers || !a.has_graph)) {
+                if (hi_digits <= (0xffffffffu - lo_key) >> 21) hi = lo_key + (hi_digits << 21) - 1u;
+            } else {
+                bs::block_range(s.val, n, s.wcnt, lo, hi);
+            }
+            const bs::Kept th = bs::block_kth(s.val, n, (uint32_t)B, lo, hi, s.hist, s.wcnt, s.misc);
             pc.mark();
-            uint32_t gt, eq;
-            kept_counts(s.val, n, th, gt, eq);
-            kept_prefix(s.wcnt, gt, eq);
             int *idx = a.idx_out + (long long)unit * d.B;
-            emit_kept(s.val, n, th, gt, eq, [&](int t, int i) {
+            bs::emit_kept(s.val, n, th, s.wcnt, [&](int t, int i) {
                 const int j = a.dense ? i : s.pos[i];
                 idx[t] = j;
                 s.kept[t] = j;
