@@ -18,6 +18,7 @@
 #include "score_simt.cuh"
 #include "score_tc.cuh"
 #include "select.cuh"
+#include "sim_stream.cuh"
 #include "sim_tc.cuh"
 
 using namespace graphkv;
@@ -44,6 +45,7 @@ struct Layout {
     size_t nbr_e;
     size_t cand;        // per-chunk neighbour candidates [units][K_src][sim_chunks][kCandCap]
     size_t cand_hist;   // [units][K_src][kCandBins]
+    size_t tau;         // bounds of the sources' m-th edges [units][K_src]
     size_t total;
     int max_parts;      // partial statistics per row the region can hold
 };
@@ -191,11 +193,13 @@ struct SimPlan {
     int chunks;     // CTAs (key chunks) per unit
     int n_tiles;    // 128-key tiles per unit
     int stages;
+    bool stream;    // bounds from a sample, then one sweep for all sources (NP: up to 256)
+    int sample, sample_ctas;    // sample tiles, and the CTAs that share them
 };
 
 SimPlan sim_plan(const Dims &d, bool bf16)
 {
-    SimPlan p{false, 16, 1, ceil_div(d.N, tc::kTileKeys), 5};
+    SimPlan p{false, 16, 1, ceil_div(d.N, tc::kTileKeys), 5, false, 0, 0};
     if (!bf16 || d.K_src < 1 || d.K_src > kSimMaxSources || d.m < 1 ||
         d.m > tc::kSimMaxNeighbors)
         return p;
@@ -213,6 +217,24 @@ SimPlan sim_plan(const Dims &d, bool bf16)
     const int cap = 512 / p.NP;
     p.chunks = sweep_chunks(group * ceil_div(d.K_src, p.NP), p.n_tiles, ceil_div(p.n_tiles, cap), 1 << 20);
     p.ok = true;
+    // A head's sources in one streaming sweep, with bounds from a sample (sim_stream.cuh), where that form would take more
+    // than one wave of CTAs: the sample costs 20 us, which one wave does not (32 sources at 32K x 8 heads: 92 against 104
+    // us a call), but two waves do (40 sources 107 -> 106, 64 118 -> 115, 154 179 -> 141; 32 sources at 128K x 32 heads
+    // 1082 -> 1031, 16K x 128 with 40 sources 566 -> 444, with 100 846 -> 594).  Not with up to 16 sources, of which that form
+    // holds 32 tiles (16K x 128: 481 against 507).
+    if (group >= d.units && d.K_src > 16 && p.n_tiles >= 16 && (long long)d.units * ceil_div(d.K_src, p.NP) * p.chunks > sm_count()) {
+        p.stream = true;
+        const int sweeps = ceil_div(d.K_src, tc::kStreamMaxSources);
+        p.NP = ceil_div(ceil_div(d.K_src, sweeps), 32) * 32;
+        p.chunks = sweep_chunks(d.units * sweeps, p.n_tiles, ceil_div(p.n_tiles, tc::kStreamMaxTiles), 1 << 20);
+        for (p.stages = 6; p.stages > 3; --p.stages)
+            if ((d.D == 64 ? tc::stream_layout<64>(p.NP, p.stages) : tc::stream_layout<128>(p.NP, p.stages)).bytes <= kMaxSmem) break;
+        // the larger the sample, the fewer edges reach the bounds (about 1.1 m n_tiles / sample of a row's); a cluster of up to
+        // four CTAs, 16 tiles each, takes it
+        p.sample_ctas = std::max(1, std::min(4, sm_count() / (d.units * ceil_div(d.K_src, 32))));
+        p.sample = std::min(16 * p.sample_ctas, ceil_div(p.n_tiles, 2));
+        p.sample_ctas = std::min(p.sample_ctas, p.sample);
+    }
     return p;
 }
 
@@ -241,6 +263,7 @@ Layout layout_of(const Dims &d)
     const size_t slots = sp.ok ? (size_t)d.units * d.K_src * sp.chunks : 1;
     l.cand = take(slots * kCandCap * sizeof(Cand));
     l.cand_hist = take((size_t)d.units * (d.K_src > 0 ? d.K_src : 1) * kCandBins * sizeof(uint32_t));
+    l.tau = take((size_t)d.units * (d.K_src > 0 ? d.K_src : 1) * sizeof(float));
     l.total = off;
     return l;
 }
@@ -747,6 +770,30 @@ graphkv_status launch_similarity(const CUtensorMap &tmK, const tc::SimTcArgs &sa
                      sa.wait_prior != 0, 1, tmK, sa);
 }
 
+// Bounds from a sample of the row, then one sweep for all sources (sim_stream.cuh).
+template <int kD>
+graphkv_status run_stream(const Dims &d, const Layout &l, const SimPlan &sp, const CUtensorMap &tmK, const __nv_bfloat16 *S,
+                          const long long *ss, const int *src, void *ws, cudaStream_t st)
+{
+    static std::mutex mu;
+    static signed char state[64] = {};
+    if (!once_per_device(mu, state, [] {
+            return set_smem(tc::similarity_tc<32, kD, true>, tc::sim_smem_bytes<32, kD>()) && set_smem(tc::sim_stream_tc<kD>, kMaxSmem);
+        }))
+        return GRAPHKV_ERR_CUDA;
+    tc::SimTcArgs ba{d, S, {ss[0], ss[1], ss[2]}, src, nullptr, nullptr, at<int>(ws, l.status), 0, sp.sample_ctas, sp.sample,
+                     d.D == 64 ? 8 : 5, 0, wait_cycles(), sp.n_tiles, at<float>(ws, l.tau)};
+    ba.wait_prior = next_launch_is_dependent();
+    const graphkv_status rc = launch_ex("similarity_bounds", tc::similarity_tc<32, kD, true>, dim3(sp.sample_ctas, d.units, ceil_div(d.K_src, 32)),
+                                        dim3(tc::kSimThreads), tc::sim_smem_bytes<32, kD>(), st, ba.wait_prior != 0, sp.sample_ctas, tmK, ba);
+    if (rc != GRAPHKV_OK) return rc;
+    tc::SimStreamArgs sa{d, S, {ss[0], ss[1], ss[2]}, src, at<float>(ws, l.tau), at<Cand>(ws, l.cand), at<uint32_t>(ws, l.cand_hist),
+                         at<int>(ws, l.status), sp.chunks, sp.n_tiles, sp.NP, sp.stages, 0, wait_cycles()};
+    sa.wait_prior = next_launch_is_dependent();
+    return launch_ex("similarity_tc", tc::sim_stream_tc<kD>, dim3(sp.chunks, d.units, ceil_div(d.K_src, sp.NP)), dim3(tc::kStreamThreads),
+                     tc::stream_layout<kD>(sp.NP, sp.stages).bytes, st, sa.wait_prior != 0, 1, tmK, sa);
+}
+
 template <typename T>
 graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &eo, const int *src, void *ws,
                          cudaStream_t st)
@@ -755,13 +802,17 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
     if (sp.ok) {
         CUtensorMap tmK;
         if (!make_k_tensormap(&tmK, eo.A, d, d.L, eo.as)) return GRAPHKV_ERR_CUDA;
+        if (sp.stream) {
+            const auto *S = reinterpret_cast<const __nv_bfloat16 *>(eo.S);
+            return d.D == 64 ? run_stream<64>(d, l, sp, tmK, S, eo.ss, src, ws, st) : run_stream<128>(d, l, sp, tmK, S, eo.ss, src, ws, st);
+        }
         const int group = units_per_group(d);
         for (int u0 = 0; u0 < d.units; u0 += group) {
             const int nu = std::min(group, d.units - u0);
             // one launch takes every source: grid.z counts the sweeps of sp.NP sources each
             tc::SimTcArgs sa{d, reinterpret_cast<const __nv_bfloat16 *>(eo.S), {eo.ss[0], eo.ss[1], eo.ss[2]}, src, at<Cand>(ws, l.cand),
                              at<uint32_t>(ws, l.cand_hist), at<int>(ws, l.status), u0, sp.chunks,
-                             sp.n_tiles, sp.stages, 0, wait_cycles()};
+                             sp.n_tiles, sp.stages, 0, wait_cycles(), sp.n_tiles, nullptr};
             sa.wait_prior = next_launch_is_dependent();
             const dim3 grid(sp.chunks, nu, ceil_div(d.K_src, sp.NP)), block(tc::kSimThreads);
             const auto launch = d.D == 64 ? (sp.NP == 16 ? launch_similarity<16, 64> : sp.NP == 32 ? launch_similarity<32, 64>

@@ -26,6 +26,8 @@
 // with the cosines of 16 sources staged in shared memory and searched there, 9 and 17.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "edge_search.cuh"
@@ -54,6 +56,8 @@ struct SimTcArgs {
     int stages;
     int wait_prior;        // launched with programmatic stream serialization
     long long wait_cycles; // limit of every wait of the kernel, in clocks
+    int row_tiles;         // sampling form: n_tiles tiles spread evenly over the row's, shared by the `chunks` CTAs of a cluster
+    float *tau;            // sampling form: [units][K_src] per source, a value that at least m of its edges reach
 };
 
 template <int NP> __host__ __device__ constexpr int sim_tiles_cap() { return 512 / NP; }
@@ -149,7 +153,9 @@ __device__ __noinline__ void list_anew(uint8_t *gen, uint32_t tmem_base, int n_l
     __syncwarp();
 }
 
-template <int NP, int kD>
+// kSample: bounds only, of a sample of the row: the CTAs of a cluster (one unit and NP sources) take sample tiles in turn
+// and combine their maxima, each for its share of the sources.
+template <int NP, int kD, bool kSample = false>
 __global__ void __launch_bounds__(kSimThreads, 1)
 similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
 {
@@ -181,6 +187,9 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     const int per = a.n_tiles / a.chunks, rem = a.n_tiles % a.chunks;
     const int t0 = chunk * per + min(chunk, rem);
     const int n_local = per + (chunk < rem ? 1 : 0);
+    auto tile_of = [&](int i) {
+        return kSample ? (int)((long long)(chunk + i * a.chunks) * a.row_tiles / a.n_tiles) : t0 + i;
+    };
     const __nv_bfloat16 *src_rows = a.S + b * a.ss[0] + (long long)h * a.ss[1];
     // a head with more than NP sources is swept once per NP of them: grid.z counts those sweeps
     const int src0 = blockIdx.z * NP;
@@ -201,7 +210,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
         // input of the call: no wait for the kernels before)
         n_ahead = min(a.stages, n_local);
         for (int i = 0; i < n_ahead; ++i)
-            tma_load_tile<kD>(s_stage0 + i * tile_bytes<kD>(), &tmK, s_full0 + 8 * i, (t0 + i) * kTileKeys, h, b);
+            tma_load_tile<kD>(s_stage0 + i * tile_bytes<kD>(), &tmK, s_full0 + 8 * i, tile_of(i) * kTileKeys, h, b);
     }
     if (warp == 1) {
         tmem_alloc(s_tmem, 512);
@@ -255,7 +264,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             for (int i = n_ahead; i < n_local; ++i) {
                 const int st = i % a.stages, ph = (i / a.stages) & 1;
                 if (!mbar_wait(s_empty0 + 8 * st, ph ^ 1, lim)) { ok = false; break; }
-                tma_load_tile<kD>(s_stage0 + st * tile_bytes<kD>(), &tmK, s_full0 + 8 * st, (t0 + i) * kTileKeys, h, b);
+                tma_load_tile<kD>(s_stage0 + st * tile_bytes<kD>(), &tmK, s_full0 + 8 * st, tile_of(i) * kTileKeys, h, b);
                 ++issued;
             }
             if (!ok)        // gave up: let the copies already in flight land before the CTA exits
@@ -320,7 +329,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
                     }
                 }
                 const int key = i * kTileKeys + key_lane;
-                const bool in = t0 * kTileKeys + key < d.N;
+                const bool in = tile_of(i) * kTileKeys + key_lane < d.N;
                 // (a key past the end of the row: NaN, which no comparison and no maximum takes)
                 const float inv = in ? 1.0f / fmaxf(sqrtf(n0 + n1), kNormEps) : __int_as_float(0x7fc00000);
                 if (col0 == 0) inv_norm[key] = inv;
@@ -341,7 +350,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
         const bool all_ok = *reinterpret_cast<volatile int *>(failed) == 0;
         const int keys = n_local * kTileKeys, j0 = t0 * kTileKeys;
         asm volatile("bar.sync 1, 512;" ::: "memory");
-        if (all_ok) {
+        if (!kSample && all_ok) {
             // 1. bounds
             for (int c = ew; c < n_src; c += 16) {
                 const float bound = warp_bound_of_maxima<kParts>(maxima + c * kParts, d.m);
@@ -470,7 +479,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             }
             pc.mark();
         }
-        if (!all_ok)
+        if (!kSample && !all_ok)
             // a wait ran out: publish empty lists so the merge reads nothing undefined
             for (int i = et; i < n_src * kCandCap; i += kSimEpiThreads) {
                 const long long slot = ((long long)unit * d.K_src + src0 + i / kCandCap) * a.chunks + chunk;
@@ -480,6 +489,36 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     }
     if (!ok && a.status) atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
     tc_fence_before();
+    if constexpr (kSample) {
+        // (where a wait ran out, the maxima are of fewer keys, whose edges reach the bound all the same)
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        if (warp >= 2)
+            for (int c = chunk + a.chunks * (warp - 2); c < n_src; c += a.chunks * 16) {
+                float *row = maxima + c * kParts;
+                float4 x[kParts / 128], y[3][kParts / 128];               // (clusters of up to four: all loads in flight)
+#pragma unroll
+                for (int q = 0; q < kParts / 128; ++q) x[q] = reinterpret_cast<float4 *>(row)[q * 32 + lane];
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {
+                    const float4 *other = reinterpret_cast<const float4 *>(cl.map_shared_rank(row, (chunk + 1 + min(p, a.chunks - 1)) % a.chunks));
+#pragma unroll
+                    for (int q = 0; q < kParts / 128; ++q) y[p][q] = other[q * 32 + lane];
+                }
+#pragma unroll
+                for (int q = 0; q < kParts / 128; ++q) {
+#pragma unroll
+                    for (int p = 0; p < 3; ++p)
+                        x[q] = make_float4(fmaxf(x[q].x, y[p][q].x), fmaxf(x[q].y, y[p][q].y), fmaxf(x[q].z, y[p][q].z), fmaxf(x[q].w, y[p][q].w));
+                    reinterpret_cast<float4 *>(row)[q * 32 + lane] = x[q];
+                }
+                __syncwarp();
+                const float bound = warp_bound_of_maxima<kParts>(row, d.m);
+                if (lane == 0) a.tau[(long long)unit * d.K_src + src0 + c] = bound;
+            }
+        cl.sync();                              // (nobody leaves while its maxima are read)
+    }
     __syncthreads();
     if (warp == 1) {
         __syncwarp();
@@ -487,7 +526,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
         tmem_dealloc(tmem_base, 512);
     }
     pc.mark();
-    pc.flush(2);
+    pc.flush(kSample ? 1 : 2);
 }
 
 }  // namespace tc
