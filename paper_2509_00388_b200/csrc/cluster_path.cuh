@@ -24,6 +24,7 @@
 #include "block_select.cuh"
 #include "edge_search.cuh"
 #include "row_finish.cuh"
+#include "score_simt.cuh"
 #include "score_tc.cuh"
 
 namespace graphkv {
@@ -45,7 +46,7 @@ constexpr int kMaxNeighbours = 32;
 // [C][GW] the cosines [rows][N].  Those come from other CTAs, which do not know whether this one's sweep is over:
 // in the tiles' place (behind the lists) they cost one more cluster barrier, so only where nothing else fits.
 struct Layout {
-    int tiles, mass, row, inv, row_c, parts, cosines, scratch, small, bars, total;
+    int tiles, lists, mass, row, inv, row_c, parts, cosines, scratch, small, bars, total;
 };
 constexpr int kScratch = 6656;                  // partial statistics or exchange (4 KB each), histogram, groups' lists
 static_assert(kScratch >= 4 * bs::GroupScratch<128>::kBytes && kScratch >= bs::GroupScratch<kThreads>::kBytes &&
@@ -59,7 +60,7 @@ template <int kD, int kTiles> __host__ __device__ inline Layout layout(const Siz
     const int row = (z.N + 3) / 4 * 16, parts = (z.C * z.GW * 8 + 15) / 16 * 16, queries = 128 * kTiles * 2 * kD;
     const int cosines = z.rows * row, region = z.lists + z.kept + (z.cosines_in_tiles ? cosines : 0);
     int off = queries;
-    l.tiles = off;
+    l.tiles = l.lists = off;
     off += z.tiles * tc::tile_bytes<kD>() > region ? z.tiles * tc::tile_bytes<kD>() : region;
     l.mass = off;    off += row;                // the unit's attention mass before pooling
     l.row = z.np * 2 * kD;                      // the unit's scores
@@ -81,7 +82,7 @@ template <int kD, int kTiles> __host__ __device__ inline Layout layout(const Siz
 
 struct PathArgs {
     Dims d;
-    const __nv_bfloat16 *Q, *K;
+    const void *Q, *K;         // bf16 or fp32
     int C;                     // CTAs per unit, and key chunks of the row statistics
     int n_tiles;               // key tiles per unit
     Sizes z;                   // tiles: most key tiles a CTA owns; np: sources padded to 16, 32 or 64; rows: sources whose
@@ -118,6 +119,222 @@ __device__ __forceinline__ void peer_store(uint32_t addr, float2 x)
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x.x), "f"(x.y) : "memory");
 }
 
+// The small arrays.
+struct Small {
+    uint32_t *wcnt, *misc;     // [2 * kWarps], [32]
+    int *src_pos;              // [kMaxSources]
+    float *src_inv;            // [kMaxSources]
+    uint32_t *range;           // [2 * kWarps] least and greatest pooled score per warp
+    __device__ __forceinline__ explicit Small(uint8_t *p)
+        : wcnt(reinterpret_cast<uint32_t *>(p)), misc(wcnt + 2 * kWarps), src_pos(reinterpret_cast<int *>(misc + 32)),
+          src_inv(reinterpret_cast<float *>(src_pos + kMaxSources)), range(reinterpret_cast<uint32_t *>(src_inv + kMaxSources)) {}
+};
+
+// What follows the masses, in both forms of the kernel: pooling, sources, neighbourhoods, decay, selection and gather.
+// kEs: bytes per element.  base: first key of this CTA.  prepare(src_pos): the products of the sources with this CTA's
+// keys (sources known, ends with a barrier); push(c0, c1, put): put(c, c / C, c % C, i, cosine) for sources c0 .. c1 and every
+// key i of this CTA.
+template <int kEs, typename Prepare, typename Push>
+__device__ __forceinline__ void finish_path(const PathArgs &a, const Layout &lay, cg::cluster_group &cl, uint8_t *gen, uint32_t base_s,
+                                            int base, const bool &alive, PhaseClock &pc, Prepare prepare, Push push)
+{
+    const Dims &d = a.d;
+    const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C, b = unit / d.hkv, h = unit % d.hkv, N = d.N;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tc::warp_index();
+    const float *mass = reinterpret_cast<const float *>(gen + lay.mass);  // [N] the unit's masses, written by all its CTAs
+    float *row = reinterpret_cast<float *>(gen + lay.row);                // [N] the unit's scores, whole
+    uint8_t *scratch = gen + lay.scratch;
+    uint32_t *hist = reinterpret_cast<uint32_t *>(scratch);
+    const Small sm(gen + lay.small);
+    uint32_t *wcnt = sm.wcnt, *misc = sm.misc, *range = sm.range;
+    int *src_pos = sm.src_pos;
+    // ---- the row of masses, which every CTA now has, pooled ----
+    auto unit_sync = [&]() { if (C > 1) cl.sync(); else __syncthreads(); };
+    unit_sync();
+    pc.mark();
+    const int half = (d.kp - 1) / 2;
+    uint32_t key_lo = 0xffffffffu, key_hi = 0u;
+    for (int i = tid; i < N; i += kThreads) {
+        float best;
+        if (d.pool_avg) {
+            best = i >= half ? mass[i - half] : 0.f;
+            for (int t = 1 - half; t <= half; ++t) best += i + t >= 0 && i + t < N ? mass[i + t] : 0.f;
+            if (d.kp > 1) best /= (float)(2 * half + 1);
+        } else {
+            best = mass[i];
+#pragma unroll 4
+            for (int j = max(i - half, 0); j <= min(i + half, N - 1); ++j) best = fmaxf(best, mass[j]);
+        }
+        row[i] = best;
+        key_lo = min(key_lo, float_to_key(best));
+        key_hi = max(key_hi, float_to_key(best));
+    }
+    key_lo = __reduce_min_sync(0xffffffffu, key_lo);
+    key_hi = __reduce_max_sync(0xffffffffu, key_hi);
+    if (lane == 0) {
+        range[warp] = key_lo;
+        range[kWarps + warp] = key_hi;
+    }
+    __syncthreads();
+    key_lo = __reduce_min_sync(0xffffffffu, range[lane & (kWarps - 1)]);
+    key_hi = __reduce_max_sync(0xffffffffu, range[kWarps + (lane & (kWarps - 1))]);
+    const int s0 = (int)((long long)N * rank / C), s1 = (int)((long long)N * (rank + 1) / C);      // this CTA's share of what is written
+    if (a.scores_only)
+        for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
+    pc.mark();
+
+    uint8_t *region = gen + lay.lists;                                    // once the sweeps are over
+    if (a.has_graph && !a.scores_only) {
+        // ---- Eq. 2 ----
+        const int k = d.K_src;
+        auto take = [&](int t, int i) {
+            src_pos[t] = i;
+            if (rank == 0) a.src_out[(long long)unit * k + t] = i;
+        };
+        bool found = false;
+        if (k <= bs::kTopMax) {
+            const bs::GroupScratch<kThreads> gs(scratch);
+            found = bs::group_top<kThreads>(row, N, k, 0, tid, gs) <= kThreads;
+            if (found && warp == 0) {
+                const int pos = lane < k ? rf::position_of(gs.top[lane]) : 0x7fffffff;
+                int t = 0;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) t += __shfl_sync(0xffffffffu, pos, u) < pos;
+                if (lane < k) take(t, pos);
+            }
+        }
+        if (!found) {
+            const bs::Kept th = bs::block_kth(row, N, (uint32_t)k, key_lo, key_hi, hist, wcnt, misc);
+            bs::emit_kept(row, N, th, wcnt, take);
+        }
+        __syncthreads();
+        pc.mark();
+
+        prepare(src_pos);
+        pc.mark();
+
+        // ---- Eq. 3: source c belongs to CTA c % C, which gets its cosines with all keys; a.z.rows sources per CTA at a time ----
+        const int m = d.m, per_cta = ceil_div(k, C);
+        int *nb_j = reinterpret_cast<int *>(region);                                  // [k m] the unit's lists, in every CTA
+        float *nb_f = reinterpret_cast<float *>(nb_j + k * m);                        // [k m]
+        const float *cosines = reinterpret_cast<const float *>(gen + lay.cosines);    // [rows][row_step]
+        const int row_step = (N + 3) & ~3;
+        for (int r0 = 0; r0 < per_cta; r0 += a.z.rows) {
+            const int c_first = r0 * C, c_last = min(k, (r0 + a.z.rows) * C);
+            if (r0 > 0 || a.z.cosines_in_tiles) unit_sync();    // (the round before has been read; nobody reads tiles any more)
+            push(c_first, c_last, [&](int c, int slot, int owner, int i, float e) {
+                peer_store(peer_addr(base_s + lay.cosines + ((slot - r0) * row_step + base + i) * 4, owner),
+                           base + i == src_pos[c] || !alive ? kCandEmpty : e);
+            });
+            unit_sync();
+            pc.mark();
+            // the sources' lists, a group of threads each, and each list to all CTAs of the unit
+            constexpr int T = 128;
+            const int mine = min(a.z.rows, per_cta - r0), gang = tid / T, gt = tid % T;
+            const bs::GroupScratch<T> gs(scratch + gang * bs::GroupScratch<T>::kBytes);
+            for (int s = gang; s < mine; s += kThreads / T) {
+                const int c = (r0 + s) * C + rank;
+                if (c >= k) break;
+                const float *x = cosines + s * row_step;
+                if (bs::group_top<T>(x, N, m, 1 + gang, gt, gs) > T) {
+                    // ties: one warp finds exactly the m
+                    if (gt < 32) {
+                        float reached;
+                        const int n = warp_list_top(N, m, -1.0f, [&](int i) { return x[i]; },
+                                                    [&](int at, float e, int i) { gs.cand[at] = edge_key(e, i); }, &reached);
+                        if (lane == 0) gs.word[0] = (uint32_t)n;
+                    }
+                    bs::group_bar<T>(1 + gang);
+                    bs::group_rank(gs, (int)gs.word[0], m, 1 + gang, gt);
+                }
+                if (lane < m) {
+                    const unsigned long long key = gs.top[lane];
+                    const float e = rf::edge_of(key);
+                    const bool is = key != 0ull && e >= -1.0f;
+                    const int j = is ? rf::position_of(key) : -1;
+                    const float f = is ? signal_factor(e, d.lambda, d.T, d.signal) : 1.f;
+                    if (gt < 32 && is) {
+                        a.nbr_idx[((long long)unit * k + c) * m + lane] = j;
+                        a.nbr_e[((long long)unit * k + c) * m + lane] = e;
+                    }
+                    const uint32_t to = base_s + lay.lists + (c * m + lane) * 4;
+                    for (int p = gt >> 5; p < C; p += T / 32) {
+                        peer_store(peer_addr(to, p), __int_as_float(j));
+                        peer_store(peer_addr(to + k * m * 4, p), f);
+                    }
+                }
+                bs::group_bar<T>(1 + gang);
+            }
+        }
+        unit_sync();
+        pc.mark();
+
+        // ---- Eq. 5: every CTA applies the unit's lists to its copy of the row, sources in order ----
+        const bool evict = d.signal == GRAPHKV_SIGNAL_EVICT;
+        for (int q0 = 0; q0 < k; q0 += 4) {
+            int slot[4];
+            float f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = lane < m && q0 + u < k;
+                slot[u] = in ? nb_j[(q0 + u) * m + lane] : -1;
+                f[u] = in ? nb_f[(q0 + u) * m + lane] : 1.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if ((uint32_t)slot[u] < (uint32_t)N && (slot[u] & (kWarps - 1)) == warp)
+                    row[slot[u]] = evict ? -INFINITY : row[slot[u]] * f[u];
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        pc.mark();
+    }
+    if (!a.scores_only) {
+        if (a.scores)
+            for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
+        // ---- the B largest, in ascending position; a CTA takes its share of them ----
+        const int B = a.per_batch_budget ? a.budget_of[b] : d.B;
+        const bs::Kept th = bs::block_kth(row, N, (uint32_t)B, key_lo, key_hi, hist, wcnt, misc);
+        pc.mark();
+        const int first = B * rank / C, count = B * (rank + 1) / C - first;
+        int *kept = reinterpret_cast<int *>(region + a.z.lists + (a.z.cosines_in_tiles ? a.z.rows * ((N + 3) / 4 * 16) : 0));         // [count]
+        int *idx = a.idx_out + (long long)unit * d.B;
+        bs::emit_kept(row, N, th, wcnt, [&](int t, int i) {
+            if (t >= first && t < first + count) {
+                idx[t] = i;
+                kept[t - first] = i;
+            }
+        });
+        __syncthreads();
+        pc.mark();
+        // ---- gather: the CTA's share of the kept rows and of the window rows ----
+        const int vl = a.vpr_log2;
+        const unsigned char *k0 = a.Kb + (b * d.ks[0] + h * d.ks[1]) * kEs, *v0 = a.V + (b * d.vs[0] + h * d.vs[1]) * kEs;
+        const long long out0 = (long long)unit * (d.B + d.W);
+        const int w0 = d.W * rank / C, w1 = d.W * (rank + 1) / C, n_rows = count + (w1 - w0);
+        for (int p0 = tid; p0 < n_rows << (vl + 1); p0 += 4 * kThreads) {
+            uint4 v[4];
+            unsigned char *dst[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = p0 + u * kThreads, t = p >> (vl + 1), c = p & ((1 << vl) - 1);
+                dst[u] = nullptr;
+                if (t < n_rows) {
+                    const bool is_v = (p >> vl) & 1;
+                    const int w = w0 + (t - count);
+                    const long long from = t < count ? kept[t] : N + w, to = out0 + (t < count ? first + t : B + w);
+                    v[u] = *reinterpret_cast<const uint4 *>((is_v ? v0 + from * d.vs[2] * kEs : k0 + from * d.ks[2] * kEs) + c * 16);
+                    dst[u] = (is_v ? a.V_out : a.K_out) + ((to << vl) + c) * 16;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (dst[u]) *reinterpret_cast<uint4 *>(dst[u]) = v[u];
+        }
+    }
+}
+
 // kTiles = 1 (G*W <= 128) or 2 (G*W <= 256).  grid = units * C CTAs in clusters of C.
 template <int kD, int kTiles>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -137,17 +354,10 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const uint32_t base_s = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base_s - smem_u32(smem_raw));
     const Layout lay = layout<kD, kTiles>(a.z);
-    const float *mass = reinterpret_cast<const float *>(gen + lay.mass);  // [N] the unit's masses, written by all its CTAs
     float *inv_norm = reinterpret_cast<float *>(gen + lay.inv);
-    float *row = reinterpret_cast<float *>(gen + lay.row);                // [N] the unit's scores, whole
     float *row_c = reinterpret_cast<float *>(gen + lay.row_c), *row_w = row_c + kRowsPad;
     uint8_t *scratch = gen + lay.scratch;
-    uint32_t *hist = reinterpret_cast<uint32_t *>(scratch);
-    uint32_t *wcnt = reinterpret_cast<uint32_t *>(gen + lay.small);       // [2 * kWarps]
-    uint32_t *misc = wcnt + 2 * kWarps;                                   // [32]
-    int *src_pos = reinterpret_cast<int *>(misc + 32);                    // [kMaxSources]
-    float *src_inv = reinterpret_cast<float *>(src_pos + kMaxSources);    // [kMaxSources]
-    uint32_t *range = reinterpret_cast<uint32_t *>(src_inv + kMaxSources);      // [2 * kWarps] least and greatest pooled score per warp
+    float *src_inv = Small(gen + lay.small).src_inv;
     const uint32_t bar_full = base_s + lay.bars, bar_done = bar_full + 8 * kMaxTiles, tmem_slot = bar_done + 16;
     PhaseClock pc(tid == 0);
     pc.mark();
@@ -180,7 +390,7 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             tma_load_tile<kD>(base_s + lay.tiles + t * kTile, &tmK, bar_full + 8 * t, (t0 + t) * kTileKeys, h, b);
         if (rank == 0 && unit == 0) *a.status = 0;
     }
-    stage_q<kD>(gen, kRowsPad, d, a.Q, b, h, tid, kThreads);
+    stage_q<kD>(gen, kRowsPad, d, static_cast<const __nv_bfloat16 *>(a.Q), b, h, tid, kThreads);
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -387,71 +597,10 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     }
     pc.mark();
 
-    // ---- the row of masses, which every CTA now has, pooled ----
-    auto unit_sync = [&]() { if (C > 1) cl.sync(); else __syncthreads(); };
-    unit_sync();
-    pc.mark();
-    const int half = (d.kp - 1) / 2;
-    uint32_t key_lo = 0xffffffffu, key_hi = 0u;
-    for (int i = tid; i < N; i += kThreads) {
-        float best;
-        if (d.pool_avg) {
-            best = i >= half ? mass[i - half] : 0.f;
-            for (int t = 1 - half; t <= half; ++t) best += i + t >= 0 && i + t < N ? mass[i + t] : 0.f;
-            if (d.kp > 1) best /= (float)(2 * half + 1);
-        } else {
-            best = mass[i];
-#pragma unroll 4
-            for (int j = max(i - half, 0); j <= min(i + half, N - 1); ++j) best = fmaxf(best, mass[j]);
-        }
-        row[i] = best;
-        key_lo = min(key_lo, float_to_key(best));
-        key_hi = max(key_hi, float_to_key(best));
-    }
-    key_lo = __reduce_min_sync(0xffffffffu, key_lo);
-    key_hi = __reduce_max_sync(0xffffffffu, key_hi);
-    if (lane == 0) {
-        range[warp] = key_lo;
-        range[kWarps + warp] = key_hi;
-    }
-    __syncthreads();
-    key_lo = __reduce_min_sync(0xffffffffu, range[lane & (kWarps - 1)]);
-    key_hi = __reduce_max_sync(0xffffffffu, range[kWarps + (lane & (kWarps - 1))]);
-    const int s0 = (int)((long long)N * rank / C), s1 = (int)((long long)N * (rank + 1) / C);      // this CTA's share of what is written
-    if (a.scores_only)
-        for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
-    pc.mark();
-
-    uint8_t *region = gen + lay.tiles;                                    // once the sweeps are over
-    if (a.has_graph && !a.scores_only) {
-        // ---- Eq. 2 ----
-        const int k = d.K_src;
-        auto take = [&](int t, int i) {
-            src_pos[t] = i;
-            if (rank == 0) a.src_out[(long long)unit * k + t] = i;
-        };
-        bool found = false;
-        if (k <= bs::kTopMax) {
-            const bs::GroupScratch<kThreads> gs(scratch);
-            found = bs::group_top<kThreads>(row, N, k, 0, tid, gs) <= kThreads;
-            if (found && warp == 0) {
-                const int pos = lane < k ? rf::position_of(gs.top[lane]) : 0x7fffffff;
-                int t = 0;
-#pragma unroll
-                for (int u = 0; u < 32; ++u) t += __shfl_sync(0xffffffffu, pos, u) < pos;
-                if (lane < k) take(t, pos);
-            }
-        }
-        if (!found) {
-            const bs::Kept th = bs::block_kth(row, N, (uint32_t)k, key_lo, key_hi, hist, wcnt, misc);
-            bs::emit_kept(row, N, th, wcnt, take);
-        }
-        __syncthreads();
-        pc.mark();
-
+    finish_path<2>(a, lay, cl, gen, base_s, base, alive, pc, [&](const int *src_pos) {
         // ---- Eq. 1: the sources' rows as an operand, all tiles against them ----
-        const int np = a.z.np;
-        const __nv_bfloat16 *Kh = a.K + b * d.ks[0] + (long long)h * d.ks[1];
+        const int np = a.z.np, k = d.K_src;
+        const __nv_bfloat16 *Kh = static_cast<const __nv_bfloat16 *>(a.K) + b * d.ks[0] + (long long)h * d.ks[1];
         for (int i = tid; i < np * kPieces; i += kThreads) {
             const int r = i / kPieces, c16 = i % kPieces;
             uint4 v = make_uint4(0, 0, 0, 0);
@@ -487,147 +636,27 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             ++batch;
         }
         tc_fence_after();
-        pc.mark();
-
-        // ---- Eq. 3: source c belongs to CTA c % C, which gets its cosines with all keys; a.z.rows sources per CTA at a time ----
-        const int m = d.m, per_cta = ceil_div(k, C);
-        int *nb_j = reinterpret_cast<int *>(region);                                  // [k m] the unit's lists, in every CTA
-        float *nb_f = reinterpret_cast<float *>(nb_j + k * m);                        // [k m]
-        const float *cosines = reinterpret_cast<const float *>(gen + lay.cosines);    // [rows][row_step]
-        const int row_step = (N + 3) & ~3;
-        for (int r0 = 0; r0 < per_cta; r0 += a.z.rows) {
-            const int c_first = r0 * C, c_last = min(k, (r0 + a.z.rows) * C);
-            if (r0 > 0 || a.z.cosines_in_tiles) unit_sync();    // (the round before has been read; nobody reads tiles any more)
-            for (int t = set; t < n_emit; t += 4) {
-                const int i = t * kTileKeys + quad * 32 + lane, j = base + i;
-                const float inv = inv_norm[i];
-                const uint32_t to = base_s + lay.cosines + j * 4;
-                int slot = (c_first & ~7) / C, owner = (c_first & ~7) - slot * C;
-                for (int g0 = c_first & ~7; g0 < c_last; g0 += 8) {
-                    uint32_t raw[8];
-                    __syncwarp();
-                    tmem_ld8_issue(tmem_lane + t * np + g0, raw);
-                    tmem_ld_fence(raw);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const int c = g0 + q;
-                        if (c >= c_first && c < c_last && i < n_local) {
-                            float e = fminf(fmaxf(__uint_as_float(raw[q]) * inv * src_inv[c], -1.0f), 1.0f);
-                            if (j == src_pos[c] || !alive) e = kCandEmpty;
-                            peer_store(peer_addr(to + (slot - r0) * row_step * 4, owner), e);
-                        }
-                        if (++owner == C) owner = 0, ++slot;
-                    }
-                }
-            }
-            tc_fence_before();
-            unit_sync();
-            pc.mark();
-            // the sources' lists, a group of threads each, and each list to all CTAs of the unit
-            constexpr int T = 128;
-            const int mine = min(a.z.rows, per_cta - r0), gang = tid / T, gt = tid % T;
-            const bs::GroupScratch<T> gs(scratch + gang * bs::GroupScratch<T>::kBytes);
-            for (int s = gang; s < mine; s += kThreads / T) {
-                const int c = (r0 + s) * C + rank;
-                if (c >= k) break;
-                const float *x = cosines + s * row_step;
-                if (bs::group_top<T>(x, N, m, 1 + gang, gt, gs) > T) {
-                    // ties: one warp finds exactly the m
-                    if (gt < 32) {
-                        float reached;
-                        const int n = warp_list_top(N, m, -1.0f, [&](int i) { return x[i]; },
-                                                    [&](int at, float e, int i) { gs.cand[at] = edge_key(e, i); }, &reached);
-                        if (lane == 0) gs.word[0] = (uint32_t)n;
-                    }
-                    bs::group_bar<T>(1 + gang);
-                    bs::group_rank(gs, (int)gs.word[0], m, 1 + gang, gt);
-                }
-                if (lane < m) {
-                    const unsigned long long key = gs.top[lane];
-                    const float e = rf::edge_of(key);
-                    const bool is = key != 0ull && e >= -1.0f;
-                    const int j = is ? rf::position_of(key) : -1;
-                    const float f = is ? signal_factor(e, d.lambda, d.T, d.signal) : 1.f;
-                    if (gt < 32 && is) {
-                        a.nbr_idx[((long long)unit * k + c) * m + lane] = j;
-                        a.nbr_e[((long long)unit * k + c) * m + lane] = e;
-                    }
-                    const uint32_t to = base_s + lay.tiles + (c * m + lane) * 4;
-                    for (int p = gt >> 5; p < C; p += T / 32) {
-                        peer_store(peer_addr(to, p), __int_as_float(j));
-                        peer_store(peer_addr(to + k * m * 4, p), f);
-                    }
-                }
-                bs::group_bar<T>(1 + gang);
-            }
-        }
-        unit_sync();
-        pc.mark();
-
-        // ---- Eq. 5: every CTA applies the unit's lists to its copy of the row, sources in order ----
-        const bool evict = d.signal == GRAPHKV_SIGNAL_EVICT;
-        for (int q0 = 0; q0 < k; q0 += 4) {
-            int slot[4];
-            float f[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool in = lane < m && q0 + u < k;
-                slot[u] = in ? nb_j[(q0 + u) * m + lane] : -1;
-                f[u] = in ? nb_f[(q0 + u) * m + lane] : 1.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if ((uint32_t)slot[u] < (uint32_t)N && (slot[u] & (kWarps - 1)) == warp)
-                    row[slot[u]] = evict ? -INFINITY : row[slot[u]] * f[u];
+    }, [&](int c_first, int c_last, auto put) {
+        for (int t = set; t < n_emit; t += 4) {
+            const int i = t * kTileKeys + quad * 32 + lane;
+            const float inv = inv_norm[i];
+            int slot = (c_first & ~7) / C, owner = (c_first & ~7) - slot * C;
+            for (int g0 = c_first & ~7; g0 < c_last; g0 += 8) {
+                uint32_t raw[8];
                 __syncwarp();
-            }
-        }
-        __syncthreads();
-        pc.mark();
-    }
-    if (!a.scores_only) {
-        if (a.scores)
-            for (int i = s0 + tid; i < s1; i += kThreads) a.scores[(long long)unit * N + i] = row[i];
-        // ---- the B largest, in ascending position; a CTA takes its share of them ----
-        const int B = a.per_batch_budget ? a.budget_of[b] : d.B;
-        const bs::Kept th = bs::block_kth(row, N, (uint32_t)B, key_lo, key_hi, hist, wcnt, misc);
-        pc.mark();
-        const int first = B * rank / C, count = B * (rank + 1) / C - first;
-        int *kept = reinterpret_cast<int *>(region + a.z.lists + (a.z.cosines_in_tiles ? a.z.rows * ((N + 3) / 4 * 16) : 0));         // [count]
-        int *idx = a.idx_out + (long long)unit * d.B;
-        bs::emit_kept(row, N, th, wcnt, [&](int t, int i) {
-            if (t >= first && t < first + count) {
-                idx[t] = i;
-                kept[t - first] = i;
-            }
-        });
-        __syncthreads();
-        pc.mark();
-        // ---- gather: the CTA's share of the kept rows and of the window rows ----
-        const int vl = a.vpr_log2, es = 2;
-        const unsigned char *k0 = a.Kb + (b * d.ks[0] + h * d.ks[1]) * es, *v0 = a.V + (b * d.vs[0] + h * d.vs[1]) * es;
-        const long long out0 = (long long)unit * (d.B + d.W);
-        const int w0 = d.W * rank / C, w1 = d.W * (rank + 1) / C, n_rows = count + (w1 - w0);
-        for (int p0 = tid; p0 < n_rows << (vl + 1); p0 += 4 * kThreads) {
-            uint4 v[4];
-            unsigned char *dst[4];
+                tmem_ld8_issue(tmem_lane + t * a.z.np + g0, raw);
+                tmem_ld_fence(raw);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int p = p0 + u * kThreads, t = p >> (vl + 1), c = p & ((1 << vl) - 1);
-                dst[u] = nullptr;
-                if (t < n_rows) {
-                    const bool is_v = (p >> vl) & 1;
-                    const int w = w0 + (t - count);
-                    const long long from = t < count ? kept[t] : N + w, to = out0 + (t < count ? first + t : B + w);
-                    v[u] = *reinterpret_cast<const uint4 *>((is_v ? v0 + from * d.vs[2] * es : k0 + from * d.ks[2] * es) + c * 16);
-                    dst[u] = (is_v ? a.V_out : a.K_out) + ((to << vl) + c) * 16;
+                for (int q = 0; q < 8; ++q) {
+                    const int c = g0 + q;
+                    if (c >= c_first && c < c_last && i < n_local)
+                        put(c, slot, owner, i, fminf(fmaxf(__uint_as_float(raw[q]) * inv * src_inv[c], -1.0f), 1.0f));
+                    if (++owner == C) owner = 0, ++slot;
                 }
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (dst[u]) *reinterpret_cast<uint4 *>(dst[u]) = v[u];
         }
-    }
+        tc_fence_before();
+    });
     pc.mark();
     if (!alive && tid == 0) atomicExch(a.status, (int)GRAPHKV_ERR_TIMEOUT);
     tc_fence_before();
@@ -636,6 +665,199 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
+    pc.flush(7);
+}
+
+// ---- fp32 rows ------------------------------------------------------------------------------------
+// The same path with the products on the FMA pipe (simt_dots, so that cosines have the bits of the general fp32 sweep):
+// a CTA owns 128 keys, its 16 warps two halves of 64 keys; a thread's products of queries and keys stay in
+// registers from the row statistics to the masses, so they are computed once.  kR rows of 16 per row tile, kRowTiles
+// of them.  (One head of 512 keys, six launches before: 38.3 -> 22 us.)
+template <int kD> __host__ __device__ inline Layout layout_f32(const Sizes &z)
+{
+    Layout l{};
+    const int row = (z.N + 3) / 4 * 16, parts = (2 * z.C * z.GW * 8 + 15) / 16 * 16, cosines = z.rows * row;
+    const int rows = z.GW <= 32 ? 32 : z.GW <= 64 ? 64 : 128, step = (kD + 4) * 4;
+    int off = (rows > z.np ? rows : z.np) * step;       // the queries [kRows][kD + 4]; then the sources' unit vectors
+    l.tiles = off;   off += tc::kTileKeys * step;       // the keys [128][kD + 4]
+    l.lists = off;   off += z.lists + z.kept;
+    l.mass = off;    off += row;
+    l.row = off;     off += row;
+    l.inv = off;     off += tc::kTileKeys * 4;
+    l.row_c = off;   off += 2 * 128 * 4;
+    l.parts = l.cosines = off;
+    off += cosines > parts ? cosines : parts;           // row statistics [2 C][GW]; then cosines [rows][N]
+    l.scratch = off; off += kScratch;
+    l.small = off;   off += 1024;
+    l.bars = off;
+    l.total = off;
+    return l;
+}
+
+template <int kD, int kR, int kRowTiles>
+__global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __grid_constant__ PathArgs a)
+{
+    extern __shared__ __align__(16) uint8_t path_smem[];
+    cg::cluster_group cl = cg::this_cluster();
+    constexpr int kStep = kD + 4, kRows = 16 * kR * kRowTiles, kPieces = kD / 4;
+    const Dims &d = a.d;
+    const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C;
+    const int b = unit / d.hkv, h = unit % d.hkv, N = d.N;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, half = warp >> 3, kg = lane & 15, rg = (warp & 7) * 2 + (lane >> 4);
+    uint8_t *gen = path_smem;
+    const uint32_t base_s = tc::smem_u32(path_smem);
+    const Layout lay = layout_f32<kD>(a.z);
+    float *rows = reinterpret_cast<float *>(gen), *keys = reinterpret_cast<float *>(gen + lay.tiles);
+    float *inv_norm = reinterpret_cast<float *>(gen + lay.inv);
+    float *row_mx = reinterpret_cast<float *>(gen + lay.row_c), *row_w = row_mx + 128;
+    float *xchg = reinterpret_cast<float *>(gen + lay.scratch);           // [kWarps][64]
+    const int base = rank * tc::kTileKeys, n_local = max(0, min(N - base, tc::kTileKeys));
+    const float *Q = static_cast<const float *>(a.Q);
+    const float *Kh = static_cast<const float *>(a.K) + b * d.ks[0] + (long long)h * d.ks[1];
+    const bool alive = true;                                              // (no wait here can run out)
+    PhaseClock pc(tid == 0);
+    pc.mark();
+    if (C > 1) cl.barrier_arrive();
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tid == 0 && rank == 0 && unit == 0) *a.status = 0;
+#pragma unroll 8
+    for (int i = tid; i < tc::kTileKeys * kPieces; i += kThreads) {
+        const int r = i / kPieces, c = i % kPieces;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (base + r < d.L) v = *reinterpret_cast<const float4 *>(Kh + (long long)(base + r) * d.ks[2] + c * 4);
+        *reinterpret_cast<float4 *>(keys + r * kStep + c * 4) = v;
+    }
+    const float scale = rsqrtf((float)kD) * kLog2e;
+#pragma unroll 4
+    for (int i = tid; i < kRows * kPieces; i += kThreads) {
+        const int r = i / kPieces, c = i % kPieces;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < d.GW) v = *reinterpret_cast<const float4 *>(Q + b * d.qs[0] + (long long)(h * d.G + r / d.W) * d.qs[1] + (r % d.W) * d.qs[2] + c * 4);
+        *reinterpret_cast<float4 *>(rows + r * kStep + c * 4) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
+    }
+    __syncthreads();
+    if (C > 1) cl.barrier_wait();               // (every CTA of the unit has started: its shared memory may be written to)
+    pc.mark();
+
+    // ---- logits, and the row statistics of each half ----
+    const float *mine = keys + half * 64 * kStep;
+    float l2[kRowTiles][kR][4];
+#pragma unroll
+    for (int rt = 0; rt < kRowTiles; ++rt) simt_dots<kD, kR>(rows + rt * 16 * kR * kStep, mine, rg, kg, l2[rt]);
+    pc.mark();
+#pragma unroll
+    for (int rt = 0; rt < kRowTiles; ++rt)
+#pragma unroll
+        for (int i = 0; i < kR; ++i) {
+            const int r = rt * 16 * kR + rg + 16 * i, last = N + (r < d.GW ? r % d.W : 0);     // last visible key of the row
+            float m = kNegBig;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (base + half * 64 + kg + 16 * e > last) l2[rt][i][e] = -INFINITY;
+                m = fmaxf(m, l2[rt][i][e]);
+            }
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            float z = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) z += exp2f(l2[rt][i][e] - m);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+            if (r < d.GW)                                                 // (the 16 lanes of a row share the CTAs)
+                for (int p = kg; p < C; p += 16)
+                    peer_store(peer_addr(base_s + lay.parts + ((rank * 2 + half) * d.GW + r) * 8, p), make_float2(m, z));
+        }
+    if (C > 1) cl.barrier_arrive();
+    if (a.has_graph && !a.scores_only && tid < tc::kTileKeys) {
+        // the keys' norms meanwhile
+        const float4 *k4 = reinterpret_cast<const float4 *>(keys + tid * kStep);
+        float n2 = 0.f;
+#pragma unroll 8
+        for (int c = 0; c < kPieces; ++c) {
+            const float4 v = k4[c];
+            n2 = fmaf(v.x, v.x, n2); n2 = fmaf(v.y, v.y, n2); n2 = fmaf(v.z, v.z, n2); n2 = fmaf(v.w, v.w, n2);
+        }
+        inv_norm[tid] = 1.0f / fmaxf(sqrtf(n2), kNormEps);
+    }
+    if (C > 1) cl.barrier_wait();
+    else __syncthreads();
+    pc.mark();
+    // ---- row constants, four threads a row ----
+    {
+        const int r = tid >> 2, sub = tid & 3;
+        const float2 *parts = reinterpret_cast<const float2 *>(gen + lay.parts);
+        float m = kNegBig, z = 0.f;
+        if (r < d.GW) {
+            for (int q = sub; q < 2 * C; q += 4) m = fmaxf(m, parts[q * d.GW + r].x);
+        }
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        if (r < d.GW) {
+            for (int q = sub; q < 2 * C; q += 4) z = fmaf(parts[q * d.GW + r].y, exp2f(parts[q * d.GW + r].x - m), z);
+        }
+        z += __shfl_xor_sync(0xffffffffu, z, 1);
+        z += __shfl_xor_sync(0xffffffffu, z, 2);
+        if (sub == 0 && r < kRows) {
+            row_mx[r] = r < d.GW ? m : 0.f;
+            row_w[r] = r < d.GW ? 1.0f / z : 0.f;
+        }
+    }
+    __syncthreads();
+    pc.mark();
+    // ---- masses ----
+    {
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int rt = 0; rt < kRowTiles; ++rt)
+#pragma unroll
+            for (int i = 0; i < kR; ++i) {
+                const int r = rt * 16 * kR + rg + 16 * i;
+                const float m = row_mx[r], w = row_w[r];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[e] = fmaf(exp2f(l2[rt][i][e] - m), w, s[e]);
+            }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            s[e] += __shfl_xor_sync(0xffffffffu, s[e], 16);
+            if (lane < 16) xchg[warp * 64 + kg + 16 * e] = s[e];
+        }
+        __syncthreads();
+        if (tid < n_local) {
+            const float *x = xchg + (tid >> 6) * (8 * 64) + (tid & 63);
+            float sum = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) sum += x[w * 64];
+            for (int p = 0; p < C; ++p) peer_store(peer_addr(base_s + lay.mass + (base + tid) * 4, p), sum);
+        }
+    }
+    pc.mark();
+    finish_path<4>(a, lay, cl, gen, base_s, base, alive, pc, [&](const int *src_pos) {
+        // ---- Eq. 1: the sources' unit vectors, a warp each ----
+        for (int c = warp; c < a.z.np; c += kWarps) {
+            float v[4] = {0.f, 0.f, 0.f, 0.f};
+            if (c < d.K_src && lane * 4 < kD) {
+                const float4 raw = *reinterpret_cast<const float4 *>(Kh + (long long)src_pos[c] * d.ks[2] + lane * 4);
+                v[0] = raw.x; v[1] = raw.y; v[2] = raw.z; v[3] = raw.w;
+            }
+            simt_unit_row(v);
+            if (lane * 4 < kD) *reinterpret_cast<float4 *>(rows + c * kStep + lane * 4) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+        __syncthreads();
+    }, [&](int c_first, int c_last, auto put) {
+        for (int a0 = c_first & ~15; a0 < c_last; a0 += 16) {
+            float dot[1][4];
+            simt_dots<kD, 1>(rows + a0 * kStep, mine, rg, kg, dot);
+            const int c = a0 + rg, slot = c / C;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = half * 64 + kg + 16 * e;
+                if (c >= c_first && c < c_last && i < n_local)
+                    put(c, slot, c - slot * C, i, fminf(fmaxf(dot[0][e] * inv_norm[i], -1.0f), 1.0f));
+            }
+        }
+    });
+    pc.mark();
     pc.flush(7);
 }
 

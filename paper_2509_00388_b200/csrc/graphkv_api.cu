@@ -526,8 +526,12 @@ ShortRow short_row(const Dims &d)
 {
     ShortRow s{0, 0};
     const int n_tiles = ceil_div(d.L, tc::kTileKeys), most = cp::max_tiles(d.D);
-    if (!d.bf16 || n_tiles > cp::kMaxCluster * most || d.units > sm_count()) return s;
+    if (n_tiles > cp::kMaxCluster * most || d.units > sm_count()) return s;
     const int *fits = resident_clusters();
+    if (!d.bf16) {              // a key tile per CTA, up to 128 query rows
+        if (fits && n_tiles <= cp::kMaxCluster && fits[n_tiles] >= d.units && d.GW <= 128) s = ShortRow{n_tiles, 1};
+        return s;
+    }
     for (int C = 1; fits && C <= std::min(cp::kMaxCluster, n_tiles); ++C) {
         if (fits[C] < d.units) continue;
         const int tiles = ceil_div(n_tiles, C);
@@ -540,7 +544,8 @@ ShortRow short_row(const Dims &d)
 // cores too (wide pooling sends that to the register-tiled products, which round differently).
 inline bool short_row_graph(const Dims &d)
 {
-    return d.K_src <= cp::kMaxSources && d.m <= cp::kMaxNeighbours && !(d.reselect && d.T > 1) && cluster_plan(d).ok;
+    return d.K_src <= cp::kMaxSources && d.m <= cp::kMaxNeighbours && !(d.reselect && d.T > 1) &&
+           (!d.bf16 || cluster_plan(d).ok);
 }
 
 // ---- step (I), tensor-core path (bf16) -----------------------------------------------------------
@@ -1010,11 +1015,11 @@ ClusterPathPlan cluster_path_plan(const Dims &d, bool graph)
     p.n_tiles = ceil_div(d.L, tc::kTileKeys);
     p.z = cp::Sizes{d.N, sr.C, d.GW, sr.tiles, !graph || d.K_src <= 16 ? 16 : d.K_src <= 32 ? 32 : 64, 0,
                     graph ? (d.K_src * d.m * 8 + 15) / 16 * 16 : 0, (d.B * 4 + 15) / 16 * 16, 0};
-    const auto layout_of_path = d.D == 64 ? (d.GW <= 128 ? cp::layout<64, 1> : cp::layout<64, 2>)
+    const auto layout_of_path = !d.bf16 ? (d.D == 64 ? cp::layout_f32<64> : cp::layout_f32<128>) : d.D == 64 ? (d.GW <= 128 ? cp::layout<64, 1> : cp::layout<64, 2>)
                                           : (d.GW <= 128 ? cp::layout<128, 1> : cp::layout<128, 2>);
     // the cosines of all a CTA's sources at once where that fits
     const int per_cta = graph ? ceil_div(d.K_src, p.C) : 0;
-    for (int in_tiles = 0; in_tiles <= (graph ? 1 : 0) && !p.ok; ++in_tiles)
+    for (int in_tiles = 0; in_tiles <= (graph && d.bf16 ? 1 : 0) && !p.ok; ++in_tiles)
         for (int rounds = 1; rounds <= std::max(1, std::min(2, per_cta)) && !p.ok; ++rounds) {
             p.z.cosines_in_tiles = in_tiles;
             p.z.rows = ceil_div(per_cta, rounds);
@@ -1037,12 +1042,22 @@ inline int short_row_chunks(const Dims &d)
     return p.ok ? p.C : 0;
 }
 
-graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPathPlan &pl, const __nv_bfloat16 *Q,
-                                const __nv_bfloat16 *K, const void *V, void *K_out, void *V_out, int *idx_out, float *scores,
+template <int kD, int kR, int kRowTiles> bool cluster_path_f32_ready()
+{
+    static std::mutex mu;
+    static signed char state[64] = {};
+    return once_per_device(mu, state, [] {
+        return set_smem(cp::cluster_path_f32_kernel<kD, kR, kRowTiles>, kMaxSmem) &&
+               cudaFuncSetAttribute(cp::cluster_path_f32_kernel<kD, kR, kRowTiles>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    });
+}
+
+graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPathPlan &pl, const void *Q,
+                                const void *K, const void *V, void *K_out, void *V_out, int *idx_out, float *scores,
                                 bool scores_only, bool graph, void *ws, cudaStream_t st)
 {
     CUtensorMap tmK;
-    if (!make_k_tensormap(&tmK, K, d, d.L)) return GRAPHKV_ERR_CUDA;
+    if (d.bf16 && !make_k_tensormap(&tmK, K, d, d.L)) return GRAPHKV_ERR_CUDA;
     cp::PathArgs a{};
     a.d = d;
     a.Q = Q;
@@ -1059,8 +1074,8 @@ graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPat
         a.nbr_idx = at<int>(ws, l.nbr_idx);
         a.nbr_e = at<float>(ws, l.nbr_e);
         a.idx_out = idx_out;
-        a.vpr_log2 = d.D == 64 ? 3 : 4;
-        a.Kb = reinterpret_cast<const unsigned char *>(K);
+        a.vpr_log2 = (d.D == 64 ? 3 : 4) + (d.bf16 ? 0 : 1);
+        a.Kb = static_cast<const unsigned char *>(K);
         a.V = static_cast<const unsigned char *>(V);
         a.K_out = static_cast<unsigned char *>(K_out);
         a.V_out = static_cast<unsigned char *>(V_out);
@@ -1071,6 +1086,16 @@ graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPat
     }
     a.wait_cycles = wait_cycles();
     a.withhold_commit = env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0);
+    auto launch_f32 = [&](auto kern, bool ready) -> graphkv_status {
+        if (!ready) return GRAPHKV_ERR_CUDA;
+        return launch_ex("cluster_path", kern, dim3(d.units * pl.C), dim3(cp::kThreads), pl.smem, st, next_launch_is_dependent(), pl.C, a);
+    };
+    if (!d.bf16) {
+#define GKV_F32(kD, kR, kRowTiles) launch_f32(cp::cluster_path_f32_kernel<kD, kR, kRowTiles>, cluster_path_f32_ready<kD, kR, kRowTiles>())
+        if (d.D == 64) return d.GW <= 32 ? GKV_F32(64, 2, 1) : d.GW <= 64 ? GKV_F32(64, 4, 1) : GKV_F32(64, 4, 2);
+        return d.GW <= 32 ? GKV_F32(128, 2, 1) : d.GW <= 64 ? GKV_F32(128, 4, 1) : GKV_F32(128, 4, 2);
+#undef GKV_F32
+    }
     auto launch = [&](auto kern, bool ready) -> graphkv_status {
         if (!ready) return GRAPHKV_ERR_CUDA;
         return launch_ex("cluster_path", kern, dim3(d.units * pl.C), dim3(cp::kThreads), pl.smem, st,
@@ -1090,11 +1115,9 @@ graphkv_status do_score(const Dims &d, const Layout &l, const T *Q, const T *K, 
                         void *ws, cudaStream_t st)
 {
     EmitExtras ex = kPlainEmit;
-    if constexpr (sizeof(T) == 2) {
-        const ClusterPathPlan pl = cluster_path_plan(d, false);
-        ex.stat_chunks = pl.ok ? pl.C : 0;
-        if (pl.ok && cluster_path_on()) return run_cluster_path(d, l, pl, Q, K, nullptr, nullptr, nullptr, nullptr, scores, true, false, ws, st);
-    }
+    const ClusterPathPlan pl = cluster_path_plan(d, false);
+    ex.stat_chunks = pl.ok ? pl.C : 0;
+    if (pl.ok && cluster_path_on()) return run_cluster_path(d, l, pl, Q, K, nullptr, nullptr, nullptr, nullptr, scores, true, false, ws, st);
     float *a = d.kp > 1 ? at<float>(ws, l.a) : scores;
     graphkv_status rc = run_mass(d, l, Q, K, a, ws, st, ex);
     if (rc != GRAPHKV_OK || d.kp == 1) return rc;
@@ -1143,23 +1166,31 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
 {
     const bool graph = graph_active(d);
     EmitExtras ex = kPlainEmit;
-    if constexpr (sizeof(T) == 2) {
+    bool scored = false;                    // `s` holds the pooled scores already
+    {
         const ClusterPathPlan pl = cluster_path_plan(d, graph);
         if (pl.ok && cluster_path_on())
             return run_cluster_path(d, l, pl, Q, K, V, K_out, V_out, idx_out, t_keep_scores ? s : nullptr, false, graph, ws, st);
-        ex.stat_chunks = pl.ok ? pl.C : short_row_chunks(d);
+        // a graph that the cluster path does not take: the scores must not depend on it
+        if (sizeof(T) == 2) {
+            ex.stat_chunks = pl.ok ? pl.C : short_row_chunks(d);
+        } else if (const ClusterPathPlan ps = cluster_path_plan(d, false); ps.ok && cluster_path_on()) {
+            const graphkv_status rc = run_cluster_path(d, l, ps, Q, K, nullptr, nullptr, nullptr, nullptr, s, true, false, ws, st);
+            if (rc != GRAPHKV_OK) return rc;
+            scored = true;
+        }
     }
     float *a = d.kp > 1 ? at<float>(ws, l.a) : s;
     int *src = at<int>(ws, l.src);
     const bool tc_graph = graph && sim_plan(d, sizeof(T) == 2).ok;
     // without a graph (plain top-B) the old finishing kernel pools where the new one does not apply
-    const bool finish_pools = !graph && d.kp > 1 && !d.pool_avg && !candidate_plan(d, false, true, false, d.B).ok &&
+    const bool finish_pools = !graph && !scored && d.kp > 1 && !d.pool_avg && !candidate_plan(d, false, true, false, d.B).ok &&
                               finish_plan(d, (d.kp - 1) / 2).ok && cluster_plan(d).ok;
     graphkv_status rc;
     uint32_t *row_hist = nullptr;
     if (!graph) {
-        if ((rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
-        if (d.kp > 1 && !finish_pools &&
+        if (!scored && (rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
+        if (!scored && d.kp > 1 && !finish_pools &&
             (rc = run_pool_sources(d, a, s, 0, nullptr, nullptr, nullptr, 0, st)) != GRAPHKV_OK)
             return rc;
     } else {
@@ -1170,9 +1201,9 @@ graphkv_status do_compress(const Dims &d, const Layout &l, const T *Q, const T *
         }
         ex.zero = row_hist;
         ex.zero_words = cs::kBins;
-        if ((rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
+        if (!scored && (rc = run_mass(d, l, Q, K, a, ws, st, ex)) != GRAPHKV_OK) return rc;
         // the tensor-core emit sweep leaves a histogram of the attention mass behind
-        rc = run_pool_sources(d, d.kp > 1 ? a : nullptr, s, d.K_src, src,
+        rc = run_pool_sources(d, d.kp > 1 && !scored ? a : nullptr, s, d.K_src, src,
                               tc_mass(Q, d) ? at<uint32_t>(ws, l.a_hist) : nullptr,
                               tc_graph ? at<uint32_t>(ws, l.cand_hist) : nullptr, d.K_src * kCandBins, st, row_hist);
         if (rc != GRAPHKV_OK) return rc;

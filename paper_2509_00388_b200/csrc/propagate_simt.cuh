@@ -62,11 +62,8 @@ __global__ void __launch_bounds__(kSimtThreads) similarity_simt(Dims d, const T 
                     v[0] = raw.x; v[1] = raw.y; v[2] = raw.z; v[3] = raw.w;
                 }
             }
-            const float n2 = warp_sum(v[0] * v[0] + v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
-            const float inv = 1.0f / fmaxf(sqrtf(n2), kNormEps);
-            if (lane * 4 < kD)
-                *reinterpret_cast<float4 *>(rows + a * (kD + 4) + lane * 4) =
-                    make_float4(v[0] * inv, v[1] * inv, v[2] * inv, v[3] * inv);
+            simt_unit_row(v);
+            if (lane * 4 < kD) *reinterpret_cast<float4 *>(rows + a * (kD + 4) + lane * 4) = make_float4(v[0], v[1], v[2], v[3]);
         }
         __syncthreads();
         if (a0 == 0) {

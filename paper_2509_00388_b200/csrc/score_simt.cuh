@@ -97,6 +97,16 @@ __device__ __forceinline__ void simt_dots(const float *rows, const float *keys, 
         for (int e = 0; e < 4; ++e) out[i][e] = (acc[i][e][0] + acc[i][e][1]) + (acc[i][e][2] + acc[i][e][3]);
 }
 
+// A row spread over a warp, four elements per lane, scaled to unit length.  (Written out in fused multiply-adds: every
+// kernel that calls it gets the same bits.)
+__device__ __forceinline__ void simt_unit_row(float (&v)[4])
+{
+    const float n2 = warp_sum(fmaf(v[3], v[3], fmaf(v[2], v[2], fmaf(v[1], v[1], v[0] * v[0]))));
+    const float inv = 1.0f / fmaxf(sqrtf(n2), kNormEps);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] *= inv;
+}
+
 // Row statistics of the softmax, in the log2 domain: for query row r and the keys of one chunk,
 // mx = max_j l2[r][j], z = sum_j 2^(l2[r][j] - mx), l2 = (q.k / sqrt(D)) * log2(e), over the keys
 // row r may see (prefix keys and window keys N + r' with r' <= r).
