@@ -670,16 +670,17 @@ cluster_path_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
 // ---- fp32 rows ------------------------------------------------------------------------------------
 // The same path with the products on the FMA pipe (simt_dots, so that cosines have the bits of the general fp32 sweep):
-// a CTA owns 128 keys, its 16 warps two halves of 64 keys; a thread's products of queries and keys stay in
-// registers from the row statistics to the masses, so they are computed once.  kR rows of 16 per row tile, kRowTiles
-// of them.  (One head of 512 keys, six launches before: 38.3 -> 22 us.)
+// a CTA owns 128 keys, its 16 warps two halves of 64 keys, or, where clusters of that many CTAs are resident, 64 keys, its
+// warps two halves of the query rows; a thread's products of queries and keys stay in registers from the row statistics
+// to the masses, so they are computed once.  kR times 16 rows per row tile, kRowTiles of them.  (One head of 512 keys: six launches
+// 38.3 us, 128 keys per CTA 25.7, 64 keys 21.)
 template <int kD> __host__ __device__ inline Layout layout_f32(const Sizes &z)
 {
     Layout l{};
-    const int row = (z.N + 3) / 4 * 16, parts = (2 * z.C * z.GW * 8 + 15) / 16 * 16, cosines = z.rows * row;
+    const int row = (z.N + 3) / 4 * 16, parts = (z.tiles * z.C * z.GW * 8 + 15) / 16 * 16, cosines = z.rows * row;
     const int rows = z.GW <= 32 ? 32 : z.GW <= 64 ? 64 : 128, step = (kD + 4) * 4;
     int off = (rows > z.np ? rows : z.np) * step;       // the queries [kRows][kD + 4]; then the sources' unit vectors
-    l.tiles = off;   off += tc::kTileKeys * step;       // the keys [128][kD + 4]
+    l.tiles = off;   off += z.tiles * 64 * step;        // the keys [64 or 128][kD + 4]
     l.lists = off;   off += z.lists + z.kept;
     l.mass = off;    off += row;
     l.row = off;     off += row;
@@ -694,16 +695,18 @@ template <int kD> __host__ __device__ inline Layout layout_f32(const Sizes &z)
     return l;
 }
 
-template <int kD, int kR, int kRowTiles>
+template <int kD, int kR, int kRowTiles, int kKeys>
 __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __grid_constant__ PathArgs a)
 {
     extern __shared__ __align__(16) uint8_t path_smem[];
     cg::cluster_group cl = cg::this_cluster();
-    constexpr int kStep = kD + 4, kRows = 16 * kR * kRowTiles, kPieces = kD / 4;
+    constexpr int kStep = kD + 4, kHalfRows = 16 * kR * kRowTiles, kRows = kKeys == 64 ? 2 * kHalfRows : kHalfRows, kPieces = kD / 4;
+    constexpr int kParts = kKeys / 64;          // partial statistics per row and CTA
+    static_assert(kRows <= 128 && (kKeys == 64 || kKeys == 128), "four threads per row");
     const Dims &d = a.d;
     const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C;
     const int b = unit / d.hkv, h = unit % d.hkv, N = d.N;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, half = warp >> 3, kg = lane & 15, rg = (warp & 7) * 2 + (lane >> 4);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, half = warp >> 3, kh = kKeys == 128 ? half : 0, rh = kKeys == 64 ? half : 0, kg = lane & 15, rg = (warp & 7) * 2 + (lane >> 4);
     uint8_t *gen = path_smem;
     const uint32_t base_s = tc::smem_u32(path_smem);
     const Layout lay = layout_f32<kD>(a.z);
@@ -711,7 +714,7 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
     float *inv_norm = reinterpret_cast<float *>(gen + lay.inv);
     float *row_mx = reinterpret_cast<float *>(gen + lay.row_c), *row_w = row_mx + 128;
     float *xchg = reinterpret_cast<float *>(gen + lay.scratch);           // [kWarps][64]
-    const int base = rank * tc::kTileKeys, n_local = max(0, min(N - base, tc::kTileKeys));
+    const int base = rank * kKeys, n_local = max(0, min(N - base, kKeys));
     const float *Q = static_cast<const float *>(a.Q);
     const float *Kh = static_cast<const float *>(a.K) + b * d.ks[0] + (long long)h * d.ks[1];
     const bool alive = true;                                              // (no wait here can run out)
@@ -722,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
     pdl_launch_dependents();
     if (tid == 0 && rank == 0 && unit == 0) *a.status = 0;
 #pragma unroll 8
-    for (int i = tid; i < tc::kTileKeys * kPieces; i += kThreads) {
+    for (int i = tid; i < kKeys * kPieces; i += kThreads) {
         const int r = i / kPieces, c = i % kPieces;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (base + r < d.L) v = *reinterpret_cast<const float4 *>(Kh + (long long)(base + r) * d.ks[2] + c * 4);
@@ -741,20 +744,21 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
     pc.mark();
 
     // ---- logits, and the row statistics of each half ----
-    const float *mine = keys + half * 64 * kStep;
+    const float *mine = keys + kh * 64 * kStep;
+    const int row0 = rh * kHalfRows;
     float l2[kRowTiles][kR][4];
 #pragma unroll
-    for (int rt = 0; rt < kRowTiles; ++rt) simt_dots<kD, kR>(rows + rt * 16 * kR * kStep, mine, rg, kg, l2[rt]);
+    for (int rt = 0; rt < kRowTiles; ++rt) simt_dots<kD, kR>(rows + (row0 + rt * 16 * kR) * kStep, mine, rg, kg, l2[rt]);
     pc.mark();
 #pragma unroll
     for (int rt = 0; rt < kRowTiles; ++rt)
 #pragma unroll
         for (int i = 0; i < kR; ++i) {
-            const int r = rt * 16 * kR + rg + 16 * i, last = N + (r < d.GW ? r % d.W : 0);     // last visible key of the row
+            const int r = row0 + rt * 16 * kR + rg + 16 * i, last = N + (r < d.GW ? r % d.W : 0);     // last visible key of the row
             float m = kNegBig;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                if (base + half * 64 + kg + 16 * e > last) l2[rt][i][e] = -INFINITY;
+                if (base + kh * 64 + kg + 16 * e > last) l2[rt][i][e] = -INFINITY;
                 m = fmaxf(m, l2[rt][i][e]);
             }
 #pragma unroll
@@ -766,10 +770,10 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
             for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
             if (r < d.GW)                                                 // (the 16 lanes of a row share the CTAs)
                 for (int p = kg; p < C; p += 16)
-                    peer_store(peer_addr(base_s + lay.parts + ((rank * 2 + half) * d.GW + r) * 8, p), make_float2(m, z));
+                    peer_store(peer_addr(base_s + lay.parts + ((rank * kParts + kh) * d.GW + r) * 8, p), make_float2(m, z));
         }
     if (C > 1) cl.barrier_arrive();
-    if (a.has_graph && !a.scores_only && tid < tc::kTileKeys) {
+    if (a.has_graph && !a.scores_only && tid < kKeys) {
         // the keys' norms meanwhile
         const float4 *k4 = reinterpret_cast<const float4 *>(keys + tid * kStep);
         float n2 = 0.f;
@@ -789,12 +793,12 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
         const float2 *parts = reinterpret_cast<const float2 *>(gen + lay.parts);
         float m = kNegBig, z = 0.f;
         if (r < d.GW) {
-            for (int q = sub; q < 2 * C; q += 4) m = fmaxf(m, parts[q * d.GW + r].x);
+            for (int q = sub; q < kParts * C; q += 4) m = fmaxf(m, parts[q * d.GW + r].x);
         }
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
         if (r < d.GW) {
-            for (int q = sub; q < 2 * C; q += 4) z = fmaf(parts[q * d.GW + r].y, exp2f(parts[q * d.GW + r].x - m), z);
+            for (int q = sub; q < kParts * C; q += 4) z = fmaf(parts[q * d.GW + r].y, exp2f(parts[q * d.GW + r].x - m), z);
         }
         z += __shfl_xor_sync(0xffffffffu, z, 1);
         z += __shfl_xor_sync(0xffffffffu, z, 2);
@@ -812,7 +816,7 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
         for (int rt = 0; rt < kRowTiles; ++rt)
 #pragma unroll
             for (int i = 0; i < kR; ++i) {
-                const int r = rt * 16 * kR + rg + 16 * i;
+                const int r = row0 + rt * 16 * kR + rg + 16 * i;
                 const float m = row_mx[r], w = row_w[r];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) s[e] = fmaf(exp2f(l2[rt][i][e] - m), w, s[e]);
@@ -827,7 +831,7 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
             const float *x = xchg + (tid >> 6) * (8 * 64) + (tid & 63);
             float sum = 0.f;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) sum += x[w * 64];
+            for (int w = 0; w < 16 / kParts; ++w) sum += x[w * 64];
             for (int p = 0; p < C; ++p) peer_store(peer_addr(base_s + lay.mass + (base + tid) * 4, p), sum);
         }
     }
@@ -845,13 +849,13 @@ __global__ void __launch_bounds__(kThreads, 1) cluster_path_f32_kernel(const __g
         }
         __syncthreads();
     }, [&](int c_first, int c_last, auto put) {
-        for (int a0 = c_first & ~15; a0 < c_last; a0 += 16) {
+        for (int a0 = (c_first & ~15) + 16 * rh; a0 < c_last; a0 += kKeys == 64 ? 32 : 16) {
             float dot[1][4];
             simt_dots<kD, 1>(rows + a0 * kStep, mine, rg, kg, dot);
             const int c = a0 + rg, slot = c / C;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int i = half * 64 + kg + 16 * e;
+                const int i = kh * 64 + kg + 16 * e;
                 if (c >= c_first && c < c_last && i < n_local)
                     put(c, slot, c - slot * C, i, fminf(fmaxf(dot[0][e] * inv_norm[i], -1.0f), 1.0f));
             }

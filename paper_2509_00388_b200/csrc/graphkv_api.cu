@@ -528,8 +528,11 @@ ShortRow short_row(const Dims &d)
     const int n_tiles = ceil_div(d.L, tc::kTileKeys), most = cp::max_tiles(d.D);
     if (n_tiles > cp::kMaxCluster * most || d.units > sm_count()) return s;
     const int *fits = resident_clusters();
-    if (!d.bf16) {              // a key tile per CTA, up to 128 query rows
-        if (fits && n_tiles <= cp::kMaxCluster && fits[n_tiles] >= d.units && d.GW <= 128) s = ShortRow{n_tiles, 1};
+    if (!d.bf16) {              // 64 keys per CTA, or 128 where the clusters would not all be resident; up to 128 query rows
+        for (int tiles = 1; tiles <= 2 && s.C == 0; ++tiles) {
+            const int C = ceil_div(d.L, 64 * tiles);
+            if (fits && C <= cp::kMaxCluster && fits[C] >= d.units && d.GW <= 128) s = ShortRow{C, tiles};
+        }
         return s;
     }
     for (int C = 1; fits && C <= std::min(cp::kMaxCluster, n_tiles); ++C) {
@@ -1042,13 +1045,13 @@ inline int short_row_chunks(const Dims &d)
     return p.ok ? p.C : 0;
 }
 
-template <int kD, int kR, int kRowTiles> bool cluster_path_f32_ready()
+template <int kD, int kR, int kRowTiles, int kKeys> bool cluster_path_f32_ready()
 {
     static std::mutex mu;
     static signed char state[64] = {};
     return once_per_device(mu, state, [] {
-        return set_smem(cp::cluster_path_f32_kernel<kD, kR, kRowTiles>, kMaxSmem) &&
-               cudaFuncSetAttribute(cp::cluster_path_f32_kernel<kD, kR, kRowTiles>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        return set_smem(cp::cluster_path_f32_kernel<kD, kR, kRowTiles, kKeys>, kMaxSmem) &&
+               cudaFuncSetAttribute(cp::cluster_path_f32_kernel<kD, kR, kRowTiles, kKeys>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     });
 }
 
@@ -1091,9 +1094,15 @@ graphkv_status run_cluster_path(const Dims &d, const Layout &l, const ClusterPat
         return launch_ex("cluster_path", kern, dim3(d.units * pl.C), dim3(cp::kThreads), pl.smem, st, next_launch_is_dependent(), pl.C, a);
     };
     if (!d.bf16) {
-#define GKV_F32(kD, kR, kRowTiles) launch_f32(cp::cluster_path_f32_kernel<kD, kR, kRowTiles>, cluster_path_f32_ready<kD, kR, kRowTiles>())
-        if (d.D == 64) return d.GW <= 32 ? GKV_F32(64, 2, 1) : d.GW <= 64 ? GKV_F32(64, 4, 1) : GKV_F32(64, 4, 2);
-        return d.GW <= 32 ? GKV_F32(128, 2, 1) : d.GW <= 64 ? GKV_F32(128, 4, 1) : GKV_F32(128, 4, 2);
+#define GKV_F32(kD, kR, kRowTiles, kKeys) \
+    launch_f32(cp::cluster_path_f32_kernel<kD, kR, kRowTiles, kKeys>, cluster_path_f32_ready<kD, kR, kRowTiles, kKeys>())
+        const int rows = d.GW <= 32 ? 0 : d.GW <= 64 ? 1 : 2;
+        if (pl.z.tiles == 1) {
+            if (d.D == 64) return rows == 0 ? GKV_F32(64, 1, 1, 64) : rows == 1 ? GKV_F32(64, 2, 1, 64) : GKV_F32(64, 4, 1, 64);
+            return rows == 0 ? GKV_F32(128, 1, 1, 64) : rows == 1 ? GKV_F32(128, 2, 1, 64) : GKV_F32(128, 4, 1, 64);
+        }
+        if (d.D == 64) return rows == 0 ? GKV_F32(64, 2, 1, 128) : rows == 1 ? GKV_F32(64, 4, 1, 128) : GKV_F32(64, 4, 2, 128);
+        return rows == 0 ? GKV_F32(128, 2, 1, 128) : rows == 1 ? GKV_F32(128, 4, 1, 128) : GKV_F32(128, 4, 2, 128);
 #undef GKV_F32
     }
     auto launch = [&](auto kern, bool ready) -> graphkv_status {
