@@ -836,20 +836,18 @@ constexpr int kPosBits = 18;             // a row's positions (its length is at 
 static_assert(kFineBins >= kThreads && kBins >= kRankList && kTotWords >= kRankList && kStage >= kThreads, "bins, lists, kept");
 static_assert(4 * kRankDirect <= kThreads, "four threads per candidate");
 
-// Top-k of the cluster's row when a histogram of values that the row dominates elementwise is at
-// hand (the pooled scores against the histogram of the attention mass before pooling: pooling only
-// raises values, so the k-th largest pooled score is at least the k-th largest mass).  The highest
-// digit b with k histogram entries in digits >= b therefore bounds the k-th largest row value from
-// below; the row's elements with digit >= b are few (at most pool_kernel times the histogram's
-// count); each CTA lists its own, the first CTA pulls the lists through distributed shared memory
-// and ranks them by counting, more than kRankDirect of them after cutting them into bins (ranking n costs n^2:
-// 600 candidates of 38 sources took 9 us of the kernel's 13, now 4).  Returns false (in every CTA alike,
-// nothing written) when they exceed kRankList; the caller then runs the radix search.  `mass_hist`: kBins counts of the top 11 bits.
+// A key that k elements of the row reach or exceed, and how many keys lie from it to the greatest one (0: 2^32).
+struct RowBound {
+    uint32_t lo, span;
+};
+
+// From a histogram of values that the row dominates elementwise (the pooled scores against the histogram of the
+// attention mass before pooling: pooling only raises values, so the k-th largest pooled score is at least the k-th
+// largest mass): the highest digit b with k histogram entries in digits >= b bounds the k-th largest row value from
+// below, and the row's elements with digit >= b are few (at most pool_kernel times the histogram's count).
 // c0, c1: the histogram's counts of digits kBins-1-2t and kBins-2-2t for thread t (the caller loads
 // them early, ahead of the pooling).
-__device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, const Smem &s,
-                                     const float *vals, int n_local, int base, int k,
-                                     uint32_t c0, uint32_t c1, int *out)
+__device__ RowBound bound_of_histogram(const Smem &s, int k, uint32_t c0, uint32_t c1)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // digit b: walk the histogram from the top (thread t owns digits kBins-1-2t and kBins-2-2t)
@@ -857,8 +855,6 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
     if (lane == 31) s.wcnt[warp] = incl;
     if (tid == 0) {
         s.misc[0] = 0u;          // digit 0 when the histogram holds fewer than k entries
-        s.misc[7] = 0u;          // this CTA's candidate counter
-        s.misc[3] = s.misc[4] = 0u;
         s.misc[5] = kBins;       // one past the highest digit in use
     }
     __syncthreads();
@@ -870,7 +866,63 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
     else if (before1 < (uint32_t)k && before1 + c1 >= (uint32_t)k) s.misc[0] = kBins - 2 - 2 * tid;
     if (before0 == 0u && c0 + c1 > 0u) s.misc[5] = kBins - 2 * tid;
     __syncthreads();
-    const uint32_t bdigit = s.misc[0];
+    return RowBound{s.misc[0] << 21, (s.misc[5] - s.misc[0]) << 21};
+}
+
+// Without one: each CTA halves the range of its threads' maxima until little more than k of them reach the lower end
+// (k elements do then), and the cluster takes the greatest of the CTAs' bounds.  One pass over the chunk, about ten
+// counting barriers and one exchange, where the radix search takes three passes and six exchanges. 16 sources of
+// 20011 given scores x 8 heads: the key-norm path's five kernels 72.0 -> 67.8 us.
+// A function of its own: inlined, it cost the calls that have a histogram 1 us in instruction fetches.
+__device__ __noinline__ RowBound bound_of_maxima(int C, uint32_t *hist, uint32_t *tot, uint32_t *misc, const float *vals, int n_local, int k)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t top = 0u;                                     // (a thread without elements: below every number)
+    for (int i = tid; i < n_local; i += kThreads) top = max(top, float_to_key(vals[i]));
+    const uint32_t wmax = __reduce_max_sync(0xffffffffu, top), wmin = __reduce_min_sync(0xffffffffu, top);
+    if (lane == 0) {
+        hist[warp] = wmax;
+        tot[warp] = wmin;
+    }
+    __syncthreads();
+    const uint32_t cta_max = __reduce_max_sync(0xffffffffu, hist[lane]);
+    uint32_t lo = __reduce_min_sync(0xffffffffu, tot[lane]), hi = cta_max;       // all reach lo
+    for (int n = kThreads; n > k + k / 4 && lo < hi;) {
+        const uint32_t mid = lo + (hi - lo) / 2 + 1;
+        const int c = __syncthreads_count(top >= mid);
+        if (c >= k) {
+            lo = mid;
+            n = c;
+        } else {
+            hi = mid - 1;
+        }
+    }
+    if (tid == 0) {
+        misc[6] = lo;
+        misc[5] = cta_max;
+    }
+    __syncthreads();
+    uint32_t greatest = cta_max;
+    if (C > 1) {
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        const uint32_t *other = cl.map_shared_rank(misc, min(lane, C - 1));
+        lo = __reduce_max_sync(0xffffffffu, other[6]);
+        greatest = __reduce_max_sync(0xffffffffu, other[5]);
+    }
+    return RowBound{lo, greatest - lo + 1u};
+}
+
+// Top-k of the cluster's row from a bound on its k-th largest element: each CTA lists its elements from the bound on, the
+// first CTA pulls the lists through distributed shared memory
+// and ranks them by counting, more than kRankDirect of them after cutting them into bins (ranking n costs n^2:
+// 600 candidates of 38 sources took 9 us of the kernel's 13, now 4).  Returns false (in every CTA alike,
+// nothing written) when they exceed kRankList; the caller then runs the radix search.
+// misc[3], misc[4] (counters of the ranking) and misc[7] (of this CTA's candidates) are zero.
+__device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, const Smem &s,
+                                     const float *vals, int n_local, int base, int k, RowBound bound, int *out)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // this CTA's candidates -> its own lists (keys in hist, positions in tot)
     for (int i0 = 0; i0 < n_local; i0 += kThreads) {
         const int i = i0 + tid;
@@ -878,7 +930,7 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
         bool cand = false;
         if (i < n_local) {
             key = float_to_key(vals[i]);
-            cand = (key >> 21) >= bdigit;
+            cand = key >= bound.lo;
         }
         const unsigned bm = __ballot_sync(0xffffffffu, cand);
         if (bm) {
@@ -934,7 +986,7 @@ __device__ bool cluster_topk_bounded(cg::cluster_group &cl, int C, int rank, con
         int n = (int)total, need = k;
         // Cut into 1024 bins by ten bits of (value above the bound, position) at a time while there are many:
         // those above the bin that holds the last one to keep are kept, those in it go on.
-        const uint32_t lo = bdigit << 21, span = (s.misc[5] - bdigit) << 21;      // (0: 2^32)
+        const uint32_t lo = bound.lo, span = bound.span;
         for (int bits = 32 - __clz(span - 1u) + kPosBits; n > kRankDirect; bits = max(bits - 10, 0)) {
             const int shift = max(bits - 10, 0);
             s.fine[tid] = 0u;
@@ -1018,6 +1070,7 @@ __global__ void __launch_bounds__(kThreads, 1) pool_select_kernel(PoolSelectArgs
     const int n_local = max(0, min(a.chunk, N - base));
     float *vals = s.vals + a.halo;
     float *row_s = a.s + (long long)unit * N;
+    if (tid == 0) s.misc[3] = s.misc[4] = s.misc[7] = 0u;
     PhaseClock pc(threadIdx.x == 0 && rank == 0);
     pc.mark();
     if (a.wait_prior) pdl_wait();
@@ -1073,7 +1126,12 @@ __global__ void __launch_bounds__(kThreads, 1) pool_select_kernel(PoolSelectArgs
     pc.mark();
     if (a.k > 0) {
         int *out = a.src_out + (long long)unit * a.k;
-        const bool done = bounded && cluster_topk_bounded(cl, C, rank, s, vals, n_local, base, a.k, hc0, hc1, out);
+        bool done = false;
+        // (about k elements per CTA reach the bound of maxima: few enough to be listed)
+        if (bounded || C * a.k <= kThreads) {
+            const RowBound bound = bounded ? bound_of_histogram(s, a.k, hc0, hc1) : bound_of_maxima(C, s.hist, s.tot, s.misc, vals, n_local, a.k);
+            done = cluster_topk_bounded(cl, C, rank, s, vals, n_local, base, a.k, bound, out);
+        }
         if (!done) {
             const RowView row{vals, nullptr, n_local};
             const Threshold th = cluster_kth(cl, C, rank, s, row, (uint32_t)a.k);
