@@ -338,7 +338,8 @@ __global__ void __launch_bounds__(kThreads, 2) finish_kernel(FinishArgs a)
     extern __shared__ __align__(16) uint8_t rf_smem[];
     cg::cluster_group cl = cg::this_cluster();
     const Dims &d = a.d;
-    const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0, unit = blockIdx.x / C;
+    const int C = a.C, rank = C > 1 ? (int)cl.block_rank() : 0;
+    const int unit = (gridDim.x - 1 - blockIdx.x) / C;   // the last units first: their keys are still in L2
     const int N = d.N, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = unit / d.hkv, h = unit % d.hkv;
     const int B = a.per_batch_budget ? a.budget_of[b] : d.B;
