@@ -88,6 +88,7 @@ def algorithmic_bytes(cfg, kernel: str) -> float:
         "decay_select_gather": 2 * row + 4 * units * B + 4 * units * (B + W) * D * e,
         "select_gather": row + 4 * units * B + 4 * units * (B + W) * D * e,
         "select_sources": row + 4 * units * Ks,
+        "similarity_bounds": 0.0,              # a sample of the keys; the sweep after it counts them whole
         "similarity": units * N * D * e + units * Ks * D * e,
         "select_neighbors": 0.0,
         "decay_rounds": 8 * units * Ks * m * 3,
