@@ -105,8 +105,8 @@ def algorithmic_bytes(cfg, kernel: str) -> float:
 # kernel inside a running step (caches as the steps before left them); see
 # profiles/kernels_llama31_8b_32k_ncu_warm.md.  Only for the workload and kernels those captures
 # cover and only while the kernels are the ones captured; anything else reports null.
-NCU_TRAFFIC = {"llama31_8b_32k": {"score_fused_tc": 73.43e6, "pool_select_sources": 0.23e6,
-                                  "similarity_tc": 0.47e6, "decay_select_gather": 1.81e6}}
+NCU_TRAFFIC = {"llama31_8b_32k": {"score_fused_tc": 72.51e6, "pool_select_sources": 0.27e6,
+                                  "similarity_tc": 0.66e6, "decay_select_gather": 1.80e6}}
 
 
 def path_bytes(cfg) -> float:
