@@ -240,7 +240,9 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
         // ---- norms of the keys, four warps a tile ----
         for (int i = (warp - 2) >> 2; i < n_local && ok; i += 2) {
             const int st = i % S;
-            ok = __all_sync(0xffffffffu, mbar_wait(s_full0 + 8 * st, (i / S) & 1, lim));
+            // (The norms of the tile before in this stage first: with S odd the other group took it, so this group's view of
+            // the stage's barrier skips phases, and the parity of the phase it waits for could be an older one's.)
+            ok = __all_sync(0xffffffffu, (i < S || mbar_wait(s_norms0 + 8 * (i - S), 0, lim)) && mbar_wait(s_full0 + 8 * st, (i / S) & 1, lim));
             if (!ok) break;
             const uint8_t *tile = gen + l.stage + st * tile_bytes<kD>();
             uint64_t n2 = 0ull;                                         // (the same two sums as elsewhere, packed)
