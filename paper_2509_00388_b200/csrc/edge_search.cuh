@@ -8,10 +8,10 @@ namespace graphkv {
 
 // The edges of x(0 .. n) (lane-strided: element i * 32 + lane, kCandEmpty where there is none) that reach a
 // bound at which between m and kCandCap of them do; with too many near-ties, exactly the m largest (lowest
-// positions first).  put(slot, e, i).  Returns their number, and in *bound a value that m of them reach (-1
+// positions first; kOrdered = false, where i is in no order of position: none, and -1 returned).  put(slot, e, i).  Returns their number, and in *bound a value that m of them reach (-1
 // with fewer than m).  `from`: -1, or a value that at least m of them are known to reach.  Rolled loops over
 // shared memory: the code runs once per source.
-template <typename At, typename Put>
+template <bool kOrdered = true, typename At, typename Put>
 __device__ __forceinline__ int warp_list_top(int n, int m, float from, At x, Put put, float *bound)
 {
     const int lane = threadIdx.x & 31;
@@ -47,6 +47,7 @@ __device__ __forceinline__ int warp_list_top(int n, int m, float from, At x, Put
         }
     }
     if (have >= m) *bound = lo;
+    if (!kOrdered && have > kCandCap) return -1;
     uint32_t exact = 0;                         // with too many near-ties: the key of the m-th largest
     int ties = 0;                               // and how many of its ties belong to the m
     if (have > kCandCap) {

@@ -46,6 +46,7 @@ struct Layout {
     size_t cand;        // per-chunk neighbour candidates [units][K_src][sim_chunks][kCandCap]
     size_t cand_hist;   // [units][K_src][kCandBins]
     size_t tau;         // bounds of the sources' m-th edges [units][K_src]
+    size_t spill;       // edges that full lists did not take, per CTA of the streaming sweep
     size_t total;
     int max_parts;      // partial statistics per row the region can hold
 };
@@ -217,23 +218,37 @@ SimPlan sim_plan(const Dims &d, bool bf16)
     const int cap = 512 / p.NP;
     p.chunks = sweep_chunks(group * ceil_div(d.K_src, p.NP), p.n_tiles, ceil_div(p.n_tiles, cap), 1 << 20);
     p.ok = true;
-    // A head's sources in one streaming sweep, with bounds from a sample (sim_stream.cuh), where that form would take more
-    // than one wave of CTAs: the sample costs 20 us, which one wave does not (32 sources at 32K x 8 heads: 92 against 104
-    // us a call), but two waves do (40 sources 107 -> 106, 64 118 -> 115, 154 179 -> 141; 32 sources at 128K x 32 heads
-    // 1082 -> 1031, 16K x 128 with 40 sources 566 -> 444, with 100 846 -> 594).  Not with up to 16 sources, of which that form
-    // holds 32 tiles (16K x 128: 481 against 507).
-    if (group >= d.units && d.K_src > 16 && p.n_tiles >= 16 && (long long)d.units * ceil_div(d.K_src, p.NP) * p.chunks > sm_count()) {
-        p.stream = true;
-        const int sweeps = ceil_div(d.K_src, tc::kStreamMaxSources);
-        p.NP = ceil_div(ceil_div(d.K_src, sweeps), 32) * 32;
-        p.chunks = sweep_chunks(d.units * sweeps, p.n_tiles, ceil_div(p.n_tiles, tc::kStreamMaxTiles), 1 << 20);
-        for (p.stages = 6; p.stages > 3; --p.stages)
-            if ((d.D == 64 ? tc::stream_layout<64>(p.NP, p.stages) : tc::stream_layout<128>(p.NP, p.stages)).bytes <= kMaxSmem) break;
-        // the larger the sample, the fewer edges reach the bounds (about 1.1 m n_tiles / sample of a row's); a cluster of up to
-        // four CTAs, 16 tiles each, takes it
-        p.sample_ctas = std::max(1, std::min(4, sm_count() / (d.units * ceil_div(d.K_src, 32))));
-        p.sample = std::min(16 * p.sample_ctas, ceil_div(p.n_tiles, 2));
-        p.sample_ctas = std::min(p.sample_ctas, p.sample);
+    // A head's sources in one streaming sweep, with bounds from a sample (sim_stream.cuh), where that form would take
+    // more than one wave of CTAs and the estimate below is for it.
+    const int waves = ceil_div(d.units * ceil_div(d.K_src, p.NP) * p.chunks, sm_count());
+    if (group >= d.units && d.K_src > 16 && p.n_tiles >= 16 && waves > 1) {
+        SimPlan q = p;
+        q.stream = true;
+        const int sweeps = ceil_div(d.K_src, tc::kStreamMaxSources), blocks = d.units * ceil_div(d.K_src, 32);
+        q.NP = ceil_div(ceil_div(d.K_src, sweeps), 32) * 32;
+        // The larger the sample, the fewer edges reach the bounds, about 1.4 m n_tiles / sample of a row's, which all have to be
+        // listed.  A cluster of up to four CTAs takes it: a quarter of the row, 24 tiles a CTA; where a CTA has it to itself, three
+        // eighths, up to 64 tiles.
+        q.sample_ctas = std::max(1, std::min(4, sm_count() / blocks));
+        q.sample = std::max(1, q.sample_ctas > 1 ? std::min(p.n_tiles / 4, 24 * q.sample_ctas) : std::min(p.n_tiles * 3 / 8, 64));
+        q.sample_ctas = std::min(q.sample_ctas, q.sample);
+        // chunks of up to 32 tiles, with 40 such edges or fewer on the average, of the 64 that a list holds
+        const double edges = 1.4 * d.m * p.n_tiles / q.sample;
+        q.chunks = sweep_chunks(d.units * sweeps, p.n_tiles, std::max(ceil_div(p.n_tiles, tc::kStreamMaxTiles), (int)(edges / 40) + 1), 1 << 20);
+        for (q.stages = 6; q.stages > 3; --q.stages)
+            if ((d.D == 64 ? tc::stream_layout<64>(q.NP, q.stages) : tc::stream_layout<128>(q.NP, q.stages)).bytes <= kMaxSmem) break;
+        // Times in us: waves of CTAs, each some us and a time per tile; an edge above its bound 15 ns where many share a list.
+        const double resident = waves * (4 + (p.NP == 64 ? 2.4 : 1.2) * ceil_div(p.n_tiles, p.chunks));
+        const double stream = ceil_div(blocks * q.sample_ctas, sm_count()) * (7 + 0.5 * ceil_div(q.sample, q.sample_ctas)) +
+                              ceil_div(d.units * sweeps * q.chunks, sm_count()) * (6 + (0.4 + 0.012 * q.NP) * ceil_div(p.n_tiles, q.chunks)) +
+                              0.015 * edges * d.units * d.K_src / sm_count();
+        // Calls of up to two waves: the sample runs under the end of the pooling kernel, and both forms take the same time within some
+        // percent (16 x 10000 with 60 sources, at 1.49: 108 and 108 us a call, with topics of 64 tokens 108 and 122; 8 x 8192 with
+        // 160, at 1.32: 106 and 103, 117 and 125; 8 x 32K with 64, at 1.09: 123 and 123, 131 and 135).  In larger ones the estimate
+        // tells (128 x 16K with 32, at 1.30: 440 and 469, 443 and 497; 64 x 8160 with 100, at 1.17: 275 and 258, 288 and 322; with 38,
+        // at 1.05: 194 and 190, 198 and 215; 128 x 16K with 64, at 1.03: 608 and 563, 624 and 621; 32 x 16K with 154, at 0.97: 321 and
+        // 279, 334 and 332; 32 x 128K with 32, at 0.88: 822 and 802, 822 and 765).
+        if (stream < (waves <= 2 ? 1.5 : 1.05) * resident) return q;
     }
     return p;
 }
@@ -264,6 +279,7 @@ Layout layout_of(const Dims &d)
     l.cand = take(slots * kCandCap * sizeof(Cand));
     l.cand_hist = take((size_t)d.units * (d.K_src > 0 ? d.K_src : 1) * kCandBins * sizeof(uint32_t));
     l.tau = take((size_t)d.units * (d.K_src > 0 ? d.K_src : 1) * sizeof(float));
+    l.spill = take(sp.stream ? (size_t)ceil_div(d.K_src, sp.NP) * d.units * sp.chunks * tc::kStreamSpill * sizeof(uint2) : 1);
     l.total = off;
     return l;
 }
@@ -572,25 +588,38 @@ EncodeTiledFn encode_tiled_fn()
 }
 
 // Tensor map over K [batch][hkv][rows][D] bf16 with the caller's strides; boxes of 128 rows x 64
-// columns, 128-byte swizzle, zero fill past the last row.
-bool make_k_tensormap(CUtensorMap *tm, const void *K, const Dims &d, int rows, const long long *ks = nullptr)
+// columns, 128-byte swizzle, zero fill past the last row.  slice_step > 0: boxes of kSlices times kSliceKeys
+// rows, one such slice every slice_step rows (zero fill past the last whole one).
+bool make_k_tensormap(CUtensorMap *tm, const void *K, const Dims &d, int rows, const long long *ks = nullptr, int slice_step = 0)
 {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return false;
     if (!ks) ks = d.ks;
     const cuuint64_t row_b = (cuuint64_t)ks[2] * 2;
-    cuuint64_t dims[4] = {(cuuint64_t)d.D, (cuuint64_t)rows, (cuuint64_t)d.hkv, (cuuint64_t)d.batch};
     cuuint64_t head_b = (cuuint64_t)ks[1] * 2, batch_b = (cuuint64_t)ks[0] * 2;
     if (d.hkv == 1 || head_b == 0) head_b = row_b * (cuuint64_t)rows;
     if (d.batch == 1 || batch_b == 0) batch_b = head_b * (cuuint64_t)d.hkv;
-    cuuint64_t strides[3] = {row_b, head_b, batch_b};
-    cuuint32_t box[4] = {64, (cuuint32_t)tc::kTileKeys, 1, 1};
-    cuuint32_t estr[4] = {1, 1, 1, 1};
-    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(K), dims, strides, box, estr,
+    cuuint64_t dims[5] = {(cuuint64_t)d.D}, strides[4] = {row_b};
+    cuuint32_t box[5] = {64}, estr[5] = {1, 1, 1, 1, 1};
+    int n = 1;
+    auto dim = [&](cuuint64_t size, cuuint32_t taken, cuuint64_t stride) {
+        dims[n] = size;
+        box[n] = taken;
+        strides[n - 1] = stride;
+        ++n;
+    };
+    if (slice_step > 0) {
+        dim(tc::kSliceKeys, tc::kSliceKeys, row_b);
+        dim((rows - tc::kSliceKeys) / slice_step + 1, tc::kSlices, (cuuint64_t)slice_step * row_b);
+    } else {
+        dim(rows, tc::kTileKeys, row_b);
+    }
+    dim(d.hkv, 1, head_b);
+    dim(d.batch, 1, batch_b);
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, n, const_cast<void *>(K), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-
 
 // What the sweeps do besides the attention mass: words cleared for the kernels that follow.
 struct EmitExtras {
@@ -778,9 +807,12 @@ graphkv_status launch_similarity(const CUtensorMap &tmK, const tc::SimTcArgs &sa
                      sa.wait_prior != 0, 1, tmK, sa);
 }
 
+// Keys from one slice of the sample to the next.
+inline int slice_step(const Dims &d, const SimPlan &sp) { return ceil_div(d.N, sp.sample * tc::kSlices); }
+
 // Bounds from a sample of the row, then one sweep for all sources (sim_stream.cuh).
 template <int kD>
-graphkv_status run_stream(const Dims &d, const Layout &l, const SimPlan &sp, const CUtensorMap &tmK, const __nv_bfloat16 *S,
+graphkv_status run_stream(const Dims &d, const Layout &l, const SimPlan &sp, const CUtensorMap &tmK, const CUtensorMap &tmSlices, const __nv_bfloat16 *S,
                           const long long *ss, const int *src, void *ws, cudaStream_t st)
 {
     static std::mutex mu;
@@ -790,13 +822,13 @@ graphkv_status run_stream(const Dims &d, const Layout &l, const SimPlan &sp, con
         }))
         return GRAPHKV_ERR_CUDA;
     tc::SimTcArgs ba{d, S, {ss[0], ss[1], ss[2]}, src, nullptr, nullptr, at<int>(ws, l.status), 0, sp.sample_ctas, sp.sample,
-                     d.D == 64 ? 8 : 5, 0, wait_cycles(), sp.n_tiles, at<float>(ws, l.tau)};
+                     d.D == 64 ? 8 : 5, 0, wait_cycles(), slice_step(d, sp), at<float>(ws, l.tau), env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) == 3};
     ba.wait_prior = next_launch_is_dependent();
     const graphkv_status rc = launch_ex("similarity_bounds", tc::similarity_tc<32, kD, true>, dim3(sp.sample_ctas, d.units, ceil_div(d.K_src, 32)),
-                                        dim3(tc::kSimThreads), tc::sim_smem_bytes<32, kD>(), st, ba.wait_prior != 0, sp.sample_ctas, tmK, ba);
+                                        dim3(tc::kSimThreads), tc::sim_smem_bytes<32, kD>(), st, ba.wait_prior != 0, sp.sample_ctas, tmSlices, ba);
     if (rc != GRAPHKV_OK) return rc;
     tc::SimStreamArgs sa{d, S, {ss[0], ss[1], ss[2]}, src, at<float>(ws, l.tau), at<Cand>(ws, l.cand), at<uint32_t>(ws, l.cand_hist),
-                         at<int>(ws, l.status), sp.chunks, sp.n_tiles, sp.NP, sp.stages, 0, wait_cycles()};
+                         at<uint2>(ws, l.spill), at<int>(ws, l.status), sp.chunks, sp.n_tiles, sp.NP, sp.stages, 0, wait_cycles(), env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) == 4};
     sa.wait_prior = next_launch_is_dependent();
     return launch_ex("similarity_tc", tc::sim_stream_tc<kD>, dim3(sp.chunks, d.units, ceil_div(d.K_src, sp.NP)), dim3(tc::kStreamThreads),
                      tc::stream_layout<kD>(sp.NP, sp.stages).bytes, st, sa.wait_prior != 0, 1, tmK, sa);
@@ -811,8 +843,10 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
         CUtensorMap tmK;
         if (!make_k_tensormap(&tmK, eo.A, d, d.L, eo.as)) return GRAPHKV_ERR_CUDA;
         if (sp.stream) {
+            CUtensorMap tmSlices;
+            if (!make_k_tensormap(&tmSlices, eo.A, d, d.L, eo.as, slice_step(d, sp))) return GRAPHKV_ERR_CUDA;
             const auto *S = reinterpret_cast<const __nv_bfloat16 *>(eo.S);
-            return d.D == 64 ? run_stream<64>(d, l, sp, tmK, S, eo.ss, src, ws, st) : run_stream<128>(d, l, sp, tmK, S, eo.ss, src, ws, st);
+            return d.D == 64 ? run_stream<64>(d, l, sp, tmK, tmSlices, S, eo.ss, src, ws, st) : run_stream<128>(d, l, sp, tmK, tmSlices, S, eo.ss, src, ws, st);
         }
         const int group = units_per_group(d);
         for (int u0 = 0; u0 < d.units; u0 += group) {
@@ -820,7 +854,7 @@ graphkv_status run_graph(const Dims &d, const Layout &l, const EdgeOperands<T> &
             // one launch takes every source: grid.z counts the sweeps of sp.NP sources each
             tc::SimTcArgs sa{d, reinterpret_cast<const __nv_bfloat16 *>(eo.S), {eo.ss[0], eo.ss[1], eo.ss[2]}, src, at<Cand>(ws, l.cand),
                              at<uint32_t>(ws, l.cand_hist), at<int>(ws, l.status), u0, sp.chunks,
-                             sp.n_tiles, sp.stages, 0, wait_cycles(), sp.n_tiles, nullptr};
+                             sp.n_tiles, sp.stages, 0, wait_cycles(), 0, nullptr, 0};
             sa.wait_prior = next_launch_is_dependent();
             const dim3 grid(sp.chunks, nu, ceil_div(d.K_src, sp.NP)), block(tc::kSimThreads);
             const auto launch = d.D == 64 ? (sp.NP == 16 ? launch_similarity<16, 64> : sp.NP == 32 ? launch_similarity<32, 64>

@@ -56,9 +56,13 @@ struct SimTcArgs {
     int stages;
     int wait_prior;        // launched with programmatic stream serialization
     long long wait_cycles; // limit of every wait of the kernel, in clocks
-    int row_tiles;         // sampling form: n_tiles tiles spread evenly over the row's, shared by the `chunks` CTAs of a cluster
+    int slice_step;        // sampling form: n_tiles tiles shared by the `chunks` CTAs of a cluster, each of kSlices slices of the
+                           // row's, one every slice_step keys (a passage of few similar keys has its share of the sample)
     float *tau;            // sampling form: [units][K_src] per source, a value that at least m of its edges reach
+    int withhold_commit;   // test hook: the first product is never announced
 };
+
+constexpr int kSliceKeys = 8, kSlices = kTileKeys / kSliceKeys;
 
 template <int NP> __host__ __device__ constexpr int sim_tiles_cap() { return 512 / NP; }
 // Bytes of the ring's place: the tiles in flight; then maxima [NP][512 or 256]; then, with the bounds taken,
@@ -175,6 +179,10 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     int *cnt = reinterpret_cast<int *>(gen + Sh::cnt);
     Cand *list = reinterpret_cast<Cand *>(gen + Sh::list);
     constexpr int kParts = sim_parts<NP>();
+    // Tiles whose edges tensor memory holds.  The sampling form, which keeps maxima only, goes round: tile i's place is free once the
+    // same warps have given back tile i - 8, that is before tile i is copied (up to eight stages).
+    constexpr int kHeld = sim_tiles_cap<NP>();
+    static_assert(!kSample || (kHeld % 8 == 0 && NP == 32), "four sets of warps take the tiles in turn");
     float *maxima = reinterpret_cast<float *>(gen + Sh::stage);                 // [NP][kParts] after the sweep
     uint2 *queue = reinterpret_cast<uint2 *>(maxima);                           // [kSimQueue][kSimEpiThreads] after the bounds
     int *failed = reinterpret_cast<int *>(gen + Sh::tmem) + 1;
@@ -187,8 +195,17 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
     const int per = a.n_tiles / a.chunks, rem = a.n_tiles % a.chunks;
     const int t0 = chunk * per + min(chunk, rem);
     const int n_local = per + (chunk < rem ? 1 : 0);
-    auto tile_of = [&](int i) {
-        return kSample ? (int)((long long)(chunk + i * a.chunks) * a.row_tiles / a.n_tiles) : t0 + i;
+    // the sample's tile i, a tile of the chunk
+    auto load_tile = [&](int i, int st) {
+        const uint32_t dst = s_stage0 + st * tile_bytes<kD>(), bar = s_full0 + 8 * st;
+        if constexpr (kSample) {
+            mbar_expect_tx(bar, tile_bytes<kD>());
+#pragma unroll
+            for (int half = 0; half < kD / 64; ++half)
+                tma_load_5d(dst + half * kHalfBytes, &tmK, bar, half * 64, 0, (chunk + i * a.chunks) * kSlices, h, b);
+        } else {
+            tma_load_tile<kD>(dst, &tmK, bar, (t0 + i) * kTileKeys, h, b);
+        }
     };
     const __nv_bfloat16 *src_rows = a.S + b * a.ss[0] + (long long)h * a.ss[1];
     // a head with more than NP sources is swept once per NP of them: grid.z counts those sweeps
@@ -202,15 +219,14 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             mbar_init(s_full0 + 8 * i, 1);
             mbar_init(s_empty0 + 8 * i, 1 + (NP == 64 ? 8 : 4));       // MMA commit + the epilogue warps of a tile
         }
-        for (int i = 0; i < n_local; ++i) mbar_init(s_done0 + 8 * i, 1);
+        for (int i = 0; i < min(n_local, kHeld); ++i) mbar_init(s_done0 + 8 * i, 1);
         *failed = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmK);
         // the first ring-full of key tiles is under way while the sources are gathered (keys are an
         // input of the call: no wait for the kernels before)
         n_ahead = min(a.stages, n_local);
-        for (int i = 0; i < n_ahead; ++i)
-            tma_load_tile<kD>(s_stage0 + i * tile_bytes<kD>(), &tmK, s_full0 + 8 * i, tile_of(i) * kTileKeys, h, b);
+        for (int i = 0; i < n_ahead; ++i) load_tile(i, i);
     }
     if (warp == 1) {
         tmem_alloc(s_tmem, 512);
@@ -264,7 +280,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             for (int i = n_ahead; i < n_local; ++i) {
                 const int st = i % a.stages, ph = (i / a.stages) & 1;
                 if (!mbar_wait(s_empty0 + 8 * st, ph ^ 1, lim)) { ok = false; break; }
-                tma_load_tile<kD>(s_stage0 + st * tile_bytes<kD>(), &tmK, s_full0 + 8 * st, tile_of(i) * kTileKeys, h, b);
+                load_tile(i, st);
                 ++issued;
             }
             if (!ok)        // gave up: let the copies already in flight land before the CTA exits
@@ -282,9 +298,9 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
             if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
             tc_fence_after();
             if (elect_one()) {
-                umma_tile<kD>(tmem_base + i * NP, ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, src_lo, NP * 128 >> 4, idesc);
+                umma_tile<kD>(tmem_base + i % kHeld * NP, ring_lo + st * (tile_bytes<kD>() >> 4), kHalfBytes >> 4, src_lo, NP * 128 >> 4, idesc);
                 umma_commit(s_empty0 + 8 * st);
-                umma_commit(s_done0 + 8 * i);
+                if (!(a.withhold_commit && i == 0)) umma_commit(s_done0 + 8 * (i % kHeld));
             }
             __syncwarp();
             if (++st == a.stages) st = 0, ph ^= 1u;
@@ -309,11 +325,11 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
                 const int st = i % a.stages, ph = (i / a.stages) & 1;
                 // (The MMA of the tile first, on a barrier of its own: a set sees only some of the tiles, so its view
                 // of a stage's barrier skips phases, and the parity of a phase it waits for could be an older one's.)
-                ok = __all_sync(0xffffffffu, mbar_wait(s_done0 + 8 * i, 0, lim) && mbar_wait(s_full0 + 8 * st, ph, lim));
+                ok = __all_sync(0xffffffffu, mbar_wait(s_done0 + 8 * (i % kHeld), (i / kHeld) & 1, lim) && mbar_wait(s_full0 + 8 * st, ph, lim));
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t raw[kCols];
-                load(i, raw);
+                load(i % kHeld, raw);
                 // squared norm of this thread's key from the staged tile
                 const uint8_t *tile = gen + Sh::stage + st * tile_bytes<kD>();
                 float n0 = 0.f, n1 = 0.f;
@@ -329,10 +345,12 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
                     }
                 }
                 const int key = i * kTileKeys + key_lane;
-                const bool in = tile_of(i) * kTileKeys + key_lane < d.N;
+                const bool in = (kSample ? ((chunk + i * a.chunks) * kSlices + key_lane / kSliceKeys) * a.slice_step + key_lane % kSliceKeys
+                                        : (t0 + i) * kTileKeys + key_lane) < d.N;
                 // (a key past the end of the row: NaN, which no comparison and no maximum takes)
                 const float inv = in ? 1.0f / fmaxf(sqrtf(n0 + n1), kNormEps) : __int_as_float(0x7fc00000);
-                if (col0 == 0) inv_norm[key] = inv;
+                if (!kSample && col0 == 0) inv_norm[key] = inv;
+                if constexpr (kSample) tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(s_empty0 + 8 * st);
                 tmem_ld_fence(raw);

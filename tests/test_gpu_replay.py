@@ -53,11 +53,13 @@ def test_captured_decode_attention(gk, rows, batch, hkv, dtype):
 
 # every form of the score sweeps and of the rest of the path: one kernel whose CTAs wait for one another (one and
 # two row tiles, both head dimensions, one and several units), two kernels (by switch, and more units than the GPU
-# holds at once), short rows in one kernel, fp32, sources re-picked, budgets per layer
+# holds at once), short rows in one kernel, fp32, sources re-picked, budgets per layer, the streaming
+# similarity sweep
 @pytest.mark.parametrize("n,batch,hkv,over", [
     (16384, 1, 8, {}), (6013, 2, 2, {"window": 64}), (8191, 1, 8, {"head_dim": 64}), (5000, 1, 1, {"topk_nodes": 100}),
     (6013, 1, 2, {"two": True}), (4100, 40, 8, {}), (1003, 1, 8, {}), (700, 1, 2, {"dtype": torch.float32}),
-    (9000, 1, 2, {"reselect": 1}), (6000, 3, 2, {"budgets": [300, 100, 7]}), (4500, 1, 4, {"rounds": 0})])
+    (9000, 1, 2, {"reselect": 1}), (6000, 3, 2, {"budgets": [300, 100, 7]}), (4500, 1, 4, {"rounds": 0}),
+    (16384, 2, 8, {"topk_nodes": 150})])
 def test_captured_compress(gk, monkeypatch, n, batch, hkv, over):
     if over.get("two"):
         monkeypatch.setenv("GRAPHKV_TWO_SCORE_KERNELS", "1")

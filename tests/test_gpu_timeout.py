@@ -54,3 +54,35 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_exact(hook, two_k
     gk.graphkv_score(p, Qd, Kd, got, ws)
     assert gk.graphkv_read_status(ws) == gk.OK
     assert torch.equal(got, want)
+
+
+# the streaming similarity sweep: the kernel that takes its bounds from a sample (3) and the sweep itself (4) leave out the
+# arrival that announces their first product
+@pytest.mark.parametrize("hook", ["3", "4"])
+def test_a_wait_of_the_streaming_sweep_that_runs_out(hook):
+    from paper_2509_00388_b200 import binding as gk
+    gk.lib()
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(7)
+    K, V = (torch.randn((1, 8, 8192 + 32, 128), generator=gen, device=dev).to(torch.bfloat16) for _ in range(2))
+    Q = torch.randn((1, 32, 32, 128), generator=gen, device=dev).to(torch.bfloat16)
+    p = gk.make_params(K, Qw=Q, V=V, window=32, budget=512, pool_kernel=7, topk_nodes=160, neighbors=32, rounds=2)
+    ws = gk.alloc_workspace(p, dev)
+    want, got = gk.alloc_outputs(p, K), gk.alloc_outputs(p, K)
+    gk.graphkv_compress(p, Q, K, V, *want, ws)
+    assert gk.graphkv_read_status(ws) == gk.OK
+    os.environ["GRAPHKV_WAIT_CYCLES"] = "2000000"           # about a millisecond
+    os.environ["GRAPHKV_DEBUG_WITHHOLD_COMMIT"] = hook
+    try:
+        gk.graphkv_compress(p, Q, K, V, *got, ws)
+        status = gk.graphkv_read_status(ws)                 # synchronises: the kernels returned
+    finally:
+        os.environ.pop("GRAPHKV_WAIT_CYCLES", None)
+        os.environ.pop("GRAPHKV_DEBUG_WITHHOLD_COMMIT", None)
+    assert status == gk.ERR_TIMEOUT
+
+    # the same workspace, a normal call: the status is clean again and the results are the same to the bit
+    gk.graphkv_compress(p, Q, K, V, *got, ws)
+    assert gk.graphkv_read_status(ws) == gk.OK
+    for a, b in zip(got, want):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
