@@ -310,7 +310,7 @@ def graphkv_trace_read(capacity: int = 1 << 16):
 def graphkv_phase_timing_read():
     """Per-kernel phase times of a library built with GRAPHKV_PHASE_TIMING, or None.
     Returns {kernel index: (CTAs, [(mean ns, max ns) per phase])}; phase 0 is the whole CTA."""
-    n_k, n_s = 8, 24
+    n_k, n_s = 10, 24
     buf = (C.c_uint64 * (n_k * n_s * 2 + n_k))()
     if not lib().graphkv_phase_timing_read(buf):
         return None

@@ -97,7 +97,7 @@ __device__ __forceinline__ void pdl_wait()
 // One thread per CTA stamps %globaltimer at phase boundaries; at the end of the kernel the
 // differences are added into per-kernel tables that graphkv_phase_timing_read copies out.  In the
 // normal build the marks compile to nothing.
-constexpr int kPhaseKernels = 8, kPhaseSlots = 24;
+constexpr int kPhaseKernels = 10, kPhaseSlots = 24;
 #ifdef GRAPHKV_PHASE_TIMING
 __device__ unsigned long long g_phase_sum[kPhaseKernels][kPhaseSlots];
 __device__ unsigned long long g_phase_max[kPhaseKernels][kPhaseSlots];

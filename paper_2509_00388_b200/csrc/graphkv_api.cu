@@ -830,7 +830,7 @@ graphkv_status run_stream(const Dims &d, const Layout &l, const SimPlan &sp, con
     tc::SimStreamArgs sa{d, S, {ss[0], ss[1], ss[2]}, src, at<float>(ws, l.tau), at<Cand>(ws, l.cand), at<uint32_t>(ws, l.cand_hist),
                          at<uint2>(ws, l.spill), at<int>(ws, l.status), sp.chunks, sp.n_tiles, sp.NP, sp.stages, 0, wait_cycles(), env_int("GRAPHKV_DEBUG_WITHHOLD_COMMIT", 0) == 4};
     sa.wait_prior = next_launch_is_dependent();
-    return launch_ex("similarity_tc", tc::sim_stream_tc<kD>, dim3(sp.chunks, d.units, ceil_div(d.K_src, sp.NP)), dim3(tc::kStreamThreads),
+    return launch_ex("similarity_stream", tc::sim_stream_tc<kD>, dim3(sp.chunks, d.units, ceil_div(d.K_src, sp.NP)), dim3(tc::kStreamThreads),
                      tc::stream_layout<kD>(sp.NP, sp.stages).bytes, st, sa.wait_prior != 0, 1, tmK, sa);
 }
 

@@ -671,7 +671,7 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
         tmem_dealloc(tmem_base, 512);
     }
     pc.mark();
-    pc.flush(0);
+    pc.flush(8);
 }
 
 }  // namespace tc

@@ -544,7 +544,7 @@ similarity_tc(const __grid_constant__ CUtensorMap tmK, SimTcArgs a)
         tmem_dealloc(tmem_base, 512);
     }
     pc.mark();
-    pc.flush(kSample ? 1 : 2);
+    pc.flush(kSample ? 9 : 2);
 }
 
 }  // namespace tc

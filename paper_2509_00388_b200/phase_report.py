@@ -20,10 +20,10 @@ import torch  # noqa: E402
 from . import binding as gk  # noqa: E402
 from . import workloads as wl  # noqa: E402
 
-KERNELS = {0: "score_stats_tc (with many sources or long rows also sim_stream_tc)",
-           1: "score_emit_tc (and similarity_tc on a sample)", 2: "similarity_tc", 3: "pool_select_kernel",
+KERNELS = {0: "score_stats_tc", 1: "score_emit_tc", 2: "similarity_tc", 3: "pool_select_kernel",
            4: "finish_kernel (first CTA of a cluster)", 5: "score_fused_tc",
-           6: "finish_kernel (other CTAs)", 7: "cluster_path_kernel"}
+           6: "finish_kernel (other CTAs)", 7: "cluster_path_kernel", 8: "sim_stream_tc",
+           9: "similarity_tc on a sample"}
 
 
 def main(name: str = "llama31_8b_32k", steps: int = 5) -> None:
