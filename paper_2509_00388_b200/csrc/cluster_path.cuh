@@ -44,7 +44,7 @@ constexpr int kMaxNeighbours = 32;
 // and, behind them, the unit's scores where they fit; the tiles' place, once the sweeps are over, the unit's
 // neighbour lists [k][m] (position, factor) and, at its end, the kept positions [B]; the place of the row statistics
 // [C][GW] the cosines [rows][N].  Those come from other CTAs, which do not know whether this one's sweep is over:
-// in the tiles' place (behind the lists) they cost one more cluster barrier, so only where nothing else fits.
+// in the tiles' place (behind the lists) they cost one more cluster barrier, so only where they do not fit otherwise.
 struct Layout {
     int tiles, lists, mass, row, inv, row_c, parts, cosines, scratch, small, bars, total;
 };
