@@ -266,8 +266,7 @@ def test_one_score_kernel_and_two_agree_to_the_bit(gk, window):
 
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_head_dimension_64(gk, dtype):
-    # heads of 64 dimensions take the general kernels for the scores, the edges and the gather
-    # (the tensor-core kernels are written for 128) and the same row kernels
+    # heads of 64 dimensions: the tensor-core kernels in bf16, the register-tiled ones in fp32, and the same row kernels
     cfg = wl.scaled(wl.LLAMA_32K, head_dim=64, dtype=dtype, n_prefix=3000 + 21, budget=200, n_q_heads=8,
                     n_kv_heads=2, n_clusters=24, neighbors=8, batch=2)
     check(gk, cfg, strict_overlap=False)
