@@ -227,10 +227,10 @@ SimPlan sim_plan(const Dims &d, bool bf16)
         const int sweeps = ceil_div(d.K_src, tc::kStreamMaxSources), blocks = d.units * ceil_div(d.K_src, 32);
         q.NP = ceil_div(ceil_div(d.K_src, sweeps), 32) * 32;
         // The larger the sample, the fewer edges reach the bounds, about 1.4 m n_tiles / sample of a row's, which all have to be
-        // listed.  A cluster of up to four CTAs takes it: a quarter of the row, 24 tiles a CTA; where a CTA has it to itself, three
+        // listed.  A cluster of up to four CTAs takes it: a quarter of the row, 16 tiles a CTA; where a CTA has it to itself, three
         // eighths, up to 64 tiles.
         q.sample_ctas = std::max(1, std::min(4, sm_count() / blocks));
-        q.sample = std::max(1, q.sample_ctas > 1 ? std::min(p.n_tiles / 4, 24 * q.sample_ctas) : std::min(p.n_tiles * 3 / 8, 64));
+        q.sample = std::max(1, q.sample_ctas > 1 ? std::min(p.n_tiles / 4, 16 * q.sample_ctas) : std::min(p.n_tiles * 3 / 8, 64));
         q.sample_ctas = std::min(q.sample_ctas, q.sample);
         // chunks of up to 32 tiles, with 40 such edges or fewer on the average, of the 64 that a list holds
         const double edges = 1.4 * d.m * p.n_tiles / q.sample;

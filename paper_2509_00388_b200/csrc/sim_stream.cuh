@@ -4,12 +4,12 @@
 // similarity_tc keeps a chunk's whole edge block in tensor memory until bounds for the chunk are known, so its loads stop
 // for half of its time, and a head with more than 64 sources is swept several times.  Here the bounds come first: a
 // sample of the row (similarity_tc in its sampling form, a cluster of CTAs per 32 sources) gives per source a
-// value that at least m of its edges reach; with a quarter of the row sampled about 5.6 m edges of the row reach it.  The sweep
+// value that at least m of its edges reach; with a fifth of the row sampled about 7 m edges of the row reach it.  The sweep
 // then streams: up to 192 sources are the columns of one product per key tile, two to four accumulators rotate, eight warps take
 // the keys' norms, and 16 epilogue warps (thread = key) push the edges that reach their source's bound into queues of
 // their own, with predicated stores and no branch, and list them from there, by source and chunk.
 //
-// In a text, keys that are alike stand together, so most of a source's 5.6 m edges can fall to few tiles.  So the sample is slices
+// In a text, keys that are alike stand together, so most of a source's 7 m edges can fall to few tiles.  So the sample is slices
 // of eight keys all along the row, a chunk's tiles are spread over the row, and a list that is full (kCandCap) spills: the
 // CTA keeps up to kStreamSpill more edges in memory, and a warp picks from those of a source when the sweep is done.  What does
 // not fit there either is counted in bins, and the sources concerned are swept again with the bound that the bins give.  Where
@@ -18,10 +18,10 @@
 // Bound: the comparisons.  128 keys x 160 sources take 1.8 us per SM, of which the products are 0.35 and the arrival of the tile
 // 0.4; per 32 sources a warp spends about 400 issue slots on the comparisons of its 32 keys and on the edges found.  At 32
 // sources a tile takes 0.8 us, near the 0.72 at which HBM delivers it.  Whole calls, with similarity_tc and with this (keys drawn
-// independently; topics that last 64 tokens; 512): 154 sources at 32K x 8 heads 189 -> 159, 195 -> 185, 214 -> 172 us; 100 sources
+// independently; topics that last 64 tokens; 512): 154 sources at 32K x 8 heads 189 -> 154, 195 -> 183, 214 -> 173 us; 100 sources
 // at 128K x 32 heads 1692 -> 1001, 1703 -> 1111, 1703 -> 1118; 32 sources there 822 -> 780, 822 -> 765, 854 -> 780; 100 at 16K x 128
 // 878 -> 705, 901 -> 805, 904 -> 754.  A sample of whole tiles, chunks of adjacent tiles and lists without spill took, in place of
-// 159, 185 and 172, 153, 326 and 463.  Tried: setp and a predicated store per edge instead of the sums of bits (the same time),
+// 154, 183 and 173, 152, 326 and 463.  Tried: setp and a predicated store per edge instead of the sums of bits (the same time),
 // queues listed at four instead of nine edges (2 us more), four warps for the norms (they held up the sweep of 32 sources),
 // another sweep in place of the spilled edges (topics of 256 tokens: 20 to 60 us more), spilled edges without the bins (where they
 // do not suffice, up to ten times the time).
@@ -39,7 +39,6 @@ namespace tc {
 constexpr int kStreamThreads = 64 + 256 + 512;          // producer, MMA, 8 norm warps, 16 epilogue warps
 constexpr int kStreamMaxSources = 192;
 constexpr int kStreamMaxTiles = 32;                     // tiles per chunk: the exact search holds 16 sources' edges with them
-constexpr int kStreamPasses = 2;                        // sweeps of a chunk before the exact search
 constexpr int kStreamSpill = 4096;                      // edges that full lists do not take, kept by a CTA
 constexpr int kStreamBins = 64;                         // per source, in which those beyond are counted
 // Edges per thread's queue, and how many make it be listed: a listing takes four edges of each thread at a time, so the
@@ -67,7 +66,7 @@ struct SimStreamArgs {
 
 // Dynamic shared memory, byte offsets from a 1024-byte aligned base.
 struct StreamLayout {
-    uint32_t stage, queue, inv_norm, src_pos, src_inv, theta, cnt, lo, scale, col, exact, hist, bars, bytes;
+    uint32_t stage, queue, inv_norm, own_key, src_inv, theta, cnt, lo, scale, col, exact, hist, bars, bytes;
 };
 template <int kD> __host__ __device__ inline StreamLayout stream_layout(int np, int stages)
 {
@@ -75,8 +74,8 @@ template <int kD> __host__ __device__ inline StreamLayout stream_layout(int np, 
     l.stage = np * 2 * kD;                               // source keys | key tiles in flight
     l.queue = l.stage + stages * tile_bytes<kD>();       // [stream_queue][512]; between sweeps the next one's columns [3][np]
     l.inv_norm = l.queue + stream_queue(np) * 512 * 8;   // [kStreamMaxTiles][128]
-    l.src_pos = l.inv_norm + kStreamMaxTiles * 128 * 4;  // per column of the sweep: position, 1 / norm, bound (negated), edges
-    l.src_inv = l.src_pos + np * 4;                      // found, source
+    l.own_key = l.inv_norm + kStreamMaxTiles * 128 * 4;  // per column of the sweep: own key, 1 / norm, bound (negated), edges
+    l.src_inv = l.own_key + np * 4;                      // found, source
     l.theta = l.src_inv + np * 4;
     l.cnt = l.theta + np * 4;
     l.lo = l.cnt + np * 4;                               // bound, and bins per unit above it, of the histogram
@@ -90,10 +89,11 @@ template <int kD> __host__ __device__ inline StreamLayout stream_layout(int np, 
 }
 __host__ __device__ inline int stream_bufs(int np) { return np <= 128 ? 4 : np <= 160 ? 3 : 2; }
 
-// What the listing of edges needs.
+// What the listing of edges needs.  (Put together where edges are listed, from the arguments: kept through the sweep, its
+// registers cost 2 us of a call of 154 sources.)
 struct StreamColumns {
-    int chunk, chunks;
-    const int *src_pos, *col;    // per column of the sweep: the source's position, the source
+    int chunk, chunks, again;
+    const int *own_key, *col;    // per column of the sweep: the source's own key of the chunk or -1, the source (the first sweep's: itself)
     int *cnt;                    // edges found
     Cand *cand;                  // source c's list of this chunk at c * source_stride
     long long source_stride;
@@ -102,29 +102,36 @@ struct StreamColumns {
     int *spilled;                // their number, kept or not
     const float *lo, *scale;     // the bins: the bound, bins per unit above it
     uint32_t *hist;              // [np][kStreamBins] 16-bit counts of those not kept
+    __device__ __forceinline__ int position(int key) const { return ((key >> 7) * chunks + chunk) * kTileKeys + (key & 127); }
+    __device__ __forceinline__ int key_of(int pos) const
+    {
+        const int tile = pos >> 7;
+        return tile % chunks == chunk ? tile / chunks * kTileKeys + (pos & 127) : -1;
+    }
     __device__ __forceinline__ void count(int c, float e) const
     {
         const int b = min(max(static_cast<int>((e - lo[c]) * scale[c]), 0), kStreamBins - 1);
         atomicAdd(hist + c * (kStreamBins / 2) + (b >> 1), 1u << (16 * (b & 1)));
     }
-    __device__ __forceinline__ int position(int key) const { return ((key >> 7) * chunks + chunk) * kTileKeys + (key & 127); }
-    // edge `at` of the column, `place` among those spilled where the list is full
-    __device__ __forceinline__ void put(int c, int at, int place, int key, float x) const
+    // edge `at` of the column, below kCandCap
+    __device__ __forceinline__ void list(int c, int at, int key, float x) const
     {
         const float e = clamped_edge(x);
-        if (at < kCandCap) {
-            const int src = col[c];
-            cand[src * source_stride + at] = Cand{e, position(key)};
-            atomicAdd(row_hist + src * kCandBins + cand_bin(e), 1u);
-        } else if (place < kStreamSpill) {
-            spill[place] = make_uint2(__float_as_uint(e), (uint32_t)c << 16 | (uint32_t)key);
-        } else {
-            count(c, e);
-        }
+        const int src = again ? col[c] : c;
+        cand[src * source_stride + at] = Cand{e, position(key)};
+        atomicAdd(row_hist + src * kCandBins + cand_bin(e), 1u);
+    }
+    // an edge beyond the list, the place-th of the chunk
+    __device__ __forceinline__ void put_aside(int c, int place, int key, float x) const
+    {
+        const float e = clamped_edge(x);
+        if (place < kStreamSpill) spill[place] = make_uint2(__float_as_uint(e), (uint32_t)c << 16 | (uint32_t)key);
+        else count(c, e);
     }
 };
 
-// Edges (column c, key of the chunk, cosine before clamping x; c < 0: none) into the lists of their sources.
+// Edges (column c, key of the chunk, cosine before clamping x; c < 0: none) into the lists of their sources.  (Their number is
+// small, but a warp goes through this for whichever lane has one: 30 instructions more took 3 us of a call of 154 sources.)
 template <int kN>
 __device__ __forceinline__ void stream_list(const int (&c)[kN], const int (&key)[kN], const float (&x)[kN], const StreamColumns &s)
 {
@@ -132,18 +139,26 @@ __device__ __forceinline__ void stream_list(const int (&c)[kN], const int (&key)
 #pragma unroll
     for (int q = 0; q < kN; ++q) {
         at[q] = -1;
-        if (c[q] >= 0 && s.position(key[q]) != s.src_pos[c[q]]) at[q] = atomicAdd(s.cnt + c[q], 1);
+        if (c[q] >= 0 && key[q] != s.own_key[c[q]]) at[q] = atomicAdd(s.cnt + c[q], 1);
     }
+    bool beyond = false;
 #pragma unroll
-    for (int q = 0; q < kN; ++q)
-        if (at[q] >= 0) s.put(c[q], at[q], at[q] < kCandCap ? 0 : atomicAdd(s.spilled, 1), key[q], x[q]);
+    for (int q = 0; q < kN; ++q) {
+        if ((uint32_t)at[q] < (uint32_t)kCandCap) s.list(c[q], at[q], key[q], x[q]);
+        beyond |= at[q] >= kCandCap;
+    }
+    if (beyond) {
+#pragma unroll
+        for (int q = 0; q < kN; ++q)
+            if (at[q] >= kCandCap) s.put_aside(c[q], atomicAdd(s.spilled, 1), key[q], x[q]);
+    }
 }
 
 // One column's edges of a warp's keys (in: the edge reaches the bound), counted together.
 __device__ __forceinline__ void stream_list_column(int c, int key, bool in, float x, const StreamColumns &s)
 {
     const int lane = threadIdx.x & 31;
-    in = in && s.position(key) != s.src_pos[c];
+    in = in && key != s.own_key[c];
     const unsigned all = __ballot_sync(0xffffffffu, in);
     if (all == 0u) return;
     const int n = __popc(all), rank = __popc(all & ((1u << lane) - 1u));
@@ -154,13 +169,153 @@ __device__ __forceinline__ void stream_list_column(int c, int key, bool in, floa
     }
     first = __shfl_sync(0xffffffffu, first, 0);
     place = __shfl_sync(0xffffffffu, place, 0);
-    if (in) s.put(c, first + rank, place + rank - max(kCandCap - first, 0), key, x);
+    if (in && first + rank < kCandCap) s.list(c, first + rank, key, x);
+    else if (in) s.put_aside(c, place + rank - max(kCandCap - first, 0), key, x);
+}
+
+template <int kD>
+__device__ __forceinline__ StreamColumns stream_columns(const SimStreamArgs &a, uint8_t *gen, int again)
+{
+    const StreamLayout l = stream_layout<kD>(a.np, a.stages);
+    const int unit = blockIdx.y, chunk = blockIdx.x;
+    const long long source0 = (long long)unit * a.d.K_src + blockIdx.z * a.np;
+    return StreamColumns{chunk, a.chunks, again, reinterpret_cast<int *>(gen + l.own_key), reinterpret_cast<int *>(gen + l.col),
+                         reinterpret_cast<int *>(gen + l.cnt), a.cand + (source0 * a.chunks + chunk) * kCandCap, (long long)a.chunks * kCandCap,
+                         a.cand_hist + source0 * kCandBins,
+                         a.spill + ((long long)(blockIdx.z * gridDim.y + unit) * a.chunks + chunk) * kStreamSpill,
+                         reinterpret_cast<int *>(gen + l.bars + 28 * 8) + 3, reinterpret_cast<float *>(gen + l.lo),
+                         reinterpret_cast<float *>(gen + l.scale), reinterpret_cast<uint32_t *>(gen + l.hist)};
+}
+
+// The edges of this thread's queue listed.
+template <int kD>
+__device__ __forceinline__ void stream_flush(const SimStreamArgs &a, uint8_t *gen, int queued, int again)
+{
+    const StreamLayout l = stream_layout<kD>(a.np, a.stages);
+    const StreamColumns columns = stream_columns<kD>(a, gen, again);
+    const float *src_inv = reinterpret_cast<const float *>(gen + l.src_inv);
+    const uint2 *q0 = reinterpret_cast<const uint2 *>(gen + l.queue) + ((int)threadIdx.x - 320);
+    const int queue = stream_queue(a.np);
+#pragma unroll 1
+    for (int k = 0; k < queued; k += 4) {
+        int c[4], key[4];
+        float x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint2 en = q0[min(k + q, queue - 1) * 512];
+            const bool in = k + q < queued;
+            c[q] = in ? (int)(en.y >> 16) : -1;
+            key[q] = (int)(en.y & 0xffffu);
+            x[q] = __uint_as_float(en.x) * src_inv[max(c[q], 0)];
+        }
+        stream_list<4>(c, key, x, columns);
+    }
+    __syncwarp();
+}
+
+// The edges of a slice that are more than the queues take, listed from tensor memory.
+template <int kD>
+__device__ __forceinline__ void stream_slice(const SimStreamArgs &a, uint8_t *gen, uint32_t taddr, int col0, int n_col, int key, float inv, int again)
+{
+    const StreamLayout l = stream_layout<kD>(a.np, a.stages);
+    const StreamColumns columns = stream_columns<kD>(a, gen, again);
+    const float *src_inv = reinterpret_cast<const float *>(gen + l.src_inv), *theta = reinterpret_cast<const float *>(gen + l.theta);
+#pragma unroll 1
+    for (int c0 = col0; c0 < col0 + 32 && c0 < n_col; c0 += 8) {
+        uint32_t r[8];
+        __syncwarp();
+        tmem_ld8_issue(taddr + c0 - col0, r);
+        tmem_ld_fence(r);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            stream_list_column(c0 + q, key, fmaf(__uint_as_float(r[q]), inv, theta[c0 + q]) > 0.f,
+                               __uint_as_float(r[q]) * inv * src_inv[c0 + q], columns);
+    }
+    __syncwarp();
+}
+
+// After a sweep in which lists were full: what was spilled, put in order by column (sorted, in the place of the ring; the columns'
+// counts behind it), and for every column concerned its list, or its place among those to sweep again (`last`: none) or to
+// search exactly.  By all threads; a function of its own, which keeps its registers out of the sweep's.
+__device__ __noinline__ void stream_resolve(StreamColumns s, uint2 *sorted, int *next, int *exact, int *words, int np, int n_col, int m, bool last)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_spilled = min(*reinterpret_cast<volatile int *>(words + 3), kStreamSpill);
+    float *bound = reinterpret_cast<float *>(next + np), *bins_of = bound + np;
+    int *kept = reinterpret_cast<int *>(sorted + kStreamSpill), *end = kept + np;       // [np] a column's edges, and their end
+    for (int c = threadIdx.x; c < n_col; c += kStreamThreads) kept[c] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_spilled; i += kStreamThreads) atomicAdd(kept + (__ldcg(&s.spill[i].y) >> 16), 1);
+    __syncthreads();
+    if (warp == 0) {
+        int run = 0;
+        for (int c0 = 0; c0 < n_col; c0 += 32) {
+            const int mine = c0 + lane < n_col ? kept[c0 + lane] : 0, incl = (int)bs::incl_scan((uint32_t)mine, lane);
+            if (c0 + lane < n_col) end[c0 + lane] = run + incl - mine;
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_spilled; i += kStreamThreads) {
+        const uint2 en = __ldcg(s.spill + i);
+        sorted[atomicAdd(end + (en.y >> 16), 1)] = make_uint2(en.x, en.y & 0xffffu);
+    }
+    __syncthreads();
+    // A source with more edges than slots, by a warp: those that reach a bound at which a list holds them.  Where some
+    // were not kept, another sweep with a bound from the counts; where too many tie, the exact search.
+    for (int c = warp; c < n_col; c += kStreamThreads / 32) {
+        const int excess = s.cnt[c] - kCandCap, have = kept[c];
+        if (excess <= 0) continue;
+        Cand *list = s.cand + s.col[c] * s.source_stride;
+        uint32_t *bins = s.row_hist + s.col[c] * kCandBins;
+        Cand own[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int2 raw = __ldcg(reinterpret_cast<const int2 *>(list + q * 32 + lane));
+            own[q] = Cand{__int_as_float(raw.x), raw.y};
+            atomicAdd(bins + cand_bin(own[q].e), 0xffffffffu);          // (counted anew)
+        }
+        const uint2 *more = sorted + end[c] - have - kCandCap;
+        if (have == excess) {
+            float reached;
+            const int n = warp_list_top<false>(kCandCap + have, m, -1.0f,
+                [&](int i) { return i < 32 ? own[0].e : i < 64 ? own[1].e : __uint_as_float(more[i].x); },
+                [&](int at, float e, int i) {
+                    list[at] = Cand{e, i < 32 ? own[0].j : i < 64 ? own[1].j : s.position((int)more[i].y)};
+                    atomicAdd(bins + cand_bin(e), 1u);
+                }, &reached);
+            if (n >= 0) {
+                for (int q = n + lane; q < kCandCap; q += 32) list[q] = Cand{kCandEmpty, -1};
+                continue;
+            }
+        } else if (!last) {
+            // all of the column's edges counted, two bins per lane: the highest bin from which on there are m of them
+            // (its lower end less what a rounding may be)
+            s.count(c, own[0].e);
+            s.count(c, own[1].e);
+            for (int i = kCandCap + lane; i < kCandCap + have; i += 32) s.count(c, __uint_as_float(more[i].x));
+            __syncwarp();
+            const uint32_t two = s.hist[c * (kStreamBins / 2) + lane];
+            const int from = (int)bs::incl_scan(__shfl_sync(0xffffffffu, (two & 0xffffu) + (two >> 16), 31 - lane), lane);
+            const int run = __shfl_sync(0xffffffffu, from, 31 - lane);           // in this lane's bins and above
+            const int word = 31 - __clz(__ballot_sync(0xffffffffu, run >= m));
+            const int above = __shfl_sync(0xffffffffu, run - (int)(two & 0xffffu), word);
+            const int bin = 2 * word + (above >= m ? 1 : 0);
+            if (lane == 0) {
+                const int at = atomicAdd(words + 2, 1);
+                next[at] = s.col[c];
+                bound[at] = s.lo[c] + bin / s.scale[c] - (bin > 0 ? 4e-7f : 0.f);
+                bins_of[at] = s.scale[c] * kStreamBins;
+            }
+            continue;
+        }
+        if (lane == 0) exact[atomicAdd(words + 4, 1)] = s.col[c];
+    }
 }
 
 // grid (chunks, units, sweeps of np sources).
 template <int kD>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
+sim_stream_tc(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ SimStreamArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const Dims &d = a.d;
@@ -170,7 +325,7 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
     const int np = a.np, S = a.stages;
     const StreamLayout l = stream_layout<kD>(np, S);
     float *inv_norm = reinterpret_cast<float *>(gen + l.inv_norm);
-    int *src_pos = reinterpret_cast<int *>(gen + l.src_pos), *col = reinterpret_cast<int *>(gen + l.col);
+    int *own_key = reinterpret_cast<int *>(gen + l.own_key), *col = reinterpret_cast<int *>(gen + l.col);
     float *src_inv = reinterpret_cast<float *>(gen + l.src_inv), *theta = reinterpret_cast<float *>(gen + l.theta);
     int *cnt = reinterpret_cast<int *>(gen + l.cnt), *exact = reinterpret_cast<int *>(gen + l.exact);
     int *next = reinterpret_cast<int *>(gen + l.queue);                 // [np] the next sweep's sources,
@@ -192,7 +347,6 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
     const long long source0 = (long long)unit * d.K_src + src0, source_stride = (long long)a.chunks * kCandCap;
     Cand *cand = a.cand + (source0 * a.chunks + chunk) * kCandCap;      // source c's list of this chunk at c * source_stride
     uint32_t *hist = a.cand_hist + source0 * kCandBins;
-    uint2 *spill = a.spill + ((long long)(blockIdx.z * gridDim.y + unit) * a.chunks + chunk) * kStreamSpill;
 
     int n_ahead = 0;
     // barriers for a sweep of n columns (the first: with the keys' norms); those before are at rest
@@ -233,7 +387,7 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
     // rows of sources -> swizzled operand of n rows, `of(r)`: the source of row r or -1
     constexpr int kPieces = kD / 8;
     auto stage_sources = [&](int n, auto of, auto put) {
-        constexpr int kU = 3;                            // pieces in flight per thread: a position, then the row's piece
+        constexpr int kU = 4;                            // pieces in flight per thread: a position, then the row's piece
         for (int i0 = threadIdx.x; i0 - (int)threadIdx.x < n * kPieces; i0 += kU * kStreamThreads) {
             int pos[kU];
             uint4 v[kU];
@@ -265,32 +419,29 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
             }
         }
     };
-    for (int i = threadIdx.x; i < n_src; i += kStreamThreads) {
-        next[i] = i;
-        bound[i] = fmaxf(__ldcg(a.tau + source0 + i), -1.0f);
-        bins_of[i] = kStreamBins / fmaxf(1.0f - bound[i], 1e-6f);
-    }
-    __syncthreads();
     bool ok = true, all_ok = true;
     uint32_t tmem_base = 0u;
     const int ew = warp - 10, quad = warp & 3, et = (int)threadIdx.x - 320;
     const int key_lane = quad * 32 + lane;
     // Sweeps: the first of all sources with the sample's bounds; then of those whose edges were not all kept, with bounds from
-    // the counts of the sweep before.
+    // the counts of the first.  (Each with code of its own: in one loop the first took 3 us more.)
     int n_col = n_src;
-    for (int pass = 0;; ++pass) {
+    auto sweep = [&](auto again) {
+        constexpr int pass = decltype(again)::value;
         const int width = pass == 0 ? np : (n_col + 31) & ~31, bufs = stream_bufs(width), n_slices = width / 32;
-        stage_sources(width, [&](int r) { return r < n_col ? next[r] : -1; }, [&](int r, int pos, float n2) {
+        stage_sources(width, [&](int r) { return r >= n_col ? -1 : pass == 0 ? r : next[r]; }, [&](int r, int pos, float n2) {
             const float norm = fmaxf(sqrtf(n2), kNormEps);
-            src_pos[r] = pos;
+            const bool in = r < n_col;
+            const float least = !in ? 0.f : pass == 0 ? fmaxf(__ldcg(a.tau + source0 + r), -1.0f) : bound[r];
+            own_key[r] = pos < 0 ? -1 : StreamColumns{chunk, a.chunks}.key_of(pos);
             src_inv[r] = 1.0f / norm;
             cnt[r] = 0;
-            col[r] = r < n_col ? next[r] : 0;
-            lo[r] = r < n_col ? bound[r] : 0.f;
-            scale[r] = r < n_col ? bins_of[r] : 0.f;
+            col[r] = !in ? 0 : pass == 0 ? r : next[r];
+            lo[r] = least;
+            scale[r] = pass == 0 ? kStreamBins / fmaxf(1.0f - least, 1e-6f) : in ? bins_of[r] : 0.f;
             // the bound brought to the scale of dot / |k_j|, lowered so that no edge whose cosine rounds up to it is missed
             // (kept negated; an infinite bound would make a difference of infinities)
-            const float q = r < n_col ? ((bound[r] <= -1.0f ? -2.0f : bound[r]) - 2.4e-7f) * norm : 3.0e38f;
+            const float q = in ? ((least <= -1.0f ? -2.0f : least) - 2.4e-7f) * norm : 3.0e38f;
             theta[r] = -(q - fabsf(q) * 3.6e-7f - 1e-30f);
         });
         for (int i = threadIdx.x; i < width * (kStreamBins / 2); i += kStreamThreads) counts[i] = 0u;
@@ -299,7 +450,6 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
         __syncthreads();
         tc_fence_after();
         tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t *>(gen + (s_tmem - base)), 0);
-        const StreamColumns columns{chunk, a.chunks, src_pos, col, cnt, cand, source_stride, hist, spill, words + 3, lo, scale, counts};
         pc.mark();
         if (warp == 0) {
             if (lane == 0) {
@@ -374,23 +524,8 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
             const uint32_t q_first = smem_u32(q0), q_last = q_first + (queue - 1) * kStep;
             uint32_t qa = q_first;
             auto flush = [&]() {
-                const int queued = static_cast<int>((qa - q_first) / kStep);
-#pragma unroll 1
-                for (int k = 0; k < queued; k += 4) {
-                    int c[4], key[4];
-                    float x[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint2 en = q0[min(k + q, queue - 1) * 512];
-                        const bool in = k + q < queued;
-                        c[q] = in ? (int)(en.y >> 16) : -1;
-                        key[q] = (int)(en.y & 0xffffu);
-                        x[q] = __uint_as_float(en.x) * src_inv[max(c[q], 0)];
-                    }
-                    stream_list<4>(c, key, x, columns);
-                }
+                stream_flush<kD>(a, gen, static_cast<int>((qa - q_first) / kStep), pass);
                 qa = q_first;
-                __syncwarp();
             };
             int i = set / n_slices, sl = set % n_slices;
             while (i < n_local) {
@@ -454,18 +589,7 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
                     // a key close to many sources: what the queues held before this slice, then the slice without queues
                     qa = before;
                     flush();
-#pragma unroll 1
-                    for (int c0 = col0; c0 < col0 + 32 && c0 < n_col; c0 += 8) {
-                        uint32_t r[8];
-                        __syncwarp();
-                        tmem_ld8_issue(lane_addr + buf * width + c0, r);
-                        tmem_ld_fence(r);
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            stream_list_column(c0 + q, key, fmaf(__uint_as_float(r[q]), inv, theta[c0 + q]) > 0.f,
-                                               __uint_as_float(r[q]) * inv * src_inv[c0 + q], columns);
-                    }
-                    __syncwarp();
+                    stream_slice<kD>(a, gen, lane_addr + buf * width + col0, col0, n_col, key, inv, pass);
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -490,86 +614,20 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
         }
         const int n_spilled = min(*reinterpret_cast<volatile int *>(words + 3), kStreamSpill);
         if (n_spilled > 0 && all_ok) {
-            uint2 *sorted = reinterpret_cast<uint2 *>(gen + l.stage);           // [kStreamSpill]
-            int *kept = reinterpret_cast<int *>(sorted + kStreamSpill), *end = kept + np;       // [np] a column's edges, and their end
-            for (int c = threadIdx.x; c < width; c += kStreamThreads) kept[c] = 0;
-            __syncthreads();
-            for (int i = threadIdx.x; i < n_spilled; i += kStreamThreads) atomicAdd(kept + (__ldcg(&spill[i].y) >> 16), 1);
-            __syncthreads();
-            if (warp == 0) {
-                int run = 0;
-                for (int c0 = 0; c0 < width; c0 += 32) {
-                    const int mine = kept[c0 + lane], incl = (int)bs::incl_scan((uint32_t)mine, lane);
-                    end[c0 + lane] = run + incl - mine;
-                    run += __shfl_sync(0xffffffffu, incl, 31);
-                }
-            }
-            __syncthreads();
-            for (int i = threadIdx.x; i < n_spilled; i += kStreamThreads) {
-                const uint2 en = __ldcg(spill + i);
-                sorted[atomicAdd(end + (en.y >> 16), 1)] = make_uint2(en.x, en.y & 0xffffu);
-            }
-            __syncthreads();
-            // A source with more edges than slots, by a warp: those that reach a bound at which a list holds them.  Where some
-            // were not kept, another sweep with a bound from the counts; where too many tie, the exact search.
-            for (int c = warp; c < n_col; c += kStreamThreads / 32) {
-                const int excess = cnt[c] - kCandCap, have = kept[c];
-                if (excess <= 0) continue;
-                Cand *list = cand + col[c] * source_stride;
-                uint32_t *bins = hist + col[c] * kCandBins;
-                Cand own[2];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int2 raw = __ldcg(reinterpret_cast<const int2 *>(list + q * 32 + lane));
-                    own[q] = Cand{__int_as_float(raw.x), raw.y};
-                    atomicAdd(bins + cand_bin(own[q].e), 0xffffffffu);          // (counted anew)
-                }
-                const uint2 *more = sorted + end[c] - have - kCandCap;
-                if (have == excess) {
-                    float reached;
-                    const int n = warp_list_top<false>(kCandCap + have, d.m, -1.0f,
-                        [&](int i) { return i < 32 ? own[0].e : i < 64 ? own[1].e : __uint_as_float(more[i].x); },
-                        [&](int at, float e, int i) {
-                            list[at] = Cand{e, i < 32 ? own[0].j : i < 64 ? own[1].j : columns.position((int)more[i].y)};
-                            atomicAdd(bins + cand_bin(e), 1u);
-                        }, &reached);
-                    if (n >= 0) {
-                        for (int q = n + lane; q < kCandCap; q += 32) list[q] = Cand{kCandEmpty, -1};
-                        continue;
-                    }
-                } else if (pass + 1 < kStreamPasses) {
-                    // all of the column's edges counted, two bins per lane: the highest bin from which on there are m of them
-                    // (its lower end less what a rounding may be)
-                    columns.count(c, own[0].e);
-                    columns.count(c, own[1].e);
-                    for (int i = kCandCap + lane; i < kCandCap + have; i += 32) columns.count(c, __uint_as_float(more[i].x));
-                    __syncwarp();
-                    const uint32_t two = counts[c * (kStreamBins / 2) + lane];
-                    const int from = (int)bs::incl_scan(__shfl_sync(0xffffffffu, (two & 0xffffu) + (two >> 16), 31 - lane), lane);
-                    const int run = __shfl_sync(0xffffffffu, from, 31 - lane);           // in this lane's bins and above
-                    const int word = 31 - __clz(__ballot_sync(0xffffffffu, run >= d.m));
-                    const int above = __shfl_sync(0xffffffffu, run - (int)(two & 0xffffu), word);
-                    const int bin = 2 * word + (above >= d.m ? 1 : 0);
-                    if (lane == 0) {
-                        const int at = atomicAdd(words + 2, 1);
-                        next[at] = col[c];
-                        bound[at] = lo[c] + bin / scale[c] - (bin > 0 ? 4e-7f : 0.f);
-                        bins_of[at] = scale[c] * kStreamBins;
-                    }
-                    continue;
-                }
-                if (lane == 0) exact[atomicAdd(words + 4, 1)] = col[c];
-            }
+            stream_resolve(stream_columns<kD>(a, gen, pass), reinterpret_cast<uint2 *>(gen + l.stage), next, exact, words, np, n_col, d.m, pass == 1);
         }
         __syncthreads();
         n_col = *reinterpret_cast<volatile int *>(words + 2);
-        if (n_col == 0) break;
+    };
+    sweep(std::integral_constant<int, 0>{});
+    if (n_col > 0) {
         n_ahead = 0;
         __syncthreads();
         if (threadIdx.x == 0) {
             words[2] = words[3] = 0;
             init_barriers((n_col + 31) & ~31, false);
         }
+        sweep(std::integral_constant<int, 1>{});
     }
     const int n_exact = *reinterpret_cast<volatile int *>(words + 4);
     if (n_exact > 0) {
@@ -583,7 +641,7 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
     for (int f0 = 0; f0 < n_exact && alive; f0 += 16) {
         const int nf = min(16, n_exact - f0);
         stage_sources(16, [&](int r) { return r < nf ? exact[f0 + r] : -1; }, [&](int r, int pos, float n2) {
-            src_pos[r] = pos;
+            own_key[r] = pos;                       // (here its position)
             src_inv[r] = 1.0f / fmaxf(sqrtf(n2), kNormEps);
         });
         fence_proxy_async();
@@ -640,7 +698,7 @@ sim_stream_tc(const __grid_constant__ CUtensorMap tmK, SimStreamArgs a)
                             const int g = h0 + q;
                             if (g >= g0 && g < min(nf, g0 + round)) {
                                 const float e = clamped_edge(__uint_as_float(r[q]) * inv * src_inv[g]);
-                                cosines[(g - g0) * keys + key] = tile_of(i) * kTileKeys + key_lane == src_pos[g] ? kCandEmpty : e;
+                                cosines[(g - g0) * keys + key] = tile_of(i) * kTileKeys + key_lane == own_key[g] ? kCandEmpty : e;
                             }
                         }
                     }
